@@ -10,19 +10,16 @@
 //   Division is monotone (correctly rounded, positive operands), so
 //   kv / min(a, b) == max(kv / a, kv / b) exactly; each block therefore divides once per
 //   (instance, level) it touches and the per-pair work is a tier test, a max and an
-//   add.  Each block owns one snapshot and 1024 consecutive decode ranks (4 per
-//   thread, kept in registers) and walks every prefill rank, staged 1024 at a time in
-//   shared memory; every warp store writes 512 contiguous bytes of a C row with an
-//   evict-first hint.  No scratch memory: the quotients of the block's instances are
-//   recomputed from the utilisation row.
+//   add.  No scratch memory: the quotients of the block's instances are recomputed from
+//   the utilisation row.  When the call also asks for UB, the blocks that hold an
+//   instance's bottlenecks first write them, so both outputs take one launch.
 #include "netkv_internal.cuh"
 
 namespace {
 
 constexpr int kBlock = 256;
 constexpr int kPerThread = 4;
-constexpr int kDChunk = kBlock * kPerThread;
-constexpr int kPTile = 1024;
+constexpr int kPTile = 256;  // prefill ranks staged at a time, one a thread
 
 __device__ __forceinline__ bool util_ok(float u) { return u >= 0.0f && u < 1.0f; }
 
@@ -72,54 +69,90 @@ __global__ void __launch_bounds__(kBlock) level_bottleneck_kernel(
   }
 }
 
+// A block takes one snapshot, the prefill ranks [y * p_span, (y + 1) * p_span) and
+// 4 * tx decode ranks: tx = 2^log2_tx thread columns own four decodes each, kept in
+// registers, and the 256 / tx thread rows walk the staged prefill ranks side by side, so
+// that small pools fill a block too.  Bound by the writes of C: a warp stores 512
+// contiguous bytes of a row (kVec), or four times 128 where rows are not 16-byte
+// aligned, with an evict-first hint.  Instances are numbered pod by pod, so a prefill
+// whose pod lies outside the pods of the thread's decodes is of tier 3 with all of them:
+// that test replaces four tier tests and the selections by tier for all but the few
+// pairs that share a pod (issue slots: about 20 instructions per four pairs, not 80).
 // util_down: the decode side's rows (the downward utilisations of directed links; the
 // same pointer as util for undirected links).
-template <bool kVec, bool kTier = false>
+template <bool kVec, bool kTier>
 __global__ void __launch_bounds__(kBlock) oracle_build_kernel(
     TopoArgs t, const float* __restrict__ util, const float* __restrict__ util_down,
-    uint32_t n_snap, float kv, float* __restrict__ C, int* status) {
+    uint32_t n_snap, float kv, float* __restrict__ C, float4* __restrict__ UB, uint32_t p_span,
+    uint32_t log2_tx, int* status) {
   __shared__ float4 s_q[kPTile];
   __shared__ uint4 s_l[kPTile];
+  __shared__ float2 s_far[kPTile];  // tier-3 quotient and pod link
   const float4 lat = make_float4(t.lat[0], t.lat[1], t.lat[2], t.lat[3]);
-  const uint32_t d0 = blockIdx.x * kDChunk + threadIdx.x * kPerThread;
+  const uint32_t tx = 1u << log2_tx, ty = kBlock >> log2_tx;
+  const uint32_t col = threadIdx.x & (tx - 1), row = threadIdx.x >> log2_tx;
+  // decode of slot j: d0 + j * dstep
+  const uint32_t dstep = kVec ? 1u : min(tx, 32u);
+  const uint32_t d0 = blockIdx.x * (kPerThread * tx) +
+                      (kVec ? col * kPerThread
+                            : col / dstep * (kPerThread * dstep) + col % dstep);
+  const uint32_t p_beg = blockIdx.y * p_span, p_end = min(t.P, p_beg + p_span);
 
-  for (uint32_t s = blockIdx.y; s < n_snap; s += gridDim.y) {
-    const float* row = util + (uint64_t)s * t.n_links;
-    const float* row_d = util_down + (uint64_t)s * t.n_links;
+  for (uint32_t s = blockIdx.z; s < n_snap; s += gridDim.z) {
+    const float* row_u = util + (uint64_t)s * (kTier ? 4u : t.n_links);
+    const float* row_d = util_down + (uint64_t)s * (kTier ? 4u : t.n_links);
     uint4 ld[kPerThread];
     float4 qd[kPerThread];
+    uint32_t pod_lo = 0xffffffffu, pod_hi = 0u;
 #pragma unroll
     for (int j = 0; j < kPerThread; ++j) {
-      const uint32_t d = d0 + j;
+      const uint32_t d = d0 + j * dstep;
+      ld[j] = make_uint4(0, 0, 0, 0);
+      qd[j] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (d < t.D) {
-        ld[j] = __ldg(t.links + __ldg(t.dec + d));
-        qd[j] = quotients(kv, kTier ? tier_bandwidths(t, util + (uint64_t)s * 4, status)
-                                    : level_bottlenecks(t, row_d, ld[j], status));
-      } else {
-        ld[j] = make_uint4(0, 0, 0, 0);
-        qd[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const uint32_t inst = __ldg(t.dec + d);
+        ld[j] = __ldg(t.links + inst);
+        const float4 b = kTier ? tier_bandwidths(t, row_u, status)
+                               : level_bottlenecks(t, row_d, ld[j], status);
+        if (UB && blockIdx.y == 0 && row == 0) UB[(uint64_t)s * t.N + inst] = b;
+        qd[j] = quotients(kv, b);
+        pod_lo = min(pod_lo, ld[j].w);
+        pod_hi = max(pod_hi, ld[j].w);
       }
     }
     float* crow = C + (uint64_t)s * t.P * t.D;
-    for (uint32_t p0 = 0; p0 < t.P; p0 += kPTile) {
-      const uint32_t np = min((uint32_t)kPTile, t.P - p0);
+    for (uint32_t p0 = p_beg; p0 < p_end; p0 += kPTile) {
+      const uint32_t np = min((uint32_t)kPTile, p_end - p0);
       __syncthreads();
-      for (uint32_t k = threadIdx.x; k < np; k += kBlock) {
-        const uint4 l = __ldg(t.links + __ldg(t.pre + p0 + k));
-        s_l[k] = l;
-        s_q[k] = quotients(kv, kTier ? tier_bandwidths(t, util + (uint64_t)s * 4, status)
-                                     : level_bottlenecks(t, row, l, status));
+      if (threadIdx.x < np) {
+        const uint32_t inst = __ldg(t.pre + p0 + threadIdx.x);
+        const uint4 l = __ldg(t.links + inst);
+        const float4 b = kTier ? tier_bandwidths(t, row_u, status)
+                               : level_bottlenecks(t, row_u, l, status);
+        if (UB && blockIdx.x == 0) UB[(uint64_t)s * t.N + inst] = b;
+        const float4 q = quotients(kv, b);
+        s_l[threadIdx.x] = l;
+        s_q[threadIdx.x] = q;
+        s_far[threadIdx.x] = make_float2(q.w, __uint_as_float(l.w));
       }
       __syncthreads();
       if (d0 >= t.D) continue;
-      for (uint32_t k = 0; k < np; ++k) {
-        const float4 qp = s_q[k];
-        const uint4 lp = s_l[k];
+#pragma unroll 4
+      for (uint32_t k = row; k < np; k += ty) {
+        const float2 far = s_far[k];
+        const uint32_t pod = __float_as_uint(far.y);
         float c[kPerThread];
+        if (pod < pod_lo || pod > pod_hi) {
 #pragma unroll
-        for (int j = 0; j < kPerThread; ++j) {
-          const int tau = tier_of(lp, ld[j]);
-          c[j] = fmaxf(pick4(qp, tau), pick4(qd[j], tau)) + pick4(lat, tau);
+          for (int j = 0; j < kPerThread; ++j) c[j] = fmaxf(far.x, qd[j].w) + lat.w;
+        } else {
+          const float4 qp = s_q[k];
+          const uint4 lp = s_l[k];
+#pragma unroll
+          for (int j = 0; j < kPerThread; ++j) {
+            const int tau = tier_of(lp, ld[j]);
+            c[j] = fmaxf(pick4(qp, tau), pick4(qd[j], tau)) + pick4(lat, tau);
+          }
         }
         float* out = crow + (uint64_t)(p0 + k) * t.D + d0;
         if (kVec) {
@@ -127,7 +160,7 @@ __global__ void __launch_bounds__(kBlock) oracle_build_kernel(
         } else {
 #pragma unroll
           for (int j = 0; j < kPerThread; ++j)
-            if (d0 + j < t.D) __stcs(out + j, c[j]);
+            if (d0 + j * dstep < t.D) __stcs(out + j * dstep, c[j]);
         }
       }
     }
@@ -149,7 +182,7 @@ static netkv_status oracle_build(netkv_topology_t topo, const float* d_util, con
   if (n_snap == 0) return NETKV_OK;
   const TopoArgs t = topo_args(topo);
   cudaStream_t s = (cudaStream_t)stream;
-  if (d_UB) {
+  if (!d_C) {
     const uint64_t total = (uint64_t)n_snap * t.N;
     const uint64_t blocks = (total + kBlock - 1) / kBlock;
     const unsigned grid = (unsigned)(blocks < (1u << 20) ? blocks : (1u << 20));
@@ -162,26 +195,45 @@ static netkv_status oracle_build(netkv_topology_t topo, const float* d_util, con
     else
       level_bottleneck_kernel<false><<<grid, kBlock, 0, s>>>(
           t, d_util, d_util, n_snap, reinterpret_cast<float4*>(d_UB), d_status);
-    if (netkv_launch_status() != NETKV_OK) return NETKV_ECUDA;
+    return netkv_launch_status();
   }
-  if (d_C) {
-    const dim3 grid((t.D + kDChunk - 1) / kDChunk, n_snap < 65535u ? n_snap : 65535u);
-    const bool vec = (t.D % 4 == 0) && aligned_to(d_C, 16);
-    if (mode == kTiers && vec)
-      oracle_build_kernel<true, true><<<grid, kBlock, 0, s>>>(t, d_util, d_util, n_snap,
-                                                              (float)kv_bytes, d_C, d_status);
-    else if (mode == kTiers)
-      oracle_build_kernel<false, true><<<grid, kBlock, 0, s>>>(t, d_util, d_util, n_snap,
-                                                               (float)kv_bytes, d_C, d_status);
-    else if (vec)
-      oracle_build_kernel<true><<<grid, kBlock, 0, s>>>(t, d_util, d_util_down, n_snap,
-                                                        (float)kv_bytes, d_C, d_status);
-    else
-      oracle_build_kernel<false><<<grid, kBlock, 0, s>>>(t, d_util, d_util_down, n_snap,
-                                                         (float)kv_bytes, d_C, d_status);
-    if (netkv_launch_status() != NETKV_OK) return NETKV_ECUDA;
+  // Thread columns to cover D four decodes a thread, at most 256; then the prefill ranks are
+  // split until the card has kBlocksPerSm blocks an SM.  A block's set-up (16 gathers
+  // and divisions a thread) is worth at least kMinRows prefill ranks per thread row.
+  // 2,048 x 8,192 pairs with UB: one snapshot, 26.6 us a call (499 us as 8 blocks of all
+  // prefill ranks); 32 snapshots, 323 us = 6.65 TB/s (539 us as 256 blocks).
+  constexpr uint32_t kBlocksPerSm = 8, kMinRows = 16;
+  uint32_t log2_tx = 0;
+  while (log2_tx < 8 && (uint32_t)kPerThread << log2_tx < t.D) ++log2_tx;
+  const uint32_t gx = (t.D + (kPerThread << log2_tx) - 1) / (kPerThread << log2_tx);
+  const uint32_t gz = n_snap < 65535u ? n_snap : 65535u;
+  int dev = 0, sms = 0;
+  NETKV_CUDA_TRY(cudaGetDevice(&dev));
+  NETKV_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const uint64_t have = (uint64_t)gx * gz, want = (uint64_t)sms * kBlocksPerSm;
+  const uint32_t rows = kMinRows * (kBlock >> log2_tx);
+  const uint32_t most = (t.P + rows - 1) / rows;
+  const uint64_t need = (want + have - 1) / have;
+  uint32_t gy = need < most ? (uint32_t)need : most;
+  if (gy > 65535u) gy = 65535u;
+  const uint32_t p_span = (t.P + gy - 1) / gy;
+  const dim3 grid(gx, (t.P + p_span - 1) / p_span, gz);
+  const bool vec = (t.D % 4 == 0) && aligned_to(d_C, 16);
+  const float* down = mode == kDirected ? d_util_down : d_util;
+  float4* ub = reinterpret_cast<float4*>(d_UB);
+#define NETKV_BUILD(VEC, TIER)                                                             \
+  oracle_build_kernel<VEC, TIER><<<grid, kBlock, 0, s>>>(t, d_util, down, n_snap,          \
+                                                         (float)kv_bytes, d_C, ub, p_span, \
+                                                         log2_tx, d_status)
+  if (mode == kTiers) {
+    if (vec) NETKV_BUILD(true, true);
+    else NETKV_BUILD(false, true);
+  } else {
+    if (vec) NETKV_BUILD(true, false);
+    else NETKV_BUILD(false, false);
   }
-  return NETKV_OK;
+#undef NETKV_BUILD
+  return netkv_launch_status();
 }
 
 extern "C" netkv_status netkv_oracle_build(netkv_topology_t topo, const float* d_util,
