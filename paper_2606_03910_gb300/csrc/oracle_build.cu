@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(kBlock) level_bottleneck_kernel(
 // util_down: the decode side's rows (the downward utilisations of directed links; the
 // same pointer as util for undirected links).
 template <bool kVec, bool kTier>
-__global__ void __launch_bounds__(kBlock) oracle_build_kernel(
+__global__ void __launch_bounds__(kBlock, 4) oracle_build_kernel(
     TopoArgs t, const float* __restrict__ util, const float* __restrict__ util_down,
     uint32_t n_snap, float kv, float* __restrict__ C, float4* __restrict__ UB, uint32_t p_span,
     uint32_t log2_tx, int* status) {
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kBlock) oracle_build_kernel(
       }
       __syncthreads();
       if (d0 >= t.D) continue;
-#pragma unroll 4
+#pragma unroll 2
       for (uint32_t k = row; k < np; k += ty) {
         const float2 far = s_far[k];
         const uint32_t pod = __float_as_uint(far.y);
@@ -200,9 +200,10 @@ static netkv_status oracle_build(netkv_topology_t topo, const float* d_util, con
   // Thread columns to cover D four decodes a thread, at most 256; then the prefill ranks are
   // split until the card has kBlocksPerSm blocks an SM.  A block's set-up (16 gathers
   // and divisions a thread) is worth at least kMinRows prefill ranks per thread row.
-  // 2,048 x 8,192 pairs with UB: one snapshot, 26.6 us a call (499 us as 8 blocks of all
-  // prefill ranks); 32 snapshots, 323 us = 6.65 TB/s (539 us as 256 blocks).
-  constexpr uint32_t kBlocksPerSm = 8, kMinRows = 16;
+  // 2,048 x 8,192 pairs with UB (kernel time): one snapshot, 21.2 us (24.5 us at 3 blocks
+  // resident an SM; 491 us as 8 blocks of all prefill ranks); 32 snapshots, 323 us = 6.65
+  // TB/s (528 us as 256 blocks; 387 us at 4 blocks an SM).
+  constexpr uint32_t kBlocksPerSm = 16, kMinRows = 16;
   uint32_t log2_tx = 0;
   while (log2_tx < 8 && (uint32_t)kPerThread << log2_tx < t.D) ++log2_tx;
   const uint32_t gx = (t.D + (kPerThread << log2_tx) - 1) / (kPerThread << log2_tx);

@@ -10,9 +10,8 @@
 //   hash table  open addressing, 16-byte slots {hash, position in the run array}.
 // Caches are filled with whole prefixes of chains, so a cached prefix sits in the run
 // array as a contiguous run in chain order.
-//   cache_build_kernel: one CTA per index; it walks the lists in order in chunks of 1024
-//   keys, claims new hashes with atomicCAS, numbers them with a block-wide scan and
-//   appends them to the run array, and ORs each decode's bit into the hashes it lists.
+// The build numbers the distinct hashes of an index by their first position in its lists
+// (see "Cache build" below).
 //
 // Match.  One warp per (request, decode group).  The warp looks up the block at the
 // current position in the hash table (one random access), then compares the chain with
@@ -73,38 +72,372 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t flag, uint32_t* warp_sum
   return warp_sums[wid] + in_warp;
 }
 
-__global__ void __launch_bounds__(kBuildBlock) cache_build_kernel(
-    void* __restrict__ index, uint32_t n_sets, uint32_t D, uint32_t log2_cap,
-    const uint64_t* __restrict__ keys, const uint64_t* __restrict__ key_off, int* status) {
+// ---- Cache build -------------------------------------------------------------------
+// The lists of an index's decodes, one after another, are its elements 0 .. T - 1.  A hash's
+// run position is the number of distinct hashes that appear before it, so cached prefixes
+// stay contiguous.  Every pass is parallel over the elements or slots of all indices:
+//   insert  each element claims its hash's slot and keeps the first position there
+//           (atomicMax on its complement, since a cleared slot holds 0), unless it is seen
+//           to repeat an earlier element: a warp looks one hash up and follows the list
+//           from its first position;
+//   mark    each occupied slot sets the bit of its first position in a bitmap of T bits,
+//           which borrows the index's run masks;
+//   count   one block per index: how many bits are set before every 256 of them, at the
+//           end of the index's run keys, and the number of distinct hashes n;
+//   place   each occupied slot takes its position's rank as its run position and writes
+//           its run key;
+//   wipe    the bitmap and the counts are cleared;
+//   masks   each element adds its decode's bit to its hash's run mask; a warp looks one
+//           hash up and follows the run for the next ones.
+// Bound by random accesses to the slots (one sector per lane and probe), which stay in L2
+// where the blocks in flight cover few indices: kPartsMax blocks per index keep them so.
+// 256 decodes of 50,000 keys (4 indices, 12.8 M elements): 0.28 ms, insert 0.125 and masks
+// 0.060 of it; one block per index walking its lists in chunks of 1,024 took 14.85 ms.
+// An index whose lists are too long for the borrowed memory (T over 8 bits per mask byte,
+// lists that repeat hashes many times) or whose table is nearly full is built by
+// build_serial_kernel instead: one block walks the lists in chunks.
+struct GroupLists {
+  uint64_t pre[kGroup + 1];  // elements before each decode's list
+  uint64_t beg[kGroup];      // where the list starts in the keys
+  bool in_order;             // the lists follow one another in the keys
+};
+constexpr int kPassBlock = 256;
+constexpr uint32_t kPartsMax = 512;
+
+struct BuildArgs {
+  void* index;
+  uint64_t n_index;
+  uint32_t D, log2_cap, parts;
+  const uint64_t* keys;
+  const uint64_t* key_off;
+  int* status;
+};
+
+// The lists of index idx, by the whole block; ends with a barrier.
+__device__ __forceinline__ void load_lists(GroupLists& L, const BuildArgs& a, uint64_t idx,
+                                           bool report) {
+  const uint32_t n_dgroups = (a.D + kGroup - 1) / kGroup;
+  const uint64_t g = idx / n_dgroups;
+  const uint32_t q0 = (uint32_t)(idx - g * n_dgroups) * kGroup;
+  const uint32_t ng = min(kGroup, a.D - q0);
+  __syncthreads();  // the lists of the index before are no longer read
+  if (threadIdx.x < 32) {
+    const uint32_t lane = threadIdx.x;
+    uint64_t len[2];
+    bool bad = false;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint32_t j = 2 * lane + h;
+      len[h] = 0;
+      if (j < ng) {
+        const uint64_t t = g * a.D + q0 + j;
+        const uint64_t beg = __ldg(a.key_off + t), end = __ldg(a.key_off + t + 1);
+        if (end >= beg) len[h] = end - beg;
+        else bad = true;
+        L.beg[j] = beg;
+      }
+    }
+    if (bad && report) flag_status(a.status, NETKV_DEV_ERANGE);
+    const bool any_bad = __any_sync(0xffffffffu, bad);
+    uint64_t x = len[0] + len[1];
+    const uint64_t own = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= (uint32_t)o) x += y;
+    }
+    L.pre[2 * lane] = x - own;
+    L.pre[2 * lane + 1] = x - own + len[0];
+    if (lane == 31) L.pre[kGroup] = x;
+    if (lane == 0) L.in_order = !any_bad;
+  }
+  __syncthreads();
+}
+
+// Words of the counts of an index: one per 256 elements, then n; they end the run keys.
+__device__ __forceinline__ uint64_t count_words(uint64_t T) { return (T + 255) / 256 + 1; }
+__device__ __forceinline__ uint32_t* build_counts(const IndexView& v, uint64_t cap, uint64_t T) {
+  return reinterpret_cast<uint32_t*>(v.keys + cap) - count_words(T);
+}
+// Whether the bitmap fits the masks, and the counts the run keys.
+__device__ __forceinline__ bool lists_fit(uint64_t T, uint64_t cap, uint32_t mask_bytes) {
+  return T <= 8u * mask_bytes * cap && count_words(T) <= 2 * cap;
+}
+__device__ __forceinline__ bool counts_fit(uint64_t n, uint64_t T, uint64_t cap) {
+  return 2 * n + count_words(T) <= 2 * cap;
+}
+
+__global__ void __launch_bounds__(kPassBlock) build_insert_kernel(BuildArgs a) {
+  __shared__ GroupLists L;
+  const uint64_t cap = 1ull << a.log2_cap, mask = cap - 1;
+  const uint32_t mb = mask_bytes_of(a.D), lane = threadIdx.x & 31;
+  constexpr uint32_t kRow = 64;
+  for (uint64_t b = blockIdx.x; b < a.n_index * a.parts; b += gridDim.x) {
+    const uint64_t idx = b / a.parts;
+    const uint32_t part = (uint32_t)(b - idx * a.parts);
+    load_lists(L, a, idx, part == 0);
+    const uint64_t T = L.pre[kGroup];
+    if (!lists_fit(T, cap, mb)) continue;
+    IndexSlot* hash = index_view(a.index, idx, a.log2_cap, mb).hash;
+    // the key of element e, e < T
+    auto key_of = [&](uint64_t e) -> unsigned long long {
+      if (L.in_order) return __ldg(a.keys + L.beg[0] + e);
+      uint32_t d = 0;
+      while (e >= L.pre[d + 1]) ++d;
+      return __ldg(a.keys + L.beg[d] + (e - L.pre[d]));
+    };
+    // warps take kRow consecutive elements; the warps of all blocks pass over the lists
+    // together, so that most elements meet an earlier list's entries in the table (rows of
+    // 32, 64, 128 and 256 elements: 135, 125, 126 and 132 us)
+    for (uint64_t row = (uint64_t)part * (kPassBlock / 32) + (threadIdx.x >> 5); row * kRow < T;
+         row += (uint64_t)a.parts * (kPassBlock / 32)) {
+      uint64_t f = kNotFound;  // an earlier element that may equal lane 0's
+      for (uint64_t e0 = row * kRow; e0 < min(T, (row + 1) * kRow); e0 += 32) {
+        const uint64_t e = e0 + lane;
+        const unsigned long long key = e < T ? key_of(e) : 0ull;
+        if (e < T && key == 0ull) flag_status(a.status, NETKV_DEV_EDOMAIN);
+        if (f == kNotFound) {
+          if (lane == 0 && key != 0ull) {
+            uint64_t slot = home_slot(key, a.log2_cap);
+            for (uint64_t step = 0; step < cap; ++step) {
+              const ulonglong2 s = __ldcg(reinterpret_cast<const ulonglong2*>(hash + slot));
+              if (s.x == key && s.y != 0ull) f = ~s.y;
+              if (s.x == key || s.x == 0ull) break;
+              slot = (slot + 1) & mask;
+            }
+          }
+          f = __shfl_sync(0xffffffffu, f, 0);
+        }
+        // an element that repeats an earlier one needs no slot: the earlier one, or the
+        // first of its kind, takes care of it
+        const bool repeat = f < e0 && key != 0ull && key_of(f + lane) == key;
+        if (key != 0ull && !repeat) {
+          uint64_t slot = home_slot(key, a.log2_cap);
+          bool placed = false;
+          for (uint64_t step = 0; step < cap; ++step) {
+            const ulonglong2 s = __ldcg(reinterpret_cast<const ulonglong2*>(hash + slot));
+            unsigned long long k = s.x;
+            if (k == 0ull) {
+              const unsigned long long prev = atomicCAS(&hash[slot].key, 0ull, key);
+              k = prev == 0ull ? key : prev;
+            }
+            if (k == key) {
+              if (s.x != key || s.y < ~e) atomicMax(&hash[slot].pos, (unsigned long long)~e);
+              placed = true;
+              break;
+            }
+            slot = (slot + 1) & mask;
+          }
+          if (!placed) flag_status(a.status, NETKV_DEV_EFULL);
+        }
+        f = __ballot_sync(0xffffffffu, repeat) >> 31 ? f + 32 : kNotFound;
+      }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kPassBlock) build_mark_kernel(BuildArgs a) {
+  __shared__ GroupLists L;
+  const uint64_t cap = 1ull << a.log2_cap;
+  const uint32_t mb = mask_bytes_of(a.D);
+  for (uint64_t b = blockIdx.x; b < a.n_index * a.parts; b += gridDim.x) {
+    const uint64_t idx = b / a.parts;
+    const uint32_t part = (uint32_t)(b - idx * a.parts);
+    load_lists(L, a, idx, false);
+    if (!lists_fit(L.pre[kGroup], cap, mb)) continue;
+    const IndexView v = index_view(a.index, idx, a.log2_cap, mb);
+    uint32_t* bits = reinterpret_cast<uint32_t*>(v.masks);
+    for (uint64_t s = (uint64_t)part * kPassBlock + threadIdx.x; s < cap;
+         s += (uint64_t)a.parts * kPassBlock) {
+      const ulonglong2 x = __ldcg(reinterpret_cast<const ulonglong2*>(v.hash + s));
+      if (x.x != 0ull) atomicOr(bits + (~x.y >> 5), 1u << (uint32_t)(~x.y & 31u));
+    }
+  }
+}
+
+// Bits set in the 256-bit group i of a bitmap.  The bitmap starts on a 16-byte boundary, and
+// its last group lies inside the index: masks and padding, cleared past the last element.
+__device__ __forceinline__ uint32_t bits_of(const uint4* __restrict__ bits, uint64_t i) {
+  const uint4 x = __ldcg(bits + 2 * i), y = __ldcg(bits + 2 * i + 1);
+  return __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w) + __popc(y.x) + __popc(y.y) +
+         __popc(y.z) + __popc(y.w);
+}
+
+__global__ void __launch_bounds__(kBuildBlock) build_count_kernel(BuildArgs a) {
+  __shared__ GroupLists L;
+  __shared__ uint32_t warp_sums[2][32];
+  const uint64_t cap = 1ull << a.log2_cap;
+  const uint32_t mb = mask_bytes_of(a.D), lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (uint64_t idx = blockIdx.x; idx < a.n_index; idx += gridDim.x) {
+    load_lists(L, a, idx, false);
+    const uint64_t T = L.pre[kGroup];
+    if (!lists_fit(T, cap, mb)) continue;
+    const IndexView v = index_view(a.index, idx, a.log2_cap, mb);
+    uint32_t* counts = build_counts(v, cap, T);
+    const uint4* bits = reinterpret_cast<const uint4*>(v.masks);
+    const uint64_t groups = (T + 255) / 256;
+    uint32_t before = 0;  // bits of the chunks before; n < 2^32 (at most 2^31 slots)
+    uint32_t parity = 0;
+    uint32_t next = threadIdx.x < groups ? bits_of(bits, threadIdx.x) : 0u;
+    for (uint64_t c = 0; c < groups; c += kBuildBlock) {
+      const uint32_t own = next;
+      const uint64_t i = c + threadIdx.x, in_next = i + kBuildBlock;
+      next = in_next < groups ? bits_of(bits, in_next) : 0u;
+      uint32_t in = own;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, in, o);
+        if (lane >= (uint32_t)o) in += y;
+      }
+      if (lane == 31) warp_sums[parity][wid] = in;
+      __syncthreads();  // one barrier a chunk: the sums are double-buffered
+      const uint32_t w = warp_sums[parity][lane];
+      const uint32_t below = __reduce_add_sync(0xffffffffu, lane < wid ? w : 0u);
+      if (i < groups) counts[i] = before + below + in - own;
+      before += __reduce_add_sync(0xffffffffu, w);
+      parity ^= 1u;
+    }
+    if (threadIdx.x == 0) counts[groups] = before;
+  }
+}
+
+__global__ void __launch_bounds__(kPassBlock) build_place_kernel(BuildArgs a) {
+  __shared__ GroupLists L;
+  const uint64_t cap = 1ull << a.log2_cap;
+  const uint32_t mb = mask_bytes_of(a.D);
+  for (uint64_t b = blockIdx.x; b < a.n_index * a.parts; b += gridDim.x) {
+    const uint64_t idx = b / a.parts;
+    const uint32_t part = (uint32_t)(b - idx * a.parts);
+    load_lists(L, a, idx, false);
+    const uint64_t T = L.pre[kGroup];
+    if (!lists_fit(T, cap, mb)) continue;
+    const IndexView v = index_view(a.index, idx, a.log2_cap, mb);
+    const uint32_t* counts = build_counts(v, cap, T);
+    if (!counts_fit(__ldcg(counts + (T + 255) / 256), T, cap)) continue;
+    const uint4* bits = reinterpret_cast<const uint4*>(v.masks);
+    for (uint64_t s = (uint64_t)part * kPassBlock + threadIdx.x; s < cap;
+         s += (uint64_t)a.parts * kPassBlock) {
+      const ulonglong2 x = __ldcg(reinterpret_cast<const ulonglong2*>(v.hash + s));
+      if (x.x == 0ull) continue;
+      const uint64_t e = ~x.y;
+      uint32_t rank = __ldcg(counts + (e >> 8));
+      const uint4 lo = __ldcg(bits + (e >> 8) * 2), hi = __ldcg(bits + (e >> 8) * 2 + 1);
+      const uint32_t word[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+      const uint32_t w = (uint32_t)(e >> 5) & 7u;  // the element's word in its group
+      const uint32_t below = (1u << (uint32_t)(e & 31u)) - 1u;
+#pragma unroll
+      for (uint32_t j = 0; j < 8; ++j)
+        rank += __popc(word[j] & (j < w ? ~0u : j == w ? below : 0u));
+      v.hash[s].pos = rank;
+      v.keys[rank] = x.x;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kPassBlock) build_wipe_kernel(BuildArgs a) {
+  __shared__ GroupLists L;
+  const uint64_t cap = 1ull << a.log2_cap;
+  const uint32_t mb = mask_bytes_of(a.D);
+  for (uint64_t b = blockIdx.x; b < a.n_index * a.parts; b += gridDim.x) {
+    const uint64_t idx = b / a.parts;
+    const uint32_t part = (uint32_t)(b - idx * a.parts);
+    load_lists(L, a, idx, false);
+    const uint64_t T = L.pre[kGroup];
+    if (!lists_fit(T, cap, mb)) continue;
+    const IndexView v = index_view(a.index, idx, a.log2_cap, mb);
+    uint32_t* counts = build_counts(v, cap, T);
+    // another block may have cleared n already: 0 fits, and only an index that fits is
+    // cleared
+    if (!counts_fit(__ldcg(counts + (T + 255) / 256), T, cap)) continue;
+    uint32_t* bits = reinterpret_cast<uint32_t*>(v.masks);
+    const uint64_t words = (T + 31) / 32, all = words + count_words(T);
+    for (uint64_t i = (uint64_t)part * kPassBlock + threadIdx.x; i < all;
+         i += (uint64_t)a.parts * kPassBlock) {
+      if (i < words) bits[i] = 0u;
+      else counts[i - words] = 0u;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kPassBlock) build_masks_kernel(BuildArgs a) {
+  __shared__ GroupLists L;
+  const uint64_t cap = 1ull << a.log2_cap;
+  const uint32_t mb = mask_bytes_of(a.D), lane = threadIdx.x & 31;
+  constexpr uint32_t kRow = 256;  // consecutive elements a warp takes at a time
+  for (uint64_t b = blockIdx.x; b < a.n_index * a.parts; b += gridDim.x) {
+    const uint64_t idx = b / a.parts;
+    const uint32_t part = (uint32_t)(b - idx * a.parts);
+    load_lists(L, a, idx, false);
+    const uint64_t T = L.pre[kGroup];
+    if (!lists_fit(T, cap, mb)) continue;
+    const IndexView v = index_view(a.index, idx, a.log2_cap, mb);
+    if (__ldcg(build_counts(v, cap, T) + (T + 255) / 256) != 0u) continue;  // not cleared: serial
+    uint32_t d = 0;
+    const uint64_t n_warps = (uint64_t)a.parts * (kPassBlock / 32);
+    for (uint64_t row = (uint64_t)part * (kPassBlock / 32) + (threadIdx.x >> 5);
+         row * kRow < T; row += n_warps) {
+      unsigned long long next = kNotFound;  // run position that lane 0's element may have
+      for (uint64_t e0 = row * kRow; e0 < min(T, (row + 1) * kRow); e0 += 32) {
+        const uint64_t e = e0 + lane;
+        unsigned long long key = 0ull;
+        if (e < T) {
+          while (e >= L.pre[d + 1]) ++d;
+          key = __ldcs(a.keys + L.beg[d] + (e - L.pre[d]));
+        }
+        if (next == kNotFound) {
+          if (lane == 0 && key != 0ull) next = lookup(v.hash, key, a.log2_cap, a.status);
+          next = __shfl_sync(0xffffffffu, next, 0);
+        }
+        unsigned long long pos = kNotFound;
+        if (key != 0ull) {
+          const unsigned long long at = next + lane;  // kNotFound + lane wraps: checked below
+          if (next != kNotFound && at < cap && __ldg(v.keys + at) == key) pos = at;
+          else pos = lookup(v.hash, key, a.log2_cap, a.status);
+        }
+        if (pos != kNotFound) run_mask_or(v, pos, 1ull << d);
+        next = __shfl_sync(0xffffffffu, pos, 31);
+        if (next != kNotFound) ++next;
+      }
+    }
+  }
+}
+
+// The indices that the passes above left out: one block each, the lists walked in order in
+// chunks; new hashes are claimed by atomicCAS and numbered by a block scan.
+__global__ void __launch_bounds__(kBuildBlock) build_serial_kernel(BuildArgs a) {
+  __shared__ GroupLists L;
   __shared__ uint32_t warp_sums[32];
   __shared__ uint32_t chunk_new;
-  const uint64_t cap = 1ull << log2_cap, mask = cap - 1;
-  const uint32_t n_dgroups = (D + kGroup - 1) / kGroup;
-  const uint32_t mb = mask_bytes_of(D);
-  const uint64_t n_index = (uint64_t)n_sets * n_dgroups;
-  for (uint64_t idx = blockIdx.x; idx < n_index; idx += gridDim.x) {
-    const uint64_t g = idx / n_dgroups;
-    const uint32_t q = (uint32_t)(idx - g * n_dgroups);
-    const IndexView v = index_view(index, idx, log2_cap, mb);
+  const uint64_t cap = 1ull << a.log2_cap, mask = cap - 1;
+  const uint32_t mb = mask_bytes_of(a.D);
+  for (uint64_t idx = blockIdx.x; idx < a.n_index; idx += gridDim.x) {
+    load_lists(L, a, idx, true);
+    const uint64_t T = L.pre[kGroup];
+    const IndexView v = index_view(a.index, idx, a.log2_cap, mb);
     IndexSlot* hash = v.hash;
+    if (lists_fit(T, cap, mb)) {
+      if (__ldcg(build_counts(v, cap, T) + (T + 255) / 256) == 0u) continue;  // built
+      // the table was nearly full: start over
+      uint4* w = reinterpret_cast<uint4*>(v.hash);
+      __syncthreads();  // every thread has read the count
+      for (uint64_t i = threadIdx.x; i < index_stride(a.log2_cap, mb) / 16; i += kBuildBlock)
+        w[i] = make_uint4(0u, 0u, 0u, 0u);
+      __syncthreads();
+    }
     uint32_t run_len = 0;  // same value in every thread
-    for (uint32_t d = q * kGroup; d < min(D, (q + 1) * kGroup); ++d) {
-      const uint64_t t = g * D + d;
-      const uint64_t beg = __ldg(key_off + t), end = __ldg(key_off + t + 1);
-      if (end < beg) {
-        if (threadIdx.x == 0) flag_status(status, NETKV_DEV_ERANGE);
-        continue;
-      }
-      const unsigned long long bit = 1ull << (d % kGroup);
+    for (uint32_t d = 0; d < kGroup; ++d) {
+      const uint64_t beg = L.beg[d], end = beg + (L.pre[d + 1] - L.pre[d]);
+      if (L.pre[d + 1] == L.pre[d]) continue;
+      const unsigned long long bit = 1ull << d;
       for (uint64_t c = beg; c < end; c += kBuildBlock) {
         const uint64_t j = c + threadIdx.x;
-        unsigned long long key = j < end ? __ldg(keys + j) : 0ull;
-        if (j < end && key == 0ull) flag_status(status, NETKV_DEV_EDOMAIN);
+        unsigned long long key = j < end ? __ldg(a.keys + j) : 0ull;
+        if (j < end && key == 0ull) flag_status(a.status, NETKV_DEV_EDOMAIN);
         bool is_new = false;
         uint64_t slot = 0;
         bool placed = false;
         if (key != 0ull) {
-          slot = home_slot(key, log2_cap);
+          slot = home_slot(key, a.log2_cap);
           for (uint64_t step = 0; step < cap; ++step) {
             const unsigned long long prev = atomicCAS(&hash[slot].key, 0ull, key);
             if (prev == 0ull || prev == key) {
@@ -114,7 +447,7 @@ __global__ void __launch_bounds__(kBuildBlock) cache_build_kernel(
             }
             slot = (slot + 1) & mask;
           }
-          if (!placed) flag_status(status, NETKV_DEV_EFULL);
+          if (!placed) flag_status(a.status, NETKV_DEV_EFULL);
         }
         const uint32_t pos = run_len + block_scan(is_new ? 1u : 0u, warp_sums, &chunk_new);
         if (is_new) {
@@ -798,10 +1131,33 @@ extern "C" netkv_status netkv_cache_build(void* d_index, uint32_t n_sets, uint32
   cudaStream_t s = (cudaStream_t)stream;
   NETKV_CUDA_TRY(cudaMemsetAsync(d_index, 0, netkv_cache_index_bytes(n_sets, D, log2_capacity), s));
   if (!d_keys) return NETKV_OK;
-  const uint64_t n_index = (uint64_t)n_sets * ((D + kGroup - 1) / kGroup);
-  const unsigned grid = (unsigned)(n_index < (1u << 20) ? n_index : (1u << 20));
-  cache_build_kernel<<<grid, kBuildBlock, 0, s>>>(d_index, n_sets, D, log2_capacity, d_keys,
-                                                  d_key_off, d_status);
+  BuildArgs a;
+  a.index = d_index;
+  a.n_index = (uint64_t)n_sets * ((D + kGroup - 1) / kGroup);
+  a.D = D;
+  a.log2_cap = log2_capacity;
+  a.keys = d_keys;
+  a.key_off = d_key_off;
+  a.status = d_status;
+  // blocks per index: one per 2,048 slots, more where the indices alone leave SMs idle
+  int dev = 0, sms = 0;
+  NETKV_CUDA_TRY(cudaGetDevice(&dev));
+  NETKV_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  uint64_t parts = (1ull << log2_capacity) / 2048;
+  const uint64_t fill = ((uint64_t)sms * 8 + a.n_index - 1) / a.n_index;
+  if (parts > kPartsMax) parts = kPartsMax;
+  if (parts < fill) parts = fill;
+  a.parts = (uint32_t)parts;
+  const uint64_t blocks = a.n_index * a.parts;
+  const unsigned grid = (unsigned)(blocks < (1u << 30) ? blocks : (1u << 30));
+  const unsigned per_index = (unsigned)(a.n_index < (1u << 20) ? a.n_index : (1u << 20));
+  build_insert_kernel<<<grid, kPassBlock, 0, s>>>(a);
+  build_mark_kernel<<<grid, kPassBlock, 0, s>>>(a);
+  build_count_kernel<<<per_index, kBuildBlock, 0, s>>>(a);
+  build_place_kernel<<<grid, kPassBlock, 0, s>>>(a);
+  build_wipe_kernel<<<grid, kPassBlock, 0, s>>>(a);
+  build_masks_kernel<<<grid, kPassBlock, 0, s>>>(a);
+  build_serial_kernel<<<per_index, kBuildBlock, 0, s>>>(a);
   return netkv_launch_status();
 }
 
