@@ -194,10 +194,11 @@ netkv_status netkv_cache_build(void* d_index, uint32_t n_sets, uint32_t D,
  *                [d_set_off[g], d_set_off[g+1]); may be NULL when n_sets == 1
  *   d_workspace  NULL, or a device buffer of at least
  *                netkv_prefix_match_workspace_size(R) bytes, 256-byte aligned, owned by
- *                the caller and overwritten by the call.  With a workspace, requests are
- *                grouped by (table set, first block hash); each group's longest chain is
- *                matched in full and the others reuse its answers over their common
- *                prefix (exactly: the result is identical to the NULL-workspace call).
+ *                the caller and overwritten by the call.  For pools of more than 64
+ *                decodes, requests are then grouped by (table set, first block hash); one
+ *                chain of each group is matched in full and the others reuse its answers
+ *                over their common prefix (exactly: the result is identical to the
+ *                NULL-workspace call).  Smaller pools match every chain directly.
  *                Calls that overlap on the GPU need distinct workspaces.
  *   d_M          [R][D] uint16 output
  * A zero hash in a chain sets EDOMAIN and counts as a miss.  A chain longer than 65535

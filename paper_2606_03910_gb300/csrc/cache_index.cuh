@@ -56,17 +56,14 @@ __device__ __forceinline__ IndexView index_view(const void* index, uint64_t idx,
   return v;
 }
 
-// Mask of run position p (read-only path).  kMB: the mask width when the caller knows it
-// at compile time (pools of more than 32 decodes: 8), 0 to read it from the view.
-template <int kMB = 0>
+// Mask of run position p (read-only path), kMB bytes wide.
+template <int kMB>
 __device__ __forceinline__ unsigned long long run_mask(const IndexView& v, uint64_t p) {
-  if (kMB == 8) return __ldg(reinterpret_cast<const unsigned long long*>(v.masks) + p);
-  switch (v.mask_bytes) {
-    case 1: return __ldg(v.masks + p);
-    case 2: return __ldg(reinterpret_cast<const unsigned short*>(v.masks) + p);
-    case 4: return __ldg(reinterpret_cast<const unsigned int*>(v.masks) + p);
-    default: return __ldg(reinterpret_cast<const unsigned long long*>(v.masks) + p);
-  }
+  static_assert(kMB == 1 || kMB == 2 || kMB == 4 || kMB == 8, "mask width");
+  if (kMB == 1) return __ldg(v.masks + p);
+  if (kMB == 2) return __ldg(reinterpret_cast<const unsigned short*>(v.masks) + p);
+  if (kMB == 4) return __ldg(reinterpret_cast<const unsigned int*>(v.masks) + p);
+  return __ldg(reinterpret_cast<const unsigned long long*>(v.masks) + p);
 }
 
 // Adds decode bit `bit` (bit d mod 64 of the group) to the mask of run position p.

@@ -15,39 +15,43 @@
 //
 // Match.  One warp per (request, decode group).  The warp looks up the block at the
 // current position in the hash table (one random access), then compares the chain with
-// the run keys from that position on, 32 blocks per step (coalesced loads of 256 chain
-// bytes, 256 key bytes and 32 .. 256 mask bytes): every block that equals the next run key
-// is cached exactly on the decodes of that position's mask, and one ballot per live decode
-// finds its first missing block.  Where chain and run part, the next block is looked up
-// in the hash table again; a block absent from the table is missing on every decode.
-// The answer never depends on the run order (any key order is exact); the order only
-// decides how many random lookups a chain needs.  A decode leaves once its first miss is
-// known and the warp stops when every decode of the group has missed.
+// the run keys from that position on, 128 blocks per step (coalesced loads of chain, key
+// and mask bytes): every block that equals the next run key is cached exactly on the
+// decodes of that position's mask.  A step whose blocks all match and are cached on every
+// live decode costs one vote; otherwise ballots find each decode's first missing block.
+// Where chain and run part, the next block is looked up in the hash table again; a block
+// absent from the table is missing on every decode.  The answer never depends on the run
+// order (any key order is exact); the order only decides how many lookups a chain needs.
+// A decode leaves once its first miss is known and the warp stops when every decode of the
+// group has missed.
+//   match_kernel: pools of one decode group (D <= 64), and any pool without a workspace.
 //
-// Prefix sharing.  Requests that share leading blocks have the same membership answers
-// on those blocks, so with a workspace the match runs in three steps:
+// Prefix sharing.  Requests that share leading blocks have the same membership answers on
+// those blocks, so for pools of several groups, whose every group would read the chain
+// again, a match with a workspace runs in three steps:
 //   group_insert_kernel / group_resolve_kernel: requests are grouped by (table set,
 //     first block hash) in an open-addressing table; each group's leader is its
 //     longest chain (lowest index among equals); leaders go to a compact list (chains of
-//     2,048 blocks or more first), and each member gets a record of its own and its
-//     leader's chain offsets and lengths.
+//     2,048 blocks or more first).
 //   match_leaders_kernel: leaders (and ungrouped requests) run the full match, one task
 //     per (leader, decode group) taken in order from a counter.
-//   match_members_kernel: a member r with leader L compares chains to get
+//   match_members_wide_kernel: one warp per member r with leader L compares chains to get
 //     lcp = |common prefix of h_r and h_L| (capped at max_d M_L[d] + 1).  For a decode
 //     with M_L[d] < lcp the first missing block of L lies inside the common prefix, so
-//     M_r[d] = M_L[d] exactly; otherwise blocks [0, lcp) are all cached and the walk
-//     resumes at block lcp.  The result equals the full match whatever the grouping.
-//   match_members_wide_kernel: the same for pools of more than one decode group, one
-//     warp per member: the common prefix is read once, the member's row is
-//     min(M_L, lcp) elementwise, and block lcp is probed only in the groups where a
-//     leader hit reaches lcp, up to 32 groups at a time.
+//     M_r[d] = M_L[d] exactly; otherwise blocks [0, lcp) are all cached.  So the member's
+//     row is min(M_L, lcp) elementwise, and block lcp is probed only in the groups where a
+//     leader hit reaches lcp, up to 32 groups at a time.  The result equals the full match
+//     whatever the grouping.
+#include <algorithm>
+#include <type_traits>
+
 #include "cache_index.cuh"
 
 namespace {
 
 constexpr int kBuildBlock = 1024;
 constexpr int kMatchBlock = 256;
+constexpr uint32_t kNoRun = 0xffffffffu;  // no run position (they are at most 2^31)
 // Exclusive scan of one flag per thread over a 1024-thread block; returns the prefix and
 // writes the block total to *total (shared).
 __device__ __forceinline__ uint32_t block_scan(uint32_t flag, uint32_t* warp_sums,
@@ -496,84 +500,210 @@ __device__ __forceinline__ void miss_all(GroupHits& h, uint32_t lane, unsigned l
   if ((alive >> (lane + 32)) & 1ull) h.hi = v;
 }
 
+// Run position of `key` (non-zero) in one index, or kNotFound, by the whole warp: four
+// consecutive slots (two sectors) per step, so that most probes take one round trip.
+__device__ __forceinline__ unsigned long long lookup_warp(const IndexSlot* __restrict__ hash,
+                                                          uint64_t key, uint32_t log2_cap,
+                                                          uint32_t lane, int* status) {
+  const uint64_t cap = 1ull << log2_cap;
+  const uint64_t home = home_slot(key, log2_cap);
+  for (uint64_t seen = 0; seen < cap; seen += 4) {
+    ulonglong2 s = make_ulonglong2(~key, 0ull);
+    if (lane < 4)
+      s = __ldg(reinterpret_cast<const ulonglong2*>(hash + ((home + seen + lane) & (cap - 1))));
+    const uint32_t end = __ballot_sync(0xffffffffu, lane < 4 && (s.x == key || s.x == 0ull));
+    if (end) {  // the first of the four that holds the key or nothing decides
+      const uint32_t at = __ffs(end) - 1;
+      const bool found = __shfl_sync(0xffffffffu, s.x == key, at);
+      const unsigned long long pos = __shfl_sync(0xffffffffu, s.y, at);
+      return found ? pos : kNotFound;
+    }
+  }
+  if (lane == 0) flag_status(status, NETKV_DEV_EFULL);
+  return kNotFound;
+}
+
 // First-miss scan of blocks [start, n) of one chain for the `alive` decodes of a group.
 // Decodes found missing at position p get p; decodes never missing keep their value.
+// A step compares 32 * U chain blocks with the run; where a looked-up block's run ends at
+// once (lists that are not in chain order) the next 32 blocks are looked up side by side.
 // start_pos: the run position of block `start` when the caller has already looked it up.
-// kMB: the run masks' width when known at compile time (see run_mask), else 0.
-template <int kMB = 0>
-__device__ __forceinline__ void scan_chain(const IndexView& ix, uint32_t log2_cap,
-                                           const uint64_t* __restrict__ chain, uint64_t start,
-                                           uint64_t n, unsigned long long alive, GroupHits& h,
-                                           uint32_t lane, int* status,
-                                           unsigned long long start_pos = kNotFound) {
-  const uint64_t cap = 1ull << log2_cap;
-  const IndexSlot* __restrict__ hash = ix.hash;
-  const unsigned long long* __restrict__ run_keys = ix.keys;
-  uint64_t p = start;
-  uint64_t seg_run = 0, seg_p = 0;  // run position matched with chain position seg_p
-  bool in_run = false, fresh = false;
-  if (start_pos != kNotFound) {
-    seg_run = start_pos;
-    seg_p = start;
-    in_run = fresh = true;
+// n is at most 65,535.  U: a wide step has more loads in flight per warp, but reads up to 32 * U - 1 blocks past
+// the last one needed.  kMB: the run masks' width.
+template <int kMB>  // masks of at most 32 decodes are reduced as one word
+using DecodeMask = std::conditional_t<kMB == 8, unsigned long long, uint32_t>;
+
+// The decodes of nm[u] miss block p + 32 u + lane: the first miss of each counts, and the
+// decode leaves `alive`.
+template <int N, typename Mask>
+__device__ __forceinline__ void settle(const Mask (&nm)[N], uint32_t p, GroupHits& h, Mask& alive,
+                                       uint32_t lane) {
+  Mask m = nm[0];
+#pragma unroll
+  for (int u = 1; u < N; ++u) m |= nm[u];
+  Mask a = __reduce_or_sync(0xffffffffu, (uint32_t)m);
+  if (sizeof(Mask) == 8)
+    a |= (Mask)((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)((uint64_t)m >> 32)) << 32);
+  while (a) {  // usually none
+    const uint32_t j = __ffsll((long long)a) - 1;
+    a &= a - 1;
+    uint32_t first = 0;
+#pragma unroll
+    for (int u = N - 1; u >= 0; --u) {
+      const uint32_t miss = __ballot_sync(0xffffffffu, (uint32_t)(nm[u] >> j) & 1u);
+      if (miss) first = 32u * u + (uint32_t)(__ffs(miss) - 1);
+    }
+    set_hit(h, lane, j, p + first);
+    alive &= ~((Mask)1 << j);
   }
+}
+
+// Where the lists are not in chain order: blocks from p on looked up 32 at a time, side by
+// side, until the scan is done (p = n) or a run can be followed again from `run`.  Out of
+// line, with its state by value, so that the common path keeps its registers.
+template <int kMB>
+struct SideScan {
+  GroupHits h;
+  DecodeMask<kMB> alive;
+  uint32_t p, run;
+};
+template <int kMB>
+__device__ __noinline__ SideScan<kMB> scan_side_by_side(const IndexSlot* __restrict__ hash,
+                                                        const unsigned char* __restrict__ masks,
+                                                        const uint64_t* __restrict__ chain,
+                                                        uint32_t n, uint32_t log2_cap,
+                                                        SideScan<kMB> s, int* status) {
+  using Mask = DecodeMask<kMB>;
+  const uint32_t lane = threadIdx.x & 31;
+  IndexView ix;
+  ix.masks = const_cast<unsigned char*>(masks);
+  while (s.p < n && s.alive) {
+    const uint32_t i = s.p + lane;
+    const uint64_t key = i < n ? __ldcs(chain + i) : 0ull;
+    const unsigned long long pos = key != 0ull ? lookup(hash, key, log2_cap, status) : kNotFound;
+    const uint32_t ok = __ballot_sync(0xffffffffu, pos != kNotFound);
+    const uint32_t lead = ~ok ? (uint32_t)(__ffs(~ok) - 1) : 32u;
+    const Mask nm[1] = {lane < lead ? (Mask)(s.alive & ~(Mask)run_mask<kMB>(ix, pos)) : (Mask)0};
+    settle(nm, s.p, s.h, s.alive, lane);
+    if (lead < 32u) {
+      if (s.p + lead < n) {  // block p + lead is absent from every cache of the group
+        if (lane == lead && key == 0ull && s.alive) flag_status(status, NETKV_DEV_EDOMAIN);
+        miss_all(s.h, lane, s.alive, s.p + lead);
+      }
+      s.p = n;
+      return s;
+    }
+    s.p += 32;
+    const unsigned long long before = __shfl_up_sync(0xffffffffu, pos, 1);
+    const uint32_t follows = __ballot_sync(0xffffffffu, lane > 0 && pos == before + 1);
+    if (__popc(follows) >= 16) {  // in order here
+      s.run = (uint32_t)__shfl_sync(0xffffffffu, pos, 31) + 1;
+      return s;
+    }
+  }
+  s.p = n;
+  return s;
+}
+
+template <int U, int kMB>
+__device__ __forceinline__ void scan_chain(const IndexView& ix, uint32_t log2_cap,
+                                           const uint64_t* __restrict__ chain, uint32_t start,
+                                           uint32_t n, unsigned long long alive_decodes,
+                                           GroupHits& h, uint32_t lane, int* status,
+                                           unsigned long long start_pos = kNotFound) {
+  using Mask = DecodeMask<kMB>;
+  const uint32_t cap = 1u << log2_cap;  // at most 2^31
+  Mask alive = (Mask)alive_decodes;
+  uint32_t p = start;
+  uint32_t run = (uint32_t)min(start_pos, (unsigned long long)cap);  // block p's run position
+  bool in_run = start_pos != kNotFound, looked_up = in_run;
   while (p < n && alive) {
-    const bool looked_up = !in_run || fresh;
-    fresh = false;
-    if (!in_run) {  // locate block p in the hash table
+    if (!in_run) {
       const uint64_t key = __ldg(chain + p);
       unsigned long long pos = kNotFound;
-      if (lane == 0) {
-        if (key == 0ull) flag_status(status, NETKV_DEV_EDOMAIN);
-        else pos = lookup(hash, key, log2_cap, status);
-      }
-      pos = __shfl_sync(0xffffffffu, pos, 0);
+      if (key != 0ull) pos = lookup_warp(ix.hash, key, log2_cap, lane, status);
+      else if (lane == 0) flag_status(status, NETKV_DEV_EDOMAIN);
       if (pos == kNotFound) {  // absent from every cache of the group
-        miss_all(h, lane, alive, (uint32_t)p);
+        miss_all(h, lane, alive, p);
         return;
       }
-      seg_run = pos;
-      seg_p = p;
-      in_run = true;
+      run = (uint32_t)min(pos, (unsigned long long)cap);
+      looked_up = true;
     }
-    // blocks p .. p+31 against the run from seg_run
-    const uint64_t i = p + lane;
-    const uint64_t rp = seg_run + (i - seg_p);
-    const bool in = i < n;
-    const uint64_t ck = in ? __ldcs(chain + i) : 0ull;
-    unsigned long long rkey = 0ull, rmask = 0ull;
-    if (in && rp < cap) {
-      rkey = __ldg(run_keys + rp);
-      rmask = run_mask<kMB>(ix, rp);
+    // blocks p .. p + 32 U - 1 against the run: as long as whole steps match and no live
+    // decode misses, a step costs its loads, the comparisons and one vote
+    unsigned long long ck[U], rk[U];
+    Mask rm[U];
+    for (;;) {
+      const bool whole = p + 32u * U <= n && run + 32u * U <= cap;
+      const uint64_t* cp = chain + p + lane;
+      const unsigned long long* kp = ix.keys + run + lane;
+      if (whole) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          ck[u] = __ldcs(cp + 32 * u);
+          rk[u] = __ldg(kp + 32 * u);
+          rm[u] = (Mask)run_mask<kMB>(ix, run + lane + 32 * u);
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          ck[u] = rk[u] = 0ull;
+          rm[u] = 0;
+          if (p + 32 * u + lane < n) {
+            ck[u] = __ldcs(cp + 32 * u);
+            if (run + 32 * u + lane < cap) {
+              rk[u] = __ldg(kp + 32 * u);
+              rm[u] = (Mask)run_mask<kMB>(ix, run + lane + 32 * u);
+            }
+          }
+        }
+      }
+      bool same = true;
+      Mask all = rm[0];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        same &= ck[u] == rk[u] && ck[u] != 0ull;
+        all &= rm[u];
+      }
+      if (!whole || !__all_sync(0xffffffffu, same && !(alive & ~all))) break;
+      p += 32u * U;
+      run += 32u * U;
+      looked_up = false;
     }
-    const bool same = in && ck != 0ull && rkey == ck;
-    const uint32_t run_ok = __ballot_sync(0xffffffffu, same);
-    const uint32_t lead = (~run_ok) ? (uint32_t)(__ffs(~run_ok) - 1) : 32u;  // leading matches
-    const bool counted = lane < lead;
-    // decodes missing at some counted position of this step (usually none)
-    const unsigned long long nm = counted ? (alive & ~rmask) : 0ull;
-    unsigned long long a = ((unsigned long long)__reduce_or_sync(0xffffffffu, (uint32_t)(nm >> 32))
-                            << 32) |
-                           __reduce_or_sync(0xffffffffu, (uint32_t)nm);
-    while (a) {
-      const uint32_t j = __ffsll((long long)a) - 1;
-      a &= a - 1;
-      const uint32_t miss = __ballot_sync(0xffffffffu, (nm >> j) & 1ull);
-      set_hit(h, lane, j, (uint32_t)(p + (uint64_t)(__ffs(miss) - 1)));
-      alive &= ~(1ull << j);
+    uint32_t lead = 32u * U;  // leading blocks that match
+#pragma unroll
+    for (int u = U - 1; u >= 0; --u) {
+      const uint32_t part = ~__ballot_sync(0xffffffffu, ck[u] != 0ull && rk[u] == ck[u]);
+      if (part) lead = 32u * u + (uint32_t)(__ffs(part) - 1);
     }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      rm[u] = 32u * u + lane < lead ? (Mask)(alive & ~rm[u]) : (Mask)0;
+    settle(rm, p, h, alive, lane);
     if (lead == 0 && looked_up) {
       // the run entry the table points to does not hold the key: a corrupted index.
       // Report it and count the block as missing, so the walk always advances.
       if (lane == 0) flag_status(status, NETKV_DEV_EFULL);
-      miss_all(h, lane, alive, (uint32_t)p);
+      miss_all(h, lane, alive, p);
       return;
     }
+    const bool out_of_order = looked_up && lead < 3;
+    looked_up = false;
     p += lead;
-    if (lead < 32) in_run = false;  // the run parts here: look the next block up
+    run += lead;
+    in_run = lead == 32u * U;  // else the run parts here: look the next block up
+    if (out_of_order) {
+      const SideScan<kMB> s = scan_side_by_side<kMB>(ix.hash, ix.masks, chain, n, log2_cap,
+                                                     SideScan<kMB>{h, alive, p, run}, status);
+      h = s.h;
+      alive = s.alive;
+      p = s.p;
+      run = s.run;
+      in_run = true;
+    }
   }
 }
-
 
 // Group key of a request: its table set and first block hash, never zero.
 __device__ __forceinline__ uint64_t group_key(uint64_t h0, uint32_t set) {
@@ -594,7 +724,6 @@ struct MatchCounters {
   unsigned long long n_long;       // leaders listed from the front of the leader list
   unsigned long long n_short;      // leaders listed from its back
   unsigned long long next_task;    // next (leader, decode group) task of the leader pass
-  unsigned long long next_member;  // next chunk of requests of the member pass
 };
 
 // Leaders with chains of at least this many blocks are listed first, so that the leader
@@ -602,13 +731,13 @@ struct MatchCounters {
 // a long one started last.
 constexpr uint64_t kLongLeader = 2048;
 
-// One thread per request: its table set (set_of) and group key (in rec[r].x, for the
-// resolve pass) are recorded, and the group's slot keeps the longest chain.
+// One thread per request: its table set (set_of) and group key (gkey, for the resolve pass)
+// are recorded, and the group's slot keeps the longest chain.
 __global__ void group_insert_kernel(GroupSlot* __restrict__ tab, uint32_t log2_slots,
                                     const uint64_t* __restrict__ chains,
                                     const uint64_t* __restrict__ chain_off, uint32_t R,
                                     const uint32_t* __restrict__ set_off, uint32_t n_sets,
-                                    int32_t* __restrict__ set_of, ulonglong2* __restrict__ rec) {
+                                    int32_t* __restrict__ set_of, uint64_t* __restrict__ gkey) {
   const uint64_t mask = (1ull << log2_slots) - 1;
   for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < R; r += gridDim.x * blockDim.x) {
     const uint64_t c0 = __ldg(chain_off + r), c1 = __ldg(chain_off + r + 1);
@@ -617,7 +746,7 @@ __global__ void group_insert_kernel(GroupSlot* __restrict__ tab, uint32_t log2_s
     if (c1 <= c0 || set < 0) continue;
     const uint64_t n = c1 - c0;
     const uint64_t key = group_key(__ldg(chains + c0), (uint32_t)set);
-    rec[r].x = key;
+    gkey[r] = key;
     const unsigned long long code =
         ((unsigned long long)(n < 0xffffffffull ? n : 0xffffffffull) << 32) | (0xffffffffu - r);
     uint64_t slot = home_slot(key, log2_slots);
@@ -632,24 +761,20 @@ __global__ void group_insert_kernel(GroupSlot* __restrict__ tab, uint32_t log2_s
   }
 }
 
-// A member's record: its chain offset and length (clamped to 65,535 blocks) and its
-// leader's, 48 + 16 bits each, so that the member pass fetches both chains' first blocks
-// and the leader's hits in its first round trip.
-constexpr uint64_t kOff48 = (1ull << 48) - 1;
-
 __global__ void group_resolve_kernel(const GroupSlot* __restrict__ tab, uint32_t log2_slots,
                                      const uint64_t* __restrict__ chain_off, uint32_t R,
                                      uint32_t* __restrict__ leader_of,
                                      const int32_t* __restrict__ set_of,
-                                     uint32_t* __restrict__ leaders, ulonglong2* __restrict__ rec,
-                                     MatchCounters* counters, int* status) {
+                                     uint32_t* __restrict__ leaders,
+                                     const uint64_t* __restrict__ gkey,
+                                     MatchCounters* counters) {
   const uint64_t mask = (1ull << log2_slots) - 1;
   for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < R; r += gridDim.x * blockDim.x) {
     const uint64_t c0 = __ldg(chain_off + r), c1 = __ldg(chain_off + r + 1);
     const int32_t set = __ldg(set_of + r);
     uint32_t lead = r;
     if (c1 > c0 && set >= 0) {
-      const uint64_t key = rec[r].x;  // written by the insert pass
+      const uint64_t key = gkey[r];  // written by the insert pass
       uint64_t slot = home_slot(key, log2_slots);
       for (uint64_t step = 0; step <= mask; ++step) {
         const unsigned long long k = tab[slot].key;
@@ -661,17 +786,6 @@ __global__ void group_resolve_kernel(const GroupSlot* __restrict__ tab, uint32_t
         }
         if (k == 0ull) break;
         slot = (slot + 1) & mask;
-      }
-    }
-    if (lead != r) {
-      const uint64_t l0 = __ldg(chain_off + lead), l1 = __ldg(chain_off + lead + 1);
-      if (c1 <= kOff48 && l1 <= kOff48 && l1 > l0) {
-        const uint64_t n = c1 - c0, nl = l1 - l0;
-        if (n > 65535) flag_status(status, NETKV_DEV_EDOMAIN);  // counted up to 65,535 blocks
-        rec[r] = make_ulonglong2(c0 | (min(n, (uint64_t)65535) << 48),
-                                 l0 | (min(nl, (uint64_t)65535) << 48));
-      } else {
-        lead = r;  // offsets beyond 48 bits: matched in full by the leader pass
       }
     }
     leader_of[r] = lead;
@@ -739,183 +853,83 @@ __global__ void __launch_bounds__(kMatchBlock, 8) match_leaders_kernel(
     if (chain_extent(chain_off, set_off, n_sets, set_of, r, lane, status, set, c0, n)) {
       h.lo = h.hi = (uint32_t)n;
       const unsigned long long alive = ng >= 64 ? ~0ull : ((1ull << ng) - 1);
-      const IndexView ix = index_view(index, (uint64_t)set * n_dgroups + q, log2_cap,
-                                      mask_bytes_of(D));
-      scan_chain(ix, log2_cap, chains + c0, 0, n, alive, h, lane, status);
+      const IndexView ix = index_view(index, (uint64_t)set * n_dgroups + q, log2_cap, 8u);
+      scan_chain<2, 8>(ix, log2_cap, chains + c0, 0, n, alive, h, lane, status);
     }
     store_hits(M, (uint64_t)r * D, q0, ng, lane, h);
   }
 }
 
-// Full match without a workspace: one warp per (request, decode group).
-__global__ void __launch_bounds__(kMatchBlock, 8) match_kernel(
+// Full match, one task per (request, decode group): pools of one group, and any pool without
+// a workspace.  A warp takes `per` <= 32 consecutive tasks: first lane i reads task i's
+// chain extent and first block and looks the block up, all tasks side by side; then the
+// warp scans one chain after another, whose first step needs no further address.
+// Blocks are small so that a long chain holds back few other warps, and steps of 128
+// blocks keep enough loads in flight at 32 warps an SM (64 registers).  Bound by latency and
+// issue: 1,024 replicas (8 decodes, 1.02 M requests) 1.05 ms, 4.8 KB of DRAM traffic a
+// request (4.7 TB/s).  Matching the members of a group against their leader's chain, after
+// a grouping and a leader pass, took 1.38 ms there, 130 us against 14 for 1,000 requests,
+// 37 against 4 for one, and 1.20 ms against 0.60 for 32,000 requests whose chains lie in
+// host memory, where the leader's chain crosses the link for every member.  Steps of 64 and
+// 96 blocks: 1.10 and 1.01 ms; 24 blocks an SM (40 registers): spills, no faster.
+constexpr int kDirectBlock = 64;
+
+template <int kMB>
+__global__ void __launch_bounds__(kDirectBlock, 16) match_kernel(
     const void* __restrict__ index, uint32_t D, uint32_t log2_cap, uint32_t n_sets,
     const uint64_t* __restrict__ chains, const uint64_t* __restrict__ chain_off, uint32_t R,
-    const uint32_t* __restrict__ set_off, uint16_t* __restrict__ M, int* status) {
+    const uint32_t* __restrict__ set_off, uint32_t per, uint16_t* __restrict__ M, int* status) {
   const uint32_t lane = threadIdx.x & 31;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   const uint32_t n_dgroups = (D + kGroup - 1) / kGroup;
   const uint64_t total = (uint64_t)R * n_dgroups;
-
-  for (uint64_t task = warp; task < total; task += n_warps) {
-    const uint32_t r = (uint32_t)(n_dgroups == 1 ? task : task / n_dgroups);
-    const uint32_t q = (uint32_t)(task - (uint64_t)r * n_dgroups);
-    const uint32_t q0 = q * kGroup, ng = min(kGroup, D - q0);
-    GroupHits h = {0u, 0u};
-    int32_t set;
-    uint64_t c0, n;
-    if (chain_extent(chain_off, set_off, n_sets, nullptr, r, lane, status, set, c0, n)) {
-      h.lo = h.hi = (uint32_t)n;
-      const unsigned long long alive = ng >= 64 ? ~0ull : ((1ull << ng) - 1);
-      const IndexView ix = index_view(index, (uint64_t)set * n_dgroups + q, log2_cap,
-                                      mask_bytes_of(D));
-      scan_chain(ix, log2_cap, chains + c0, 0, n, alive, h, lane, status);
+  for (uint64_t t0 = warp * per; t0 < total; t0 += n_warps * per) {
+    const uint32_t count = (uint32_t)min((uint64_t)per, total - t0);
+    uint64_t my_c0 = 0;  // lane i: task t0 + i
+    uint32_t my_n = 0, my_pos = 0;
+    int32_t my_set = -1;  // < 0: a bad request, hits 0
+    if (lane < count) {
+      const uint64_t task = t0 + lane;
+      const uint32_t r = (uint32_t)(n_dgroups == 1 ? task : task / n_dgroups);
+      const uint32_t q = (uint32_t)(task - (uint64_t)r * n_dgroups);
+      my_c0 = __ldg(chain_off + r);
+      const uint64_t c1 = __ldg(chain_off + r + 1);
+      my_set = find_set(set_off, n_sets, r);
+      if (my_set < 0 || c1 < my_c0) {
+        flag_status(status, NETKV_DEV_ERANGE);
+        my_set = -1;
+      } else if (c1 > my_c0) {
+        if (c1 - my_c0 > 65535) flag_status(status, NETKV_DEV_EDOMAIN);
+        my_n = (uint32_t)min(c1 - my_c0, (uint64_t)65535);
+        const uint64_t key = __ldg(chains + my_c0);
+        unsigned long long pos = kNotFound;
+        if (key != 0ull)
+          pos = lookup(index_view(index, (uint64_t)my_set * n_dgroups + q, log2_cap, kMB).hash,
+                       key, log2_cap, status);
+        else
+          flag_status(status, NETKV_DEV_EDOMAIN);
+        my_pos = pos == kNotFound ? kNoRun : (uint32_t)min(pos, 1ull << log2_cap);
+      }
     }
-    store_hits(M, (uint64_t)r * D, q0, ng, lane, h);
-  }
-}
-
-// Member pass of pools of one decode group (D <= 64), for member r with leader `lead`.
-// The record written by the grouping gives both chains' offsets and lengths, so the
-// leader's hits and the first 128 blocks of both chains are fetched in one round trip (the
-// cap on the common prefix, min(n_r, n_L, max_d M_L[d] + 1), is known once the hits
-// arrive).  Then as the leader pass: decodes whose leader missed inside the common prefix
-// take the leader's answer, the rest walk on from the common prefix.
-__device__ __forceinline__ void member_match(const void* __restrict__ index, uint32_t D,
-                                             uint32_t log2_cap,
-                                             const uint64_t* __restrict__ chains, uint32_t r,
-                                             uint32_t lead, int32_t set, ulonglong2 rc,
-                                             uint16_t* __restrict__ M, uint32_t lane,
-                                             int* status) {
-  const uint32_t ng = D;  // one group
-  const uint64_t c0 = rc.x & kOff48, n = rc.x >> 48;
-  const uint64_t l0 = rc.y & kOff48, nl = rc.y >> 48;
-  const uint64_t capn = min(n, nl);
-  const uint64_t lrow = (uint64_t)lead * D;
-  const uint32_t mlo = lane < ng ? (uint32_t)__ldg(M + lrow + lane) : 0u;
-  const uint32_t mhi = lane + 32 < ng ? (uint32_t)__ldg(M + lrow + lane + 32) : 0u;
-  uint64_t a[4], b[4];
-  const uint64_t first = min(capn, (uint64_t)128);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const uint64_t i = 32 * k + lane;
-    a[k] = i < first ? __ldcs(chains + c0 + i) : 0ull;
-    b[k] = i < first ? __ldg(chains + l0 + i) : 0ull;
-  }
-  uint32_t mmax = max(mlo, mhi);
-#pragma unroll
-  for (int o = 16; o; o >>= 1) mmax = max(mmax, __shfl_xor_sync(0xffffffffu, mmax, o));
-  const uint64_t cap = min(capn, (uint64_t)mmax + 1);
-  uint64_t lcp = cap;  // common prefix, 128 blocks per step
-  for (uint64_t base = 0; base < cap;) {
-    uint64_t found = cap;
-#pragma unroll
-    for (int k = 3; k >= 0; --k) {
-      const uint64_t i = base + 32 * k + lane;
-      const uint32_t diff = __ballot_sync(0xffffffffu, i < cap && a[k] != b[k]);
-      if (diff) found = base + 32 * k + (uint64_t)(__ffs(diff) - 1);
+    for (uint32_t i = 0; i < count; ++i) {
+      const uint64_t task = t0 + i;
+      const uint32_t r = (uint32_t)(n_dgroups == 1 ? task : task / n_dgroups);
+      const uint32_t q = (uint32_t)(task - (uint64_t)r * n_dgroups);
+      const uint32_t q0 = q * kGroup, ng = min(kGroup, D - q0);
+      const int32_t set = __shfl_sync(0xffffffffu, my_set, i);
+      const uint32_t n = __shfl_sync(0xffffffffu, my_n, i);
+      const uint32_t pos = __shfl_sync(0xffffffffu, my_pos, i);
+      const uint64_t c0 = __shfl_sync(0xffffffffu, my_c0, i);
+      GroupHits h = {0u, 0u};
+      if (set >= 0 && pos != kNoRun) {  // else every decode misses block 0
+        h.lo = h.hi = n;
+        const unsigned long long alive = ng >= 64 ? ~0ull : ((1ull << ng) - 1);
+        scan_chain<4, kMB>(index_view(index, (uint64_t)set * n_dgroups + q, log2_cap, kMB),
+                           log2_cap, chains + c0, 0, n, alive, h, lane, status, pos);
+      }
+      store_hits(M, (uint64_t)r * D, q0, ng, lane, h);
     }
-    if (found < cap) {
-      lcp = found;
-      break;
-    }
-    base += 128;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const uint64_t i = base + 32 * k + lane;
-      a[k] = i < cap ? __ldcs(chains + c0 + i) : 0ull;
-      b[k] = i < cap ? __ldg(chains + l0 + i) : 0ull;
-    }
-  }
-  GroupHits h = {(uint32_t)n, (uint32_t)n};
-  // decodes whose leader missed inside the common prefix copy the leader's answer
-  const uint32_t clo = __ballot_sync(0xffffffffu, lane < ng && (uint64_t)mlo < lcp);
-  const uint32_t chi = __ballot_sync(0xffffffffu, lane + 32 < ng && (uint64_t)mhi < lcp);
-  if ((clo >> lane) & 1u) h.lo = mlo;
-  if ((chi >> lane) & 1u) h.hi = mhi;
-  unsigned long long alive = ng >= 64 ? ~0ull : ((1ull << ng) - 1);
-  alive &= ~((unsigned long long)clo | ((unsigned long long)chi << 32));
-  scan_chain(index_view(index, (uint64_t)set, log2_cap, mask_bytes_of(D)), log2_cap,
-             chains + c0, lcp, n, alive, h, lane, status);
-  store_hits(M, (uint64_t)r * D, 0, ng, lane, h);
-}
-
-constexpr uint32_t kMemberChunk = 8;  // consecutive requests a warp takes at a time
-
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-}
-
-// A request's record, leader and table set, staged in shared memory per warp.
-struct __align__(16) MemberSlot {
-  ulonglong2 rc;
-  uint32_t lead;
-  int32_t set;
-  uint32_t pad[2];
-};
-
-// Persistent member pass of pools of one decode group: every warp takes chunks of 8
-// consecutive requests from a global counter (fetched one chunk ahead), so a warp that
-// finishes early takes more work instead of idling until its block ends.  The next
-// request's record, leader and table set are copied into the warp's shared-memory slot
-// with cp.async while the current one is matched, so they cost no round trip of their own.
-__global__ void __launch_bounds__(kMatchBlock, 8) match_members_kernel(
-    const void* __restrict__ index, uint32_t D, uint32_t log2_cap,
-    const uint64_t* __restrict__ chains, uint32_t R, const uint32_t* __restrict__ leader_of,
-    const int32_t* __restrict__ set_of, const ulonglong2* __restrict__ rec,
-    MatchCounters* counters, uint16_t* __restrict__ M, int* status) {
-  __shared__ MemberSlot slots[kMatchBlock / 32];
-  MemberSlot& slot = slots[threadIdx.x >> 5];
-  const uint32_t lane = threadIdx.x & 31;
-  const unsigned long long n_chunks = ((unsigned long long)R + kMemberChunk - 1) / kMemberChunk;
-  // request rr's record into the slot (a leader's record is not written and not used)
-  auto fetch = [&](uint64_t rr) {
-    if (lane == 0) {
-      cp_async16(&slot.rc, rec + rr);
-      cp_async4(&slot.lead, leader_of + rr);
-      cp_async4(&slot.set, set_of + rr);
-      cp_async_commit();
-    }
-  };
-  unsigned long long c = 0, c_next = 0;
-  if (lane == 0) c = atomicAdd(&counters->next_member, 1ull);
-  c = __shfl_sync(0xffffffffu, c, 0);
-  if (c >= n_chunks) return;
-  if (lane == 0) c_next = atomicAdd(&counters->next_member, 1ull);  // the chunk after
-  uint64_t r = c * kMemberChunk;
-  uint64_t end = min(r + kMemberChunk, (uint64_t)R);
-  fetch(r);
-  for (;;) {
-    if (lane == 0) cp_async_wait_all();  // request r's record has landed
-    __syncwarp();
-    const ulonglong2 rc = slot.rc;
-    const uint32_t lead = slot.lead;
-    const int32_t set = slot.set;
-    __syncwarp();  // every lane has read the slot before it is refilled
-    uint64_t rn = r + 1;
-    if (rn >= end) {  // this chunk is done: take the one fetched ahead, and fetch the next
-      const unsigned long long cn = __shfl_sync(0xffffffffu, c_next, 0);
-      rn = cn < n_chunks ? cn * kMemberChunk : (uint64_t)R;
-      end = min(rn + kMemberChunk, (uint64_t)R);
-      if (lane == 0 && cn < n_chunks) c_next = atomicAdd(&counters->next_member, 1ull);
-    }
-    if (rn < R) fetch(rn);
-    if (lead != (uint32_t)r)  // leaders were matched by the leader pass
-      member_match(index, D, log2_cap, chains, (uint32_t)r, lead, set, rc, M, lane, status);
-    if (rn >= R) break;
-    r = rn;
   }
 }
 
@@ -1022,7 +1036,7 @@ __global__ void __launch_bounds__(kMatchBlock, 6) match_members_wide_kernel(
         const uint32_t alo = __ballot_sync(0xffffffffu, lane < ng && (uint64_t)mlo >= lcp);
         const uint32_t ahi = __ballot_sync(0xffffffffu, lane + 32 < ng && (uint64_t)mhi >= lcp);
         const unsigned long long alive = (unsigned long long)alo | ((unsigned long long)ahi << 32);
-        scan_chain<8>(index_view(index, (uint64_t)set * n_dgroups + q, log2_cap, 8u),
+        scan_chain<2, 8>(index_view(index, (uint64_t)set * n_dgroups + q, log2_cap, 8u),
                    log2_cap, own, lcp, n, alive, h, lane, status, pj);
         store_hits(M, row, q0, ng, lane, h);
       }
@@ -1081,10 +1095,10 @@ uint32_t group_log2_slots(uint32_t R) {
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Workspace: group table | leader_of [R] | set_of [R] | leader list [R] | member records [R]
-// | counters.
+// Workspace: group table | leader_of [R] | set_of [R] | leader list [R] | group keys [R]
+// | counters.  Used for pools of several decode groups.
 struct WorkspaceLayout {
-  size_t table, leader_of, set_of, leaders, rec, counters, total;
+  size_t table, leader_of, set_of, leaders, gkey, counters, total;
 };
 
 WorkspaceLayout workspace_layout(uint32_t R) {
@@ -1093,23 +1107,50 @@ WorkspaceLayout workspace_layout(uint32_t R) {
   w.leader_of = align_up(sizeof(GroupSlot) << group_log2_slots(R), 256);
   w.set_of = w.leader_of + align_up(sizeof(uint32_t) * (size_t)R, 256);
   w.leaders = w.set_of + align_up(sizeof(int32_t) * (size_t)R, 256);
-  w.rec = w.leaders + align_up(sizeof(uint32_t) * (size_t)R, 256);
-  w.counters = w.rec + align_up(sizeof(ulonglong2) * (size_t)R, 256);
+  w.gkey = w.leaders + align_up(sizeof(uint32_t) * (size_t)R, 256);
+  w.counters = w.gkey + align_up(sizeof(uint64_t) * (size_t)R, 256);
   w.total = w.counters + align_up(sizeof(MatchCounters), 256);
   return w;
 }
 
 // Blocks of a persistent grid: every SM filled to the kernel's occupancy.
 template <typename Kernel>
-int persistent_grid(Kernel kernel) {
+int persistent_grid(Kernel kernel, int block) {
   int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kMatchBlock, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, 0);
   return (sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
 }
-int leader_grid() { return persistent_grid(match_leaders_kernel); }
-int member_grid() { return persistent_grid(match_members_kernel); }
+int leader_grid() { return persistent_grid(match_leaders_kernel, kMatchBlock); }
+
+// The direct match.  A warp takes several tasks where every resident warp still gets
+// kWaves turns (the card's last turns are then short), at most kPerWarp.
+constexpr uint32_t kPerWarp = 8, kWaves = 8;
+netkv_status launch_match(const void* index, uint32_t D, uint32_t log2_cap, uint32_t n_sets,
+                          const uint64_t* chains, const uint64_t* chain_off, uint32_t R,
+                          const uint32_t* set_off, uint16_t* M, int* status, cudaStream_t s) {
+  int dev = 0, sms = 0;
+  NETKV_CUDA_TRY(cudaGetDevice(&dev));
+  NETKV_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const uint64_t tasks = (uint64_t)R * ((D + kGroup - 1) / kGroup);
+  const uint64_t turns = tasks / ((uint64_t)sms * 32 * kWaves);
+  const uint32_t per = turns < 1 ? 1u : turns < kPerWarp ? (uint32_t)turns : kPerWarp;
+  const uint64_t per_block = (uint64_t)per * (kDirectBlock / 32);
+  const uint64_t blocks = (tasks + per_block - 1) / per_block;
+  const unsigned grid = (unsigned)(blocks < (1u << 24) ? blocks : (1u << 24));
+#define NETKV_MATCH(MB)                                                                      \
+  match_kernel<MB><<<grid, kDirectBlock, 0, s>>>(index, D, log2_cap, n_sets, chains,         \
+                                                 chain_off, R, set_off, per, M, status)
+  switch (mask_bytes_of(D)) {
+    case 1: NETKV_MATCH(1); break;
+    case 2: NETKV_MATCH(2); break;
+    case 4: NETKV_MATCH(4); break;
+    default: NETKV_MATCH(8); break;
+  }
+#undef NETKV_MATCH
+  return netkv_launch_status();
+}
 
 }  // namespace
 
@@ -1184,15 +1225,9 @@ extern "C" netkv_status netkv_prefix_match(const void* d_index, uint32_t D,
   if (d_workspace && workspace_bytes < netkv_prefix_match_workspace_size(R)) return NETKV_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
   const void* index = d_index;
-  const uint64_t tasks = (uint64_t)R * ((D + kGroup - 1) / kGroup);
-  const uint64_t warps_per_block = kMatchBlock / 32;
-  const uint64_t blocks = (tasks + warps_per_block - 1) / warps_per_block;
-  const unsigned grid = (unsigned)(blocks < (1u << 24) ? blocks : (1u << 24));
-  if (!d_workspace) {
-    match_kernel<<<grid, kMatchBlock, 0, s>>>(index, D, log2_capacity, n_sets, d_chains,
-                                              d_chain_off, R, d_set_off, d_M, d_status);
-    return netkv_launch_status();
-  }
+  if (!d_workspace || D <= kGroup)
+    return launch_match(index, D, log2_capacity, n_sets, d_chains, d_chain_off, R, d_set_off, d_M,
+                        d_status, s);
   const uint32_t lg = group_log2_slots(R);
   const WorkspaceLayout L = workspace_layout(R);
   char* ws = reinterpret_cast<char*>(d_workspace);
@@ -1200,28 +1235,24 @@ extern "C" netkv_status netkv_prefix_match(const void* d_index, uint32_t D,
   uint32_t* leader_of = reinterpret_cast<uint32_t*>(ws + L.leader_of);
   int32_t* set_of = reinterpret_cast<int32_t*>(ws + L.set_of);
   uint32_t* leaders = reinterpret_cast<uint32_t*>(ws + L.leaders);
-  ulonglong2* rec = reinterpret_cast<ulonglong2*>(ws + L.rec);
+  uint64_t* gkey = reinterpret_cast<uint64_t*>(ws + L.gkey);
   MatchCounters* counters = reinterpret_cast<MatchCounters*>(ws + L.counters);
   NETKV_CUDA_TRY(cudaMemsetAsync(tab, 0, sizeof(GroupSlot) << lg, s));
   NETKV_CUDA_TRY(cudaMemsetAsync(counters, 0, sizeof(MatchCounters), s));
   const unsigned rgrid = (unsigned)((R + 255) / 256 < 65535u * 16 ? (R + 255) / 256 : 65535u * 16);
   group_insert_kernel<<<rgrid, 256, 0, s>>>(tab, lg, d_chains, d_chain_off, R, d_set_off, n_sets,
-                                            set_of, rec);
+                                            set_of, gkey);
   group_resolve_kernel<<<rgrid, 256, 0, s>>>(tab, lg, d_chain_off, R, leader_of, set_of, leaders,
-                                             rec, counters, d_status);
+                                             gkey, counters);
   match_leaders_kernel<<<leader_grid(), kMatchBlock, 0, s>>>(
       index, D, log2_capacity, n_sets, d_chains, d_chain_off, R, d_set_off, set_of, leaders,
       counters, d_M, d_status);
-  if (D <= kGroup) {
-    match_members_kernel<<<member_grid(), kMatchBlock, 0, s>>>(
-        index, D, log2_capacity, d_chains, R, leader_of, set_of, rec, counters, d_M, d_status);
-  } else {
-    const uint64_t mblocks = ((uint64_t)R + warps_per_block - 1) / warps_per_block;
-    const unsigned mgrid = (unsigned)(mblocks < (1u << 24) ? mblocks : (1u << 24));
-    match_members_wide_kernel<<<mgrid, kMatchBlock, 0, s>>>(index, D, log2_capacity, n_sets,
-                                                            d_chains, d_chain_off, R, d_set_off,
-                                                            leader_of, set_of, d_M, d_status);
-  }
+  const uint64_t warps_per_block = kMatchBlock / 32;
+  const uint64_t mblocks = ((uint64_t)R + warps_per_block - 1) / warps_per_block;
+  const unsigned mgrid = (unsigned)(mblocks < (1u << 24) ? mblocks : (1u << 24));
+  match_members_wide_kernel<<<mgrid, kMatchBlock, 0, s>>>(index, D, log2_capacity, n_sets,
+                                                          d_chains, d_chain_off, R, d_set_off,
+                                                          leader_of, set_of, d_M, d_status);
   return netkv_launch_status();
 }
 
