@@ -29,19 +29,22 @@
 // Prefix sharing.  Requests that share leading blocks have the same membership answers on
 // those blocks, so for pools of several groups, whose every group would read the chain
 // again, a match with a workspace runs in three steps:
-//   group_insert_kernel / group_resolve_kernel: requests are grouped by (table set,
-//     first block hash) in an open-addressing table; each group's leader is its
-//     longest chain (lowest index among equals); leaders go to a compact list (chains of
-//     2,048 blocks or more first).
+//   group_scan_kernel: every chain is followed through the run keys of its set's first
+//     index (no masks), which gives how many of its blocks that group caches at all.
+//     Requests are grouped by (table set, first block hash) in an open-addressing table, and
+//     each group's leader is the chain with the most such blocks (then the longest, then the
+//     lowest index): the one whose cached prefix the others' are prefixes of.
+//   group_resolve_kernel: leaders go to a compact list; a member r with leader L gets
+//     lcp = |common prefix of h_r and h_L| from how far both chains followed the same run,
+//     without reading them again (exactly, unless both left the run at the same block).
 //   match_leaders_kernel: leaders (and ungrouped requests) run the full match, one task
 //     per (leader, decode group) taken in order from a counter.
-//   match_members_wide_kernel: one warp per member r with leader L compares chains to get
-//     lcp = |common prefix of h_r and h_L| (capped at max_d M_L[d] + 1).  For a decode
-//     with M_L[d] < lcp the first missing block of L lies inside the common prefix, so
-//     M_r[d] = M_L[d] exactly; otherwise blocks [0, lcp) are all cached.  So the member's
-//     row is min(M_L, lcp) elementwise, and block lcp is probed only in the groups where a
-//     leader hit reaches lcp, up to 32 groups at a time.  The result equals the full match
-//     whatever the grouping.
+//   match_members_wide_kernel: one warp per member.  For a decode with M_L[d] < lcp the
+//     first missing block of L lies inside the common prefix, so M_r[d] = M_L[d] exactly;
+//     otherwise blocks [0, lcp) are all cached.  So the member's row is min(M_L, lcp)
+//     elementwise, and block lcp is probed only in the groups where a leader hit reaches
+//     lcp, up to 32 groups at a time.  The result equals the full match whatever the
+//     grouping.
 #include <algorithm>
 #include <type_traits>
 
@@ -51,6 +54,7 @@ namespace {
 
 constexpr int kBuildBlock = 1024;
 constexpr int kMatchBlock = 256;
+constexpr int kDirectBlock = 64;
 constexpr uint32_t kNoRun = 0xffffffffu;  // no run position (they are at most 2^31)
 // Exclusive scan of one flag per thread over a 1024-thread block; returns the prefix and
 // writes the block total to *total (shared).
@@ -716,7 +720,7 @@ __device__ __forceinline__ uint64_t group_key(uint64_t h0, uint32_t set) {
 
 struct GroupSlot {
   unsigned long long key;
-  unsigned long long code;  // (chain length << 32) | (0xffffffff - r): max = longest, lowest r
+  unsigned long long code;  // cached blocks << 48 | chain length << 32 | (0xffffffff - r)
 };
 
 // Work counters at the end of the workspace.
@@ -726,62 +730,150 @@ struct MatchCounters {
   unsigned long long next_task;    // next (leader, decode group) task of the leader pass
 };
 
-// Leaders with chains of at least this many blocks are listed first, so that the leader
-// pass, which takes its tasks in list order, ends on short chains instead of waiting for
-// a long one started last.
-constexpr uint64_t kLongLeader = 2048;
+// Leaders with at least this many cached blocks are listed first, so that the leader pass,
+// which takes its tasks in list order, ends on short chains instead of waiting for a long
+// one started last.
+constexpr uint32_t kLongLeader = 2048;
 
-// One thread per request: its table set (set_of) and group key (gkey, for the resolve pass)
-// are recorded, and the group's slot keeps the longest chain.
-__global__ void group_insert_kernel(GroupSlot* __restrict__ tab, uint32_t log2_slots,
-                                    const uint64_t* __restrict__ chains,
-                                    const uint64_t* __restrict__ chain_off, uint32_t R,
-                                    const uint32_t* __restrict__ set_off, uint32_t n_sets,
-                                    int32_t* __restrict__ set_of, uint64_t* __restrict__ gkey) {
-  const uint64_t mask = (1ull << log2_slots) - 1;
-  for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < R; r += gridDim.x * blockDim.x) {
-    const uint64_t c0 = __ldg(chain_off + r), c1 = __ldg(chain_off + r + 1);
-    const int32_t set = find_set(set_off, n_sets, r);
-    set_of[r] = set;
-    if (c1 <= c0 || set < 0) continue;
-    const uint64_t n = c1 - c0;
-    const uint64_t key = group_key(__ldg(chains + c0), (uint32_t)set);
-    gkey[r] = key;
-    const unsigned long long code =
-        ((unsigned long long)(n < 0xffffffffull ? n : 0xffffffffull) << 32) | (0xffffffffu - r);
-    uint64_t slot = home_slot(key, log2_slots);
-    for (uint64_t step = 0; step <= mask; ++step) {
-      const unsigned long long prev = atomicCAS(&tab[slot].key, 0ull, key);
-      if (prev == 0ull || prev == key) {
-        atomicMax(&tab[slot].code, code);
-        break;
+// Blocks of one chain from p on that follow the run from position `run`, by one warp.
+__device__ __forceinline__ uint32_t follow_run(const unsigned long long* __restrict__ run_keys,
+                                               uint32_t cap, const uint64_t* __restrict__ chain,
+                                               uint32_t p, uint32_t n, uint32_t run,
+                                               uint32_t lane) {
+  constexpr int U = 4;
+  const uint32_t start = p;
+  for (;;) {
+    bool same[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint32_t i = p + 32 * u + lane, rp = run + 32 * u + lane;
+      const uint64_t ck = i < n ? __ldg(chain + i) : 0ull;
+      const unsigned long long rk = i < n && rp < cap ? __ldg(run_keys + rp) : 1ull;
+      same[u] = ck != 0ull && ck == rk && rp < cap;
+    }
+    if (!__all_sync(0xffffffffu, same[0] && same[1] && same[2] && same[3])) {
+      uint32_t lead = 0;
+#pragma unroll
+      for (int u = U - 1; u >= 0; --u) {
+        const uint32_t part = ~__ballot_sync(0xffffffffu, same[u]);
+        if (part) lead = 32u * u + (uint32_t)(__ffs(part) - 1);
       }
-      slot = (slot + 1) & mask;
+      return p + lead - start;
+    }
+    p += 32 * U;
+    run += 32 * U;
+  }
+}
+
+// What a chain's walk through its set's first index found: the run position of its first
+// block (kNoRun: not there) and how many blocks follow the run from it.
+struct FirstRun {
+  uint32_t pos, len;
+};
+
+constexpr int kMaxRuns = 8;  // runs followed per chain: more only refine the choice of leader
+
+// A warp takes `per` <= 32 consecutive requests, as match_kernel does.
+__global__ void __launch_bounds__(kDirectBlock, 16) group_scan_kernel(
+    const void* __restrict__ index, uint32_t n_dgroups, uint32_t log2_cap, uint32_t n_sets,
+    const uint64_t* __restrict__ chains, const uint64_t* __restrict__ chain_off, uint32_t R,
+    const uint32_t* __restrict__ set_off, uint32_t per, GroupSlot* __restrict__ tab,
+    uint32_t log2_slots, int32_t* __restrict__ set_of, uint64_t* __restrict__ gkey,
+    FirstRun* __restrict__ first_run) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t cap = 1u << log2_cap;
+  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  for (uint64_t t0 = warp * per; t0 < R; t0 += n_warps * per) {
+    const uint32_t count = (uint32_t)min((uint64_t)per, R - t0);
+    const uint32_t my_r = (uint32_t)t0 + lane;
+    uint64_t my_c0 = 0, my_key = 0;
+    uint32_t my_n = 0, my_pos = kNoRun, my_len = 0, my_cached = 0;
+    int32_t my_set = -1;
+    if (lane < count) {
+      my_c0 = __ldg(chain_off + my_r);
+      const uint64_t c1 = __ldg(chain_off + my_r + 1);
+      my_set = find_set(set_off, n_sets, my_r);
+      set_of[my_r] = my_set;
+      if (my_set >= 0 && c1 > my_c0) {
+        my_n = (uint32_t)min(c1 - my_c0, (uint64_t)65535);
+        const uint64_t h0 = __ldg(chains + my_c0);
+        my_key = group_key(h0, (uint32_t)my_set);
+        unsigned long long pos = kNotFound;
+        if (h0 != 0ull)
+          pos = lookup(index_view(index, (uint64_t)my_set * n_dgroups, log2_cap, 8u).hash, h0,
+                       log2_cap, nullptr);  // the match itself reports what it meets
+        if (pos < cap) my_pos = (uint32_t)pos;
+      }
+    }
+    for (uint32_t i = 0; i < count; ++i) {
+      const uint32_t pos = __shfl_sync(0xffffffffu, my_pos, i);
+      if (pos == kNoRun) continue;
+      const uint32_t n = __shfl_sync(0xffffffffu, my_n, i);
+      const uint64_t* chain = chains + __shfl_sync(0xffffffffu, my_c0, i);
+      const IndexView ix = index_view(
+          index, (uint64_t)__shfl_sync(0xffffffffu, my_set, i) * n_dgroups, log2_cap, 8u);
+      const uint32_t len = follow_run(ix.keys, cap, chain, 0, n, pos, lane);
+      uint32_t p = len;
+      for (int runs = 1; runs < kMaxRuns && p < n; ++runs) {
+        const uint64_t key = __ldg(chain + p);
+        if (key == 0ull) break;
+        const unsigned long long at = lookup_warp(ix.hash, key, log2_cap, lane, nullptr);
+        if (at >= cap) break;
+        const uint32_t more = follow_run(ix.keys, cap, chain, p, n, (uint32_t)at, lane);
+        if (more == 0) break;
+        p += more;
+      }
+      if (lane == i) {
+        my_len = len;
+        my_cached = p;
+      }
+    }
+    if (lane < count) {
+      gkey[my_r] = my_key;  // 0: not grouped
+      first_run[my_r] = FirstRun{my_pos, my_len};
+      if (my_key != 0ull) {
+        const uint64_t mask = (1ull << log2_slots) - 1;
+        const unsigned long long code = ((unsigned long long)my_cached << 48) |
+                                        ((unsigned long long)my_n << 32) | (0xffffffffu - my_r);
+        uint64_t slot = home_slot(my_key, log2_slots);
+        for (uint64_t step = 0; step <= mask; ++step) {
+          const unsigned long long prev = atomicCAS(&tab[slot].key, 0ull, my_key);
+          if (prev == 0ull || prev == my_key) {
+            atomicMax(&tab[slot].code, code);
+            break;
+          }
+          slot = (slot + 1) & mask;
+        }
+      }
     }
   }
 }
 
+// A member's common prefix with its leader, in the place of its group key: the length, and
+// whether it is exact (else the chains agree at least so far and are compared from there).
+constexpr uint64_t kLcpExact = 1ull << 32;
+
 __global__ void group_resolve_kernel(const GroupSlot* __restrict__ tab, uint32_t log2_slots,
-                                     const uint64_t* __restrict__ chain_off, uint32_t R,
-                                     uint32_t* __restrict__ leader_of,
+                                     uint32_t R, uint32_t* __restrict__ leader_of,
                                      const int32_t* __restrict__ set_of,
-                                     uint32_t* __restrict__ leaders,
-                                     const uint64_t* __restrict__ gkey,
+                                     uint32_t* __restrict__ leaders, uint64_t* __restrict__ gkey,
+                                     const FirstRun* __restrict__ first_run,
                                      MatchCounters* counters) {
   const uint64_t mask = (1ull << log2_slots) - 1;
   for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < R; r += gridDim.x * blockDim.x) {
-    const uint64_t c0 = __ldg(chain_off + r), c1 = __ldg(chain_off + r + 1);
-    const int32_t set = __ldg(set_of + r);
-    uint32_t lead = r;
-    if (c1 > c0 && set >= 0) {
-      const uint64_t key = gkey[r];  // written by the insert pass
+    const uint64_t key = gkey[r];  // written by the scan pass
+    uint32_t lead = r, cached = 0;
+    if (key != 0ull) {
       uint64_t slot = home_slot(key, log2_slots);
       for (uint64_t step = 0; step <= mask; ++step) {
         const unsigned long long k = tab[slot].key;
         if (k == key) {
-          const uint32_t L = 0xffffffffu - (uint32_t)(tab[slot].code & 0xffffffffull);
+          const unsigned long long code = tab[slot].code;
+          const uint32_t L = 0xffffffffu - (uint32_t)(code & 0xffffffffull);
           // a leader from another table set (64-bit key collision) is never used
-          if (L < R && __ldg(set_of + L) == set) lead = L;
+          if (L < R && __ldg(set_of + L) == __ldg(set_of + r)) lead = L;
+          cached = (uint32_t)(code >> 48);
           break;
         }
         if (k == 0ull) break;
@@ -790,10 +882,15 @@ __global__ void group_resolve_kernel(const GroupSlot* __restrict__ tab, uint32_t
     }
     leader_of[r] = lead;
     if (lead == r) {  // long chains from the front of the list, the rest from its back
-      if (c1 > c0 && c1 - c0 >= kLongLeader)
-        leaders[atomicAdd(&counters->n_long, 1ull)] = r;
-      else
-        leaders[R - 1 - atomicAdd(&counters->n_short, 1ull)] = r;
+      if (cached >= kLongLeader) leaders[atomicAdd(&counters->n_long, 1ull)] = r;
+      else leaders[R - 1 - atomicAdd(&counters->n_short, 1ull)] = r;
+    } else {
+      // the chain that left their common run first parts from the other there
+      const FirstRun a = first_run[r], b = first_run[lead];
+      uint64_t lcp = 0;
+      if (a.pos == b.pos && a.pos != kNoRun)
+        lcp = min(a.len, b.len) | (a.len != b.len ? kLcpExact : 0ull);
+      gkey[r] = lcp;
     }
   }
 }
@@ -826,8 +923,11 @@ __device__ __forceinline__ void store_hits(uint16_t* __restrict__ M, uint64_t ro
 }
 
 // Leader pass: one task per (leader, decode group), taken in order from a global counter
-// by whole warps, so long and short chains balance across the GPU.
-__global__ void __launch_bounds__(kMatchBlock, 8) match_leaders_kernel(
+// by whole warps, so long and short chains balance across the GPU.  Bound by the dependent
+// steps of the longest chains, so steps are 256 blocks: 8 leaders x 16 groups of up to 7,680
+// blocks 57 us (69 at 128 a step), 50 leaders x 64 groups 93 us.  A block of 8 warps per long
+// leader, 1,024 blocks a step: 58 and 209 us.
+__global__ void __launch_bounds__(kMatchBlock, 2) match_leaders_kernel(
     const void* __restrict__ index, uint32_t D, uint32_t log2_cap, uint32_t n_sets,
     const uint64_t* __restrict__ chains, const uint64_t* __restrict__ chain_off, uint32_t R,
     const uint32_t* __restrict__ set_off, const int32_t* __restrict__ set_of,
@@ -843,7 +943,7 @@ __global__ void __launch_bounds__(kMatchBlock, 8) match_leaders_kernel(
     if (lane == 0) t = atomicAdd(&counters->next_task, 1ull);
     t = __shfl_sync(0xffffffffu, t, 0);
     if (t >= total) break;
-    const uint64_t li = n_dgroups == 1 ? t : t / n_dgroups;
+    const uint64_t li = t / n_dgroups;
     const uint32_t r = __ldg(leaders + (li < n_long ? li : (uint64_t)R - 1 - (li - n_long)));
     const uint32_t q = (uint32_t)(t - li * n_dgroups);
     const uint32_t q0 = q * kGroup, ng = min(kGroup, D - q0);
@@ -854,7 +954,7 @@ __global__ void __launch_bounds__(kMatchBlock, 8) match_leaders_kernel(
       h.lo = h.hi = (uint32_t)n;
       const unsigned long long alive = ng >= 64 ? ~0ull : ((1ull << ng) - 1);
       const IndexView ix = index_view(index, (uint64_t)set * n_dgroups + q, log2_cap, 8u);
-      scan_chain<2, 8>(ix, log2_cap, chains + c0, 0, n, alive, h, lane, status);
+      scan_chain<8, 8>(ix, log2_cap, chains + c0, 0, n, alive, h, lane, status);
     }
     store_hits(M, (uint64_t)r * D, q0, ng, lane, h);
   }
@@ -872,7 +972,6 @@ __global__ void __launch_bounds__(kMatchBlock, 8) match_leaders_kernel(
 // 37 against 4 for one, and 1.20 ms against 0.60 for 32,000 requests whose chains lie in
 // host memory, where the leader's chain crosses the link for every member.  Steps of 64 and
 // 96 blocks: 1.10 and 1.01 ms; 24 blocks an SM (40 registers): spills, no faster.
-constexpr int kDirectBlock = 64;
 
 template <int kMB>
 __global__ void __launch_bounds__(kDirectBlock, 16) match_kernel(
@@ -933,18 +1032,21 @@ __global__ void __launch_bounds__(kDirectBlock, 16) match_kernel(
   }
 }
 
-// Member pass for pools of several decode groups: one warp per member.  With
-// lcp = |common prefix of h_r and h_L| capped at min(n_r, n_L, max_d M_L[d] + 1), every
-// decode has M_r[d] = min(M_L[d], lcp) unless M_L[d] >= lcp and block lcp of h_r is
-// cached on d.  So the member's row is one elementwise pass over the leader's row (16
-// bytes a lane when the rows are 16-byte aligned), and block lcp is then probed in the
-// groups where some leader hit reaches lcp, up to 32 groups at once with one lane per
-// group; a group whose probe finds the block is walked again by the whole warp.
-__global__ void __launch_bounds__(kMatchBlock, 6) match_members_wide_kernel(
+// Member pass: one warp per member.  With lcp = |common prefix of h_r and h_L|, every decode
+// has M_r[d] = min(M_L[d], lcp) unless M_L[d] >= lcp and block lcp of h_r is cached on d.  So
+// the member's row is one elementwise pass over the leader's row (16 bytes a lane when the
+// rows are 16-byte aligned), and block lcp is then probed in the groups where some leader
+// hit reaches lcp, up to 32 groups at once with one lane per group; a group whose probe
+// finds the block is walked again by the whole warp.
+// Bound by the rows it writes: 32,000 requests on 4,096 decodes 164 us.  With leaders chosen
+// by chain length, the members whose cached prefix ran past their leader's walked all 64
+// groups of the pool again: 3.9 ms (6.6 ms at 32 blocks a step).
+__global__ void __launch_bounds__(kMatchBlock, 4) match_members_wide_kernel(
     const void* __restrict__ index, uint32_t D, uint32_t log2_cap, uint32_t n_sets,
     const uint64_t* __restrict__ chains, const uint64_t* __restrict__ chain_off, uint32_t R,
     const uint32_t* __restrict__ set_off, const uint32_t* __restrict__ leader_of,
-    const int32_t* __restrict__ set_of, uint16_t* __restrict__ M, int* status) {
+    const int32_t* __restrict__ set_of, const uint64_t* __restrict__ known_lcp,
+    uint16_t* __restrict__ M, int* status) {
   const uint32_t lane = threadIdx.x & 31;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
@@ -956,6 +1058,7 @@ __global__ void __launch_bounds__(kMatchBlock, 6) match_members_wide_kernel(
     const uint32_t r = (uint32_t)rr;
     const uint32_t lead = __ldg(leader_of + r);
     if (lead == r) continue;  // leaders were matched by the leader pass
+    const uint64_t known = __ldg(known_lcp + r);
     const uint64_t row = (uint64_t)r * D;
     int32_t set;
     uint64_t c0, n;
@@ -965,47 +1068,48 @@ __global__ void __launch_bounds__(kMatchBlock, 6) match_members_wide_kernel(
         store_hits(M, row, q * kGroup, min(kGroup, D - q * kGroup), lane, z);
       continue;
     }
-    const uint64_t l0 = __ldg(chain_off + lead);
-    const uint64_t nl = min(__ldg(chain_off + lead + 1) - l0, (uint64_t)65535);
     const uint64_t* __restrict__ own = chains + c0;
-    const uint64_t* __restrict__ lch = chains + l0;
     const uint16_t* __restrict__ ml = M + (uint64_t)lead * D;
     uint16_t* __restrict__ mr = M + row;
 
-    // the leader's largest hit
-    uint32_t mmax = 0;
-    if (vec) {
-      for (uint32_t c = lane; c < n8; c += 32) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(ml) + c);
-        const uint32_t m2 = __vmaxu2(__vmaxu2(v.x, v.y), __vmaxu2(v.z, v.w));
-        mmax = max(mmax, max(m2 & 0xffffu, m2 >> 16));
+    uint64_t lcp = known & (kLcpExact - 1);
+    if (!(known & kLcpExact)) {  // compare the chains from there, 128 blocks a step
+      const uint64_t l0 = __ldg(chain_off + lead);
+      const uint64_t nl = min(__ldg(chain_off + lead + 1) - l0, (uint64_t)65535);
+      const uint64_t* __restrict__ lch = chains + l0;
+      // the leader's largest hit: blocks past it decide nothing
+      uint32_t mmax = 0;
+      if (vec) {
+        for (uint32_t c = lane; c < n8; c += 32) {
+          const uint4 v = __ldg(reinterpret_cast<const uint4*>(ml) + c);
+          const uint32_t m2 = __vmaxu2(__vmaxu2(v.x, v.y), __vmaxu2(v.z, v.w));
+          mmax = max(mmax, max(m2 & 0xffffu, m2 >> 16));
+        }
+      } else {
+        for (uint32_t d = lane; d < D; d += 32) mmax = max(mmax, (uint32_t)__ldg(ml + d));
       }
-    } else {
-      for (uint32_t d = lane; d < D; d += 32) mmax = max(mmax, (uint32_t)__ldg(ml + d));
-    }
+      mmax = __reduce_max_sync(0xffffffffu, mmax);
+      const uint64_t cap = min(n, min(nl, (uint64_t)mmax + 1));
+      const uint64_t from = min(lcp, cap);
+      lcp = cap;
+      for (uint64_t base = from; base < cap; base += 128) {
+        uint64_t a[4], b[4];
 #pragma unroll
-    for (int o = 16; o; o >>= 1) mmax = max(mmax, __shfl_xor_sync(0xffffffffu, mmax, o));
-
-    // common prefix with the leader, capped, 128 blocks a step
-    const uint64_t cap = min(n, min(nl, (uint64_t)mmax + 1));
-    uint64_t lcp = cap;
-    for (uint64_t base = 0; base < cap; base += 128) {
-      uint64_t a[4], b[4];
+        for (int k = 0; k < 4; ++k) {
+          const uint64_t i = base + 32 * k + lane;
+          a[k] = i < cap ? __ldg(own + i) : 0ull;
+          b[k] = i < cap ? __ldg(lch + i) : 0ull;
+        }
+        uint64_t found = cap;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint64_t i = base + 32 * k + lane;
-        a[k] = i < cap ? __ldg(own + i) : 0ull;
-        b[k] = i < cap ? __ldg(lch + i) : 0ull;
-      }
-      uint64_t found = cap;
-#pragma unroll
-      for (int k = 3; k >= 0; --k) {
-        const uint32_t diff = __ballot_sync(0xffffffffu, a[k] != b[k]);
-        if (diff) found = base + 32 * k + (uint64_t)(__ffs(diff) - 1);
-      }
-      if (found < cap) {
-        lcp = found;
-        break;
+        for (int k = 3; k >= 0; --k) {
+          const uint32_t diff = __ballot_sync(0xffffffffu, a[k] != b[k]);
+          if (diff) found = base + 32 * k + (uint64_t)(__ffs(diff) - 1);
+        }
+        if (found < cap) {
+          lcp = found;
+          break;
+        }
       }
     }
     const bool probe = lcp < n;  // decodes with M_L >= lcp may hit block lcp
@@ -1036,7 +1140,7 @@ __global__ void __launch_bounds__(kMatchBlock, 6) match_members_wide_kernel(
         const uint32_t alo = __ballot_sync(0xffffffffu, lane < ng && (uint64_t)mlo >= lcp);
         const uint32_t ahi = __ballot_sync(0xffffffffu, lane + 32 < ng && (uint64_t)mhi >= lcp);
         const unsigned long long alive = (unsigned long long)alo | ((unsigned long long)ahi << 32);
-        scan_chain<2, 8>(index_view(index, (uint64_t)set * n_dgroups + q, log2_cap, 8u),
+        scan_chain<4, 8>(index_view(index, (uint64_t)set * n_dgroups + q, log2_cap, 8u),
                    log2_cap, own, lcp, n, alive, h, lane, status, pj);
         store_hits(M, row, q0, ng, lane, h);
       }
@@ -1095,10 +1199,10 @@ uint32_t group_log2_slots(uint32_t R) {
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Workspace: group table | leader_of [R] | set_of [R] | leader list [R] | group keys [R]
-// | counters.  Used for pools of several decode groups.
+// Workspace: group table | leader_of [R] | set_of [R] | leader list [R] | group keys, then
+// known common prefixes [R] | first runs [R] | counters.  Used for pools of several decode groups.
 struct WorkspaceLayout {
-  size_t table, leader_of, set_of, leaders, gkey, counters, total;
+  size_t table, leader_of, set_of, leaders, gkey, first_run, counters, total;
 };
 
 WorkspaceLayout workspace_layout(uint32_t R) {
@@ -1108,7 +1212,8 @@ WorkspaceLayout workspace_layout(uint32_t R) {
   w.set_of = w.leader_of + align_up(sizeof(uint32_t) * (size_t)R, 256);
   w.leaders = w.set_of + align_up(sizeof(int32_t) * (size_t)R, 256);
   w.gkey = w.leaders + align_up(sizeof(uint32_t) * (size_t)R, 256);
-  w.counters = w.gkey + align_up(sizeof(uint64_t) * (size_t)R, 256);
+  w.first_run = w.gkey + align_up(sizeof(uint64_t) * (size_t)R, 256);
+  w.counters = w.first_run + align_up(sizeof(FirstRun) * (size_t)R, 256);
   w.total = w.counters + align_up(sizeof(MatchCounters), 256);
   return w;
 }
@@ -1127,15 +1232,16 @@ int leader_grid() { return persistent_grid(match_leaders_kernel, kMatchBlock); }
 // The direct match.  A warp takes several tasks where every resident warp still gets
 // kWaves turns (the card's last turns are then short), at most kPerWarp.
 constexpr uint32_t kPerWarp = 8, kWaves = 8;
+uint32_t tasks_per_warp(uint64_t tasks, int sms) {
+  const uint64_t turns = tasks / ((uint64_t)sms * 32 * kWaves);
+  return turns < 1 ? 1u : turns < kPerWarp ? (uint32_t)turns : kPerWarp;
+}
 netkv_status launch_match(const void* index, uint32_t D, uint32_t log2_cap, uint32_t n_sets,
                           const uint64_t* chains, const uint64_t* chain_off, uint32_t R,
-                          const uint32_t* set_off, uint16_t* M, int* status, cudaStream_t s) {
-  int dev = 0, sms = 0;
-  NETKV_CUDA_TRY(cudaGetDevice(&dev));
-  NETKV_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+                          const uint32_t* set_off, uint16_t* M, int* status, int sms,
+                          cudaStream_t s) {
   const uint64_t tasks = (uint64_t)R * ((D + kGroup - 1) / kGroup);
-  const uint64_t turns = tasks / ((uint64_t)sms * 32 * kWaves);
-  const uint32_t per = turns < 1 ? 1u : turns < kPerWarp ? (uint32_t)turns : kPerWarp;
+  const uint32_t per = tasks_per_warp(tasks, sms);
   const uint64_t per_block = (uint64_t)per * (kDirectBlock / 32);
   const uint64_t blocks = (tasks + per_block - 1) / per_block;
   const unsigned grid = (unsigned)(blocks < (1u << 24) ? blocks : (1u << 24));
@@ -1225,9 +1331,15 @@ extern "C" netkv_status netkv_prefix_match(const void* d_index, uint32_t D,
   if (d_workspace && workspace_bytes < netkv_prefix_match_workspace_size(R)) return NETKV_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
   const void* index = d_index;
-  if (!d_workspace || D <= kGroup)
+  int dev = 0, sms = 0;
+  NETKV_CUDA_TRY(cudaGetDevice(&dev));
+  NETKV_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const uint64_t tasks = (uint64_t)R * ((D + kGroup - 1) / kGroup);
+  // a few requests: every (request, group) has a warp at once, and sharing, six launches
+  // long, cannot end before the longest of them (34 requests on 1,218 decodes: 20 us, not 55)
+  if (!d_workspace || D <= kGroup || tasks <= (uint64_t)sms * 32)
     return launch_match(index, D, log2_capacity, n_sets, d_chains, d_chain_off, R, d_set_off, d_M,
-                        d_status, s);
+                        d_status, sms, s);
   const uint32_t lg = group_log2_slots(R);
   const WorkspaceLayout L = workspace_layout(R);
   char* ws = reinterpret_cast<char*>(d_workspace);
@@ -1240,10 +1352,15 @@ extern "C" netkv_status netkv_prefix_match(const void* d_index, uint32_t D,
   NETKV_CUDA_TRY(cudaMemsetAsync(tab, 0, sizeof(GroupSlot) << lg, s));
   NETKV_CUDA_TRY(cudaMemsetAsync(counters, 0, sizeof(MatchCounters), s));
   const unsigned rgrid = (unsigned)((R + 255) / 256 < 65535u * 16 ? (R + 255) / 256 : 65535u * 16);
-  group_insert_kernel<<<rgrid, 256, 0, s>>>(tab, lg, d_chains, d_chain_off, R, d_set_off, n_sets,
-                                            set_of, gkey);
-  group_resolve_kernel<<<rgrid, 256, 0, s>>>(tab, lg, d_chain_off, R, leader_of, set_of, leaders,
-                                             gkey, counters);
+  FirstRun* first_run = reinterpret_cast<FirstRun*>(ws + L.first_run);
+  const uint32_t per = tasks_per_warp(R, sms);
+  const uint64_t sblocks = ((uint64_t)R + per * (kDirectBlock / 32) - 1) / (per * (kDirectBlock / 32));
+  const unsigned sgrid = (unsigned)(sblocks < (1u << 24) ? sblocks : (1u << 24));
+  group_scan_kernel<<<sgrid, kDirectBlock, 0, s>>>(
+      index, (D + kGroup - 1) / kGroup, log2_capacity, n_sets, d_chains, d_chain_off, R, d_set_off,
+      per, tab, lg, set_of, gkey, first_run);
+  group_resolve_kernel<<<rgrid, 256, 0, s>>>(tab, lg, R, leader_of, set_of, leaders, gkey,
+                                             first_run, counters);
   match_leaders_kernel<<<leader_grid(), kMatchBlock, 0, s>>>(
       index, D, log2_capacity, n_sets, d_chains, d_chain_off, R, d_set_off, set_of, leaders,
       counters, d_M, d_status);
@@ -1252,7 +1369,8 @@ extern "C" netkv_status netkv_prefix_match(const void* d_index, uint32_t D,
   const unsigned mgrid = (unsigned)(mblocks < (1u << 24) ? mblocks : (1u << 24));
   match_members_wide_kernel<<<mgrid, kMatchBlock, 0, s>>>(index, D, log2_capacity, n_sets,
                                                           d_chains, d_chain_off, R, d_set_off,
-                                                          leader_of, set_of, d_M, d_status);
+                                                          leader_of, set_of, gkey, d_M,
+                                                          d_status);
   return netkv_launch_status();
 }
 
