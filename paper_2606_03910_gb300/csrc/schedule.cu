@@ -25,8 +25,6 @@
 
 namespace {
 
-constexpr uint32_t kNone = 0xffffffffu;
-
 __device__ __forceinline__ void combine(float& b, uint32_t& i, float& s, float b2, uint32_t i2,
                                         float s2) {
   const bool other = (b2 < b) || (b2 == b && i2 < i);
@@ -49,55 +47,6 @@ __device__ __forceinline__ void seg_argmin(float& b, uint32_t& i, float& s, uint
     const float s2 = __shfl_xor_sync(mask, s, o, LPS);
     combine(b, i, s, b2, i2, s2);
   }
-}
-
-// Order-preserving 32-bit keys of fp32 scores, so that warp-wide redux minima give the
-// (score, rank) argmin; kNoKey (above every float's key) stands for "no candidate".
-constexpr uint32_t kNoKey = 0xffffffffu;
-__device__ __forceinline__ uint32_t score_key(float x) {
-  const uint32_t u = __float_as_uint(__fadd_rn(x, 0.0f));  // -0 and +0 tie, as compared
-  return u ^ ((uint32_t)((int32_t)u >> 31) | 0x80000000u);
-}
-__device__ __forceinline__ float key_score(uint32_t k) {
-  if (k == kNoKey) return __int_as_float(0x7f800000);
-  return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xffffffffu));
-}
-// Block-free argmin over the 32 lanes of a warp: (best key, its lowest rank, second key),
-// where a lane offers (key, rank, key of its own runner-up).
-__device__ __forceinline__ void warp_argmin_keys(uint32_t& key, uint32_t& rank, uint32_t& key2) {
-  const uint32_t bk = __reduce_min_sync(0xffffffffu, key);
-  const uint32_t br = __reduce_min_sync(0xffffffffu, key == bk ? rank : kNone);
-  // the winning lane offers its runner-up; every other lane its best
-  const uint32_t sk = __reduce_min_sync(0xffffffffu, (key == bk && rank == br) ? key2 : key);
-  key = bk;
-  rank = br;
-  key2 = sk;
-}
-
-// The paper's compute-load model (Sec. III-C, IV-B) as kernel parameters.
-struct LoadModel {
-  float t_a, t_b;      // t_iter(beta) = t_a + t_b * beta
-  int32_t beta_max;
-  int64_t m_min, m0;
-};
-
-// Self-contention (Eq. 4's n_inflight, Algorithm 1 lines 5 and 14, Sec. V-C): the
-// candidate's bandwidth is divided by 1 + n; T is returned for the completion time.
-__device__ __forceinline__ float contended_score(const netkv_weights& w, uint32_t l, uint32_t m,
-                                                 float ub_p, float ub_d, float lat_tau,
-                                                 uint32_t n, float& T, int* status) {
-  uint32_t lam = 16u * m;
-  if (m > l / 16u) {
-    flag_status(status, NETKV_DEV_EDOMAIN);
-    lam = lam < l ? lam : l;
-  }
-  const uint32_t miss_tok = l - lam;
-  const float bb = fminf(ub_p, ub_d);
-  const float b_eff = n ? bb / (float)(1u + n) : bb;
-  const float s_eff = (float)((int64_t)miss_tok * (int64_t)w.bytes_per_token);
-  T = s_eff / b_eff + lat_tau;
-  const float miss = (float)miss_tok / (float)l;
-  return w.w_net * T + w.w_prefix * miss;
 }
 
 // combine() carrying the winner's transfer time along
@@ -125,39 +74,6 @@ __device__ __forceinline__ void seg_argmin_t(float& b, uint32_t& i, float& s, fl
     combine_t(b, i, s, tt, b2, i2, s2, t2);
   }
 }
-
-// Pending transfer completions of one stream: a binary min-heap in shared memory kept by
-// the stream's lead thread, keys (completion time in us << 16) | (prefill rank << 2) | tier.
-struct DoneHeap {
-  unsigned long long* a;
-  uint32_t n, cap;
-  __device__ bool push(unsigned long long k) {
-    if (n == cap) return false;
-    uint32_t i = n++;
-    while (i > 0) {
-      const uint32_t p = (i - 1) >> 1;
-      if (a[p] <= k) break;
-      a[i] = a[p];
-      i = p;
-    }
-    a[i] = k;
-    return true;
-  }
-  __device__ void pop() {
-    const unsigned long long k = a[--n];
-    if (n == 0) return;
-    uint32_t i = 0;
-    for (;;) {
-      uint32_t c = 2 * i + 1;
-      if (c >= n) break;
-      if (c + 1 < n && a[c + 1] < a[c]) ++c;
-      if (a[c] >= k) break;
-      a[i] = a[c];
-      i = c;
-    }
-    a[i] = k;
-  }
-};
 
 // s_eff / Bbot, the factor self-contention multiplies by 1 + n (Eq. 4): written beside
 // the base scores when the greedy runs with self-contention.
@@ -956,12 +872,8 @@ __global__ void __launch_bounds__(BLOCK) schedule_kernel(
         if (kLoad) {  // Sec. IV-B: T_queue + T_decode; Sec. IV-A: m_d >= s_eff + m_min
           const uint32_t lam = min(16u * m[j], l);
           feasible = load[j] >= (int64_t)(l - lam) * (int64_t)w.bytes_per_token + lm.m_min;
-          const int32_t beta = min(held[j], lm.beta_max);
-          const int32_t blocked = (held[j] - beta) - (lm.beta_max - beta);
-          const float t_queue = (blocked > 0 ? (float)blocked : 0.0f) * (lm.t_a + lm.t_b * (float)beta);
-          const float t_decode = lm.t_a + lm.t_b * (float)(beta + 1);
           sc = base_score(w, l, m[j], pick4(ubp, tau[j]), ubd[j], pick4(lat, tau[j]), status) +
-               w.w_load * (t_queue + t_decode);
+               w.w_load * load_term(lm, held[j]);
         } else if (kBase && kInfl) {  // base + w_net (s_eff / Bbot) n: Eq. 4's 1 + n
           const uint32_t n = (cw >> (8 * tau[j])) & 0xffu;
           sc = (__uint_as_float(m[j]) + w.w_net * (xv[j] * (float)n)) +
@@ -2075,6 +1987,7 @@ __global__ void __launch_bounds__(32 * kWinWarps) schedule_window_kernel(
   if (mine) load_final[(uint64_t)stream * D + sl] = load;
 }
 
+constexpr uint32_t kSmallMaxStreams = 4096;
 constexpr int kStages = 8;
 constexpr uint32_t kHeapPerStream = 4096;       // pending completions, one stream per CTA
 constexpr uint32_t kHeapPerPackedStream = 256;  // pending completions, packed streams
@@ -2219,6 +2132,13 @@ netkv_status launch(const TopoArgs& t, uint32_t n_streams, const netkv_weights* 
                            d_event_off, d_load_init, d_dec, d_best, d_second, d_load_final,
                            d_base, lw->lists, lw->bounds, d_status, s);
     }
+    if (t.D <= 32 && n_streams <= kSmallMaxStreams) {
+      netkv_status st;
+      if (launch_small_plain(t, n_streams, d_w, R, d_len, d_prefill, d_snap, n_snap, d_events,
+                             d_event_off, d_load_init, d_dec, d_best, d_second, d_load_final,
+                             d_base, d_status, s, &st))
+        return st;
+    }
     if (LPS == 32) {
       // one CTA per stream: the walk is bound by each warp's chain of dependent
       // instructions per event; 16 warps (4 per scheduler) measured best on 4,096 decodes
@@ -2274,6 +2194,14 @@ netkv_status launch_inflight(const TopoArgs& t, uint32_t n_streams, const netkv_
   const uint32_t infl_bytes = ((t.P * 4u + 15u) & ~15u) + heap_cap * 8u;
   const size_t smem = (size_t)per_cta * infl_bytes;
   if (smem > kInflightSmemMax) return NETKV_EINVAL;
+  // without a workspace, pools whose candidates fit in shared memory take the walk that
+  // prepares them a window ahead
+  netkv_status st;
+  if (!d_base && launch_model_inflight(t, n_streams, d_w, R, d_len, d_prefill, d_snap,
+                                       d_arrival_us, d_M, d_UB, n_snap, d_events, d_event_off,
+                                       inflight_cap, heap_cap, d_load_init, d_dec, d_best,
+                                       d_second, d_xfer_us, d_load_final, d_status, s, &st))
+    return st;
   if (d_base) {  // base scores and s_eff / Bbot of every arrival first, in parallel
     if (launch_base(t, n_streams, d_w, R, d_len, d_prefill, d_snap, d_M, d_UB, n_snap, d_events,
                     d_event_off, d_base, d_X, d_status, s) != NETKV_OK)
@@ -2495,6 +2423,12 @@ extern "C" netkv_status netkv_schedule_streams_load(
   cudaStream_t s = (cudaStream_t)stream;
   const LoadModel lm = {model->t_a_s, model->t_b_s, model->beta_max, model->m_min_bytes,
                         model->m0_bytes};
+  netkv_status st;
+  if (launch_model_load(t, n_streams, d_w, model->t_a_s, model->t_b_s, model->beta_max,
+                        model->m_min_bytes, model->m0_bytes, R, d_len, d_prefill, d_snap, d_M,
+                        d_UB, n_snap, d_events, d_event_off, d_m_init, d_n_init, d_dec, d_best,
+                        d_second, d_m_final, d_n_final, d_status, s, &st))
+    return st;
 #define NETKV_LOAD(NPT, BLOCK, LPS)                                                             \
   do {                                                                                          \
     const uint32_t per_cta = LPS == 32 ? 1u : 32u / LPS;                                        \

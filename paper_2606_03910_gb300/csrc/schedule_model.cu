@@ -1,0 +1,1025 @@
+// The greedy's walks with one CTA per stream: warp 0 walks the stream's events in order, the
+// other warps ("producers") work one window of events ahead and put what an arrival's
+// candidates contribute besides the stream's own state into shared memory.
+//
+//   plain            base scores precomputed in global memory (base_kernel): copied
+//   self-contention  Eq. 4's n_inflight: network and prefix terms without contention, and
+//                    the parts contention needs, computed by the producers
+//   load model       Sec. IV-B: network and prefix terms and missed tokens, by the producers
+//
+// So an arrival costs the walker one or two shared-memory loads, a fused multiply-add and a
+// comparison per decode, and a warp reduction; windows are double-buffered and the two
+// sides meet at one block barrier a window.  Scores are those of schedule_kernel bit for
+// bit (the same expressions on the same values); that kernel, which evaluates the
+// candidates between two events, spends 1.3 us an event on the last two forms.
+//   schedule_small_kernel  pools of at most 32 decodes: lane d holds decode d's state in
+//                          registers and the argmin is one reduction and one ballot
+//   schedule_model_kernel  larger pools, self-contention and load model: the state lies in
+//                          shared memory, lane i takes decodes i, i + 32, ...
+// Bound by the walker's chain of dependent instructions per event.
+#include <math.h>
+
+#include "score.cuh"
+
+namespace {
+
+constexpr uint32_t kBadCode = 0xffffffffu;
+constexpr uint32_t kSlotBit = 0x40000000u;  // a departure whose arrival is in its window: the slot
+constexpr uint32_t kMaxWindow = 32;         // events per window: one a lane
+constexpr int kAhead = 4;                   // candidates a producer thread has in flight
+constexpr size_t kModelSmem = 227u * 1024u; // dynamic shared memory of one CTA
+
+enum EventType : uint32_t { kNoEvent = 0, kArrival = 1, kDeparture = 2, kBadArrival = 3 };
+
+// An event with what its candidates share, filled one window ahead.
+struct __align__(16) ModelEvent {
+  uint4 lp;        // the prefill's links
+  float4 ubp;      // and level bottlenecks
+  uint32_t code, type, l, pr;
+  long long now;   // arrival time (self-contention)
+  int32_t dd;      // a departure's decode as recorded in global memory
+  uint32_t miss;   // and the missed tokens of its request there (load model)
+  uint32_t k, pad[3];
+};
+
+enum Walk { kPlain = 0, kContend = 1, kModel = 2 };
+
+// A candidate under self-contention: apart from its score without contention, the parts
+// that contention needs (read only while a counter of the prefill is up).
+struct __align__(16) XferRow {
+  float s_eff, bb, miss;
+  uint32_t tau;
+};
+// Whole microseconds of a transfer time (at most 2^31 - 1).
+__device__ __forceinline__ int32_t whole_us(float T) {
+  const float us = T * 1.0e6f;
+  return (int32_t)(us < 2147483520.0f ? __float2ll_rn(us) : 2147483647ll);
+}
+// (float)x of a load: through int32 when it fits (the same value, without the slow 64-bit
+// conversion, which stays out of line so that it is not evaluated on the common path)
+__device__ __noinline__ float wide_to_float(int64_t x) { return (float)x; }
+__device__ __forceinline__ float load_to_float(int64_t x) {
+  if (__builtin_expect(x == (int64_t)(int32_t)x, 1)) return (float)(int32_t)x;
+  return wide_to_float(x);
+}
+__device__ __forceinline__ float latency_of(const TopoArgs& t, uint32_t tau) {
+  return tau == 0 ? t.lat[0] : tau == 1 ? t.lat[1] : tau == 2 ? t.lat[2] : t.lat[3];
+}
+
+// Byte offsets of the dynamic shared memory.
+struct ModelLayout {
+  uint32_t win;
+  uint32_t ev, arr, narr, wd, wmiss, wb, ws, wx, state, term, held, cnt, heap, rel, base, rows, dt,
+      total;
+};
+
+ModelLayout model_layout(Walk walk, bool small, uint32_t D, uint32_t P, uint32_t heap_cap,
+                         uint32_t win) {
+  ModelLayout a;
+  uint32_t at = 0;
+  auto take = [&](size_t bytes) {
+    const uint32_t o = at;
+    at += (uint32_t)((bytes + 15) / 16 * 16);
+    return o;
+  };
+  const bool infl = walk == kContend;
+  const size_t cand = (size_t)2 * win * D;
+  a.win = win;
+  a.ev = take(2 * win * sizeof(ModelEvent));
+  a.arr = take(2 * kMaxWindow * 4);
+  a.narr = take(2 * 4);
+  // state and results of the larger pools; the small walk keeps both in registers
+  a.wd = take(small ? 0 : 2 * kMaxWindow * 4);
+  a.wmiss = take(small ? 0 : 2 * kMaxWindow * 4);
+  a.wb = take(small ? 0 : kMaxWindow * 4);
+  a.ws = take(small ? 0 : kMaxWindow * 4);
+  a.wx = take(small ? 0 : kMaxWindow * 4);
+  a.state = take(small ? 0 : (size_t)D * 8);              // load or free bytes
+  a.term = take(small ? 0 : (size_t)D * (infl ? 8 : 4));  // (headroom, theta * load) or load term
+  a.held = take(small || infl ? 0 : (size_t)D * 4);
+  a.cnt = take(infl ? (size_t)P * 4 : 0);
+  a.heap = take(infl ? (size_t)heap_cap * 8 : 0);
+  a.rel = take(small ? (size_t)(kMaxWindow + 1) * 32 * (walk == kModel ? 8 : 4) : 0);
+  a.base = take(cand * (walk == kModel ? 8 : 4));
+  a.rows = take(infl ? cand * sizeof(XferRow) : 0);
+  a.dt = take(infl ? cand * sizeof(int2) : 0);
+  a.total = at;
+  return a;
+}
+
+struct ModelArgs {
+  TopoArgs t;
+  const netkv_weights* W;
+  uint32_t R, n_snap;
+  const uint32_t *len, *prefill, *snap;
+  const uint16_t* M;
+  const float* UB;
+  const float* base;          // plain: [R][D] base scores
+  const uint32_t* events;
+  const uint64_t* event_off;
+  const int64_t* state_init;  // loads, or free bytes
+  int32_t* dec;
+  float *best, *second;
+  int64_t* state_final;
+  int* status;
+  const int64_t* arrival_us;  // self-contention
+  uint32_t inflight_cap, heap_cap;
+  int32_t* xfer_us;
+  LoadModel lm;               // load model
+  const int32_t* held_init;
+  int32_t* held_final;
+  ModelLayout lay;
+};
+
+// The shared memory of a block, by name.
+struct ModelShared {
+  ModelEvent* ev;    // [2][win]
+  uint32_t* arr;     // [2][kMaxWindow] slots of a window's arrivals
+  uint32_t* narr;    // [2]
+  float* base;       // [2][win][D]
+  uint2* cand;       // load model: (score, missed tokens)
+  XferRow* rows;     // [2][win][D]
+  int2* dt;          // [2][win][D] uncontended transfer time in us, tier
+  uint32_t* cnt;     // self-contention: n_inflight, byte `tier` of cnt[prefill rank]
+  __device__ ModelShared(unsigned char* smem, const ModelLayout& l)
+      : ev(reinterpret_cast<ModelEvent*>(smem + l.ev)),
+        arr(reinterpret_cast<uint32_t*>(smem + l.arr)),
+        narr(reinterpret_cast<uint32_t*>(smem + l.narr)),
+        base(reinterpret_cast<float*>(smem + l.base)),
+        cand(reinterpret_cast<uint2*>(smem + l.base)),
+        rows(reinterpret_cast<XferRow*>(smem + l.rows)),
+        dt(reinterpret_cast<int2*>(smem + l.dt)),
+        cnt(reinterpret_cast<uint32_t*>(smem + l.cnt)) {}
+};
+
+// The producers: in step k of the block they fill window k while the walker walks window
+// k - 1; every step ends with a block barrier.
+template <Walk kWalk, int BT>
+__device__ __forceinline__ void produce(const ModelArgs& a, const netkv_weights& w,
+                                        const ModelShared& S, uint64_t e0, uint64_t e1,
+                                        uint64_t n_win) {
+  constexpr uint32_t NP = BT - 32;
+  const TopoArgs& t = a.t;
+  const uint32_t D = t.D, win = a.lay.win, ptid = threadIdx.x - 32;
+  const uint32_t step_q = NP / D, step_d = NP % D;
+  uint32_t code = ptid < win && e0 + ptid < e1 ? __ldg(a.events + e0 + ptid) : kBadCode;
+  for (uint64_t k = 0; k <= n_win; ++k) {
+    if (k < n_win) {
+      ModelEvent* ev = S.ev + (k & 1) * win;
+      uint32_t* arr = S.arr + (k & 1) * kMaxWindow;
+      if (ptid < 32) {
+        uint32_t type = kNoEvent;
+        if (ptid < win) {
+          ModelEvent x;
+          x.lp = make_uint4(0, 0, 0, 0);
+          x.ubp = make_float4(0.f, 0.f, 0.f, 0.f);
+          x.code = code;
+          x.l = x.pr = x.miss = x.k = 0;
+          x.now = 0;
+          x.dd = -1;
+          const uint32_t r = code & 0x7fffffffu;
+          const uint64_t e = e0 + (k + 1) * win + ptid;
+          const uint32_t next = e < e1 ? __ldg(a.events + e) : kBadCode;
+          if (code == kBadCode) {
+          } else if (r >= a.R) {
+            flag_status(a.status, NETKV_DEV_ERANGE);
+          } else if (code >> 31) {
+            type = kDeparture;
+            x.l = __ldg(a.len + r);
+            x.dd = __ldcg(a.dec + r);  // by the walker, up to the window before the walked one
+            if (kWalk == kModel && x.dd >= 0 && (uint32_t)x.dd < D)
+              x.miss = x.l - min(16u * (uint32_t)__ldg(a.M + (uint64_t)r * D + x.dd), x.l);
+          } else {
+            x.l = __ldg(a.len + r);
+            x.pr = __ldg(a.prefill + r);
+            x.k = __ldg(a.snap + r);
+            if (kWalk == kContend) x.now = __ldg(a.arrival_us + r);
+            if (x.pr < t.P && x.k < a.n_snap && x.l != 0) {
+              type = kArrival;
+              if (kWalk != kPlain) {
+                const uint32_t pinst = __ldg(t.pre + x.pr);
+                x.lp = __ldg(t.links + pinst);
+                x.ubp = __ldg(reinterpret_cast<const float4*>(a.UB) + (uint64_t)x.k * t.N + pinst);
+              }
+            } else {
+              type = kBadArrival;
+              flag_status(a.status, x.l == 0 ? NETKV_DEV_EDOMAIN : NETKV_DEV_ERANGE);
+            }
+          }
+          x.type = type;
+          ev[ptid] = x;
+          code = next;
+        }
+        // the window's arrivals, in order
+        const uint32_t list = __ballot_sync(0xffffffffu, type == kArrival);
+        if (type == kArrival) arr[__popc(list & ((1u << ptid) - 1u))] = ptid;
+        if (ptid == 0) S.narr[k & 1] = __popc(list);
+      }
+      if (BT == 64) __syncwarp();
+      else asm volatile("bar.sync 1, %0;" ::"n"(BT - 32) : "memory");
+      // candidates (arrival, decode), decodes fastest, kAhead of a thread in flight
+      const uint32_t na = S.narr[k & 1];
+      uint32_t q = ptid / D, d = ptid % D;
+      while (q < na) {
+        uint32_t ci[kAhead], cd[kAhead], m[kAhead], inst[kAhead];
+        uint4 ld[kAhead];
+        float ubd[kAhead];
+        int tau[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+          ci[u] = q < na ? arr[q] : kNone;
+          cd[u] = d;
+          if (ci[u] != kNone) {
+            const uint64_t at = (uint64_t)(ev[ci[u]].code & 0x7fffffffu) * D + d;
+            if (kWalk == kPlain) {
+              ubd[u] = __ldg(a.base + at);
+            } else {
+              inst[u] = __ldg(t.dec + d);
+              m[u] = __ldg(a.M + at);
+            }
+          }
+          q += step_q;
+          d += step_d;
+          if (d >= D) {
+            d -= D;
+            ++q;
+          }
+        }
+        if (kWalk != kPlain) {
+#pragma unroll
+          for (int u = 0; u < kAhead; ++u)
+            if (ci[u] != kNone) ld[u] = __ldg(t.links + inst[u]);
+#pragma unroll
+          for (int u = 0; u < kAhead; ++u)
+            if (ci[u] != kNone) {
+              const ModelEvent& x = ev[ci[u]];
+              tau[u] = tier_of(x.lp, ld[u]);
+              ubd[u] = __ldg(a.UB + ((uint64_t)x.k * t.N + inst[u]) * 4 + tau[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+          if (ci[u] == kNone) continue;
+          const size_t at = ((k & 1) * win + ci[u]) * (size_t)D + cd[u];
+          if (kWalk == kPlain) {
+            S.base[at] = ubd[u];
+            continue;
+          }
+          const ModelEvent& x = ev[ci[u]];
+          const float ubp = pick4(x.ubp, tau[u]), lat = latency_of(t, (uint32_t)tau[u]);
+          if (kWalk == kContend) {
+            const XferParts p = xfer_parts(w, x.l, m[u], ubp, ubd[u], a.status);
+            const float T = xfer_time(p, 0u, lat);
+            S.base[at] = w.w_net * T + w.w_prefix * p.miss;
+            S.rows[at] = XferRow{p.s_eff, p.bb, p.miss, (uint32_t)tau[u]};
+            S.dt[at] = make_int2(whole_us(T), tau[u]);
+          } else {
+            const float b = base_score(w, x.l, m[u], ubp, ubd[u], lat, a.status);
+            S.cand[at] = make_uint2(__float_as_uint(b), x.l - min(16u * m[u], x.l));
+          }
+        }
+      }
+    }
+    __syncthreads();  // window k is ready, window k - 1 has been walked
+  }
+}
+
+// The pending completions of a stream and its counters.  The lanes of the walker hold 32 of
+// them, one each, in no order (lowering a counter, floored at zero, commutes); more go to a
+// heap kept by lane 0.
+struct Completions {
+  static constexpr unsigned long long kFree = ~0ull;  // above every key: prefill < 2^14 - 1
+  unsigned long long key;  // time in us << 16 | prefill rank << 2 | tier
+  DoneHeap heap;
+  uint32_t in_heap, cap;   // the same in every lane; cap: pending in all
+  uint32_t* cnt;
+  int* status;
+  __device__ Completions(const ModelArgs& a, unsigned char* smem, uint32_t* c)
+      : key(kFree), in_heap(0), cap(a.heap_cap), cnt(c), status(a.status) {
+    heap.a = reinterpret_cast<unsigned long long*>(smem + a.lay.heap);
+    heap.n = 0;
+    heap.cap = a.heap_cap;
+  }
+  __device__ __forceinline__ void lower(uint32_t pt) {
+    uint32_t* c = cnt + (pt >> 2);
+    const uint32_t sh = 8u * (pt & 3u);
+    if ((*c >> sh) & 0xffu) *c -= 1u << sh;
+  }
+  // Transfers completed by `now` lower their counters (Algorithm 1 line 14's callback).
+  __device__ __forceinline__ void settle(long long now, uint32_t lane) {
+    const bool due = key != kFree && (int64_t)(key >> 16) <= now;
+    uint32_t dm = __ballot_sync(0xffffffffu, due);
+    if (!dm && !in_heap) return;
+    while (dm) {
+      const uint32_t j = __ffs(dm) - 1;
+      dm &= dm - 1;
+      const uint32_t pt = __shfl_sync(0xffffffffu, (uint32_t)key & 0xffffu, j);
+      if (lane == 0) lower(pt);
+    }
+    if (due) key = kFree;
+    if (in_heap) {
+      if (lane == 0) {
+        while (heap.n > 0 && (int64_t)(heap.a[0] >> 16) <= now) {
+          lower((uint32_t)(heap.a[0] & 0xffffu));
+          heap.pop();
+        }
+      }
+      in_heap = __shfl_sync(0xffffffffu, heap.n, 0);
+    }
+    __syncwarp();
+  }
+  // A dispatch on tier tau of prefill pr, whose counters are cw: the counter and the
+  // completion at now + dt.
+  __device__ __forceinline__ void dispatch(long long now, int32_t dt, uint32_t pr, uint32_t tau,
+                                           uint32_t cw, uint32_t most, uint32_t lane) {
+    const unsigned long long k = ((unsigned long long)(now + dt) << 16) |
+                                 ((unsigned long long)pr << 2) | tau;
+    const uint32_t sh = 8u * tau;
+    if (lane == 0 && ((cw >> sh) & 0xffu) < most) cnt[pr] = cw + (1u << sh);
+    const uint32_t free = __ballot_sync(0xffffffffu, key == kFree);
+    if (32u - __popc(free) + in_heap >= cap) {
+      if (lane == 0) flag_status(status, NETKV_DEV_EFULL);
+    } else if (free) {
+      if (lane == (uint32_t)(__ffs(free) - 1)) key = k;
+    } else {
+      if (lane == 0) heap.push(k);
+      ++in_heap;
+    }
+    __syncwarp();
+  }
+};
+
+// The score of a candidate under contention cw (the counters of its prefill's tiers).
+__device__ __forceinline__ float contended(const TopoArgs& t, const netkv_weights& w,
+                                           const XferRow& x, uint32_t cw, float uncontended) {
+  const uint32_t n = (cw >> (8u * x.tau)) & 0xffu;
+  if (n == 0) return uncontended;
+  const XferParts p = {x.s_eff, x.bb, x.miss};
+  const float T = xfer_time(p, n, latency_of(t, x.tau));
+  return w.w_net * T + w.w_prefix * p.miss;
+}
+
+constexpr uint32_t kSumTokens = 1u << 27;  // below: a window's sum of 32 fits in 32 bits
+
+template <Walk kWalk, int BT>
+__global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const TopoArgs& t = a.t;
+  const uint32_t D = t.D, win = a.lay.win, lane = threadIdx.x & 31;
+  const uint32_t stream = blockIdx.x;
+  const netkv_weights w = a.W[stream];
+  const ModelShared S(smem, a.lay);
+  const uint64_t e0 = a.event_off[stream], e1 = a.event_off[stream + 1];
+  const uint64_t n_win = e1 > e0 ? (e1 - e0 + win - 1) / win : 0;
+  if (threadIdx.x >= 32) {
+    produce<kWalk, BT>(a, w, S, e0, e1, n_win);
+    return;
+  }
+
+  // ---- the walker: lane d holds decode d
+  const bool mine = lane < D;
+  uint32_t* rel = reinterpret_cast<uint32_t*>(smem + a.lay.rel);  // [kMaxWindow + 1][32]
+  uint32_t* reln = rel + (kMaxWindow + 1) * 32;                   // load model: departures
+  for (uint32_t q = lane; q < (kMaxWindow + 1) * 32; q += 32) {
+    rel[q] = 0u;
+    if (kWalk == kModel) reln[q] = 0u;
+  }
+  int64_t state = kWalk == kModel ? a.lm.m0 : 0;  // load, or free bytes
+  int32_t held = 0;
+  if (mine && a.state_init) state = a.state_init[(uint64_t)stream * D + lane];
+  if (kWalk == kModel && mine && a.held_init) held = a.held_init[(uint64_t)stream * D + lane];
+  const int64_t bpt = (int64_t)w.bytes_per_token;
+  // what the last dispatch took on its decode's lane (tokens, or missed tokens of one
+  // request), applied with the releases before the next arrival
+  uint32_t own = 0, own_n = 0;
+  Completions done_at(a, smem, S.cnt);
+  if (kWalk == kContend)
+    for (uint32_t p = lane; p < t.P; p += 32) S.cnt[p] = 0u;
+  __syncwarp();
+
+  uint32_t prev_r = kBadCode;  // lane j: event j of the window before: its request, if an arrival,
+  int32_t prev_d = -1;         // its decision and its missed tokens there
+  uint32_t prev_miss = 0;
+  for (uint64_t k = 0; k <= n_win; ++k) {
+    if (k > 0) {
+      const uint32_t buf = (uint32_t)((k - 1) & 1);
+      const ModelEvent* ev = S.ev + buf * win;
+      // lane i prepares event i
+      uint32_t type = kNoEvent, r = kBadCode, l_ev = 0, miss_ev = 0, pr_ev = 0;
+      int32_t dd = -1;
+      long long now_ev = 0;
+      if (lane < win) {
+        const ModelEvent& x = ev[lane];
+        type = x.type;
+        l_ev = x.l;
+        dd = x.dd;
+        miss_ev = x.miss;
+        if (kWalk == kContend) {
+          pr_ev = x.pr;
+          now_ev = x.now;
+        }
+        if (type != kNoEvent) r = x.code & 0x7fffffffu;
+      }
+      const bool is_arr = type == kArrival || type == kBadArrival, is_dep = type == kDeparture;
+      const uint32_t any_arr = __ballot_sync(0xffffffffu, is_arr);
+      const uint32_t arrivals = __ballot_sync(0xffffffffu, type == kArrival);
+      const uint32_t dep_mask = __ballot_sync(0xffffffffu, is_dep);
+      const uint32_t below = (1u << lane) - 1u;
+      bool slow = false;     // a departure released one by one
+      uint32_t my_bj = 0;    // an arrival whose request departs in this window: 1 + the number
+                             // of arrivals before that departure
+      if (dep_mask) {
+        // a departure's arrival may lie in the window before (its decision there) or
+        // earlier in this one (its slot), after the recorded decision was read
+        for (uint32_t j = 0; j < win; ++j) {
+          const uint32_t rj = __shfl_sync(0xffffffffu, prev_r, j);
+          const int32_t dj = __shfl_sync(0xffffffffu, prev_d, j);
+          if (is_dep && rj == r) dd = dj;
+          if (kWalk == kModel) {
+            const uint32_t mj = __shfl_sync(0xffffffffu, prev_miss, j);
+            if (is_dep && rj == r) miss_ev = mj;
+          }
+        }
+        const uint32_t same = __match_any_sync(0xffffffffu, r);
+        const uint32_t mate = same & any_arr & below;  // the departure's arrival
+        const uint32_t leave = same & dep_mask & ~below & ~(1u << lane);  // the arrival's departures
+        if (type == kArrival && __popc(leave) == 1 && l_ev < kSumTokens)
+          my_bj = 1u + __popc(arrivals & ((1u << (__ffs(leave) - 1)) - 1u));
+        if (is_dep && mate) {
+          const uint32_t slot = 31u - __clz(mate);
+          dd = (int32_t)(kSlotBit | slot);
+          // the arrival's dispatch releases it, unless it is large or departs twice
+          slow = l_ev >= kSumTokens || __popc(same & dep_mask & ~((2u << slot) - 1u)) != 1;
+        } else if (is_dep && dd >= 0 && (uint32_t)dd < D) {
+          // tokens released before the window's b-th arrival
+          const uint32_t amount = kWalk == kModel ? miss_ev : l_ev;
+          const uint32_t b = __popc(arrivals & below);
+          if (amount >= kSumTokens) {
+            slow = true;
+          } else {
+            atomicAdd(&rel[b * 32 + dd], amount);
+            if (kWalk == kModel) atomicAdd(&reln[b * 32 + dd], 1u);
+          }
+        }
+        __syncwarp();
+      }
+      const uint32_t leaving = __ballot_sync(0xffffffffu, my_bj != 0u);
+      uint32_t left = __ballot_sync(0xffffffffu, slow);  // slow departures not applied yet
+      int32_t my_d = -1, my_x = -1;  // lane i: event i's decision, transfer time,
+      uint32_t my_miss = 0, my_b = kNoKey, my_s = kNoKey;  // missed tokens there, score keys
+      // the departures of slots in `bits`, one by one
+      auto apply = [&](uint32_t bits) {
+        while (bits) {
+          const uint32_t j = __ffs(bits) - 1;
+          bits &= bits - 1;
+          int32_t d = __shfl_sync(0xffffffffu, dd, j);
+          const uint32_t l = __shfl_sync(0xffffffffu, l_ev, j);
+          uint32_t m = __shfl_sync(0xffffffffu, miss_ev, j);
+          const uint32_t slot = (uint32_t)d & 31u;
+          const int32_t ds = __shfl_sync(0xffffffffu, my_d, slot);
+          const uint32_t ms = __shfl_sync(0xffffffffu, my_miss, slot);
+          if (d >= 0 && ((uint32_t)d & kSlotBit)) {
+            d = ds;
+            m = ms;
+          }
+          if (mine && d == (int32_t)lane) {
+            if (kWalk == kModel) {
+              state += (int64_t)m * bpt;
+              held -= 1;
+            } else {
+              state -= (int64_t)l;
+            }
+          }
+        }
+      };
+      // an arrival's length, this lane's candidate and the releases before it: read one
+      // arrival ahead
+      uint32_t l_n = 0, rel_n = 0, reln_n = 0, miss_n = 0;
+      float net_n = 0.f;
+      auto fetch = [&](uint32_t i) {
+        const size_t row = (buf * win + i) * (size_t)D;
+        l_n = __shfl_sync(0xffffffffu, l_ev, i);
+        if (mine) {
+          if (kWalk == kModel) {
+            const uint2 c = S.cand[row + lane];
+            net_n = __uint_as_float(c.x);
+            miss_n = c.y;
+          } else {
+            net_n = S.base[row + lane];
+          }
+        }
+      };
+      auto fetch_rel = [&](uint32_t b) {
+        rel_n = rel[b * 32 + lane];
+        rel[b * 32 + lane] = 0u;
+        if (kWalk == kModel) {
+          reln_n = reln[b * 32 + lane];
+          reln[b * 32 + lane] = 0u;
+        }
+      };
+      // the last dispatch and the releases since
+      auto advance = [&]() {
+        if (kWalk == kModel) {
+          state += ((int64_t)rel_n - (int64_t)own) * bpt;
+          held += (int32_t)own_n - (int32_t)reln_n;
+          own_n = 0;
+        } else {
+          state += (int64_t)own - (int64_t)rel_n;
+        }
+        own = 0;
+      };
+      uint32_t todo = arrivals, b = 0;
+      if (todo) fetch(__ffs(todo) - 1);
+      fetch_rel(0);
+      while (todo) {
+        const uint32_t i = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const uint32_t l = l_n, miss = miss_n;
+        float net = net_n;
+        advance();
+        const uint32_t before = left & ((1u << i) - 1u);
+        if (before) {
+          apply(before);
+          left &= ~before;
+        }
+        ++b;
+        if (todo) fetch(__ffs(todo) - 1);
+        fetch_rel(b);
+        uint32_t pr = 0, cw = 0;
+        long long now = 0;
+        const size_t row = (buf * win + i) * (size_t)D;
+        if (kWalk == kContend) {
+          pr = __shfl_sync(0xffffffffu, pr_ev, i);
+          now = __shfl_sync(0xffffffffu, now_ev, i);
+          done_at.settle(now, lane);
+          cw = S.cnt[pr];
+          if (cw && mine) net = contended(t, w, S.rows[row + lane], cw, net);
+        }
+        bool feasible;
+        float sc;
+        if (kWalk == kModel) {
+          feasible = mine && state >= (int64_t)miss * bpt + a.lm.m_min;
+          sc = net + w.w_load * load_term(a.lm, held);
+        } else {
+          feasible = mine && state + (int64_t)l <= w.cap_tokens;
+          sc = __fmaf_rn(w.w_load, w.theta_s_per_token * load_to_float(state), net);
+        }
+        const uint32_t key = feasible ? score_key(sc) : kNoKey;
+        const uint32_t kb = __reduce_min_sync(0xffffffffu, key);
+        const uint32_t at_best = __ballot_sync(0xffffffffu, key == kb);
+        const uint32_t one = __reduce_min_sync(0xffffffffu, key == kb ? kNoKey : key);
+        const int32_t dstar = kb == kNoKey ? -1 : (int32_t)(__ffs(at_best) - 1);
+        if (dstar == (int32_t)lane) {
+          own = kWalk == kModel ? miss : l;
+          own_n = 1;
+        }
+        if (leaving >> i & 1u) {
+          // the request departs in this window: its release waits with the others, or
+          // cancels the dispatch where no arrival lies between
+          const uint32_t bj = __shfl_sync(0xffffffffu, my_bj, i) - 1u;
+          if (dstar == (int32_t)lane) {
+            if (bj == b) {
+              own = own_n = 0;
+            } else {
+              rel[bj * 32 + lane] += own;
+              if (kWalk == kModel) reln[bj * 32 + lane] += 1u;
+            }
+          }
+        }
+        int32_t xfer = -1;
+        if (kWalk == kContend && dstar >= 0) {
+          const int2 tt = S.dt[row + dstar];
+          const uint32_t tau = (uint32_t)tt.y, n = (cw >> (8u * tau)) & 0xffu;
+          xfer = tt.x;
+          if (n) {
+            const XferRow x = S.rows[row + dstar];
+            xfer = whole_us(xfer_time(XferParts{x.s_eff, x.bb, x.miss}, n, latency_of(t, tau)));
+          }
+          done_at.dispatch(now, xfer, pr, tau, cw, a.inflight_cap, lane);
+        }
+        const uint32_t taken =
+            kWalk == kModel ? __shfl_sync(0xffffffffu, miss, dstar < 0 ? 0 : dstar) : 0u;
+        if (lane == i) {
+          my_d = dstar;
+          my_miss = taken;
+          my_x = xfer;
+          my_b = kb;
+          my_s = __popc(at_best) >= 2 ? kb : one;
+        }
+      }
+      advance();  // after the window's last arrival
+      apply(left);
+      if (is_arr) {
+        a.dec[r] = my_d;
+        a.best[r] = key_score(my_b);
+        a.second[r] = key_score(my_s);
+        if (kWalk == kContend) a.xfer_us[r] = my_x;
+      }
+      prev_r = is_arr ? r : kBadCode;
+      prev_d = my_d;
+      prev_miss = my_miss;
+    }
+    __syncthreads();
+  }
+  if (mine) {
+    a.state_final[(uint64_t)stream * D + lane] = state;
+    if (kWalk == kModel) a.held_final[(uint64_t)stream * D + lane] = held;
+  }
+}
+
+template <bool kInfl, int BT>
+__global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr Walk kWalk = kInfl ? kContend : kModel;
+  const TopoArgs& t = a.t;
+  const uint32_t D = t.D, win = a.lay.win, lane = threadIdx.x & 31;
+  const uint32_t stream = blockIdx.x;
+  const netkv_weights w = a.W[stream];
+  const ModelShared S(smem, a.lay);
+  const uint64_t e0 = a.event_off[stream], e1 = a.event_off[stream + 1];
+  const uint64_t n_win = e1 > e0 ? (e1 - e0 + win - 1) / win : 0;
+  if (threadIdx.x >= 32) {
+    produce<kWalk, BT>(a, w, S, e0, e1, n_win);
+    return;
+  }
+
+  // ---- the walker
+  int32_t* s_wd = reinterpret_cast<int32_t*>(smem + a.lay.wd);          // [2][kMaxWindow]
+  uint32_t* s_wmiss = reinterpret_cast<uint32_t*>(smem + a.lay.wmiss);  // [2][kMaxWindow]
+  uint32_t* s_wb = reinterpret_cast<uint32_t*>(smem + a.lay.wb);
+  uint32_t* s_ws = reinterpret_cast<uint32_t*>(smem + a.lay.ws);
+  int32_t* s_wx = reinterpret_cast<int32_t*>(smem + a.lay.wx);
+  int64_t* s_state = reinterpret_cast<int64_t*>(smem + a.lay.state);
+  uint2* s_hl = reinterpret_cast<uint2*>(smem + a.lay.term);
+  float* s_term = reinterpret_cast<float*>(smem + a.lay.term);
+  int32_t* s_held = reinterpret_cast<int32_t*>(smem + a.lay.held);
+  auto hl_of = [&](int64_t ld) -> uint2 {  // headroom clamped to 32 bits, theta * load
+    const int64_t h = w.cap_tokens - ld;
+    const uint32_t hr = h <= 0 ? 0u : h >= 0xffffffffll ? 0xffffffffu : (uint32_t)h;
+    return make_uint2(hr, __float_as_uint(w.theta_s_per_token * load_to_float(ld)));
+  };
+  for (uint32_t d = lane; d < D; d += 32) {
+    int64_t x = kInfl ? 0 : a.lm.m0;
+    if (a.state_init) x = a.state_init[(uint64_t)stream * D + d];
+    s_state[d] = x;
+    if (kInfl) {
+      s_hl[d] = hl_of(x);
+    } else {
+      const int32_t n = a.held_init ? a.held_init[(uint64_t)stream * D + d] : 0;
+      s_held[d] = n;
+      s_term[d] = load_term(a.lm, n);
+    }
+  }
+  Completions done_at(a, smem, S.cnt);
+  if (kInfl)
+    for (uint32_t p = lane; p < t.P; p += 32) S.cnt[p] = 0u;
+  __syncwarp();
+  uint32_t prev_r = kBadCode;  // lane j: the request of the window before's event j, if an arrival
+  for (uint64_t k = 0; k <= n_win; ++k) {
+    if (k > 0) {
+      const uint32_t buf = (uint32_t)((k - 1) & 1);
+      const ModelEvent* ev = S.ev + buf * win;
+      int32_t* wd = s_wd + buf * kMaxWindow;
+      uint32_t* wmiss = s_wmiss + buf * kMaxWindow;
+      const int32_t* pd = s_wd + (buf ^ 1) * kMaxWindow;
+      const uint32_t* pmiss = s_wmiss + (buf ^ 1) * kMaxWindow;
+      // lane i prepares event i
+      uint32_t type = kNoEvent, r = kBadCode, my_l = 0, my_miss = 0;
+      int32_t my_dd = -1;
+      long long my_now = 0;
+      uint32_t my_pr = 0;
+      if (lane < win) {
+        const ModelEvent& x = ev[lane];
+        type = x.type;
+        my_l = x.l;
+        my_pr = x.pr;
+        my_now = x.now;
+        my_dd = x.dd;
+        my_miss = x.miss;
+        if (type != kNoEvent) r = x.code & 0x7fffffffu;
+        if (type == kBadArrival) {
+          wd[lane] = -1;
+          s_wb[lane] = s_ws[lane] = kNoKey;
+          s_wx[lane] = -1;
+        }
+      }
+      const bool is_arr = type == kArrival || type == kBadArrival;
+      const uint32_t any_arr = __ballot_sync(0xffffffffu, is_arr);
+      const uint32_t dep_mask = __ballot_sync(0xffffffffu, type == kDeparture);
+      if (dep_mask) {
+        // a departure's arrival may lie in the window before (its decision there) or
+        // earlier in this one (its slot), after the recorded decision was read
+        for (uint32_t j = 0; j < win; ++j) {
+          const uint32_t pr_j = __shfl_sync(0xffffffffu, prev_r, j);
+          if (type == kDeparture && pr_j == r) {
+            my_dd = pd[j];
+            my_miss = pmiss[j];
+          }
+        }
+        const uint32_t same = __match_any_sync(0xffffffffu, r) & any_arr & ((1u << lane) - 1u);
+        if (type == kDeparture && same) my_dd = (int32_t)(kSlotBit | (31u - __clz(same)));
+      }
+      uint32_t arr_mask = __ballot_sync(0xffffffffu, type == kArrival);
+      uint32_t done = 0;  // events before `done` are applied
+      __syncwarp();       // results of bad arrivals are visible
+      // the departures between the last arrival and event `upto`, all at once: they commute
+      auto depart = [&](uint32_t upto) {
+        const uint32_t lo = done >= 32 ? 0u : ~0u << done;
+        const uint32_t hi = upto >= 32 ? ~0u : (1u << upto) - 1u;
+        const uint32_t bm = dep_mask & lo & hi;
+        done = upto;
+        if (!bm) return;
+        uint32_t d = kNone, miss = my_miss;
+        if ((bm >> lane) & 1u) {
+          int32_t dd = my_dd;
+          if (dd >= 0 && ((uint32_t)dd & kSlotBit)) {
+            const uint32_t slot = (uint32_t)dd & 31u;
+            dd = wd[slot];
+            miss = wmiss[slot];
+          }
+          if (dd >= 0 && (uint32_t)dd < D) d = (uint32_t)dd;
+        }
+        auto release = [&](uint32_t at, uint32_t l, uint32_t ms) {
+          if (kInfl) {
+            const int64_t x = s_state[at] - (int64_t)l;
+            s_state[at] = x;
+            s_hl[at] = hl_of(x);
+          } else {
+            s_state[at] += (int64_t)ms * (int64_t)w.bytes_per_token;
+            const int32_t n = s_held[at] - 1;
+            s_held[at] = n;
+            s_term[at] = load_term(a.lm, n);
+          }
+        };
+        // each lane releases its own decode; departures of one decode (rare) go one by one
+        const uint32_t peers = __match_any_sync(0xffffffffu, d);
+        if (__any_sync(0xffffffffu, d != kNone && __popc(peers) > 1)) {
+          uint32_t rest = __ballot_sync(0xffffffffu, d != kNone);
+          while (rest) {
+            const uint32_t src = __ffs(rest) - 1;
+            rest &= rest - 1;
+            if (lane == src) release(d, my_l, miss);
+            __syncwarp();
+          }
+        } else if (d != kNone) {
+          release(d, my_l, miss);
+        }
+        __syncwarp();
+      };
+      while (arr_mask) {
+        const uint32_t i = __ffs(arr_mask) - 1;
+        arr_mask &= arr_mask - 1;
+        const uint32_t l = __shfl_sync(0xffffffffu, my_l, i);
+        const size_t row = (buf * win + i) * (size_t)D;
+        depart(i);
+        done = i + 1;
+        uint32_t pr = 0, cw = 0;
+        long long now = 0;
+        if (kInfl) {
+          pr = __shfl_sync(0xffffffffu, my_pr, i);
+          now = __shfl_sync(0xffffffffu, my_now, i);
+          done_at.settle(now, lane);
+          cw = S.cnt[pr];
+        }
+        // each lane's best and second-best of decodes lane, lane + 32, ...
+        float b = __int_as_float(0x7f800000), s2 = b;
+        uint32_t ci = kNone;
+#pragma unroll 4
+        for (uint32_t d = lane; d < D; d += 32) {
+          bool feasible;
+          float sc;
+          if (kInfl) {
+            const uint2 hl = s_hl[d];
+            feasible = l <= hl.x;  // load + l <= cap (l >= 1 here)
+            float net = S.base[row + d];
+            if (cw) net = contended(t, w, S.rows[row + d], cw, net);
+            sc = net + w.w_load * __uint_as_float(hl.y);
+          } else {
+            const uint2 c = S.cand[row + d];
+            feasible = s_state[d] >= (int64_t)c.y * (int64_t)w.bytes_per_token + a.lm.m_min;
+            sc = __uint_as_float(c.x) + w.w_load * s_term[d];
+          }
+          const bool take = feasible && (ci == kNone || sc < b);
+          s2 = take ? b : (feasible ? fminf(s2, sc) : s2);
+          b = take ? sc : b;
+          ci = take ? d : ci;
+        }
+        // (key, rank) argmin and second key: the rank and the second depend only on the key
+        const uint32_t key = ci == kNone ? kNoKey : score_key(b);
+        const uint32_t kb = __reduce_min_sync(0xffffffffu, key);
+        const bool at_best = key == kb;
+        const uint32_t bi = __reduce_min_sync(0xffffffffu, at_best ? ci : kNone);
+        const uint32_t ties = __popc(__ballot_sync(0xffffffffu, at_best));
+        const uint32_t one = __reduce_min_sync(0xffffffffu, at_best ? score_key(s2) : key);
+        const uint32_t ks = ties >= 2 ? kb : one;
+        const int32_t dstar = kb == kNoKey ? -1 : (int32_t)bi;
+        int32_t xfer = -1;
+        uint32_t miss = 0;
+        if (dstar >= 0) {
+          if (kInfl) {
+            // the dispatch's transfer time, tier counter (line 14) and completion
+            const int2 tt = S.dt[row + dstar];
+            const uint32_t tau = (uint32_t)tt.y, n = (cw >> (8u * tau)) & 0xffu;
+            xfer = tt.x;
+            if (n) {
+              const XferRow x = S.rows[row + dstar];
+              xfer = whole_us(xfer_time(XferParts{x.s_eff, x.bb, x.miss}, n, latency_of(t, tau)));
+            }
+            const int64_t ld = s_state[dstar] + (int64_t)l;
+            const uint2 h = hl_of(ld);
+            __syncwarp();
+            if (lane == 0) {
+              s_state[dstar] = ld;
+              s_hl[dstar] = h;
+            }
+            done_at.dispatch(now, xfer, pr, tau, cw, a.inflight_cap, lane);
+          } else {
+            miss = S.cand[row + dstar].y;
+            const int64_t x = s_state[dstar] - (int64_t)miss * (int64_t)w.bytes_per_token;
+            const int32_t n = s_held[dstar] + 1;
+            const float term = load_term(a.lm, n);
+            __syncwarp();
+            if (lane == 0) {
+              s_state[dstar] = x;
+              s_held[dstar] = n;
+              s_term[dstar] = term;
+            }
+          }
+        }
+        if (lane == 0) {
+          wd[i] = dstar;
+          wmiss[i] = miss;
+          s_wb[i] = kb;
+          s_ws[i] = ks;
+          s_wx[i] = xfer;
+        }
+        __syncwarp();
+      }
+      depart(32);  // departures after the window's last arrival
+      if (is_arr) {
+        a.dec[r] = wd[lane];
+        a.best[r] = key_score(s_wb[lane]);
+        a.second[r] = key_score(s_ws[lane]);
+        if (kInfl) a.xfer_us[r] = s_wx[lane];
+      }
+      prev_r = is_arr ? r : kBadCode;
+    }
+    __syncthreads();
+  }
+  for (uint32_t d = lane; d < D; d += 32) {
+    a.state_final[(uint64_t)stream * D + d] = s_state[d];
+    if (!kInfl) a.held_final[(uint64_t)stream * D + d] = s_held[d];
+  }
+}
+
+template <Walk kWalk, int BT>
+netkv_status launch_walk(const ModelArgs& a, bool small, uint32_t n_streams, cudaStream_t s) {
+  // the attribute is per device: set before every launch that needs it
+  const bool big = a.lay.total > 48u * 1024u;
+  if constexpr (BT <= 128) if (small) {
+    if (big) NETKV_CUDA_TRY(cudaFuncSetAttribute(schedule_small_kernel<kWalk, BT>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)kModelSmem));
+    schedule_small_kernel<kWalk, BT><<<n_streams, BT, a.lay.total, s>>>(a);
+    return netkv_launch_status();
+  }
+  if constexpr (kWalk != kPlain) {
+    if (big) NETKV_CUDA_TRY(cudaFuncSetAttribute(schedule_model_kernel<kWalk == kContend, BT>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)kModelSmem));
+    schedule_model_kernel<kWalk == kContend, BT><<<n_streams, BT, a.lay.total, s>>>(a);
+  }
+  return netkv_launch_status();
+}
+
+// Launches the walk when the pool fits: false (and nothing launched) otherwise.  Windows of
+// 32 events hide the producers' round trips best; shorter ones where the rows of a larger
+// pool need the memory, or more streams than the card's SMs hold at once.
+template <Walk kWalk>
+bool launch_model(ModelArgs& a, uint32_t n_streams, cudaStream_t s, netkv_status* result) {
+  *result = NETKV_OK;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    *result = NETKV_ECUDA;
+    return true;
+  }
+  const uint32_t D = a.t.D;
+  const bool small = D <= 32;
+  if (!small && kWalk == kPlain) return false;
+  // producers enough for a window's candidates (about 16 arrivals) in one or two rounds
+  // while the streams leave the SMs room
+  uint32_t bt = kWalk == kPlain ? 64u : small ? 128u : D <= 96 ? 256u : 512u;
+  while (bt > 64u && (uint64_t)n_streams * bt > (uint64_t)sms * 1024u) bt /= 2;
+  const uint32_t per_sm = (n_streams + (uint32_t)sms - 1) / (uint32_t)sms;
+  const uint32_t most = 1024u / bt < per_sm ? 1024u / bt : per_sm;
+  uint32_t win = 0;
+  for (uint32_t x = kMaxWindow; x >= 8; x /= 2) {
+    const ModelLayout l = model_layout(kWalk, small, D, a.t.P, a.heap_cap, x);
+    if (l.total > kModelSmem) continue;
+    win = x;
+    if ((size_t)l.total * most <= kModelSmem) break;
+  }
+  if (win == 0) return false;
+  a.lay = model_layout(kWalk, small, D, a.t.P, a.heap_cap, win);
+  if (bt == 64) *result = launch_walk<kWalk, 64>(a, small, n_streams, s);
+  else if (bt == 128) *result = launch_walk<kWalk, 128>(a, small, n_streams, s);
+  else if (bt == 256) *result = launch_walk<kWalk, 256>(a, small, n_streams, s);
+  else *result = launch_walk<kWalk, 512>(a, small, n_streams, s);
+  return true;
+}
+
+}  // namespace
+
+bool launch_model_inflight(const TopoArgs& t, uint32_t n_streams, const netkv_weights* d_w,
+                           uint32_t R, const uint32_t* d_len, const uint32_t* d_prefill,
+                           const uint32_t* d_snap, const int64_t* d_arrival_us,
+                           const uint16_t* d_M, const float* d_UB, uint32_t n_snap,
+                           const uint32_t* d_events, const uint64_t* d_event_off,
+                           uint32_t inflight_cap, uint32_t heap_cap, const int64_t* d_load_init,
+                           int32_t* d_dec, float* d_best, float* d_second, int32_t* d_xfer_us,
+                           int64_t* d_load_final, int* d_status, cudaStream_t s,
+                           netkv_status* result) {
+  ModelArgs a = {};
+  a.t = t;
+  a.W = d_w;
+  a.R = R;
+  a.n_snap = n_snap;
+  a.len = d_len;
+  a.prefill = d_prefill;
+  a.snap = d_snap;
+  a.M = d_M;
+  a.UB = d_UB;
+  a.events = d_events;
+  a.event_off = d_event_off;
+  a.state_init = d_load_init;
+  a.dec = d_dec;
+  a.best = d_best;
+  a.second = d_second;
+  a.state_final = d_load_final;
+  a.status = d_status;
+  a.arrival_us = d_arrival_us;
+  a.inflight_cap = inflight_cap;
+  a.heap_cap = heap_cap;
+  a.xfer_us = d_xfer_us;
+  return launch_model<kContend>(a, n_streams, s, result);
+}
+
+bool launch_model_load(const TopoArgs& t, uint32_t n_streams, const netkv_weights* d_w,
+                       float t_a, float t_b, int32_t beta_max, int64_t m_min, int64_t m0,
+                       uint32_t R, const uint32_t* d_len, const uint32_t* d_prefill,
+                       const uint32_t* d_snap, const uint16_t* d_M, const float* d_UB,
+                       uint32_t n_snap, const uint32_t* d_events, const uint64_t* d_event_off,
+                       const int64_t* d_m_init, const int32_t* d_n_init, int32_t* d_dec,
+                       float* d_best, float* d_second, int64_t* d_m_final, int32_t* d_n_final,
+                       int* d_status, cudaStream_t s, netkv_status* result) {
+  ModelArgs a = {};
+  a.t = t;
+  a.W = d_w;
+  a.R = R;
+  a.n_snap = n_snap;
+  a.len = d_len;
+  a.prefill = d_prefill;
+  a.snap = d_snap;
+  a.M = d_M;
+  a.UB = d_UB;
+  a.events = d_events;
+  a.event_off = d_event_off;
+  a.state_init = d_m_init;
+  a.dec = d_dec;
+  a.best = d_best;
+  a.second = d_second;
+  a.state_final = d_m_final;
+  a.status = d_status;
+  a.lm = LoadModel{t_a, t_b, beta_max, m_min, m0};
+  a.held_init = d_n_init;
+  a.held_final = d_n_final;
+  return launch_model<kModel>(a, n_streams, s, result);
+}
+
+bool launch_small_plain(const TopoArgs& t, uint32_t n_streams, const netkv_weights* d_w,
+                        uint32_t R, const uint32_t* d_len, const uint32_t* d_prefill,
+                        const uint32_t* d_snap, uint32_t n_snap, const uint32_t* d_events,
+                        const uint64_t* d_event_off, const int64_t* d_load_init, int32_t* d_dec,
+                        float* d_best, float* d_second, int64_t* d_load_final,
+                        const float* d_base, int* d_status, cudaStream_t s,
+                        netkv_status* result) {
+  ModelArgs a = {};
+  a.t = t;
+  a.W = d_w;
+  a.R = R;
+  a.n_snap = n_snap;
+  a.len = d_len;
+  a.prefill = d_prefill;
+  a.snap = d_snap;
+  a.base = d_base;
+  a.events = d_events;
+  a.event_off = d_event_off;
+  a.state_init = d_load_init;
+  a.dec = d_dec;
+  a.best = d_best;
+  a.second = d_second;
+  a.state_final = d_load_final;
+  a.status = d_status;
+  return launch_model<kPlain>(a, n_streams, s, result);
+}
