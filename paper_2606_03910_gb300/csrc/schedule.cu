@@ -1987,7 +1987,7 @@ __global__ void __launch_bounds__(32 * kWinWarps) schedule_window_kernel(
   if (mine) load_final[(uint64_t)stream * D + sl] = load;
 }
 
-constexpr uint32_t kSmallMaxStreams = 4096;
+constexpr uint32_t kSmallMaxStreams = 1536;
 constexpr int kStages = 8;
 constexpr uint32_t kHeapPerStream = 4096;       // pending completions, one stream per CTA
 constexpr uint32_t kHeapPerPackedStream = 256;  // pending completions, packed streams
@@ -2132,9 +2132,9 @@ netkv_status launch(const TopoArgs& t, uint32_t n_streams, const netkv_weights* 
                            d_event_off, d_load_init, d_dec, d_best, d_second, d_load_final,
                            d_base, lw->lists, lw->bounds, d_status, s);
     }
-    if (t.D <= 32 && n_streams <= kSmallMaxStreams) {
+    if (t.D > 16 ? t.D <= 1024 : n_streams <= kSmallMaxStreams) {
       netkv_status st;
-      if (launch_small_plain(t, n_streams, d_w, R, d_len, d_prefill, d_snap, n_snap, d_events,
+      if (launch_model_plain(t, n_streams, d_w, R, d_len, d_prefill, d_snap, n_snap, d_events,
                              d_event_off, d_load_init, d_dec, d_best, d_second, d_load_final,
                              d_base, d_status, s, &st))
         return st;

@@ -24,7 +24,6 @@
 namespace {
 
 constexpr uint32_t kBadCode = 0xffffffffu;
-constexpr uint32_t kSlotBit = 0x40000000u;  // a departure whose arrival is in its window: the slot
 constexpr uint32_t kMaxWindow = 32;         // events per window: one a lane
 constexpr int kAhead = 4;                   // candidates a producer thread has in flight
 constexpr size_t kModelSmem = 227u * 1024u; // dynamic shared memory of one CTA
@@ -32,15 +31,22 @@ constexpr size_t kModelSmem = 227u * 1024u; // dynamic shared memory of one CTA
 enum EventType : uint32_t { kNoEvent = 0, kArrival = 1, kDeparture = 2, kBadArrival = 3 };
 
 // An event with what its candidates share, filled one window ahead.
+// ref: where a departure's decode is known from: kRefGlobal (dd, read from global memory),
+// kRefPrev | slot (its arrival in the window before), kRefOwn | slot (earlier in its own
+// window); kRefSlow: released by itself, not with the sums.  count: the window's arrivals
+// before a departure; for an arrival whose request departs once in its window, 1 + that
+// departure's count, else 0.
 struct __align__(16) ModelEvent {
   uint4 lp;        // the prefill's links
   float4 ubp;      // and level bottlenecks
   uint32_t code, type, l, pr;
   long long now;   // arrival time (self-contention)
-  int32_t dd;      // a departure's decode as recorded in global memory
-  uint32_t miss;   // and the missed tokens of its request there (load model)
-  uint32_t k, pad[3];
+  int32_t dd;
+  uint32_t miss;   // a departure's missed tokens on dd (load model)
+  uint32_t k, ref, count, pad;
 };
+constexpr uint32_t kRefGlobal = 0u, kRefPrev = 0x100u, kRefOwn = 0x200u, kRefSlow = 0x400u;
+constexpr uint32_t kSumTokens = 1u << 27;  // below: a window's sum of 32 fits in 32 bits
 
 enum Walk { kPlain = 0, kContend = 1, kModel = 2 };
 
@@ -69,7 +75,7 @@ __device__ __forceinline__ float latency_of(const TopoArgs& t, uint32_t tau) {
 // Byte offsets of the dynamic shared memory.
 struct ModelLayout {
   uint32_t win;
-  uint32_t ev, arr, narr, wd, wmiss, wb, ws, wx, state, term, held, cnt, heap, rel, base, rows, dt,
+  uint32_t ev, arr, narr, wd, wmiss, wb, ws, wx, state, tok, term, held, cnt, heap, rel, base, rows, dt,
       total;
 };
 
@@ -95,8 +101,9 @@ ModelLayout model_layout(Walk walk, bool small, uint32_t D, uint32_t P, uint32_t
   a.ws = take(small ? 0 : kMaxWindow * 4);
   a.wx = take(small ? 0 : kMaxWindow * 4);
   a.state = take(small ? 0 : (size_t)D * 8);              // load or free bytes
-  a.term = take(small ? 0 : (size_t)D * (infl ? 8 : 4));  // (headroom, theta * load) or load term
-  a.held = take(small || infl ? 0 : (size_t)D * 4);
+  a.tok = take(small || walk != kModel ? 0 : (size_t)D * 8);
+  a.term = take(small ? 0 : (size_t)D * 8);               // (tokens that fit, load term)
+  a.held = take(small || walk != kModel ? 0 : (size_t)D * 4);
   a.cnt = take(infl ? (size_t)P * 4 : 0);
   a.heap = take(infl ? (size_t)heap_cap * 8 : 0);
   a.rel = take(small ? (size_t)(kMaxWindow + 1) * 32 * (walk == kModel ? 8 : 4) : 0);
@@ -163,56 +170,84 @@ __device__ __forceinline__ void produce(const ModelArgs& a, const netkv_weights&
   const uint32_t D = t.D, win = a.lay.win, ptid = threadIdx.x - 32;
   const uint32_t step_q = NP / D, step_d = NP % D;
   uint32_t code = ptid < win && e0 + ptid < e1 ? __ldg(a.events + e0 + ptid) : kBadCode;
+  uint32_t prev_r = kBadCode;  // lane j: event j of the window before: its request, if an arrival
   for (uint64_t k = 0; k <= n_win; ++k) {
     if (k < n_win) {
       ModelEvent* ev = S.ev + (k & 1) * win;
       uint32_t* arr = S.arr + (k & 1) * kMaxWindow;
       if (ptid < 32) {
-        uint32_t type = kNoEvent;
-        if (ptid < win) {
-          ModelEvent x;
-          x.lp = make_uint4(0, 0, 0, 0);
-          x.ubp = make_float4(0.f, 0.f, 0.f, 0.f);
-          x.code = code;
-          x.l = x.pr = x.miss = x.k = 0;
-          x.now = 0;
-          x.dd = -1;
-          const uint32_t r = code & 0x7fffffffu;
-          const uint64_t e = e0 + (k + 1) * win + ptid;
-          const uint32_t next = e < e1 ? __ldg(a.events + e) : kBadCode;
-          if (code == kBadCode) {
-          } else if (r >= a.R) {
-            flag_status(a.status, NETKV_DEV_ERANGE);
-          } else if (code >> 31) {
-            type = kDeparture;
-            x.l = __ldg(a.len + r);
-            x.dd = __ldcg(a.dec + r);  // by the walker, up to the window before the walked one
-            if (kWalk == kModel && x.dd >= 0 && (uint32_t)x.dd < D)
-              x.miss = x.l - min(16u * (uint32_t)__ldg(a.M + (uint64_t)r * D + x.dd), x.l);
-          } else {
-            x.l = __ldg(a.len + r);
-            x.pr = __ldg(a.prefill + r);
-            x.k = __ldg(a.snap + r);
-            if (kWalk == kContend) x.now = __ldg(a.arrival_us + r);
-            if (x.pr < t.P && x.k < a.n_snap && x.l != 0) {
-              type = kArrival;
-              if (kWalk != kPlain) {
-                const uint32_t pinst = __ldg(t.pre + x.pr);
-                x.lp = __ldg(t.links + pinst);
-                x.ubp = __ldg(reinterpret_cast<const float4*>(a.UB) + (uint64_t)x.k * t.N + pinst);
-              }
-            } else {
-              type = kBadArrival;
-              flag_status(a.status, x.l == 0 ? NETKV_DEV_EDOMAIN : NETKV_DEV_ERANGE);
+        ModelEvent x;
+        x.lp = make_uint4(0, 0, 0, 0);
+        x.ubp = make_float4(0.f, 0.f, 0.f, 0.f);
+        x.code = code;
+        x.type = kNoEvent;
+        x.l = x.pr = x.miss = x.k = x.count = x.pad = 0;
+        x.ref = kRefGlobal;
+        x.now = 0;
+        x.dd = -1;
+        const uint32_t r = code & 0x7fffffffu;
+        const uint64_t e = e0 + (k + 1) * win + ptid;
+        const uint32_t next = ptid < win && e < e1 ? __ldg(a.events + e) : kBadCode;
+        if (code == kBadCode) {
+        } else if (r >= a.R) {
+          flag_status(a.status, NETKV_DEV_ERANGE);
+        } else if (code >> 31) {
+          x.type = kDeparture;
+          x.l = __ldg(a.len + r);
+          x.dd = __ldcg(a.dec + r);  // by the walker, up to the window before the walked one
+          if (kWalk == kModel && x.dd >= 0 && (uint32_t)x.dd < D)
+            x.miss = x.l - min(16u * (uint32_t)__ldg(a.M + (uint64_t)r * D + x.dd), x.l);
+        } else {
+          x.l = __ldg(a.len + r);
+          x.pr = __ldg(a.prefill + r);
+          x.k = __ldg(a.snap + r);
+          if (kWalk == kContend) x.now = __ldg(a.arrival_us + r);
+          if (x.pr < t.P && x.k < a.n_snap && x.l != 0) {
+            x.type = kArrival;
+            if (kWalk != kPlain) {
+              const uint32_t pinst = __ldg(t.pre + x.pr);
+              x.lp = __ldg(t.links + pinst);
+              x.ubp = __ldg(reinterpret_cast<const float4*>(a.UB) + (uint64_t)x.k * t.N + pinst);
             }
+          } else {
+            x.type = kBadArrival;
+            flag_status(a.status, x.l == 0 ? NETKV_DEV_EDOMAIN : NETKV_DEV_ERANGE);
           }
-          x.type = type;
-          ev[ptid] = x;
-          code = next;
         }
-        // the window's arrivals, in order
-        const uint32_t list = __ballot_sync(0xffffffffu, type == kArrival);
-        if (type == kArrival) arr[__popc(list & ((1u << ptid) - 1u))] = ptid;
+        code = next;
+        // the window's arrivals, in order, and each departure's arrival when that lies in
+        // this window or the one before (their decisions are not recorded yet)
+        const bool is_arr = x.type == kArrival || x.type == kBadArrival;
+        const bool is_dep = x.type == kDeparture;
+        const uint32_t any_arr = __ballot_sync(0xffffffffu, is_arr);
+        const uint32_t list = __ballot_sync(0xffffffffu, x.type == kArrival);
+        const uint32_t deps = __ballot_sync(0xffffffffu, is_dep);
+        const uint32_t below = (1u << ptid) - 1u;
+        const uint32_t er = x.type == kNoEvent ? kBadCode : r;
+        if (deps) {
+          for (uint32_t j = 0; j < win; ++j) {
+            const uint32_t rj = __shfl_sync(0xffffffffu, prev_r, j);
+            if (is_dep && rj == r) x.ref = kRefPrev | j;
+          }
+          const uint32_t same = __match_any_sync(0xffffffffu, er);
+          const uint32_t mate = same & any_arr & below;               // a departure's arrival
+          const uint32_t leave = same & deps & ~below & ~(1u << ptid);  // an arrival's departures
+          if (is_dep) {
+            x.count = __popc(list & below);
+            if (mate) {
+              const uint32_t slot = 31u - __clz(mate);
+              x.ref = kRefOwn | slot;
+              // the arrival's dispatch releases it, unless it is large or departs twice
+              if (__popc(same & deps & ~((2u << slot) - 1u)) != 1) x.ref |= kRefSlow;
+            }
+            if (x.l >= kSumTokens) x.ref |= kRefSlow;
+          } else if (x.type == kArrival && __popc(leave) == 1 && x.l < kSumTokens) {
+            x.count = 1u + __popc(list & ((1u << (__ffs(leave) - 1)) - 1u));
+          }
+        }
+        prev_r = is_arr ? r : kBadCode;
+        if (ptid < win) ev[ptid] = x;
+        if (x.type == kArrival) arr[__popc(list & below)] = ptid;
         if (ptid == 0) S.narr[k & 1] = __popc(list);
       }
       if (BT == 64) __syncwarp();
@@ -286,65 +321,69 @@ __device__ __forceinline__ void produce(const ModelArgs& a, const netkv_weights&
 
 // The pending completions of a stream and its counters.  The lanes of the walker hold 32 of
 // them, one each, in no order (lowering a counter, floored at zero, commutes); more go to a
-// heap kept by lane 0.
+// heap kept by lane 0, out of line.
+__device__ __forceinline__ void lower_counter(uint32_t* cnt, uint32_t pt) {
+  uint32_t* c = cnt + (pt >> 2);
+  const uint32_t sh = 8u * (pt & 3u);
+  if ((*c >> sh) & 0xffu) *c -= 1u << sh;
+}
+__device__ __noinline__ uint32_t heap_settle(unsigned long long* a, uint32_t n, uint32_t cap,
+                                             uint32_t* cnt, long long now) {
+  DoneHeap h = {a, n, cap};
+  while (h.n > 0 && (int64_t)(h.a[0] >> 16) <= now) {
+    lower_counter(cnt, (uint32_t)(h.a[0] & 0xffffu));
+    h.pop();
+  }
+  return h.n;
+}
+__device__ __noinline__ void heap_push(unsigned long long* a, uint32_t n, uint32_t cap,
+                                       unsigned long long key) {
+  DoneHeap h = {a, n, cap};
+  h.push(key);
+}
 struct Completions {
   static constexpr unsigned long long kFree = ~0ull;  // above every key: prefill < 2^14 - 1
   unsigned long long key;  // time in us << 16 | prefill rank << 2 | tier
-  DoneHeap heap;
-  uint32_t in_heap, cap;   // the same in every lane; cap: pending in all
-  uint32_t* cnt;
-  int* status;
-  __device__ Completions(const ModelArgs& a, unsigned char* smem, uint32_t* c)
-      : key(kFree), in_heap(0), cap(a.heap_cap), cnt(c), status(a.status) {
-    heap.a = reinterpret_cast<unsigned long long*>(smem + a.lay.heap);
-    heap.n = 0;
-    heap.cap = a.heap_cap;
-  }
-  __device__ __forceinline__ void lower(uint32_t pt) {
-    uint32_t* c = cnt + (pt >> 2);
-    const uint32_t sh = 8u * (pt & 3u);
-    if ((*c >> sh) & 0xffu) *c -= 1u << sh;
-  }
+  uint32_t in_heap;        // the same in every lane
+  __device__ Completions() : key(kFree), in_heap(0) {}
   // Transfers completed by `now` lower their counters (Algorithm 1 line 14's callback).
-  __device__ __forceinline__ void settle(long long now, uint32_t lane) {
+  __device__ __forceinline__ void settle(const ModelArgs& a, unsigned char* smem, uint32_t* cnt,
+                                         long long now, uint32_t lane) {
     const bool due = key != kFree && (int64_t)(key >> 16) <= now;
     uint32_t dm = __ballot_sync(0xffffffffu, due);
     if (!dm && !in_heap) return;
     while (dm) {
       const uint32_t j = __ffs(dm) - 1;
       dm &= dm - 1;
-      const uint32_t pt = __shfl_sync(0xffffffffu, (uint32_t)key & 0xffffu, j);
-      if (lane == 0) lower(pt);
+      if (lane == j) lower_counter(cnt, (uint32_t)key & 0xffffu);
+      __syncwarp();
     }
     if (due) key = kFree;
     if (in_heap) {
-      if (lane == 0) {
-        while (heap.n > 0 && (int64_t)(heap.a[0] >> 16) <= now) {
-          lower((uint32_t)(heap.a[0] & 0xffffu));
-          heap.pop();
-        }
-      }
-      in_heap = __shfl_sync(0xffffffffu, heap.n, 0);
+      if (lane == 0)
+        in_heap = heap_settle(reinterpret_cast<unsigned long long*>(smem + a.lay.heap), in_heap,
+                              a.heap_cap, cnt, now);
+      in_heap = __shfl_sync(0xffffffffu, in_heap, 0);
     }
-    __syncwarp();
   }
   // A dispatch on tier tau of prefill pr, whose counters are cw: the counter and the
   // completion at now + dt.
-  __device__ __forceinline__ void dispatch(long long now, int32_t dt, uint32_t pr, uint32_t tau,
-                                           uint32_t cw, uint32_t most, uint32_t lane) {
+  __device__ __forceinline__ void dispatch(const ModelArgs& a, unsigned char* smem, uint32_t* cnt,
+                                           long long now, int32_t dt, uint32_t pr, uint32_t tau,
+                                           uint32_t cw, uint32_t lane) {
+    const uint32_t free = __ballot_sync(0xffffffffu, key == kFree);
     const unsigned long long k = ((unsigned long long)(now + dt) << 16) |
                                  ((unsigned long long)pr << 2) | tau;
     const uint32_t sh = 8u * tau;
-    if (lane == 0 && ((cw >> sh) & 0xffu) < most) cnt[pr] = cw + (1u << sh);
-    const uint32_t free = __ballot_sync(0xffffffffu, key == kFree);
-    if (32u - __popc(free) + in_heap >= cap) {
-      if (lane == 0) flag_status(status, NETKV_DEV_EFULL);
-    } else if (free) {
-      if (lane == (uint32_t)(__ffs(free) - 1)) key = k;
-    } else {
-      if (lane == 0) heap.push(k);
-      ++in_heap;
+    const uint32_t at = free ? (uint32_t)(__ffs(free) - 1) : 0u;
+    const bool full = 32u - __popc(free) + in_heap >= a.heap_cap;
+    if (lane == at) {  // one lane does it all
+      if (((cw >> sh) & 0xffu) < a.inflight_cap) cnt[pr] = cw + (1u << sh);
+      if (full) flag_status(a.status, NETKV_DEV_EFULL);
+      else if (free) key = k;
+      else heap_push(reinterpret_cast<unsigned long long*>(smem + a.lay.heap), in_heap, a.heap_cap, k);
     }
+    if (!full && !free) ++in_heap;
     __syncwarp();
   }
 };
@@ -358,8 +397,6 @@ __device__ __forceinline__ float contended(const TopoArgs& t, const netkv_weight
   const float T = xfer_time(p, n, latency_of(t, x.tau));
   return w.w_net * T + w.w_prefix * p.miss;
 }
-
-constexpr uint32_t kSumTokens = 1u << 27;  // below: a window's sum of 32 fits in 32 bits
 
 template <Walk kWalk, int BT>
 __global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs a) {
@@ -392,20 +429,19 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs
   // what the last dispatch took on its decode's lane (tokens, or missed tokens of one
   // request), applied with the releases before the next arrival
   uint32_t own = 0, own_n = 0;
-  Completions done_at(a, smem, S.cnt);
+  Completions done_at;
   if (kWalk == kContend)
     for (uint32_t p = lane; p < t.P; p += 32) S.cnt[p] = 0u;
   __syncwarp();
 
-  uint32_t prev_r = kBadCode;  // lane j: event j of the window before: its request, if an arrival,
-  int32_t prev_d = -1;         // its decision and its missed tokens there
-  uint32_t prev_miss = 0;
+  int32_t prev_d = -1;  // lane j: event j of the window before: its decision
+  uint32_t prev_miss = 0;  // and its missed tokens there
   for (uint64_t k = 0; k <= n_win; ++k) {
     if (k > 0) {
       const uint32_t buf = (uint32_t)((k - 1) & 1);
       const ModelEvent* ev = S.ev + buf * win;
       // lane i prepares event i
-      uint32_t type = kNoEvent, r = kBadCode, l_ev = 0, miss_ev = 0, pr_ev = 0;
+      uint32_t type = kNoEvent, r = kBadCode, l_ev = 0, miss_ev = 0, pr_ev = 0, ref = 0, count = 0;
       int32_t dd = -1;
       long long now_ev = 0;
       if (lane < win) {
@@ -414,55 +450,32 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs
         l_ev = x.l;
         dd = x.dd;
         miss_ev = x.miss;
+        ref = x.ref;
+        count = x.count;
         if (kWalk == kContend) {
           pr_ev = x.pr;
           now_ev = x.now;
         }
-        if (type != kNoEvent) r = x.code & 0x7fffffffu;
+        r = x.code & 0x7fffffffu;
       }
-      const bool is_arr = type == kArrival || type == kBadArrival, is_dep = type == kDeparture;
-      const uint32_t any_arr = __ballot_sync(0xffffffffu, is_arr);
+      const bool is_arr = type == kArrival || type == kBadArrival;
       const uint32_t arrivals = __ballot_sync(0xffffffffu, type == kArrival);
-      const uint32_t dep_mask = __ballot_sync(0xffffffffu, is_dep);
-      const uint32_t below = (1u << lane) - 1u;
-      bool slow = false;     // a departure released one by one
-      uint32_t my_bj = 0;    // an arrival whose request departs in this window: 1 + the number
-                             // of arrivals before that departure
-      if (dep_mask) {
-        // a departure's arrival may lie in the window before (its decision there) or
-        // earlier in this one (its slot), after the recorded decision was read
-        for (uint32_t j = 0; j < win; ++j) {
-          const uint32_t rj = __shfl_sync(0xffffffffu, prev_r, j);
-          const int32_t dj = __shfl_sync(0xffffffffu, prev_d, j);
-          if (is_dep && rj == r) dd = dj;
-          if (kWalk == kModel) {
-            const uint32_t mj = __shfl_sync(0xffffffffu, prev_miss, j);
-            if (is_dep && rj == r) miss_ev = mj;
-          }
+      const bool slow = type == kDeparture && (ref & kRefSlow);
+      const uint32_t my_bj = type == kArrival ? count : 0u;
+      {
+        const int32_t pd = __shfl_sync(0xffffffffu, prev_d, ref & 31u);
+        const uint32_t pm = kWalk == kModel ? __shfl_sync(0xffffffffu, prev_miss, ref & 31u) : 0u;
+        if (ref & kRefPrev) {
+          dd = pd;
+          miss_ev = pm;
         }
-        const uint32_t same = __match_any_sync(0xffffffffu, r);
-        const uint32_t mate = same & any_arr & below;  // the departure's arrival
-        const uint32_t leave = same & dep_mask & ~below & ~(1u << lane);  // the arrival's departures
-        if (type == kArrival && __popc(leave) == 1 && l_ev < kSumTokens)
-          my_bj = 1u + __popc(arrivals & ((1u << (__ffs(leave) - 1)) - 1u));
-        if (is_dep && mate) {
-          const uint32_t slot = 31u - __clz(mate);
-          dd = (int32_t)(kSlotBit | slot);
-          // the arrival's dispatch releases it, unless it is large or departs twice
-          slow = l_ev >= kSumTokens || __popc(same & dep_mask & ~((2u << slot) - 1u)) != 1;
-        } else if (is_dep && dd >= 0 && (uint32_t)dd < D) {
-          // tokens released before the window's b-th arrival
-          const uint32_t amount = kWalk == kModel ? miss_ev : l_ev;
-          const uint32_t b = __popc(arrivals & below);
-          if (amount >= kSumTokens) {
-            slow = true;
-          } else {
-            atomicAdd(&rel[b * 32 + dd], amount);
-            if (kWalk == kModel) atomicAdd(&reln[b * 32 + dd], 1u);
-          }
-        }
-        __syncwarp();
       }
+      if (type == kDeparture && !(ref & (kRefOwn | kRefSlow)) && dd >= 0 && (uint32_t)dd < D) {
+        // tokens released before the window's count-th arrival
+        atomicAdd(&rel[count * 32 + dd], kWalk == kModel ? miss_ev : l_ev);
+        if (kWalk == kModel) atomicAdd(&reln[count * 32 + dd], 1u);
+      }
+      __syncwarp();
       const uint32_t leaving = __ballot_sync(0xffffffffu, my_bj != 0u);
       uint32_t left = __ballot_sync(0xffffffffu, slow);  // slow departures not applied yet
       int32_t my_d = -1, my_x = -1;  // lane i: event i's decision, transfer time,
@@ -475,10 +488,10 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs
           int32_t d = __shfl_sync(0xffffffffu, dd, j);
           const uint32_t l = __shfl_sync(0xffffffffu, l_ev, j);
           uint32_t m = __shfl_sync(0xffffffffu, miss_ev, j);
-          const uint32_t slot = (uint32_t)d & 31u;
-          const int32_t ds = __shfl_sync(0xffffffffu, my_d, slot);
-          const uint32_t ms = __shfl_sync(0xffffffffu, my_miss, slot);
-          if (d >= 0 && ((uint32_t)d & kSlotBit)) {
+          const uint32_t rf = __shfl_sync(0xffffffffu, ref, j);
+          const int32_t ds = __shfl_sync(0xffffffffu, my_d, rf & 31u);
+          const uint32_t ms = __shfl_sync(0xffffffffu, my_miss, rf & 31u);
+          if (rf & kRefOwn) {
             d = ds;
             m = ms;
           }
@@ -551,7 +564,7 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs
         if (kWalk == kContend) {
           pr = __shfl_sync(0xffffffffu, pr_ev, i);
           now = __shfl_sync(0xffffffffu, now_ev, i);
-          done_at.settle(now, lane);
+          done_at.settle(a, smem, S.cnt, now, lane);
           cw = S.cnt[pr];
           if (cw && mine) net = contended(t, w, S.rows[row + lane], cw, net);
         }
@@ -595,7 +608,7 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs
             const XferRow x = S.rows[row + dstar];
             xfer = whole_us(xfer_time(XferParts{x.s_eff, x.bb, x.miss}, n, latency_of(t, tau)));
           }
-          done_at.dispatch(now, xfer, pr, tau, cw, a.inflight_cap, lane);
+          done_at.dispatch(a, smem, S.cnt, now, xfer, pr, tau, cw, lane);
         }
         const uint32_t taken =
             kWalk == kModel ? __shfl_sync(0xffffffffu, miss, dstar < 0 ? 0 : dstar) : 0u;
@@ -615,7 +628,6 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs
         a.second[r] = key_score(my_s);
         if (kWalk == kContend) a.xfer_us[r] = my_x;
       }
-      prev_r = is_arr ? r : kBadCode;
       prev_d = my_d;
       prev_miss = my_miss;
     }
@@ -627,10 +639,16 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs
   }
 }
 
-template <bool kInfl, int BT>
+// A decode's feasibility and load term, 8 bytes: (headroom, theta * load), a request of l
+// tokens fits iff l <= headroom; load model: (free tokens + 1, T_queue + T_decode), a
+// candidate fits iff its missed tokens are below the first.  There the free bytes above m_min
+// are counted in whole tokens once and then change by the missed tokens of each dispatch
+// and departure: floor((f - b * S) / b) = floor(f / b) - S.  That needs 0 < bytes_per_token
+// < 2^31 (products of 32-bit token counts then stay in 63 bits); a stream with other bytes,
+// and a request of 2^32 - 1 tokens, compare bytes instead.
+template <Walk kWalk, int BT>
 __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  constexpr Walk kWalk = kInfl ? kContend : kModel;
   const TopoArgs& t = a.t;
   const uint32_t D = t.D, win = a.lay.win, lane = threadIdx.x & 31;
   const uint32_t stream = blockIdx.x;
@@ -643,38 +661,57 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs
     return;
   }
 
-  // ---- the walker
+  // ---- the walker: lane i takes decodes i, i + 32, ...
   int32_t* s_wd = reinterpret_cast<int32_t*>(smem + a.lay.wd);          // [2][kMaxWindow]
   uint32_t* s_wmiss = reinterpret_cast<uint32_t*>(smem + a.lay.wmiss);  // [2][kMaxWindow]
   uint32_t* s_wb = reinterpret_cast<uint32_t*>(smem + a.lay.wb);
   uint32_t* s_ws = reinterpret_cast<uint32_t*>(smem + a.lay.ws);
   int32_t* s_wx = reinterpret_cast<int32_t*>(smem + a.lay.wx);
-  int64_t* s_state = reinterpret_cast<int64_t*>(smem + a.lay.state);
+  int64_t* s_state = reinterpret_cast<int64_t*>(smem + a.lay.state);  // load, or free bytes
+  int64_t* s_tok = reinterpret_cast<int64_t*>(smem + a.lay.tok);      // load model: in tokens
   uint2* s_hl = reinterpret_cast<uint2*>(smem + a.lay.term);
-  float* s_term = reinterpret_cast<float*>(smem + a.lay.term);
   int32_t* s_held = reinterpret_cast<int32_t*>(smem + a.lay.held);
-  auto hl_of = [&](int64_t ld) -> uint2 {  // headroom clamped to 32 bits, theta * load
-    const int64_t h = w.cap_tokens - ld;
-    const uint32_t hr = h <= 0 ? 0u : h >= 0xffffffffll ? 0xffffffffu : (uint32_t)h;
-    return make_uint2(hr, __float_as_uint(w.theta_s_per_token * load_to_float(ld)));
+  const int64_t bpt = (int64_t)w.bytes_per_token;
+  const bool in_tokens = kWalk != kModel || (bpt > 0 && bpt < (1ll << 31));
+  auto clamp32 = [](int64_t h) -> uint32_t {
+    return h <= 0 ? 0u : h >= 0xffffffffll ? 0xffffffffu : (uint32_t)h;
+  };
+  auto hl_of_load = [&](int64_t ld) -> uint2 {
+    return make_uint2(clamp32(w.cap_tokens - ld),
+                      __float_as_uint(w.theta_s_per_token * load_to_float(ld)));
+  };
+  // decode d after `delta` tokens more (load model: `delta` missed tokens of `n` requests less)
+  auto change = [&](uint32_t d, int64_t delta, int32_t n) {
+    if (kWalk == kModel) {
+      const int64_t tok = s_tok[d] + delta;
+      const int32_t h = s_held[d] - n;
+      s_state[d] += delta * bpt;
+      s_tok[d] = tok;
+      s_held[d] = h;
+      s_hl[d] = make_uint2(clamp32(tok + 1), __float_as_uint(load_term(a.lm, h)));
+    } else {
+      const int64_t ld = s_state[d] + delta;
+      s_state[d] = ld;
+      s_hl[d] = hl_of_load(ld);
+    }
   };
   for (uint32_t d = lane; d < D; d += 32) {
-    int64_t x = kInfl ? 0 : a.lm.m0;
+    int64_t x = kWalk == kModel ? a.lm.m0 : 0;
     if (a.state_init) x = a.state_init[(uint64_t)stream * D + d];
     s_state[d] = x;
-    if (kInfl) {
-      s_hl[d] = hl_of(x);
+    if (kWalk == kModel) {
+      const int64_t f = x < INT64_MIN / 4 ? INT64_MIN / 2 : x - min(a.lm.m_min, INT64_MAX / 4);
+      s_tok[d] = !in_tokens ? 0 : f >= 0 ? f / bpt : -((-f + bpt - 1) / bpt);
+      s_held[d] = a.held_init ? a.held_init[(uint64_t)stream * D + d] : 0;
+      change(d, 0, 0);
     } else {
-      const int32_t n = a.held_init ? a.held_init[(uint64_t)stream * D + d] : 0;
-      s_held[d] = n;
-      s_term[d] = load_term(a.lm, n);
+      s_hl[d] = hl_of_load(x);
     }
   }
-  Completions done_at(a, smem, S.cnt);
-  if (kInfl)
+  Completions done_at;
+  if (kWalk == kContend)
     for (uint32_t p = lane; p < t.P; p += 32) S.cnt[p] = 0u;
   __syncwarp();
-  uint32_t prev_r = kBadCode;  // lane j: the request of the window before's event j, if an arrival
   for (uint64_t k = 0; k <= n_win; ++k) {
     if (k > 0) {
       const uint32_t buf = (uint32_t)((k - 1) & 1);
@@ -684,10 +721,9 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs
       const int32_t* pd = s_wd + (buf ^ 1) * kMaxWindow;
       const uint32_t* pmiss = s_wmiss + (buf ^ 1) * kMaxWindow;
       // lane i prepares event i
-      uint32_t type = kNoEvent, r = kBadCode, my_l = 0, my_miss = 0;
+      uint32_t type = kNoEvent, r = kBadCode, my_l = 0, my_miss = 0, my_pr = 0, ref = 0;
       int32_t my_dd = -1;
       long long my_now = 0;
-      uint32_t my_pr = 0;
       if (lane < win) {
         const ModelEvent& x = ev[lane];
         type = x.type;
@@ -696,7 +732,12 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs
         my_now = x.now;
         my_dd = x.dd;
         my_miss = x.miss;
-        if (type != kNoEvent) r = x.code & 0x7fffffffu;
+        ref = x.ref;
+        r = x.code & 0x7fffffffu;
+        if (ref & kRefPrev) {
+          my_dd = pd[ref & 31u];
+          my_miss = pmiss[ref & 31u];
+        }
         if (type == kBadArrival) {
           wd[lane] = -1;
           s_wb[lane] = s_ws[lane] = kNoKey;
@@ -704,21 +745,7 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs
         }
       }
       const bool is_arr = type == kArrival || type == kBadArrival;
-      const uint32_t any_arr = __ballot_sync(0xffffffffu, is_arr);
       const uint32_t dep_mask = __ballot_sync(0xffffffffu, type == kDeparture);
-      if (dep_mask) {
-        // a departure's arrival may lie in the window before (its decision there) or
-        // earlier in this one (its slot), after the recorded decision was read
-        for (uint32_t j = 0; j < win; ++j) {
-          const uint32_t pr_j = __shfl_sync(0xffffffffu, prev_r, j);
-          if (type == kDeparture && pr_j == r) {
-            my_dd = pd[j];
-            my_miss = pmiss[j];
-          }
-        }
-        const uint32_t same = __match_any_sync(0xffffffffu, r) & any_arr & ((1u << lane) - 1u);
-        if (type == kDeparture && same) my_dd = (int32_t)(kSlotBit | (31u - __clz(same)));
-      }
       uint32_t arr_mask = __ballot_sync(0xffffffffu, type == kArrival);
       uint32_t done = 0;  // events before `done` are applied
       __syncwarp();       // results of bad arrivals are visible
@@ -732,37 +759,26 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs
         uint32_t d = kNone, miss = my_miss;
         if ((bm >> lane) & 1u) {
           int32_t dd = my_dd;
-          if (dd >= 0 && ((uint32_t)dd & kSlotBit)) {
-            const uint32_t slot = (uint32_t)dd & 31u;
-            dd = wd[slot];
-            miss = wmiss[slot];
+          if (ref & kRefOwn) {
+            dd = wd[ref & 31u];
+            miss = wmiss[ref & 31u];
           }
           if (dd >= 0 && (uint32_t)dd < D) d = (uint32_t)dd;
         }
-        auto release = [&](uint32_t at, uint32_t l, uint32_t ms) {
-          if (kInfl) {
-            const int64_t x = s_state[at] - (int64_t)l;
-            s_state[at] = x;
-            s_hl[at] = hl_of(x);
-          } else {
-            s_state[at] += (int64_t)ms * (int64_t)w.bytes_per_token;
-            const int32_t n = s_held[at] - 1;
-            s_held[at] = n;
-            s_term[at] = load_term(a.lm, n);
-          }
-        };
+        const int64_t delta = kWalk == kModel ? (int64_t)miss : -(int64_t)my_l;
         // each lane releases its own decode; departures of one decode (rare) go one by one
-        const uint32_t peers = __match_any_sync(0xffffffffu, d);
-        if (__any_sync(0xffffffffu, d != kNone && __popc(peers) > 1)) {
+        const bool one = __popc(bm) == 1;
+        const uint32_t peers = one ? 0u : __match_any_sync(0xffffffffu, d);
+        if (!one && __any_sync(0xffffffffu, d != kNone && __popc(peers) > 1)) {
           uint32_t rest = __ballot_sync(0xffffffffu, d != kNone);
           while (rest) {
             const uint32_t src = __ffs(rest) - 1;
             rest &= rest - 1;
-            if (lane == src) release(d, my_l, miss);
+            if (lane == src) change(d, delta, 1);
             __syncwarp();
           }
         } else if (d != kNone) {
-          release(d, my_l, miss);
+          change(d, delta, 1);
         }
         __syncwarp();
       };
@@ -775,34 +791,42 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs
         done = i + 1;
         uint32_t pr = 0, cw = 0;
         long long now = 0;
-        if (kInfl) {
+        if (kWalk == kContend) {
           pr = __shfl_sync(0xffffffffu, my_pr, i);
           now = __shfl_sync(0xffffffffu, my_now, i);
-          done_at.settle(now, lane);
+          done_at.settle(a, smem, S.cnt, now, lane);
           cw = S.cnt[pr];
         }
-        // each lane's best and second-best of decodes lane, lane + 32, ...
+        // each lane's best and second-best of its decodes
         float b = __int_as_float(0x7f800000), s2 = b;
         uint32_t ci = kNone;
-#pragma unroll 4
-        for (uint32_t d = lane; d < D; d += 32) {
-          bool feasible;
-          float sc;
-          if (kInfl) {
-            const uint2 hl = s_hl[d];
-            feasible = l <= hl.x;  // load + l <= cap (l >= 1 here)
-            float net = S.base[row + d];
-            if (cw) net = contended(t, w, S.rows[row + d], cw, net);
-            sc = net + w.w_load * __uint_as_float(hl.y);
-          } else {
-            const uint2 c = S.cand[row + d];
-            feasible = s_state[d] >= (int64_t)c.y * (int64_t)w.bytes_per_token + a.lm.m_min;
-            sc = __uint_as_float(c.x) + w.w_load * s_term[d];
-          }
+        auto visit = [&](uint32_t d, bool feasible, float sc) {
           const bool take = feasible && (ci == kNone || sc < b);
           s2 = take ? b : (feasible ? fminf(s2, sc) : s2);
           b = take ? sc : b;
           ci = take ? d : ci;
+        };
+        if (kWalk == kModel && (!in_tokens || l == kNone)) {  // see clamp32: 2^32 - 1 is a bound
+          for (uint32_t d = lane; d < D; d += 32) {
+            const uint2 c = S.cand[row + d];
+            visit(d, s_state[d] >= (int64_t)c.y * bpt + a.lm.m_min,
+                  __uint_as_float(c.x) + w.w_load * __uint_as_float(s_hl[d].y));
+          }
+        } else {
+#pragma unroll 4
+          for (uint32_t d = lane; d < D; d += 32) {
+            const uint2 hl = s_hl[d];
+            if (kWalk == kModel) {
+              const uint2 c = S.cand[row + d];
+              visit(d, c.y < hl.x,
+                    __uint_as_float(c.x) + w.w_load * __uint_as_float(hl.y));
+            } else {
+              float net = S.base[row + d];
+              if (kWalk == kContend && cw) net = contended(t, w, S.rows[row + d], cw, net);
+              visit(d, l <= hl.x,  // load + l <= cap (l >= 1 here)
+                    __fmaf_rn(w.w_load, __uint_as_float(hl.y), net));
+            }
+          }
         }
         // (key, rank) argmin and second key: the rank and the second depend only on the key
         const uint32_t key = ci == kNone ? kNoKey : score_key(b);
@@ -816,8 +840,12 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs
         int32_t xfer = -1;
         uint32_t miss = 0;
         if (dstar >= 0) {
-          if (kInfl) {
-            // the dispatch's transfer time, tier counter (line 14) and completion
+          if (kWalk == kModel) miss = S.cand[row + dstar].y;
+          if (lane == 0) {
+            if (kWalk == kModel) change((uint32_t)dstar, -(int64_t)miss, -1);
+            else change((uint32_t)dstar, (int64_t)l, 0);
+          }
+          if (kWalk == kContend) {
             const int2 tt = S.dt[row + dstar];
             const uint32_t tau = (uint32_t)tt.y, n = (cw >> (8u * tau)) & 0xffu;
             xfer = tt.x;
@@ -825,25 +853,7 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs
               const XferRow x = S.rows[row + dstar];
               xfer = whole_us(xfer_time(XferParts{x.s_eff, x.bb, x.miss}, n, latency_of(t, tau)));
             }
-            const int64_t ld = s_state[dstar] + (int64_t)l;
-            const uint2 h = hl_of(ld);
-            __syncwarp();
-            if (lane == 0) {
-              s_state[dstar] = ld;
-              s_hl[dstar] = h;
-            }
-            done_at.dispatch(now, xfer, pr, tau, cw, a.inflight_cap, lane);
-          } else {
-            miss = S.cand[row + dstar].y;
-            const int64_t x = s_state[dstar] - (int64_t)miss * (int64_t)w.bytes_per_token;
-            const int32_t n = s_held[dstar] + 1;
-            const float term = load_term(a.lm, n);
-            __syncwarp();
-            if (lane == 0) {
-              s_state[dstar] = x;
-              s_held[dstar] = n;
-              s_term[dstar] = term;
-            }
+            done_at.dispatch(a, smem, S.cnt, now, xfer, pr, tau, cw, lane);
           }
         }
         if (lane == 0) {
@@ -860,15 +870,14 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs
         a.dec[r] = wd[lane];
         a.best[r] = key_score(s_wb[lane]);
         a.second[r] = key_score(s_ws[lane]);
-        if (kInfl) a.xfer_us[r] = s_wx[lane];
+        if (kWalk == kContend) a.xfer_us[r] = s_wx[lane];
       }
-      prev_r = is_arr ? r : kBadCode;
     }
     __syncthreads();
   }
   for (uint32_t d = lane; d < D; d += 32) {
     a.state_final[(uint64_t)stream * D + d] = s_state[d];
-    if (!kInfl) a.held_final[(uint64_t)stream * D + d] = s_held[d];
+    if (kWalk == kModel) a.held_final[(uint64_t)stream * D + d] = s_held[d];
   }
 }
 
@@ -883,12 +892,10 @@ netkv_status launch_walk(const ModelArgs& a, bool small, uint32_t n_streams, cud
     schedule_small_kernel<kWalk, BT><<<n_streams, BT, a.lay.total, s>>>(a);
     return netkv_launch_status();
   }
-  if constexpr (kWalk != kPlain) {
-    if (big) NETKV_CUDA_TRY(cudaFuncSetAttribute(schedule_model_kernel<kWalk == kContend, BT>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)kModelSmem));
-    schedule_model_kernel<kWalk == kContend, BT><<<n_streams, BT, a.lay.total, s>>>(a);
-  }
+  if (big) NETKV_CUDA_TRY(cudaFuncSetAttribute(schedule_model_kernel<kWalk, BT>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)kModelSmem));
+  schedule_model_kernel<kWalk, BT><<<n_streams, BT, a.lay.total, s>>>(a);
   return netkv_launch_status();
 }
 
@@ -906,10 +913,10 @@ bool launch_model(ModelArgs& a, uint32_t n_streams, cudaStream_t s, netkv_status
   }
   const uint32_t D = a.t.D;
   const bool small = D <= 32;
-  if (!small && kWalk == kPlain) return false;
   // producers enough for a window's candidates (about 16 arrivals) in one or two rounds
   // while the streams leave the SMs room
-  uint32_t bt = kWalk == kPlain ? 64u : small ? 128u : D <= 96 ? 256u : 512u;
+  uint32_t bt = kWalk == kPlain ? (small ? 64u : D <= 256 ? 128u : 256u)
+                                : small ? 128u : D <= 96 ? 256u : 512u;
   while (bt > 64u && (uint64_t)n_streams * bt > (uint64_t)sms * 1024u) bt /= 2;
   const uint32_t per_sm = (n_streams + (uint32_t)sms - 1) / (uint32_t)sms;
   const uint32_t most = 1024u / bt < per_sm ? 1024u / bt : per_sm;
@@ -997,7 +1004,7 @@ bool launch_model_load(const TopoArgs& t, uint32_t n_streams, const netkv_weight
   return launch_model<kModel>(a, n_streams, s, result);
 }
 
-bool launch_small_plain(const TopoArgs& t, uint32_t n_streams, const netkv_weights* d_w,
+bool launch_model_plain(const TopoArgs& t, uint32_t n_streams, const netkv_weights* d_w,
                         uint32_t R, const uint32_t* d_len, const uint32_t* d_prefill,
                         const uint32_t* d_snap, uint32_t n_snap, const uint32_t* d_events,
                         const uint64_t* d_event_off, const int64_t* d_load_init, int32_t* d_dec,

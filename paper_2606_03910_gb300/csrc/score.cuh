@@ -152,7 +152,7 @@ struct DoneHeap {
 
 // The walks with producers (schedule_model.cu); false when the pool or its tables do not fit:
 // nothing is launched.
-bool launch_small_plain(const TopoArgs& t, uint32_t n_streams, const netkv_weights* d_w,
+bool launch_model_plain(const TopoArgs& t, uint32_t n_streams, const netkv_weights* d_w,
                         uint32_t R, const uint32_t* d_len, const uint32_t* d_prefill,
                         const uint32_t* d_snap, uint32_t n_snap, const uint32_t* d_events,
                         const uint64_t* d_event_off, const int64_t* d_load_init, int32_t* d_dec,
