@@ -1987,6 +1987,10 @@ __global__ void __launch_bounds__(32 * kWinWarps) schedule_window_kernel(
   if (mine) load_final[(uint64_t)stream * D + sl] = load;
 }
 
+// Pools of at most 16 decodes with base scores: one stream per warp with a producer up to
+// here, else the windowed walk, which packs 2 or 4 streams into a warp.  300 requests on 8
+// decodes: one stream 70 us against 135, 1,024 streams 89 against 166, 4,096 streams 285
+// against 174.
 constexpr uint32_t kSmallMaxStreams = 1536;
 constexpr int kStages = 8;
 constexpr uint32_t kHeapPerStream = 4096;       // pending completions, one stream per CTA

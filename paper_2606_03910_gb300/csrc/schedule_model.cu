@@ -913,6 +913,14 @@ bool launch_model(ModelArgs& a, uint32_t n_streams, cudaStream_t s, netkv_status
   }
   const uint32_t D = a.t.D;
   const bool small = D <= 32;
+  // Many streams over large pools keep every SM busy with one CTA of several scoring warps per
+  // stream, and the rows of a window no longer leave room for several CTAs here.  60 requests
+  // a stream, this walk against the per-event one (us): base scores, 1,024 decodes, 400
+  // streams 137 / 151, 1,500 streams 1,374 / 464, 288 decodes 1,500 streams 176 / 463;
+  // self-contention, 288 decodes, 400 streams 245 / 422, 1,500 streams 3,137 / 1,143; load
+  // model, 1,024 decodes, 8 streams 255 / 424, 400 streams 512 / 416.
+  const uint64_t pool = (uint64_t)D * n_streams;
+  if (kWalk == kPlain ? D > 512 && pool > 512u * 1024u : D > 96 && pool > 256u * 1024u) return false;
   // producers enough for a window's candidates (about 16 arrivals) in one or two rounds
   // while the streams leave the SMs room
   uint32_t bt = kWalk == kPlain ? (small ? 64u : D <= 256 ? 128u : 256u)
