@@ -15,7 +15,7 @@
 //   schedule_small_kernel  pools of at most 32 decodes: lane d holds decode d's state in
 //                          registers and the argmin is one reduction and one ballot
 //   schedule_model_kernel  larger pools, self-contention and load model: the state lies in
-//                          shared memory, lane i takes decodes i, i + 32, ...
+//                          shared memory, a lane takes pairs of decodes
 // Bound by the walker's chain of dependent instructions per event.
 #include <math.h>
 
@@ -73,6 +73,9 @@ __device__ __forceinline__ float latency_of(const TopoArgs& t, uint32_t tau) {
 }
 
 // Byte offsets of the dynamic shared memory.
+// Rows of candidates are padded to an even number of decodes, so that pairs load as one.
+__host__ __device__ inline uint32_t row_stride(uint32_t D) { return (D + 1u) & ~1u; }
+
 struct ModelLayout {
   uint32_t win;
   uint32_t ev, arr, narr, wd, wmiss, wb, ws, wx, state, tok, term, held, cnt, heap, rel, base, rows, dt,
@@ -89,7 +92,7 @@ ModelLayout model_layout(Walk walk, bool small, uint32_t D, uint32_t P, uint32_t
     return o;
   };
   const bool infl = walk == kContend;
-  const size_t cand = (size_t)2 * win * D;
+  const size_t cand = (size_t)2 * win * row_stride(D);
   a.win = win;
   a.ev = take(2 * win * sizeof(ModelEvent));
   a.arr = take(2 * kMaxWindow * 4);
@@ -102,9 +105,9 @@ ModelLayout model_layout(Walk walk, bool small, uint32_t D, uint32_t P, uint32_t
   a.wx = take(small ? 0 : kMaxWindow * 4);
   a.state = take(small ? 0 : (size_t)D * 8);              // load or free bytes
   a.tok = take(small || walk != kModel ? 0 : (size_t)D * 8);
-  a.term = take(small ? 0 : (size_t)D * 8);               // (tokens that fit, load term)
+  a.term = take(small ? 0 : (size_t)row_stride(D) * 8);               // (tokens that fit, load term)
   a.held = take(small || walk != kModel ? 0 : (size_t)D * 4);
-  a.cnt = take(infl ? (size_t)P * 4 : 0);
+  a.cnt = take(infl ? (size_t)(P < 32 ? 32 : P) * 4 : 0);
   a.heap = take(infl ? (size_t)heap_cap * 8 : 0);
   a.rel = take(small ? (size_t)(kMaxWindow + 1) * 32 * (walk == kModel ? 8 : 4) : 0);
   a.base = take(cand * (walk == kModel ? 8 : 4));
@@ -143,10 +146,10 @@ struct ModelShared {
   ModelEvent* ev;    // [2][win]
   uint32_t* arr;     // [2][kMaxWindow] slots of a window's arrivals
   uint32_t* narr;    // [2]
-  float* base;       // [2][win][D]
+  float* base;       // [2][win][row_stride(D)]
   uint2* cand;       // load model: (score, missed tokens)
-  XferRow* rows;     // [2][win][D]
-  int2* dt;          // [2][win][D] uncontended transfer time in us, tier
+  XferRow* rows;     // [2][win][row_stride(D)]
+  int2* dt;          // [2][win][row_stride(D)] uncontended transfer time in us, tier
   uint32_t* cnt;     // self-contention: n_inflight, byte `tier` of cnt[prefill rank]
   __device__ ModelShared(unsigned char* smem, const ModelLayout& l)
       : ev(reinterpret_cast<ModelEvent*>(smem + l.ev)),
@@ -161,13 +164,22 @@ struct ModelShared {
 
 // The producers: in step k of the block they fill window k while the walker walks window
 // k - 1; every step ends with a block barrier.
+// Warps 4, 8, ... share warp 0's scheduler and only keep the barriers: a producer there took
+// issue slots from the walker (262 decodes under the load model: 459 us with all warps
+// producing, of which 68 were theirs).
 template <Walk kWalk, int BT>
 __device__ __forceinline__ void produce(const ModelArgs& a, const netkv_weights& w,
                                         const ModelShared& S, uint64_t e0, uint64_t e1,
                                         uint64_t n_win) {
-  constexpr uint32_t NP = BT - 32;
+  constexpr uint32_t NP = BT == 64 ? 32u : BT / 4 * 3;  // producing threads
   const TopoArgs& t = a.t;
-  const uint32_t D = t.D, win = a.lay.win, ptid = threadIdx.x - 32;
+  const uint32_t wid = threadIdx.x >> 5;
+  if (wid % 4 == 0) {
+    for (uint64_t k = 0; k <= n_win; ++k) __syncthreads();
+    return;
+  }
+  const uint32_t D = t.D, win = a.lay.win;
+  const uint32_t ptid = (wid - 1 - wid / 4) * 32 + (threadIdx.x & 31);
   const uint32_t step_q = NP / D, step_d = NP % D;
   uint32_t code = ptid < win && e0 + ptid < e1 ? __ldg(a.events + e0 + ptid) : kBadCode;
   uint32_t prev_r = kBadCode;  // lane j: event j of the window before: its request, if an arrival
@@ -251,7 +263,7 @@ __device__ __forceinline__ void produce(const ModelArgs& a, const netkv_weights&
         if (ptid == 0) S.narr[k & 1] = __popc(list);
       }
       if (BT == 64) __syncwarp();
-      else asm volatile("bar.sync 1, %0;" ::"n"(BT - 32) : "memory");
+      else asm volatile("bar.sync 1, %0;" ::"n"(NP) : "memory");
       // candidates (arrival, decode), decodes fastest, kAhead of a thread in flight
       const uint32_t na = S.narr[k & 1];
       uint32_t q = ptid / D, d = ptid % D;
@@ -295,7 +307,7 @@ __device__ __forceinline__ void produce(const ModelArgs& a, const netkv_weights&
 #pragma unroll
         for (int u = 0; u < kAhead; ++u) {
           if (ci[u] == kNone) continue;
-          const size_t at = ((k & 1) * win + ci[u]) * (size_t)D + cd[u];
+          const size_t at = ((k & 1) * win + ci[u]) * (size_t)row_stride(D) + cd[u];
           if (kWalk == kPlain) {
             S.base[at] = ubd[u];
             continue;
@@ -341,11 +353,17 @@ __device__ __noinline__ void heap_push(unsigned long long* a, uint32_t n, uint32
   DoneHeap h = {a, n, cap};
   h.push(key);
 }
+template <bool kRegs>  // counters of at most 32 prefill ranks: lane p holds rank p's
 struct Completions {
   static constexpr unsigned long long kFree = ~0ull;  // above every key: prefill < 2^14 - 1
   unsigned long long key;  // time in us << 16 | prefill rank << 2 | tier
   uint32_t in_heap;        // the same in every lane
-  __device__ Completions() : key(kFree), in_heap(0) {}
+  uint32_t mine;           // kRegs: the lane's counters
+  __device__ Completions() : key(kFree), in_heap(0), mine(0) {}
+  // The counters of prefill pr, a byte per tier.
+  __device__ __forceinline__ uint32_t counters(const uint32_t* cnt, uint32_t pr) const {
+    return kRegs ? __shfl_sync(0xffffffffu, mine, pr) : cnt[pr];
+  }
   // Transfers completed by `now` lower their counters (Algorithm 1 line 14's callback).
   __device__ __forceinline__ void settle(const ModelArgs& a, unsigned char* smem, uint32_t* cnt,
                                          long long now, uint32_t lane) {
@@ -355,15 +373,25 @@ struct Completions {
     while (dm) {
       const uint32_t j = __ffs(dm) - 1;
       dm &= dm - 1;
-      if (lane == j) lower_counter(cnt, (uint32_t)key & 0xffffu);
-      __syncwarp();
+      if (kRegs) {
+        const uint32_t pt = __shfl_sync(0xffffffffu, (uint32_t)key & 0xffffu, j);
+        const uint32_t sh = 8u * (pt & 3u);
+        if (lane == pt >> 2 && ((mine >> sh) & 0xffu)) mine -= 1u << sh;
+      } else {
+        if (lane == j) lower_counter(cnt, (uint32_t)key & 0xffffu);
+        __syncwarp();
+      }
     }
     if (due) key = kFree;
     if (in_heap) {
+      if (kRegs) cnt[lane] = mine;  // the heap lowers them in memory
+      __syncwarp();
       if (lane == 0)
         in_heap = heap_settle(reinterpret_cast<unsigned long long*>(smem + a.lay.heap), in_heap,
                               a.heap_cap, cnt, now);
       in_heap = __shfl_sync(0xffffffffu, in_heap, 0);
+      __syncwarp();
+      if (kRegs) mine = cnt[lane];
     }
   }
   // A dispatch on tier tau of prefill pr, whose counters are cw: the counter and the
@@ -377,14 +405,16 @@ struct Completions {
     const uint32_t sh = 8u * tau;
     const uint32_t at = free ? (uint32_t)(__ffs(free) - 1) : 0u;
     const bool full = 32u - __popc(free) + in_heap >= a.heap_cap;
-    if (lane == at) {  // one lane does it all
-      if (((cw >> sh) & 0xffu) < a.inflight_cap) cnt[pr] = cw + (1u << sh);
+    const bool up = ((cw >> sh) & 0xffu) < a.inflight_cap;
+    if (kRegs && up && lane == pr) mine += 1u << sh;
+    if (lane == at) {
+      if (!kRegs && up) cnt[pr] = cw + (1u << sh);
       if (full) flag_status(a.status, NETKV_DEV_EFULL);
       else if (free) key = k;
       else heap_push(reinterpret_cast<unsigned long long*>(smem + a.lay.heap), in_heap, a.heap_cap, k);
     }
     if (!full && !free) ++in_heap;
-    __syncwarp();
+    if (!kRegs || !free) __syncwarp();
   }
 };
 
@@ -398,8 +428,11 @@ __device__ __forceinline__ float contended(const TopoArgs& t, const netkv_weight
   return w.w_net * T + w.w_prefix * p.miss;
 }
 
-template <Walk kWalk, int BT>
-__global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs a) {
+// kRegs: at most 32 prefill ranks (self-contention).  Blocks of 128 threads are for few
+// streams: registers without spills; blocks of 64 for many: residency.
+template <Walk kWalk, int BT, bool kRegs>
+__global__ void __launch_bounds__(BT, BT >= 128 ? 512 / BT : 1024 / BT)
+    schedule_small_kernel(ModelArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const TopoArgs& t = a.t;
   const uint32_t D = t.D, win = a.lay.win, lane = threadIdx.x & 31;
@@ -429,8 +462,8 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs
   // what the last dispatch took on its decode's lane (tokens, or missed tokens of one
   // request), applied with the releases before the next arrival
   uint32_t own = 0, own_n = 0;
-  Completions done_at;
-  if (kWalk == kContend)
+  Completions<kRegs> done_at;
+  if (kWalk == kContend && !kRegs)
     for (uint32_t p = lane; p < t.P; p += 32) S.cnt[p] = 0u;
   __syncwarp();
 
@@ -507,11 +540,16 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs
       };
       // an arrival's length, this lane's candidate and the releases before it: read one
       // arrival ahead
-      uint32_t l_n = 0, rel_n = 0, reln_n = 0, miss_n = 0;
+      uint32_t l_n = 0, rel_n = 0, reln_n = 0, miss_n = 0, pr_n = 0;
+      long long now_n = 0;
       float net_n = 0.f;
       auto fetch = [&](uint32_t i) {
-        const size_t row = (buf * win + i) * (size_t)D;
+        const size_t row = (buf * win + i) * (size_t)row_stride(D);
         l_n = __shfl_sync(0xffffffffu, l_ev, i);
+        if (kWalk == kContend) {
+          pr_n = __shfl_sync(0xffffffffu, pr_ev, i);
+          now_n = __shfl_sync(0xffffffffu, now_ev, i);
+        }
         if (mine) {
           if (kWalk == kModel) {
             const uint2 c = S.cand[row + lane];
@@ -547,7 +585,8 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs
       while (todo) {
         const uint32_t i = __ffs(todo) - 1;
         todo &= todo - 1;
-        const uint32_t l = l_n, miss = miss_n;
+        const uint32_t l = l_n, miss = miss_n, pr = pr_n;
+        const long long now = now_n;
         float net = net_n;
         advance();
         const uint32_t before = left & ((1u << i) - 1u);
@@ -558,14 +597,11 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs
         ++b;
         if (todo) fetch(__ffs(todo) - 1);
         fetch_rel(b);
-        uint32_t pr = 0, cw = 0;
-        long long now = 0;
-        const size_t row = (buf * win + i) * (size_t)D;
+        uint32_t cw = 0;
+        const size_t row = (buf * win + i) * (size_t)row_stride(D);
         if (kWalk == kContend) {
-          pr = __shfl_sync(0xffffffffu, pr_ev, i);
-          now = __shfl_sync(0xffffffffu, now_ev, i);
           done_at.settle(a, smem, S.cnt, now, lane);
-          cw = S.cnt[pr];
+          cw = done_at.counters(S.cnt, pr);
           if (cw && mine) net = contended(t, w, S.rows[row + lane], cw, net);
         }
         bool feasible;
@@ -647,7 +683,8 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_small_kernel(ModelArgs
 // < 2^31 (products of 32-bit token counts then stay in 63 bits); a stream with other bytes,
 // and a request of 2^32 - 1 tokens, compare bytes instead.
 template <Walk kWalk, int BT>
-__global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs a) {
+__global__ void __launch_bounds__(BT, BT >= 256 ? 512 / BT : 1024 / BT)
+    schedule_model_kernel(ModelArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const TopoArgs& t = a.t;
   const uint32_t D = t.D, win = a.lay.win, lane = threadIdx.x & 31;
@@ -661,7 +698,7 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs
     return;
   }
 
-  // ---- the walker: lane i takes decodes i, i + 32, ...
+  // ---- the walker: lane i takes decodes 2 i, 2 i + 1, 2 i + 64, ...
   int32_t* s_wd = reinterpret_cast<int32_t*>(smem + a.lay.wd);          // [2][kMaxWindow]
   uint32_t* s_wmiss = reinterpret_cast<uint32_t*>(smem + a.lay.wmiss);  // [2][kMaxWindow]
   uint32_t* s_wb = reinterpret_cast<uint32_t*>(smem + a.lay.wb);
@@ -708,7 +745,8 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs
       s_hl[d] = hl_of_load(x);
     }
   }
-  Completions done_at;
+  Completions<false> done_at;
+  if (lane == 0 && (D & 1u)) s_hl[D] = make_uint2(0u, 0u);  // the padding fits nothing
   if (kWalk == kContend)
     for (uint32_t p = lane; p < t.P; p += 32) S.cnt[p] = 0u;
   __syncwarp();
@@ -786,7 +824,7 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs
         const uint32_t i = __ffs(arr_mask) - 1;
         arr_mask &= arr_mask - 1;
         const uint32_t l = __shfl_sync(0xffffffffu, my_l, i);
-        const size_t row = (buf * win + i) * (size_t)D;
+        const size_t row = (buf * win + i) * (size_t)row_stride(D);
         depart(i);
         done = i + 1;
         uint32_t pr = 0, cw = 0;
@@ -795,38 +833,58 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs
           pr = __shfl_sync(0xffffffffu, my_pr, i);
           now = __shfl_sync(0xffffffffu, my_now, i);
           done_at.settle(a, smem, S.cnt, now, lane);
-          cw = S.cnt[pr];
+          cw = done_at.counters(S.cnt, pr);
         }
-        // each lane's best and second-best of its decodes
-        float b = __int_as_float(0x7f800000), s2 = b;
-        uint32_t ci = kNone;
-        auto visit = [&](uint32_t d, bool feasible, float sc) {
-          const bool take = feasible && (ci == kNone || sc < b);
-          s2 = take ? b : (feasible ? fminf(s2, sc) : s2);
-          b = take ? sc : b;
-          ci = take ? d : ci;
+        // Each lane's best and second-best of its decodes: with base scores in two independent
+        // chains (even and odd ranks) merged at the end (1,024 decodes: 107 against 133 us for
+        // 128 arrivals on each of 64 streams), else in one (262 decodes under the load model:
+        // 423 against 456 us).
+        constexpr bool kTwo = kWalk == kPlain;
+        const float inf = __int_as_float(0x7f800000);
+        float b = inf, s2 = inf, bo = inf, so = inf;
+        uint32_t ci = kNone, co = kNone;
+        auto visit = [](float& cb, float& cs, uint32_t& cc, uint32_t d, bool feasible, float sc) {
+          const bool take = feasible && (cc == kNone || sc < cb);
+          cs = take ? cb : (feasible ? fminf(cs, sc) : cs);
+          cb = take ? sc : cb;
+          cc = take ? d : cc;
         };
         if (kWalk == kModel && (!in_tokens || l == kNone)) {  // see clamp32: 2^32 - 1 is a bound
-          for (uint32_t d = lane; d < D; d += 32) {
+          for (uint32_t d = lane; d < D; d += 32) {  // ranks rise within a lane, as below
             const uint2 c = S.cand[row + d];
-            visit(d, s_state[d] >= (int64_t)c.y * bpt + a.lm.m_min,
+            visit(b, s2, ci, d, s_state[d] >= (int64_t)c.y * bpt + a.lm.m_min,
                   __uint_as_float(c.x) + w.w_load * __uint_as_float(s_hl[d].y));
           }
         } else {
-#pragma unroll 4
-          for (uint32_t d = lane; d < D; d += 32) {
-            const uint2 hl = s_hl[d];
+          constexpr int kUnroll = kWalk == kPlain ? 4 : 2;
+#pragma unroll kUnroll
+          for (uint32_t d = 2 * lane; d < D; d += 64) {
+            const uint4 hl = *reinterpret_cast<const uint4*>(s_hl + d);
             if (kWalk == kModel) {
-              const uint2 c = S.cand[row + d];
-              visit(d, c.y < hl.x,
+              const uint4 c = *reinterpret_cast<const uint4*>(S.cand + row + d);
+              visit(b, s2, ci, d, c.y < hl.x,
                     __uint_as_float(c.x) + w.w_load * __uint_as_float(hl.y));
+              visit(b, s2, ci, d + 1, c.w < hl.z,
+                    __uint_as_float(c.z) + w.w_load * __uint_as_float(hl.w));
             } else {
-              float net = S.base[row + d];
-              if (kWalk == kContend && cw) net = contended(t, w, S.rows[row + d], cw, net);
-              visit(d, l <= hl.x,  // load + l <= cap (l >= 1 here)
-                    __fmaf_rn(w.w_load, __uint_as_float(hl.y), net));
+              float2 net = *reinterpret_cast<const float2*>(S.base + row + d);
+              if (kWalk == kContend && cw) {
+                net.x = contended(t, w, S.rows[row + d], cw, net.x);
+                if (d + 1 < D) net.y = contended(t, w, S.rows[row + d + 1], cw, net.y);
+              }
+              // load + l <= cap (l >= 1 here)
+              visit(b, s2, ci, d, l <= hl.x,
+                    __fmaf_rn(w.w_load, __uint_as_float(hl.y), net.x));
+              visit(kTwo ? bo : b, kTwo ? so : s2, kTwo ? co : ci, d + 1, l <= hl.z,
+                    __fmaf_rn(w.w_load, __uint_as_float(hl.w), net.y));
             }
           }
+        }
+        if (kTwo) {
+          const bool other = bo < b || (bo == b && co < ci);
+          s2 = other ? fminf(so, b) : fminf(s2, bo);
+          b = other ? bo : b;
+          ci = other ? co : ci;
         }
         // (key, rank) argmin and second key: the rank and the second depend only on the key
         const uint32_t key = ci == kNone ? kNoKey : score_key(b);
@@ -881,21 +939,14 @@ __global__ void __launch_bounds__(BT, 1024 / BT) schedule_model_kernel(ModelArgs
   }
 }
 
-template <Walk kWalk, int BT>
-netkv_status launch_walk(const ModelArgs& a, bool small, uint32_t n_streams, cudaStream_t s) {
-  // the attribute is per device: set before every launch that needs it
-  const bool big = a.lay.total > 48u * 1024u;
-  if constexpr (BT <= 128) if (small) {
-    if (big) NETKV_CUDA_TRY(cudaFuncSetAttribute(schedule_small_kernel<kWalk, BT>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)kModelSmem));
-    schedule_small_kernel<kWalk, BT><<<n_streams, BT, a.lay.total, s>>>(a);
-    return netkv_launch_status();
-  }
-  if (big) NETKV_CUDA_TRY(cudaFuncSetAttribute(schedule_model_kernel<kWalk, BT>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)kModelSmem));
-  schedule_model_kernel<kWalk, BT><<<n_streams, BT, a.lay.total, s>>>(a);
+// The attribute is per device: set before every launch that needs it.
+template <typename Kernel>
+netkv_status launch_walk(Kernel kernel, const ModelArgs& a, uint32_t n_streams, uint32_t bt,
+                         cudaStream_t s) {
+  if (a.lay.total > 48u * 1024u)
+    NETKV_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)kModelSmem));
+  kernel<<<n_streams, bt, a.lay.total, s>>>(a);
   return netkv_launch_status();
 }
 
@@ -921,11 +972,15 @@ bool launch_model(ModelArgs& a, uint32_t n_streams, cudaStream_t s, netkv_status
   // model, 1,024 decodes, 8 streams 255 / 424, 400 streams 512 / 416.
   const uint64_t pool = (uint64_t)D * n_streams;
   if (kWalk == kPlain ? D > 512 && pool > 512u * 1024u : D > 96 && pool > 256u * 1024u) return false;
-  // producers enough for a window's candidates (about 16 arrivals) in one or two rounds
-  // while the streams leave the SMs room
-  uint32_t bt = kWalk == kPlain ? (small ? 64u : D <= 256 ? 128u : 256u)
-                                : small ? 128u : D <= 96 ? 256u : 512u;
-  while (bt > 64u && (uint64_t)n_streams * bt > (uint64_t)sms * 1024u) bt /= 2;
+  // producers enough for a window's candidates (about 16 arrivals) in a few rounds while
+  // every stream is resident
+  uint32_t bt = 64u;
+  if (small) {
+    if (kWalk != kPlain && n_streams <= 4u * (uint32_t)sms) bt = 128u;
+  } else {
+    bt = D <= 96 || (kWalk == kPlain && D <= 512) ? 256u : 512u;
+    while (bt > 64u && (uint64_t)n_streams * bt > (uint64_t)sms * 512u) bt /= 2;
+  }
   const uint32_t per_sm = (n_streams + (uint32_t)sms - 1) / (uint32_t)sms;
   const uint32_t most = 1024u / bt < per_sm ? 1024u / bt : per_sm;
   uint32_t win = 0;
@@ -937,10 +992,22 @@ bool launch_model(ModelArgs& a, uint32_t n_streams, cudaStream_t s, netkv_status
   }
   if (win == 0) return false;
   a.lay = model_layout(kWalk, small, D, a.t.P, a.heap_cap, win);
-  if (bt == 64) *result = launch_walk<kWalk, 64>(a, small, n_streams, s);
-  else if (bt == 128) *result = launch_walk<kWalk, 128>(a, small, n_streams, s);
-  else if (bt == 256) *result = launch_walk<kWalk, 256>(a, small, n_streams, s);
-  else *result = launch_walk<kWalk, 512>(a, small, n_streams, s);
+  const bool regs = kWalk == kContend && a.t.P <= 32;
+  if (small && bt == 128u) {
+    if (regs) *result = launch_walk(schedule_small_kernel<kWalk, 128, kWalk == kContend>, a, n_streams, bt, s);
+    else *result = launch_walk(schedule_small_kernel<kWalk, 128, false>, a, n_streams, bt, s);
+  } else if (small) {
+    if (regs) *result = launch_walk(schedule_small_kernel<kWalk, 64, kWalk == kContend>, a, n_streams, bt, s);
+    else *result = launch_walk(schedule_small_kernel<kWalk, 64, false>, a, n_streams, bt, s);
+  } else if (bt == 64u) {
+    *result = launch_walk(schedule_model_kernel<kWalk, 64>, a, n_streams, bt, s);
+  } else if (bt == 128u) {
+    *result = launch_walk(schedule_model_kernel<kWalk, 128>, a, n_streams, bt, s);
+  } else if (bt == 256u) {
+    *result = launch_walk(schedule_model_kernel<kWalk, 256>, a, n_streams, bt, s);
+  } else {
+    *result = launch_walk(schedule_model_kernel<kWalk, 512>, a, n_streams, bt, s);
+  }
   return true;
 }
 
