@@ -75,21 +75,15 @@ __device__ __forceinline__ void seg_argmin_t(float& b, uint32_t& i, float& s, fl
   }
 }
 
-// s_eff / Bbot, the factor self-contention multiplies by 1 + n (Eq. 4): written beside
-// the base scores when the greedy runs with self-contention.
-__device__ __forceinline__ float xfer_factor(const netkv_weights& w, uint32_t l, uint32_t m,
-                                             float ub_p, float ub_d) {
-  const uint32_t lam = min(16u * m, l);
-  const float s_eff = (float)((int64_t)(l - lam) * (int64_t)w.bytes_per_token);
-  return s_eff / fminf(ub_p, ub_d);
-}
-
 // Base scores of every arrival (pools of at most 32 decodes): the events of a stream are
 // split into contiguous ranges over the segments (LPS lanes each) of grid.y blocks, and
-// lane sl of a segment owns decode sl.  As in base_wide_kernel, a lane keeps its decode's
-// quotients bytes_per_token / UB_d[k] for the current snapshot and each arrival divides
-// once per level for its prefill and once for 1 / l:
-//     base = w_net * (miss_tok * max(qp[tau], qd[tau]) + L_tau) + w_prefix * miss_tok * (1/l)
+// lane sl of a segment owns decode sl.  A lane keeps its decode's level bottlenecks for the
+// current snapshot and divides twice per arrival:
+//     base = w_net * (miss_tok * (bytes_per_token / min(UB_p[tau], UB_d[tau])) + L_tau)
+//            + w_prefix * miss_tok * (1 / l)
+// Bound by instruction issue: 1.02 M arrivals on 8 decodes, whose
+// snapshot mostly changes with each arrival, 157 us, against 176 with the decode's four
+// quotients taken per snapshot.
 // Departures and invalid events are skipped (the greedy reports them).  kUtil: `UB` holds
 // the utilisation rows [n_snap][n_links] instead of the level bottlenecks, and the
 // bottlenecks are taken from the links' entries.  X (self-contention) gets s_eff / Bbot.
@@ -131,7 +125,7 @@ __global__ void __launch_bounds__(256, 6) base_kernel(
     const uint64_t eb = e0 + ((uint64_t)blockIdx.y * kSegs + seg) * span;
     const uint64_t ee = min(e1, eb + span);
     uint32_t cur_k = 0xffffffffu;
-    float4 qd = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 ubd = make_float4(0.f, 0.f, 0.f, 0.f);
     // software pipeline: the next event's fields and the code after it are loaded while
     // the current arrival is scored, so an arrival waits for one round trip (its
     // utilisation entries) instead of three
@@ -149,9 +143,8 @@ __global__ void __launch_bounds__(256, 6) base_kernel(
       if (pr >= t.P || k >= n_snap || l == 0 || !mine) continue;
       if (k != cur_k) {  // the decode's level bottlenecks of a new snapshot
         cur_k = k;
-        const float4 ub = kUtil ? level_bottlenecks_of(t, UB + (uint64_t)k * t.n_links, ld, status)
-                                : __ldg(reinterpret_cast<const float4*>(UB) + (uint64_t)k * N + inst);
-        qd = make_float4(bpt / ub.x, bpt / ub.y, bpt / ub.z, bpt / ub.w);
+        ubd = kUtil ? level_bottlenecks_of(t, UB + (uint64_t)k * t.n_links, ld, status)
+                    : __ldg(reinterpret_cast<const float4*>(UB) + (uint64_t)k * N + inst);
       }
       const uint32_t pinst = __ldg(t.pre + pr);
       const uint4 lp = __ldg(t.links + pinst);
@@ -165,7 +158,7 @@ __global__ void __launch_bounds__(256, 6) base_kernel(
         lam = lam < l ? lam : l;
       }
       const float miss_tok = (float)(l - lam);
-      const float q = fmaxf(bpt / ubp, pick4(qd, tau));
+      const float q = bpt / fminf(ubp, pick4(ubd, tau));
       const float T = __fmaf_rn(miss_tok, q, pick4(lat, tau));
       base[(uint64_t)r * D + sl] = __fmaf_rn(w_net, T, w_prefix * (miss_tok * (1.0f / (float)l)));
       if (X) X[(uint64_t)r * D + sl] = miss_tok * q;
@@ -176,10 +169,11 @@ __global__ void __launch_bounds__(256, 6) base_kernel(
 // ---- candidate lists: a bound on every decode a walk need not rescore ----------------
 // The load term of a score is w_load * theta * load >= 0, so a decode's score is never below
 // its base score, and the fp32 score fma(w_load, theta * load, base) is monotone in both the
-// load and the base.  For each arrival the base pass lists the pool's kListLen smallest
-// (base, rank) pairs in that order and a bound (tau, tau_rank): every decode not listed has
-// (base, rank) >= (tau, tau_rank).  A walk that knows a lower bound
-// L on every decode's current load then has, for every unlisted decode d,
+// load and the base.  For each arrival chunk_lists_kernel and merge_lists_kernel list the pool's
+// kListLen smallest (base, rank) pairs in that order (fewer only where a chunk lists fewer) and
+// a bound (tau, tau_rank): every decode not listed has (base, rank) >= (tau, tau_rank).  A walk
+// that knows a lower bound L on every decode's current load then has, for every unlisted
+// decode d,
 //     score(d) >= fma(w_load, theta * L, base(d)) >= fma(w_load, theta * L, tau) =: LB,
 // so the best listed (score, rank) is the argmin of all decodes when its score is below LB, or
 // equal to tau with a rank below tau_rank (with L >= 0, an unlisted decode scores at least its
@@ -189,126 +183,159 @@ __global__ void __launch_bounds__(256, 6) base_kernel(
 // Bound keys: score_key(tau), or kNoKey when every decode of the pool is listed, or
 // kBoundInvalid (below every float's key) when the list cannot bound anything (a NaN score).
 constexpr int kListLen = 32;             // (rank, base) pairs listed per arrival: one a lane
-constexpr uint32_t kListChunk = 1024;    // decodes per base-pass block (256 threads, 4 each)
+constexpr uint32_t kListChunk = 1024;    // decodes a warp lists: 32 a lane
 constexpr uint32_t kListMinD = 1025;     // listed pools: 1,025 .. 4,096 decodes, whose
 constexpr uint32_t kListMaxD = 4096;     // 2 .. 4 chunk lists are merged into the pool's
 // The list arrays of a workspace (all null: the staged walk runs).
 struct ListWs {
   uint2 *chunk_lists = nullptr, *chunk_bounds = nullptr, *lists = nullptr, *bounds = nullptr;
 };
-constexpr int kListLevels = 8;           // distinct base scores a block walks up per arrival
+constexpr uint32_t kListCand = 64;       // pairs below a warp's threshold that it ranks
 constexpr uint32_t kBoundInvalid = 0u;
 
-// Per-level exchange of a block's NW <= 32 warps, double-buffered by barrier phase.
-template <int NW>
-struct ListShared {
-  uint32_t cnt[2][NW];  // pairs of the warp at the current key
-  uint32_t nxt[2][NW];  // the warp's smallest key above it
-};
+// ascending 32-lane bitonic sort, one value a lane
+__device__ __forceinline__ uint32_t warp_sort(uint32_t v, uint32_t lane) {
+#pragma unroll
+  for (uint32_t k = 2; k <= 32; k <<= 1) {
+#pragma unroll
+    for (uint32_t j = k >> 1; j; j >>= 1) {
+      const uint32_t o = __shfl_xor_sync(0xffffffffu, v, j);
+      v = ((lane & j) == 0) == ((lane & k) == 0) ? min(v, o) : max(v, o);
+    }
+  }
+  return v;
+}
 
-// The pool's list and bound for one arrival, by the whole block: walking up the distinct
-// keys of the pool (at most kListLevels of them), the pairs of each key are listed in rank
-// order until kListLen are listed; the next pair is the bound.  Every warp first finds its
-// smallest key and how many of its pairs hold it, so that after one block barrier the
-// pool's smallest key and its pairs are placed: when there are more than kListLen of them
-// (ties, the common case) that barrier is the only one.  Each further level costs one
-// barrier: every warp counts its pairs at the key and finds its smallest key above it, and
-// after the barrier each thread places its own pairs by the counts of the warps before it.
-// When the levels run out first, the bound is (next key, rank 0) or, with no key left, the
-// pool is listed entirely (kNoKey).  k: the thread's NPT = 4 keys (kNoKey past D) of
-// decodes d0 .. d0 + 3 (lane-major within a warp, warps in rank order).  `phase` counts the
-// block's barrier phases (uniform).  NaN scores make the bound kBoundInvalid.
-template <int NW>
-__device__ __forceinline__ void block_levels(ListShared<NW>& S, uint32_t& phase, const uint32_t (&k)[4],
-                                             bool nan, uint32_t d0, uint2* __restrict__ out,
-                                             uint2* __restrict__ bound) {
-  const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+// The list and bound of one chunk of up to 1,024 decodes of an arrival's base-score row, one
+// warp per (arrival, chunk).  Lane L holds decodes 128 q + 4 L .. + 3 of the chunk, q = 0 .. 7.
+// The 32nd smallest of the 64 minima over a lane's even and odd q is a threshold T that at
+// least 32 pairs reach and few are below: 31 minima at most are, about 44 pairs of 1,024
+// distinct scores.  The pairs below T are gathered in shared memory and each is placed by
+// counting the pairs before it; then pairs at T follow in rank order until the list and its
+// bound are full.  With more than kListCand pairs below, T falls back to smaller minima (the
+// smallest has none below it), and the list may hold fewer than kListLen pairs.
+// Bound by instruction issue: 32,000 arrivals on 4,096 decodes, 207 us (a read of the rows alone
+// takes 77); walking up at most 8 distinct scores with block barriers inside the base pass
+// added 463 us to it and could leave shorter lists.
+__global__ void __launch_bounds__(256, 4) chunk_lists_kernel(
+    const float* __restrict__ base, uint32_t D, uint32_t n_ch, uint32_t R,
+    uint2* __restrict__ lists, uint2* __restrict__ bounds) {
+  __shared__ unsigned long long s_cand[8][kListCand];
+  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const uint32_t below = (1u << lane) - 1u;
-  // pairs of this thread at key v placed from position base_pos (in rank order)
-  auto place = [&](uint32_t v, uint32_t base_pos) {
-    uint32_t pos = base_pos;
+  unsigned long long* cand = s_cand[wid];
+  const float nan = __int_as_float(0x7fffffff);
+  const bool vec = D % 4u == 0 && (reinterpret_cast<uintptr_t>(base) & 15u) == 0;
+  const uint64_t n_tasks = (uint64_t)R * n_ch, n_warps = (uint64_t)gridDim.x * 8;
+  for (uint64_t task = (uint64_t)blockIdx.x * 8 + wid; task < n_tasks; task += n_warps) {
+    const uint32_t c0 = (uint32_t)(task % n_ch) * kListChunk;
+    const uint32_t n = min(D - c0, kListChunk);  // decodes of the chunk
+    const float* row = base + (task / n_ch) * D + c0;
+    uint2* out = lists + task * kListLen;
+    float x[8][4];  // NaN past the chunk: neither below nor at any threshold
+    bool bad = false;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) pos += __popc(__ballot_sync(0xffffffffu, k[j] == v) & below);
+    for (int q = 0; q < 8; ++q) {
+      const uint32_t d = 128u * q + 4u * lane;
+      if (vec) {
+        const float4 v = d < n ? __ldg(reinterpret_cast<const float4*>(row + d))
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
+        x[q][0] = v.x;
+        x[q][1] = v.y;
+        x[q][2] = v.z;
+        x[q][3] = v.w;
+      } else {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (k[j] == v) {
-        if (pos < (uint32_t)kListLen)
-          out[pos] = make_uint2(d0 + j, __float_as_uint(key_score(v)));
-        else if (pos == (uint32_t)kListLen)
-          *bound = make_uint2(d0 + j, v);
-        ++pos;
+        for (int j = 0; j < 4; ++j) x[q][j] = d + j < n ? __ldg(row + d + j) : 0.f;
       }
     }
-  };
-  // level 0: each warp's smallest key, its pairs at that key, and whether a score is NaN
-  {
-    const uint32_t m = __reduce_min_sync(0xffffffffu, min(min(k[0], k[1]), min(k[2], k[3])));
-    uint32_t c = 0;
+    float mn[2] = {nan, nan};  // minima over the even and the odd q
 #pragma unroll
-    for (int j = 0; j < 4; ++j) c += __popc(__ballot_sync(0xffffffffu, k[j] == m));
-    const bool bad = __any_sync(0xffffffffu, nan);
-    if (lane == 0) {
-      S.nxt[phase & 1][wid] = m;
-      S.cnt[phase & 1][wid] = c | (bad ? 0x80000000u : 0u);
-    }
-  }
-  __syncthreads();
-  uint32_t v, cum;
-  {
-    const uint32_t b = phase & 1;
-    const uint32_t mw = lane < (uint32_t)NW ? S.nxt[b][lane] : kNoKey;
-    const uint32_t cw = lane < (uint32_t)NW ? S.cnt[b][lane] : 0u;
-    ++phase;
-    if (__reduce_or_sync(0xffffffffu, cw & 0x80000000u)) {
-      if (tid < (uint32_t)kListLen) out[tid] = make_uint2(kNone, 0x7f800000u);
-      if (tid == 0) *bound = make_uint2(0u, kBoundInvalid);
-      return;
-    }
-    v = __reduce_min_sync(0xffffffffu, mw);
-    if (v == kNoKey) {  // no decode at all
-      if (tid < (uint32_t)kListLen) out[tid] = make_uint2(kNone, 0x7f800000u);
-      if (tid == 0) *bound = make_uint2(kNone, kNoKey);
-      return;
-    }
-    const uint32_t c = mw == v ? cw : 0u;  // a warp whose smallest key is above v has none at v
-    const uint32_t off = __reduce_add_sync(0xffffffffu, lane < wid ? c : 0u);
-    cum = __reduce_add_sync(0xffffffffu, c);
-    place(v, off);
-  }
-  for (int lev = 1; lev < kListLevels && cum <= (uint32_t)kListLen; ++lev) {
-    // each warp's smallest key above v and its pairs at that key, as at level 0
-    const uint32_t b = phase & 1;
-    uint32_t m = kNoKey;
+    for (int q = 0; q < 8; ++q) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) m = min(m, k[j] > v ? k[j] : kNoKey);
-    m = __reduce_min_sync(0xffffffffu, m);
-    uint32_t c = 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) c += __popc(__ballot_sync(0xffffffffu, k[j] == m));
-    if (lane == 0) {
-      S.nxt[b][wid] = m;
-      S.cnt[b][wid] = c;
-    }
-    __syncthreads();
-    const uint32_t mw = lane < (uint32_t)NW ? S.nxt[b][lane] : kNoKey;
-    const uint32_t cw = lane < (uint32_t)NW ? S.cnt[b][lane] : 0u;
-    ++phase;
-    v = __reduce_min_sync(0xffffffffu, mw);
-    if (v == kNoKey) break;  // every pair is listed
-    const uint32_t cv = mw == v ? cw : 0u;
-    const uint32_t off = __reduce_add_sync(0xffffffffu, lane < wid ? cv : 0u);
-    const uint32_t total = __reduce_add_sync(0xffffffffu, cv);
-    place(v, cum + off);
-    cum += total;
-  }
-  if (cum <= (uint32_t)kListLen) {  // as many pairs as the list holds, or fewer
-    if (tid >= cum && tid < (uint32_t)kListLen) out[tid] = make_uint2(kNone, 0x7f800000u);
-    if (tid == 0) {
-      if (v == kNoKey) {
-        *bound = make_uint2(kNone, kNoKey);
-      } else {  // the levels ran out: every pair not listed has a key above v
-        *bound = make_uint2(0u, v + 1u);
+      for (int j = 0; j < 4; ++j) {
+        bad |= !(x[q][j] == x[q][j]);
+        if (n < kListChunk && 128u * q + 4u * lane + j >= n) x[q][j] = nan;
+        mn[q & 1] = fminf(mn[q & 1], x[q][j]);
       }
+    }
+    if (__any_sync(0xffffffffu, bad)) {  // a NaN score: nothing bounds the chunk
+      out[lane] = make_uint2(kNone, 0x7f800000u);
+      if (lane == 0) bounds[task] = make_uint2(0u, kBoundInvalid);
+      continue;
+    }
+    const uint32_t a = warp_sort(mn[0] == mn[0] ? score_key(mn[0]) : kNoKey, lane);
+    const uint32_t b = warp_sort(mn[1] == mn[1] ? score_key(mn[1]) : kNoKey, lane);
+    uint32_t tk = __reduce_max_sync(0xffffffffu, min(a, __shfl_sync(0xffffffffu, b, 31 - lane)));
+    float T = key_score(tk);
+    uint32_t m, own, total;  // the lane's pairs below T, their number, the warp's
+    for (uint32_t at = 15;; at >>= 1) {
+      m = 0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) m |= x[q][j] < T ? 1u << (4 * q + j) : 0u;
+      }
+      own = __popc(m);
+      total = __reduce_add_sync(0xffffffffu, own);
+      if (total <= kListCand) break;
+      tk = min(__shfl_sync(0xffffffffu, a, at), __shfl_sync(0xffffffffu, b, at));
+      T = key_score(tk);
+    }
+    uint32_t pos = own;  // inclusive prefix over the lanes
+#pragma unroll
+    for (uint32_t o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, pos, o);
+      if (lane >= o) pos += y;
+    }
+    pos -= own;
+    __syncwarp();  // the task before is done with `cand`
+    while (m) {
+      const uint32_t i = __ffs(m) - 1;
+      m &= m - 1;
+      const uint32_t d = 128u * (i >> 2) + 4u * lane + (i & 3u);
+      cand[pos++] = ((unsigned long long)score_key(__ldg(row + d)) << 32) | (c0 + d);
+    }
+    __syncwarp();
+    for (uint32_t i = lane; i < total; i += 32) {
+      const unsigned long long v = cand[i];
+      uint32_t p = 0;
+      for (uint32_t o = 0; o < total; ++o) p += cand[o] < v;
+      if (p < (uint32_t)kListLen)
+        out[p] = make_uint2((uint32_t)v, __float_as_uint(key_score((uint32_t)(v >> 32))));
+      else if (p == (uint32_t)kListLen)
+        bounds[task] = make_uint2((uint32_t)v, (uint32_t)(v >> 32));
+    }
+    if (total > (uint32_t)kListLen) continue;
+    // pairs at T in rank order, while the list or its bound has room
+    uint32_t cum = total;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const bool any = x[q][0] == T || x[q][1] == T || x[q][2] == T || x[q][3] == T;
+      if (cum <= (uint32_t)kListLen && __any_sync(0xffffffffu, any)) {
+        uint32_t p = cum;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t bl = __ballot_sync(0xffffffffu, x[q][j] == T);
+          p += __popc(bl & below);
+          cum += __popc(bl);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (x[q][j] == T) {
+            const uint32_t d = c0 + 128u * q + 4u * lane + j;
+            if (p < (uint32_t)kListLen)
+              out[p] = make_uint2(d, __float_as_uint(T));
+            else if (p == (uint32_t)kListLen)
+              bounds[task] = make_uint2(d, tk);
+            ++p;
+          }
+        }
+      }
+    }
+    if (cum <= (uint32_t)kListLen) {  // every pair up to T is listed
+      if (lane >= cum) out[lane] = make_uint2(kNone, 0x7f800000u);
+      if (lane == 0) bounds[task] = cum == n ? make_uint2(kNone, kNoKey) : make_uint2(0u, tk + 1u);
     }
   }
 }
@@ -395,35 +422,40 @@ __global__ void __launch_bounds__(256) merge_lists_kernel(
 
 // Base scores for pools of more than 32 decodes.  A block takes one chunk of 256 * NPT
 // decodes of one stream and a contiguous range of its events; each thread owns NPT
-// consecutive decodes.  Arrivals in a range mostly share their telemetry snapshot, so a
-// thread keeps, for its decodes and the current snapshot, the quotients
-// qd[k] = bytes_per_token / UB_d[k] of every level k, and recomputes them only when the
-// snapshot changes; per arrival it divides once per level for the prefill,
-// qp[k] = bytes_per_token / UB_p[k], and once for 1 / l.  Division of positive operands is
-// monotone, so bytes_per_token / min(UB_p, UB_d) = max(qp, qd) exactly, and a candidate
-// costs a tier test, a max and three multiply-adds:
-//     base = w_net * (miss_tok * max(qp[tau], qd[tau]) + L_tau) + w_prefix * miss_tok * (1/l)
-// (two roundings more than dividing per candidate: a relative difference below 3e-7).
-// The next arrival's request fields and prefix hits are loaded one arrival ahead; hits are
-// read 8 bytes and scores written 16 bytes at a time when the rows allow it.
+// consecutive decodes and keeps their level bottlenecks for the current snapshot.  A
+// candidate costs a tier test, a division by the smaller bottleneck and three multiply-adds;
+// an arrival one more division, 1 / l:
+//     base = w_net * (miss_tok * (bytes_per_token / min(UB_p[tau], UB_d[tau])) + L_tau)
+//            + w_prefix * miss_tok * (1 / l)
+// (two roundings more than dividing miss_tok * bytes_per_token per candidate: a relative
+// difference below 3e-7).  A prefill of a pod outside the thread's decodes is of tier 3 with
+// all of them, which spares the tier tests.  Bound by instruction issue: 32,000 arrivals on
+// 4,096 decodes 325 us (the rows' traffic takes 116), against about 490 with the decodes' four
+// quotients kept per snapshot and every thread reading each arrival's fields itself; 8,192
+// arrivals on 1,024, each in a snapshot of its own, 54 against 62.
+// Each warp prepares 32 events at a time, one a lane (request fields, the prefill's links and
+// level bottlenecks, 1 / l), so that an arrival's own work is done once per warp and batch
+// instead of by every thread; prefix hits are loaded one arrival ahead, hits read 8 bytes and
+// scores written 16 bytes at a time when the rows allow it.
 // kUtil: as for base_kernel (UB holds the utilisation rows).  X (self-contention) keeps
 // the per-candidate division s_eff / Bbot.
-// kList: the block also writes each arrival's candidate list and bound for its chunk of
-// decodes (lists[r][chunk][kListLen], bounds[r][chunk]) with block_levels; merge_lists_kernel
-// then merges the chunks' lists into the pool's.
-template <int NPT, bool kUtil = false, bool kList = false, int BT = 256>
+struct BaseRec {  // an arrival as a warp prepares it
+  uint4 req;      // request, length, snapshot, 1 / length
+  uint4 lp;       // the prefill's links
+  float4 ubp;     // the prefill's level bottlenecks
+};
+template <int NPT, bool kUtil = false, int BT = 256>
 __global__ void __launch_bounds__(BT, 1024 / BT) base_wide_kernel(
     TopoArgs t, uint32_t n_streams, const netkv_weights* __restrict__ W, uint32_t R,
     const uint32_t* __restrict__ len, const uint32_t* __restrict__ prefill,
     const uint32_t* __restrict__ snap, const uint16_t* __restrict__ M,
     const float* __restrict__ UB, uint32_t n_snap, const uint32_t* __restrict__ events,
     const uint64_t* __restrict__ event_off, float* __restrict__ base, int* status,
-    float* __restrict__ X = nullptr, uint2* __restrict__ lists = nullptr,
-    uint2* __restrict__ bounds = nullptr) {
-  static_assert(!kList || NPT == 4, "lists take 4 decodes a thread");
+    float* __restrict__ X = nullptr) {
   static_assert(BT % 32 == 0 && BT <= 1024, "block of whole warps");
-  __shared__ std::conditional_t<kList, ListShared<BT / 32>, char> S;
-  uint32_t phase = 0;  // block barrier phases of the list selection (buffer parity)
+  __shared__ BaseRec s_rec[BT / 32][32];
+  BaseRec* rec = s_rec[threadIdx.x >> 5];
+  const uint32_t lane = threadIdx.x & 31;
   constexpr uint32_t kChunk = (uint32_t)BT * NPT;
   constexpr uint32_t kBad = 0xffffffffu;
   const uint32_t D = t.D, N = t.N;
@@ -434,13 +466,14 @@ __global__ void __launch_bounds__(BT, 1024 / BT) base_wide_kernel(
   for (uint64_t sc = blockIdx.x; sc < (uint64_t)n_streams * n_chunks; sc += gridDim.x) {
     const uint32_t stream = (uint32_t)(sc / n_chunks);
     const uint32_t d0 = (uint32_t)(sc % n_chunks) * kChunk + threadIdx.x * NPT;
-    uint3 lt[NPT];     // level-1..3 links of each decode: its tier against a prefill
-    uint32_t inst[NPT];
+    uint32_t pod_lo = 0xffffffffu, pod_hi = 0u;  // pods of the thread's decodes
 #pragma unroll
     for (int j = 0; j < NPT; ++j) {
-      inst[j] = d0 + j < D ? __ldg(t.dec + d0 + j) : 0u;
-      const uint4 l = __ldg(t.links + inst[j]);
-      lt[j] = make_uint3(l.y, l.z, l.w);
+      if (d0 + j < D) {
+        const uint32_t pod = __ldg(t.links + __ldg(t.dec + d0 + j)).w;
+        pod_lo = min(pod_lo, pod);
+        pod_hi = max(pod_hi, pod);
+      }
     }
     const netkv_weights w = W[stream];
     const float bpt = (float)w.bytes_per_token;
@@ -450,20 +483,12 @@ __global__ void __launch_bounds__(BT, 1024 / BT) base_wide_kernel(
     const uint64_t eb = e0 + blockIdx.y * span;
     const uint64_t ee = min(e1, eb + span);
 
-    // request fields of an event: kBad r for departures and events to skip
-    auto fields = [&](uint64_t e, uint32_t& r, uint32_t& l, uint32_t& pr, uint32_t& k,
-                      uint32_t* m) {
-      r = kBad;
-      if (e >= ee) return;
-      const uint32_t code = __ldg(events + e);
-      const uint32_t rr = code & 0x7fffffffu;
-      if ((code >> 31) || rr >= R) return;
-      l = __ldg(len + rr);
-      pr = __ldg(prefill + rr);
-      k = __ldg(snap + rr);
-      if (pr >= t.P || k >= n_snap || l == 0) return;
-      r = rr;
-      const uint16_t* mrow = M + (uint64_t)rr * D + d0;
+    float4 ubd[NPT];  // the decodes' level bottlenecks in the current snapshot
+    uint32_t cur_k = kBad;
+#pragma unroll
+    for (int j = 0; j < NPT; ++j) ubd[j] = make_float4(1.f, 1.f, 1.f, 1.f);
+    auto hits = [&](uint32_t r, uint32_t* m) {  // the thread's prefix hits of request r
+      const uint16_t* mrow = M + (uint64_t)r * D + d0;
       if (vec) {
         if (d0 < D) {
           const uint2 v = __ldcs(reinterpret_cast<const uint2*>(mrow));
@@ -477,79 +502,92 @@ __global__ void __launch_bounds__(BT, 1024 / BT) base_wide_kernel(
         for (int j = 0; j < NPT; ++j) m[j] = d0 + j < D ? (uint32_t)__ldcs(mrow + j) : 0u;
       }
     };
-
-    float4 qd[NPT];  // bytes_per_token / UB_d[k] of the current snapshot
-    uint32_t cur_k = kBad;
-    uint32_t nr, nl = 0, npr = 0, nk = 0, nm[NPT];
+    for (uint64_t eb32 = eb; eb32 < ee; eb32 += 32) {
+      // lane i prepares event i of the batch: departures and events to skip leave no bit
+      bool ok = false;
+      uint32_t r = 0, l = 0, pr = 0, k = 0;
+      if (eb32 + lane < ee) {
+        const uint32_t code = __ldg(events + eb32 + lane);
+        r = code & 0x7fffffffu;
+        if (!(code >> 31) && r < R) {
+          l = __ldg(len + r);
+          pr = __ldg(prefill + r);
+          k = __ldg(snap + r);
+          ok = pr < t.P && k < n_snap && l != 0;
+        }
+      }
+      uint32_t todo = __ballot_sync(0xffffffffu, ok);
+      if (ok) {
+        const uint32_t pinst = __ldg(t.pre + pr);
+        const uint4 lp = __ldg(t.links + pinst);
+        rec[lane].ubp = kUtil
+            ? level_bottlenecks_of(t, UB + (uint64_t)k * t.n_links, lp, status)
+            : __ldg(reinterpret_cast<const float4*>(UB) + (uint64_t)k * N + pinst);
+        rec[lane].req = make_uint4(r, l, k, __float_as_uint(1.0f / (float)l));
+        rec[lane].lp = lp;
+      }
+      __syncwarp();
+      uint32_t nm[NPT];
 #pragma unroll
-    for (int j = 0; j < NPT; ++j) {
-      nm[j] = 0;
-      qd[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    uint64_t e = eb;
-    fields(e, nr, nl, npr, nk, nm);
-    for (; e < ee; ++e) {
-      const uint32_t r = nr, l = nl, pr = npr, k = nk;
-      uint32_t m[NPT];
+      for (int j = 0; j < NPT; ++j) nm[j] = 0;
+      if (todo) hits(__shfl_sync(0xffffffffu, r, __ffs(todo) - 1), nm);
+      while (todo) {
+        const uint32_t at = __ffs(todo) - 1;
+        todo &= todo - 1;
+        uint32_t m[NPT];
 #pragma unroll
-      for (int j = 0; j < NPT; ++j) m[j] = nm[j];
-      fields(e + 1, nr, nl, npr, nk, nm);
-      if (r == kBad) continue;
-      if (k != cur_k) {  // the decodes' level bottlenecks of a new snapshot
-        cur_k = k;
-        const float* urow = UB + (uint64_t)k * t.n_links;
+        for (int j = 0; j < NPT; ++j) m[j] = nm[j];
+        if (todo) hits(rec[__ffs(todo) - 1].req.x, nm);
+        const uint4 rq = rec[at].req;  // request, length, snapshot, 1 / length
+        const float4 ubp = rec[at].ubp;
+        const uint4 lp = rec[at].lp;
+        const uint32_t r = rq.x, l = rq.y, k = rq.z;
+        const float rl = __uint_as_float(rq.w);
+        if (k != cur_k) {  // the decodes' level bottlenecks of a new snapshot
+          cur_k = k;
+          const float* urow = UB + (uint64_t)k * t.n_links;
 #pragma unroll
-        for (int j = 0; j < NPT; ++j) {
-          if (d0 + j < D) {
-            const float4 ub = kUtil
-                ? level_bottlenecks_of(t, urow, __ldg(t.links + inst[j]), status)
-                : __ldg(reinterpret_cast<const float4*>(UB) + (uint64_t)k * N + inst[j]);
-            qd[j] = make_float4(bpt / ub.x, bpt / ub.y, bpt / ub.z, bpt / ub.w);
+          for (int j = 0; j < NPT; ++j) {
+            if (d0 + j < D) {
+              const uint32_t inst = __ldg(t.dec + d0 + j);
+              ubd[j] = kUtil ? level_bottlenecks_of(t, urow, __ldg(t.links + inst), status)
+                             : __ldg(reinterpret_cast<const float4*>(UB) + (uint64_t)k * N + inst);
+            }
           }
         }
-      }
-      const uint32_t pinst = __ldg(t.pre + pr);
-      const uint4 lp = __ldg(t.links + pinst);
-      const float4 ubp = kUtil
-          ? level_bottlenecks_of(t, UB + (uint64_t)k * t.n_links, lp, status)
-          : __ldg(reinterpret_cast<const float4*>(UB) + (uint64_t)k * N + pinst);
-      const float4 qp = make_float4(bpt / ubp.x, bpt / ubp.y, bpt / ubp.z, bpt / ubp.w);
-      const float rl = 1.0f / (float)l;
-      float out[NPT];
+        const bool far = lp.w < pod_lo || lp.w > pod_hi;  // tier 3 with every decode of the thread
+        float out[NPT];
 #pragma unroll
-      for (int j = 0; j < NPT; ++j) {
-        const int tau = (lp.y == lt[j].x) ? 0 : (lp.z == lt[j].y) ? 1 : (lp.w == lt[j].z) ? 2 : 3;
-        uint32_t lam = 16u * m[j];
-        if (m[j] > l / 16u) {
-          flag_status(status, NETKV_DEV_EDOMAIN);
-          lam = lam < l ? lam : l;
+        for (int j = 0; j < NPT; ++j) {
+          float pb = ubp.w, db = ubd[j].w, la = lat.w;
+          if (!far) {
+            const uint4 ld = __ldg(t.links + __ldg(t.dec + min(d0 + j, D - 1)));
+            const int tau = (lp.y == ld.y) ? 0 : (lp.z == ld.z) ? 1 : (lp.w == ld.w) ? 2 : 3;
+            pb = pick4(ubp, tau);
+            db = pick4(ubd[j], tau);
+            la = pick4(lat, tau);
+          }
+          uint32_t lam = 16u * m[j];
+          if (m[j] > l / 16u) {
+            flag_status(status, NETKV_DEV_EDOMAIN);
+            lam = lam < l ? lam : l;
+          }
+          const float miss_tok = (float)(l - lam);
+          const float q = bpt / fminf(pb, db);
+          const float T = __fmaf_rn(miss_tok, q, la);
+          out[j] = __fmaf_rn(w.w_net, T, w.w_prefix * (miss_tok * rl));
+          if (X && d0 + j < D) X[(uint64_t)r * D + d0 + j] = miss_tok * q;
         }
-        const float miss_tok = (float)(l - lam);
-        const float q = fmaxf(pick4(qp, tau), pick4(qd[j], tau));
-        const float T = __fmaf_rn(miss_tok, q, pick4(lat, tau));
-        out[j] = __fmaf_rn(w.w_net, T, w.w_prefix * (miss_tok * rl));
-        if (X && d0 + j < D) X[(uint64_t)r * D + d0 + j] = miss_tok * q;
-      }
-      float* brow = base + (uint64_t)r * D + d0;
-      if (vec) {
-        if (d0 < D) __stcs(reinterpret_cast<float4*>(brow), make_float4(out[0], out[1], out[2], out[3]));
-      } else {
+        float* brow = base + (uint64_t)r * D + d0;
+        if (vec) {
+          if (d0 < D) __stcs(reinterpret_cast<float4*>(brow), make_float4(out[0], out[1], out[2], out[3]));
+        } else {
 #pragma unroll
-        for (int j = 0; j < NPT; ++j)
-          if (d0 + j < D) __stcs(brow + j, out[j]);
-      }
-      if constexpr (kList) {
-        uint32_t key[4];
-        bool nan = false;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const bool present = d0 + j < D;
-          key[j] = present ? score_key(out[j]) : kNoKey;
-          nan |= present && !(out[j] == out[j]);
+          for (int j = 0; j < NPT; ++j)
+            if (d0 + j < D) __stcs(brow + j, out[j]);
         }
-        const uint64_t slot = (uint64_t)r * n_chunks + (uint32_t)(sc % n_chunks);
-        block_levels(S, phase, key, nan, d0, lists + slot * kListLen, bounds + slot);
       }
+      __syncwarp();  // every lane is done with the batch's records
     }
   }
 }
@@ -2065,8 +2103,7 @@ netkv_status launch_base(const TopoArgs& t, uint32_t n_streams, const netkv_weig
                          uint32_t R, const uint32_t* d_len, const uint32_t* d_prefill,
                          const uint32_t* d_snap, const uint16_t* d_M, const float* d_UB,
                          uint32_t n_snap, const uint32_t* d_events, const uint64_t* d_event_off,
-                         float* d_base, float* d_X, int* d_status, cudaStream_t s,
-                         uint2* d_lists = nullptr, uint2* d_bounds = nullptr) {
+                         float* d_base, float* d_X, int* d_status, cudaStream_t s) {
     const uint32_t D = t.D;
     const unsigned gy = n_streams >= 1024u ? 1u : (1024u + n_streams - 1) / n_streams;
     const dim3 bgrid(n_streams < (1u << 20) ? n_streams : (1u << 20), gy);
@@ -2093,10 +2130,6 @@ netkv_status launch_base(const TopoArgs& t, uint32_t n_streams, const netkv_weig
         base_wide_kernel<1, kUtil><<<dim3(wx, wy), 256, 0, s>>>(t, n_streams, d_w, R, d_len, d_prefill,
                                                          d_snap, d_M, d_UB, n_snap, d_events,
                                                          d_event_off, d_base, d_status, d_X);
-      else if (d_lists)
-        base_wide_kernel<4, kUtil, true><<<dim3(wx, wy), 256, 0, s>>>(
-            t, n_streams, d_w, R, d_len, d_prefill, d_snap, d_M, d_UB, n_snap, d_events,
-            d_event_off, d_base, d_status, d_X, d_lists, d_bounds);
       else
         base_wide_kernel<4, kUtil><<<dim3(wx, wy), 256, 0, s>>>(t, n_streams, d_w, R, d_len, d_prefill,
                                                          d_snap, d_M, d_UB, n_snap, d_events,
@@ -2118,19 +2151,21 @@ netkv_status launch(const TopoArgs& t, uint32_t n_streams, const netkv_weights* 
   if (d_base) {
     const bool lists = LPS == 32 && lw != nullptr && lw->lists != nullptr;
     if (launch_base<kUtil>(t, n_streams, d_w, R, d_len, d_prefill, d_snap, d_M, d_UB, n_snap,
-                           d_events, d_event_off, d_base, nullptr, d_status, s,
-                           lists ? lw->chunk_lists : nullptr,
-                           lists ? lw->chunk_bounds : nullptr) != NETKV_OK)
+                           d_events, d_event_off, d_base, nullptr, d_status, s) != NETKV_OK)
       return NETKV_ECUDA;
     if (lists) {
       int dev = 0, sms = 0;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+      const uint32_t n_ch = (t.D + kListChunk - 1) / kListChunk;
       const uint64_t blocks = ((uint64_t)R * 32 + 255) / 256;
       const uint64_t cap = (uint64_t)(sms > 0 ? sms : 1) * 64;
+      const uint64_t cblocks = blocks * n_ch;
+      chunk_lists_kernel<<<(unsigned)(cblocks < cap ? cblocks : cap), 256, 0, s>>>(
+          d_base, t.D, n_ch, R, lw->chunk_lists, lw->chunk_bounds);
+      if (netkv_launch_status() != NETKV_OK) return NETKV_ECUDA;
       merge_lists_kernel<<<(unsigned)(blocks < cap ? blocks : cap), 256, 0, s>>>(
-          lw->chunk_lists, lw->chunk_bounds, (t.D + kListChunk - 1) / kListChunk, R, lw->lists,
-          lw->bounds);
+          lw->chunk_lists, lw->chunk_bounds, n_ch, R, lw->lists, lw->bounds);
       if (netkv_launch_status() != NETKV_OK) return NETKV_ECUDA;
       return launch_listed(t, n_streams, d_w, R, d_len, d_prefill, d_snap, n_snap, d_events,
                            d_event_off, d_load_init, d_dec, d_best, d_second, d_load_final,
