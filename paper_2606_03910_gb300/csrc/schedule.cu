@@ -192,6 +192,7 @@ struct ListWs {
 };
 constexpr uint32_t kListCand = 64;       // pairs below a warp's threshold that it ranks
 constexpr uint32_t kBoundInvalid = 0u;
+constexpr uint32_t kInfKey = 0xff800000u;  // score_key(infinity)
 
 // ascending 32-lane bitonic sort, one value a lane
 __device__ __forceinline__ uint32_t warp_sort(uint32_t v, uint32_t lane) {
@@ -267,6 +268,7 @@ __global__ void __launch_bounds__(256, 4) chunk_lists_kernel(
     const uint32_t a = warp_sort(mn[0] == mn[0] ? score_key(mn[0]) : kNoKey, lane);
     const uint32_t b = warp_sort(mn[1] == mn[1] ? score_key(mn[1]) : kNoKey, lane);
     uint32_t tk = __reduce_max_sync(0xffffffffu, min(a, __shfl_sync(0xffffffffu, b, 31 - lane)));
+    tk = min(tk, kInfKey);  // fewer than 32 minima: no score is above infinity
     float T = key_score(tk);
     uint32_t m, own, total;  // the lane's pairs below T, their number, the warp's
     for (uint32_t at = 15;; at >>= 1) {
@@ -279,7 +281,7 @@ __global__ void __launch_bounds__(256, 4) chunk_lists_kernel(
       own = __popc(m);
       total = __reduce_add_sync(0xffffffffu, own);
       if (total <= kListCand) break;
-      tk = min(__shfl_sync(0xffffffffu, a, at), __shfl_sync(0xffffffffu, b, at));
+      tk = min(min(__shfl_sync(0xffffffffu, a, at), __shfl_sync(0xffffffffu, b, at)), kInfKey);
       T = key_score(tk);
     }
     uint32_t pos = own;  // inclusive prefix over the lanes
