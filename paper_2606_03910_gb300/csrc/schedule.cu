@@ -1,6 +1,6 @@
 // The greedy of Algorithm 1 (Sec. V-A) over independent scheduling streams.
 //
-// One CTA per stream walks that stream's events in order.  Each thread owns NPT
+// schedule_kernel: one CTA per stream walks that stream's events in order.  Each thread owns NPT
 // consecutive decode ranks and keeps their load (active tokens) and instance links in
 // registers, so the state of a stream never leaves the SM.  An arrival scores every
 // candidate in parallel (the per-candidate work is the tier test, the bottleneck min of
@@ -12,11 +12,19 @@
 // every warp, so a later departure event is resolved by the same lanes that wrote it.
 // Events are software-pipelined (up to five events ahead) so that no global load sits
 // on the per-event critical path (see the loop below).
-// Without a workspace the network, prefix and load terms are combined on the fly from
-// the level bottlenecks UB and the prefix hits M.  With a workspace, base_kernel first
-// computes the decision-independent network + prefix term of every (arrival, decode)
-// in parallel, and the greedy only adds the load term: the sequential part of a step
-// shrinks to a load, a capacity test, one multiply-add and the argmin per candidate.
+// Without a workspace it combines the network, prefix and load terms on the fly from
+// the level bottlenecks UB and the prefix hits M.  With a workspace, base_kernel or
+// base_wide_kernel first computes the decision-independent network + prefix term of every
+// (arrival, decode) in parallel, and a walk only adds the load term: the sequential part of a
+// step shrinks to a load, a capacity test, one multiply-add and the argmin per candidate.
+// Which walk a call takes:
+//   base scores      at most 16 decodes and more than kSmallMaxStreams streams: windowed;
+//                    up to 1,024 decodes: the walk with producers (launch_model_plain), or
+//                    staged past its rule on decodes and streams; 1,025 .. 4,096: listed, or
+//                    staged where the workspace has no room for the lists
+//   no workspace     schedule_kernel; self-contention and the load model the walk with
+//                    producers first (launch_model_inflight, launch_model_load)
+//   self-contention with a workspace: schedule_kernel on base scores
 #include <math.h>
 
 #include <type_traits>
@@ -624,6 +632,7 @@ __global__ void __launch_bounds__(BLOCK) schedule_kernel(
     int32_t* __restrict__ n_final = nullptr, const float* __restrict__ xf = nullptr) {
   static_assert(LPS == 32 || (BLOCK == 32 && NPT == 1), "packed streams use one warp");
   static_assert(!(kLoad && (kBase || kInfl)), "the load model scores from UB and M alone");
+  static_assert(!kBase || kInfl, "without self-contention, base scores have walks of their own");
   constexpr int NW = BLOCK / 32;
   __shared__ float s_b[2][NW];
   __shared__ uint32_t s_i[2][NW];
@@ -756,7 +765,7 @@ __global__ void __launch_bounds__(BLOCK) schedule_kernel(
       if (lane == 0) dec_pref = *((volatile int32_t*)(dec + r));
       return;
     }
-    if ((kBase && !kInfl) || pr >= t.P || k >= n_snap) return;
+    if (pr >= t.P || k >= n_snap) return;
     const uint32_t pinst = __ldg(t.pre + pr);
     const uint4 lp = __ldg(t.links + pinst);
     if (!kBase) ubp = __ldg(reinterpret_cast<const float4*>(UB) + (uint64_t)k * N + pinst);
@@ -771,7 +780,7 @@ __global__ void __launch_bounds__(BLOCK) schedule_kernel(
   auto xrow = [&](uint32_t code, float* x) {
 #pragma unroll
     for (int j = 0; j < NPT; ++j) x[j] = 0.0f;
-    if (!(kBase && kInfl) || code == kBad || (code >> 31)) return;
+    if (!kBase || code == kBad || (code >> 31)) return;
     const uint32_t r = code & 0x7fffffffu;
     if (r >= R) return;
     const float* x_row = xf + (uint64_t)r * D;
@@ -914,13 +923,11 @@ __global__ void __launch_bounds__(BLOCK) schedule_kernel(
           feasible = load[j] >= (int64_t)(l - lam) * (int64_t)w.bytes_per_token + lm.m_min;
           sc = base_score(w, l, m[j], pick4(ubp, tau[j]), ubd[j], pick4(lat, tau[j]), status) +
                w.w_load * load_term(lm, held[j]);
-        } else if (kBase && kInfl) {  // base + w_net (s_eff / Bbot) n: Eq. 4's 1 + n
+        } else if (kBase) {  // base + w_net (s_eff / Bbot) n: Eq. 4's 1 + n
           const uint32_t n = (cw >> (8 * tau[j])) & 0xffu;
           sc = (__uint_as_float(m[j]) + w.w_net * (xv[j] * (float)n)) +
                w.w_load * (w.theta_s_per_token * (float)load[j]);
           tj = xv[j] * (float)(1u + n) + pick4(lat, tau[j]);
-        } else if (kBase) {
-          sc = __uint_as_float(m[j]) + w.w_load * (w.theta_s_per_token * (float)load[j]);
         } else if (kInfl) {
           const float net_prefix =
               contended_score(w, l, m[j], pick4(ubp, tau[j]), ubd[j], pick4(lat, tau[j]),
@@ -2184,12 +2191,6 @@ netkv_status launch(const TopoArgs& t, uint32_t n_streams, const netkv_weights* 
       // one CTA per stream: the walk is bound by each warp's chain of dependent
       // instructions per event; 16 warps (4 per scheduler) measured best on 4,096 decodes
       const uint32_t D = t.D;
-      if (D <= 32) return launch_staged<1, 32>(t, n_streams, d_w, R, d_len, d_prefill, d_snap,
-                                               n_snap, d_events, d_event_off, d_load_init, d_dec,
-                                               d_best, d_second, d_load_final, d_base, d_status, s);
-      if (D <= 256) return launch_staged<1, 256>(t, n_streams, d_w, R, d_len, d_prefill, d_snap,
-                                                 n_snap, d_events, d_event_off, d_load_init, d_dec,
-                                                 d_best, d_second, d_load_final, d_base, d_status, s);
       if (D <= 1024) return launch_staged<2, 512>(t, n_streams, d_w, R, d_len, d_prefill, d_snap,
                                                   n_snap, d_events, d_event_off, d_load_init, d_dec,
                                                   d_best, d_second, d_load_final, d_base, d_status, s);
@@ -2199,15 +2200,11 @@ netkv_status launch(const TopoArgs& t, uint32_t n_streams, const netkv_weights* 
       return launch_staged<8, 512>(t, n_streams, d_w, R, d_len, d_prefill, d_snap, n_snap,
                                    d_events, d_event_off, d_load_init, d_dec, d_best, d_second,
                                    d_load_final, d_base, d_status, s);
-    } else if (LPS == 8 || LPS == 16) {
+    } else {
       return launch_window<(LPS == 16 ? 16 : 8)>(t, n_streams, d_w, R, d_len, d_prefill, d_snap,
                                                  n_snap, d_events, d_event_off, d_load_init,
                                                  d_dec, d_best, d_second, d_load_final, d_base,
                                                  d_status, s);
-    } else {
-      schedule_kernel<NPT, BLOCK, LPS, true><<<grid, BLOCK, 0, s>>>(
-          t, n_streams, d_w, R, d_base, d_len, d_prefill, d_snap, d_M, d_UB, n_snap, d_events,
-          d_event_off, d_load_init, d_dec, d_best, d_second, d_load_final, d_status);
     }
   } else {
     schedule_kernel<NPT, BLOCK, LPS, false><<<grid, BLOCK, 0, s>>>(
