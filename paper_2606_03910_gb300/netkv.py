@@ -138,10 +138,18 @@ def _ptr(x) -> Optional[int]:
     return int(x.data_ptr())
 
 
+def current_stream() -> Optional[int]:
+    """torch's current CUDA stream, or None before CUDA is initialised."""
+    import torch
+    if not torch.cuda.is_initialized():
+        return None
+    # with the device's index given, torch skips its search for one (3.1 -> 1.6 us a call)
+    return int(torch.cuda.current_stream(torch.cuda.current_device()).cuda_stream)
+
+
 def _stream(s) -> Optional[int]:
     if s is None:
-        import torch
-        return int(torch.cuda.current_stream().cuda_stream) if torch.cuda.is_initialized() else None
+        return current_stream()
     if isinstance(s, int):
         return s
     return int(s.cuda_stream)

@@ -95,6 +95,7 @@ class Scorer:
         self.status = torch.zeros(1, dtype=torch.int32, device=self.device)
         self.share_prefixes = share_prefixes
         self.workspace = None
+        self._match_need = self._sched_need = (None, 0)  # (requests, workspace bytes for them)
         self.precompute_scores = True
         self.sched_workspace = None
         # self-contention counter cap (Eq. 4's n_inflight); 0 = the plain greedy
@@ -143,7 +144,10 @@ class Scorer:
         """Greedy workspace (base scores of every arrival), grown on demand."""
         if not self.precompute_scores:
             return None
-        need = netkv.netkv_schedule_workspace_size(R, self.D)
+        sized = self._sched_need
+        if sized[0] != R:
+            sized = self._sched_need = (R, netkv.netkv_schedule_workspace_size(R, self.D))
+        need = sized[1]
         if self.sched_workspace is None or self.sched_workspace.numel() < need:
             self.sched_workspace = torch.empty(max(need, 256), dtype=torch.uint8,
                                                device=self.device)
@@ -153,7 +157,10 @@ class Scorer:
         """Prefix-match workspace for R requests (grown on demand, reused across steps)."""
         if not self.share_prefixes:
             return None
-        need = netkv.netkv_prefix_match_workspace_size(R)
+        sized = self._match_need
+        if sized[0] != R:
+            sized = self._match_need = (R, netkv.netkv_prefix_match_workspace_size(R))
+        need = sized[1]
         if self.workspace is None or self.workspace.numel() < need:
             self.workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=self.device)
         return self.workspace
@@ -240,6 +247,8 @@ class Scorer:
                 and self.load_model is None and self.lru_cfg is None)
 
     def step(self, x: StepInputs, out: StepOutputs, stream=None) -> StepOutputs:
+        if stream is None:  # asked for once, not by every call
+            stream = netkv.current_stream()
         if self.fused(x):
             self.prefix_match(x, out, stream)
             self.schedule(x, out, stream)
