@@ -85,18 +85,26 @@ __device__ __forceinline__ void seg_argmin_t(float& b, uint32_t& i, float& s, fl
 
 // Base scores of every arrival (pools of at most 32 decodes): the events of a stream are
 // split into contiguous ranges over the segments (LPS lanes each) of grid.y blocks, and
-// lane sl of a segment owns decode sl.  A lane keeps its decode's level bottlenecks for the
-// current snapshot and divides twice per arrival:
+// lane sl of a segment owns decode sl.  The lanes of a segment prepare LPS events at a time,
+// one each (request fields, the prefill's links and level bottlenecks, 1 / l), a batch ahead for
+// the fields; then the segment scores the batch's arrivals, and departures cost nothing.  A
+// lane keeps its decode's level bottlenecks for the current snapshot and divides once per
+// arrival:
 //     base = w_net * (miss_tok * (bytes_per_token / min(UB_p[tau], UB_d[tau])) + L_tau)
 //            + w_prefix * miss_tok * (1 / l)
-// Bound by instruction issue: 1.02 M arrivals on 8 decodes, whose
-// snapshot mostly changes with each arrival, 157 us, against 176 with the decode's four
-// quotients taken per snapshot.
+// Bound by instruction issue: 1.02 M arrivals on 8 decodes, whose snapshot mostly changes with
+// each arrival, 105 us (113 with 6 blocks an SM, whose 40 registers spill), against 157 with
+// every lane reading each event's fields and 176 with four quotients per snapshot besides.
 // Departures and invalid events are skipped (the greedy reports them).  kUtil: `UB` holds
 // the utilisation rows [n_snap][n_links] instead of the level bottlenecks, and the
 // bottlenecks are taken from the links' entries.  X (self-contention) gets s_eff / Bbot.
+struct BaseRec {  // an arrival as one lane of a base pass prepares it
+  uint4 req;      // request, length, snapshot, 1 / length
+  uint4 lp;       // the prefill's links
+  float4 ubp;     // the prefill's level bottlenecks
+};
 template <int LPS, bool kUtil = false>
-__global__ void __launch_bounds__(256, 6) base_kernel(
+__global__ void __launch_bounds__(256, 4) base_kernel(
     TopoArgs t, uint32_t n_streams, const netkv_weights* __restrict__ W, uint32_t R,
     const uint32_t* __restrict__ len, const uint32_t* __restrict__ prefill,
     const uint32_t* __restrict__ snap, const uint16_t* __restrict__ M,
@@ -104,24 +112,15 @@ __global__ void __launch_bounds__(256, 6) base_kernel(
     const uint64_t* __restrict__ event_off, float* __restrict__ base, int* status,
     float* __restrict__ X = nullptr) {
   constexpr uint32_t kSegs = 256 / LPS;
-  constexpr uint32_t kNone = 0xffffffffu;  // no event (a departure code: skipped)
+  constexpr uint32_t kSegMask = LPS == 32 ? 0xffffffffu : (1u << (LPS & 31)) - 1u;
+  __shared__ BaseRec s_rec[256];
   const uint32_t seg = threadIdx.x / LPS, sl = threadIdx.x % LPS;
+  const BaseRec* rec = s_rec + seg * LPS;
   const uint32_t D = t.D, N = t.N;
   const bool mine = sl < D;  // D <= LPS: lane sl owns decode sl
   const float4 lat = make_float4(t.lat[0], t.lat[1], t.lat[2], t.lat[3]);
   const uint32_t inst = mine ? __ldg(t.dec + sl) : 0u;
   const uint4 ld = __ldg(t.links + inst);
-  // an arrival's length, prefill rank, snapshot and this lane's prefix hit
-  auto fields = [&](uint32_t code, uint32_t& l, uint32_t& pr, uint32_t& k, uint32_t& m) {
-    const uint32_t r = code & 0x7fffffffu;
-    l = pr = k = m = 0u;
-    if (!(code >> 31) && r < R) {
-      l = __ldg(len + r);
-      pr = __ldg(prefill + r);
-      k = __ldg(snap + r);
-      if (mine) m = __ldg(M + (uint64_t)r * D + sl);
-    }
-  };
   for (uint32_t stream = blockIdx.x; stream < n_streams; stream += gridDim.x) {
     const float w_net = W[stream].w_net, w_prefix = W[stream].w_prefix;
     const float bpt = (float)W[stream].bytes_per_token;
@@ -133,43 +132,67 @@ __global__ void __launch_bounds__(256, 6) base_kernel(
     const uint64_t eb = e0 + ((uint64_t)blockIdx.y * kSegs + seg) * span;
     const uint64_t ee = min(e1, eb + span);
     uint32_t cur_k = 0xffffffffu;
-    float4 ubd = make_float4(0.f, 0.f, 0.f, 0.f);
-    // software pipeline: the next event's fields and the code after it are loaded while
-    // the current arrival is scored, so an arrival waits for one round trip (its
-    // utilisation entries) instead of three
-    uint32_t c_next = eb + 1 < ee ? __ldg(events + eb + 1) : kNone;
-    uint32_t code_n = eb < ee ? __ldg(events + eb) : kNone;
-    uint32_t l_n, pr_n, k_n, m_n;
-    fields(code_n, l_n, pr_n, k_n, m_n);
-    for (uint64_t e = eb; e < ee; ++e) {
-      const uint32_t code = code_n, l = l_n, pr = pr_n, k = k_n, m = m_n;
-      code_n = c_next;
-      c_next = e + 2 < ee ? __ldg(events + e + 2) : kNone;
-      fields(code_n, l_n, pr_n, k_n, m_n);
-      const uint32_t r = code & 0x7fffffffu;
-      if ((code >> 31) || r >= R) continue;
-      if (pr >= t.P || k >= n_snap || l == 0 || !mine) continue;
-      if (k != cur_k) {  // the decode's level bottlenecks of a new snapshot
-        cur_k = k;
-        ubd = kUtil ? level_bottlenecks_of(t, UB + (uint64_t)k * t.n_links, ld, status)
-                    : __ldg(reinterpret_cast<const float4*>(UB) + (uint64_t)k * N + inst);
+    float4 ubd = make_float4(1.f, 1.f, 1.f, 1.f);
+    // a lane's event of a batch: whether it is an arrival, and its request's fields
+    auto fields = [&](uint64_t off, uint32_t& r, uint32_t& l, uint32_t& pr, uint32_t& k) {
+      r = l = pr = k = 0u;
+      if (off < span && eb + off < ee) {
+        const uint32_t code = __ldg(events + eb + off);
+        r = code & 0x7fffffffu;
+        if (!(code >> 31) && r < R) {
+          l = __ldg(len + r);
+          pr = __ldg(prefill + r);
+          k = __ldg(snap + r);
+        }
       }
-      const uint32_t pinst = __ldg(t.pre + pr);
-      const uint4 lp = __ldg(t.links + pinst);
-      const int tau = tier_of(lp, ld);
-      const float ubp = kUtil ? pick4(level_bottlenecks_of(t, UB + (uint64_t)k * t.n_links, lp,
-                                                           status), tau)
-                              : __ldg(UB + ((uint64_t)k * N + pinst) * 4 + tau);
-      uint32_t lam = 16u * m;
-      if (m > l / 16u) {
-        flag_status(status, NETKV_DEV_EDOMAIN);
-        lam = lam < l ? lam : l;
+    };
+    uint32_t r_n, l_n, pr_n, k_n;  // of the batch after
+    fields(sl, r_n, l_n, pr_n, k_n);
+    for (uint64_t off = 0; off < span; off += LPS) {
+      const uint32_t my_r = r_n, my_l = l_n, my_pr = pr_n, my_k = k_n;
+      fields(off + LPS + sl, r_n, l_n, pr_n, k_n);
+      const bool ok = my_l != 0 && my_pr < t.P && my_k < n_snap;
+      uint32_t todo = __ballot_sync(0xffffffffu, ok);
+      if (LPS < 32) todo = (todo >> ((threadIdx.x & 31) - sl)) & kSegMask;
+      if (ok) {
+        const uint32_t pinst = __ldg(t.pre + my_pr);
+        const uint4 lp = __ldg(t.links + pinst);
+        s_rec[threadIdx.x].ubp = kUtil
+            ? level_bottlenecks_of(t, UB + (uint64_t)my_k * t.n_links, lp, status)
+            : __ldg(reinterpret_cast<const float4*>(UB) + (uint64_t)my_k * N + pinst);
+        s_rec[threadIdx.x].req = make_uint4(my_r, my_l, my_k, __float_as_uint(1.0f / (float)my_l));
+        s_rec[threadIdx.x].lp = lp;
       }
-      const float miss_tok = (float)(l - lam);
-      const float q = bpt / fminf(ubp, pick4(ubd, tau));
-      const float T = __fmaf_rn(miss_tok, q, pick4(lat, tau));
-      base[(uint64_t)r * D + sl] = __fmaf_rn(w_net, T, w_prefix * (miss_tok * (1.0f / (float)l)));
-      if (X) X[(uint64_t)r * D + sl] = miss_tok * q;
+      __syncwarp();
+      if (mine) {
+        uint32_t m_n = 0;
+        if (todo) m_n = __ldg(M + (uint64_t)rec[__ffs(todo) - 1].req.x * D + sl);
+        while (todo) {
+          const uint32_t at = __ffs(todo) - 1, m = m_n;
+          todo &= todo - 1;
+          if (todo) m_n = __ldg(M + (uint64_t)rec[__ffs(todo) - 1].req.x * D + sl);
+          const uint4 rq = rec[at].req;  // request, length, snapshot, 1 / length
+          const float4 ubp = rec[at].ubp;
+          const uint32_t r = rq.x, l = rq.y, k = rq.z;
+          if (k != cur_k) {  // the decode's level bottlenecks of a new snapshot
+            cur_k = k;
+            ubd = kUtil ? level_bottlenecks_of(t, UB + (uint64_t)k * t.n_links, ld, status)
+                        : __ldg(reinterpret_cast<const float4*>(UB) + (uint64_t)k * N + inst);
+          }
+          const int tau = tier_of(rec[at].lp, ld);
+          uint32_t lam = 16u * m;
+          if (m > l / 16u) {
+            flag_status(status, NETKV_DEV_EDOMAIN);
+            lam = lam < l ? lam : l;
+          }
+          const float miss_tok = (float)(l - lam);
+          const float q = bpt / fminf(pick4(ubp, tau), pick4(ubd, tau));
+          const float T = __fmaf_rn(miss_tok, q, pick4(lat, tau));
+          base[(uint64_t)r * D + sl] = __fmaf_rn(w_net, T, w_prefix * (miss_tok * __uint_as_float(rq.w)));
+          if (X) X[(uint64_t)r * D + sl] = miss_tok * q;
+        }
+      }
+      __syncwarp();  // every lane is done with the batch's records
     }
   }
 }
@@ -449,11 +472,6 @@ __global__ void __launch_bounds__(256) merge_lists_kernel(
 // scores written 16 bytes at a time when the rows allow it.
 // kUtil: as for base_kernel (UB holds the utilisation rows).  X (self-contention) keeps
 // the per-candidate division s_eff / Bbot.
-struct BaseRec {  // an arrival as a warp prepares it
-  uint4 req;      // request, length, snapshot, 1 / length
-  uint4 lp;       // the prefill's links
-  float4 ubp;     // the prefill's level bottlenecks
-};
 template <int NPT, bool kUtil = false, int BT = 256>
 __global__ void __launch_bounds__(BT, 1024 / BT) base_wide_kernel(
     TopoArgs t, uint32_t n_streams, const netkv_weights* __restrict__ W, uint32_t R,
