@@ -557,6 +557,15 @@ def match_extent(M, chain_off, rows: int = 1 << 16):
 
 
 # ------------------------------------------------------------------ GPU arm
+def match_launches(sc, R: int, dev) -> int:
+    """Kernels of one prefix match: grouped (4) with a workspace, pools of more than 64 decodes
+    and more (request, decode group) tasks than the resident warps of the card; else 1."""
+    import torch
+    tasks = R * ((sc.D + 63) // 64)
+    resident = 32 * torch.cuda.get_device_properties(dev).multi_processor_count
+    return 4 if sc.share_prefixes and sc.D > 64 and tasks > resident else 1
+
+
 def run_netkv(args):
     import torch
     import synth
@@ -623,16 +632,13 @@ def run_netkv(args):
         raise RuntimeError(f"device status {status} in the timed region")
 
     R, D = x.R, sc.D
-    # level bottlenecks 1; prefix match 4 (group insert, group resolve, leaders, members)
-    # with a workspace or 1 without; greedy 2 (base scores + walk) with a workspace, 3 for
-    # pools of 1,025 .. 4,096 decodes (base scores with chunk lists, list merge, listed
-    # walk), or 1
+    # level bottlenecks 1; prefix match 4 (group scan, group resolve, leaders, members) or 1;
+    # greedy 2 (base scores + walk) with a workspace, 4 for pools of 1,025 .. 4,096 decodes
+    # (base scores, chunk lists, list merge, listed walk), or 1
     plain_greedy = not (sc.inflight_cap > 0 or sc.load_model is not None)
     listed = plain_greedy and sc.precompute_scores and 1025 <= sc.D <= 4096
-    launches_per_step = (0 if fused else 1) + (4 if sc.share_prefixes else 1) + (
-        1 if not plain_greedy else (3 if listed else 2) if sc.precompute_scores else 1)
-    n_input_tensors = sum(1 for f in dataclasses.fields(StepInputs)
-                          if isinstance(getattr(x, f.name), torch.Tensor))
+    launches_per_step = (0 if fused else 1) + match_launches(sc, R, dev) + (
+        1 if not plain_greedy else (4 if listed else 2) if sc.precompute_scores else 1)
     decisions = R * world
     value = decisions / (ms / 1e3)
 
@@ -640,8 +646,7 @@ def run_netkv(args):
     examined, probes = match_extent(out.M, x.chain_off)
     algo = {
         # floor: each chain block up to the request's last first miss read once (8 B) and
-        # each M entry written once (2 B); index reads are left out (prefix sharing skips
-        # them over shared prefixes and L2 serves most of the rest)
+        # each M entry written once (2 B); index reads are left out (L2 serves most of them)
         "prefix_match": 8 * examined + 2 * R * D,
         # per snapshot: the utilisation row (L floats), 16-byte UB of every instance
         "oracle_build": 0 if fused else x.n_snap * (16 + 16 * sc.N) if args.tiers else
@@ -649,10 +654,10 @@ def run_netkv(args):
         # per arrival: event, len/prefill/snap and the dec/best/second stores; per
         # departure: event, len, dec; the loads in and out.  With a workspace the base pass
         # reads M (2 B) and writes the base score (4 B) of every candidate, and the walk
-        # reads the row (staged walk) or the candidate list and bound (listed walk: the
-        # chunk lists written and merged, 264 B each); without one the walk reads M.
+        # reads the row, or the list pass does (4 B) and the walk the candidate list and bound
+        # (the chunk lists written and merged, 264 B each); without one the walk reads M.
         "schedule": R * (4 + 12 + 12) + R * 12 + 2 * 8 * D * x.n_streams + (
-            (R * 6 * D + (R * 264 * (2 * ((D + 1023) // 1024) + 2) if listed else R * 4 * D))
+            (R * 10 * D + (R * 264 * (2 * ((D + 1023) // 1024) + 2) if listed else 0))
             if sc.precompute_scores else R * 2 * D),
     }
     dom = max(per_kernel, key=per_kernel.get)
@@ -675,8 +680,8 @@ def run_netkv(args):
                              "oracle_build": "per snapshot: the utilisation row + 16 B per instance",
                              "schedule": "per arrival: event, request fields, dec/best/second, "
                                          "M read and base score written per candidate (2 + 4 B), "
-                                         "then the row (staged walk) or the 264 B candidate list "
-                                         "(listed walk); per departure: event, len, dec"}[dom],
+                                         "then the row (4 B) and, for listed pools, the 264 B "
+                                         "candidate lists; per departure: event, len, dec"}[dom],
                 "examined_blocks_per_launch": examined,
                 "survey_probe_bytes_per_launch": 16 * probes + 2 * R * D,
                 "survey_probes_per_launch": probes,
@@ -716,7 +721,7 @@ def run_netkv(args):
                "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                "host_read_in_place_bytes": zc_bytes,
                "host_read_in_place": list(zc),
-               "gpu_launches_per_step": launches_per_step + n_input_tensors - len(zc) + 4}
+               "gpu_launches_per_step": launches_per_step + 2}
 
     # ---- CPU oracle baseline, rank 0 at N=1 only
     cpu = None
@@ -807,10 +812,10 @@ def run_single(args):
         torch.cuda.synchronize()
         return g
 
-    # the stream's step: grouping, leaders and members (with the workspace), base scores
-    # (level bottlenecks from the utilisation rows) and the walk: 6 launches
+    # the stream's step: prefix match, base scores (level bottlenecks from the utilisation
+    # rows) and the walk: 3 launches
     g_step = capture(lambda st: sc.step(x, out, st), True, True)
-    step_launches = 6 if sc.fused(x) else 7
+    step_launches = (2 if sc.fused(x) else 3) + match_launches(sc, R, dev)
     # one decision: one request against the 8 decodes, no workspaces: 3 launches
     r_one = int(w.req_off[0]) + R // 2
     x1 = one_decision_inputs(x, r_one)

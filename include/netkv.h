@@ -477,6 +477,15 @@ netkv_status netkv_schedule_streams_evolving(
  */
 netkv_status netkv_copy_async(void* dst, const void* src, size_t bytes, netkv_stream_t stream);
 
+/* Several such copies in one launch per 32 of them.  `copies` is host memory, read before the
+ * call returns.  Any bad copy (NULL, misaligned, 1 TiB or more) refuses the whole call. */
+typedef struct netkv_copy {
+  void* dst;
+  const void* src;
+  uint64_t bytes;
+} netkv_copy;
+netkv_status netkv_copy_group_async(const netkv_copy* copies, uint32_t n, netkv_stream_t stream);
+
 /* Library version, for the bindings' load check. */
 uint32_t netkv_version(void);
 

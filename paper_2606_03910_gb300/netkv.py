@@ -41,7 +41,7 @@ EXPORTS = ("netkv_topology_create", "netkv_topology_destroy", "netkv_topology_qu
            "netkv_schedule_streams_load",
            "netkv_lru_state_bytes", "netkv_lru_init", "netkv_lru_export",
            "netkv_schedule_streams_evolving",
-           "netkv_copy_async", "netkv_version")
+           "netkv_copy_async", "netkv_copy_group_async", "netkv_version")
 
 
 class NetKVError(RuntimeError):
@@ -123,6 +123,7 @@ _lib.netkv_schedule_streams_evolving.argtypes = [_P, _U32, _P, _U32, _P, _P, _P,
                                                  _P, _P, _P, C.c_size_t, C.POINTER(LruConfig), _P,
                                                  _P, _P, _P, _P, _P, _P, _P]
 _lib.netkv_copy_async.argtypes = [_P, _P, C.c_size_t, _P]
+_lib.netkv_copy_group_async.argtypes = [_P, _U32, _P]
 for _f in EXPORTS:
     if _f not in ("netkv_version", "netkv_prefix_match_workspace_size", "netkv_cache_index_bytes",
                   "netkv_schedule_workspace_size", "netkv_schedule_inflight_workspace_size",
@@ -365,6 +366,13 @@ def netkv_copy_async(dst, src, nbytes: int, stream=None) -> None:
     """Kernel copy between device and/or pinned host buffers (torch tensors or addresses)."""
     _check("netkv_copy_async", _lib.netkv_copy_async(_ptr(dst), _ptr(src), int(nbytes),
                                                      _stream(stream)))
+
+
+def netkv_copy_group_async(copies, stream=None) -> None:
+    """Kernel copies (dst, src, bytes), each as for netkv_copy_async, in one launch per 32."""
+    flat = [v for dst, src, nbytes in copies for v in (_ptr(dst) or 0, _ptr(src) or 0, int(nbytes))]
+    _check("netkv_copy_group_async", _lib.netkv_copy_group_async(
+        (_U64 * len(flat))(*flat), len(flat) // 3, _stream(stream)))
 
 
 def make_weights(w: np.ndarray, theta: float, cap_tokens: int, bytes_per_token: int) -> np.ndarray:

@@ -15,7 +15,7 @@ With evolving caches (``lru_setup``), steps 2 and 3 are one call,
 LRU-managed caches that every dispatch updates (``lru_reset`` sets them from key lists).
 
 ``step_host`` is the same step from host buffers: it copies the step's inputs
-host->device (``netkv_copy_async``: SM-driven reads of pinned host memory), runs
+host->device (``netkv_copy_group_async``: SM-driven reads of pinned host memory), runs
 the step and copies the results back, all on the stream.
 Python here only marshals arguments; PyTorch provides device memory.
 """
@@ -270,17 +270,15 @@ class Scorer:
         pinned host memory (unified addressing over NVLink-C2C), so only the parts a step
         actually touches cross the link (for the chains: blocks up to each first miss)."""
         s = torch.cuda.current_stream() if stream is None else stream
-        for f in dataclasses.fields(StepInputs):
-            h = getattr(xh, f.name)
-            if isinstance(h, torch.Tensor) and f.name not in zero_copy:
-                d = getattr(xd, f.name)
-                netkv.netkv_copy_async(d, h, h.numel() * h.element_size(), s)
+        inputs = [(getattr(xd, f.name), getattr(xh, f.name)) for f in dataclasses.fields(StepInputs)
+                  if f.name not in zero_copy]
+        netkv.netkv_copy_group_async([(d, h, h.numel() * h.element_size()) for d, h in inputs
+                                      if isinstance(h, torch.Tensor)], s)
         if zero_copy:
             xd = dataclasses.replace(xd, **{name: getattr(xh, name) for name in zero_copy})
         self.step(xd, out, s)
-        for k in ("dec", "best", "second", "load_final"):
-            d = getattr(out, k)
-            netkv.netkv_copy_async(res_h[k], d, d.numel() * d.element_size(), s)
+        results = [(res_h[k], getattr(out, k)) for k in ("dec", "best", "second", "load_final")]
+        netkv.netkv_copy_group_async([(h, d, d.numel() * d.element_size()) for h, d in results], s)
         return out
 
 
