@@ -766,12 +766,17 @@ __device__ __forceinline__ uint32_t follow_run(const unsigned long long* __restr
 }
 
 // What a chain's walk through its set's first index found: the run position of its first
-// block (kNoRun: not there) and how many blocks follow the run from it.
+// block (kNoRun: not there), how many blocks follow the run from it, and how many runs were
+// followed.  The later runs' positions and lengths lie in the request's row of M, 3 entries
+// each, until the match writes the row (more than 64 entries, as pools of one decode group are
+// matched directly).
 struct FirstRun {
-  uint32_t pos, len;
+  uint32_t pos;
+  uint16_t len, runs;
 };
 
-constexpr int kMaxRuns = 8;  // runs followed per chain: more only refine the choice of leader
+constexpr uint32_t kMaxRuns = 8;  // runs followed per chain: more only refine the grouping
+static_assert(3 * (kMaxRuns - 1) <= kGroup, "the later runs fit the request's row");
 
 // A warp takes `per` <= 32 consecutive requests, as match_kernel does.
 __global__ void __launch_bounds__(kDirectBlock, 16) group_scan_kernel(
@@ -779,7 +784,7 @@ __global__ void __launch_bounds__(kDirectBlock, 16) group_scan_kernel(
     const uint64_t* __restrict__ chains, const uint64_t* __restrict__ chain_off, uint32_t R,
     const uint32_t* __restrict__ set_off, uint32_t per, GroupSlot* __restrict__ tab,
     uint32_t log2_slots, int32_t* __restrict__ set_of, uint64_t* __restrict__ gkey,
-    FirstRun* __restrict__ first_run) {
+    FirstRun* __restrict__ first_run, uint16_t* __restrict__ M, uint32_t D) {
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t cap = 1u << log2_cap;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -788,7 +793,7 @@ __global__ void __launch_bounds__(kDirectBlock, 16) group_scan_kernel(
     const uint32_t count = (uint32_t)min((uint64_t)per, R - t0);
     const uint32_t my_r = (uint32_t)t0 + lane;
     uint64_t my_c0 = 0, my_key = 0;
-    uint32_t my_n = 0, my_pos = kNoRun, my_len = 0, my_cached = 0;
+    uint32_t my_n = 0, my_pos = kNoRun, my_len = 0, my_cached = 0, my_runs = 0;
     int32_t my_set = -1;
     if (lane < count) {
       my_c0 = __ldg(chain_off + my_r);
@@ -814,24 +819,28 @@ __global__ void __launch_bounds__(kDirectBlock, 16) group_scan_kernel(
       const IndexView ix = index_view(
           index, (uint64_t)__shfl_sync(0xffffffffu, my_set, i) * n_dgroups, log2_cap, 8u);
       const uint32_t len = follow_run(ix.keys, cap, chain, 0, n, pos, lane);
-      uint32_t p = len;
-      for (int runs = 1; runs < kMaxRuns && p < n; ++runs) {
+      uint16_t* path = M + (uint64_t)(t0 + i) * D;
+      uint32_t p = len, runs = 1;
+      for (; runs < kMaxRuns && p < n; ++runs) {
         const uint64_t key = __ldg(chain + p);
         if (key == 0ull) break;
         const unsigned long long at = lookup_warp(ix.hash, key, log2_cap, lane, nullptr);
         if (at >= cap) break;
         const uint32_t more = follow_run(ix.keys, cap, chain, p, n, (uint32_t)at, lane);
         if (more == 0) break;
+        if (lane < 3)
+          path[3 * (runs - 1) + lane] = (uint16_t)(lane == 0 ? at : lane == 1 ? at >> 16 : more);
         p += more;
       }
       if (lane == i) {
         my_len = len;
         my_cached = p;
+        my_runs = runs;
       }
     }
     if (lane < count) {
       gkey[my_r] = my_key;  // 0: not grouped
-      first_run[my_r] = FirstRun{my_pos, my_len};
+      first_run[my_r] = FirstRun{my_pos, (uint16_t)my_len, (uint16_t)my_runs};
       if (my_key != 0ull) {
         const uint64_t mask = (1ull << log2_slots) - 1;
         const unsigned long long code = ((unsigned long long)my_cached << 48) |
@@ -859,6 +868,7 @@ __global__ void group_resolve_kernel(const GroupSlot* __restrict__ tab, uint32_t
                                      const int32_t* __restrict__ set_of,
                                      uint32_t* __restrict__ leaders, uint64_t* __restrict__ gkey,
                                      const FirstRun* __restrict__ first_run,
+                                     const uint16_t* __restrict__ M, uint32_t D,
                                      MatchCounters* counters) {
   const uint64_t mask = (1ull << log2_slots) - 1;
   for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < R; r += gridDim.x * blockDim.x) {
@@ -885,11 +895,30 @@ __global__ void group_resolve_kernel(const GroupSlot* __restrict__ tab, uint32_t
       if (cached >= kLongLeader) leaders[atomicAdd(&counters->n_long, 1ull)] = r;
       else leaders[R - 1 - atomicAdd(&counters->n_short, 1ull)] = r;
     } else {
-      // the chain that left their common run first parts from the other there
+      // Chains that agree follow the same runs.  So the chain that left their common run
+      // first parts from the other there, and so do chains whose next runs differ, or of
+      // which only one goes on: a block's run depends on its hash alone.
       const FirstRun a = first_run[r], b = first_run[lead];
       uint64_t lcp = 0;
-      if (a.pos == b.pos && a.pos != kNoRun)
-        lcp = min(a.len, b.len) | (a.len != b.len ? kLcpExact : 0ull);
+      if (a.pos == b.pos && a.pos != kNoRun) {
+        uint32_t x = a.len, y = b.len;
+        lcp = min(x, y);
+        bool parted = x != y;
+        for (uint32_t i = 1; !parted; ++i) {
+          if (i == a.runs && i == b.runs) break;  // they agree so far
+          parted = i == a.runs || i == b.runs;
+          if (parted) break;
+          const uint16_t* pa = M + (uint64_t)r * D + 3 * (i - 1);
+          const uint16_t* pb = M + (uint64_t)lead * D + 3 * (i - 1);
+          parted = pa[0] != pb[0] || pa[1] != pb[1];
+          if (parted) break;
+          x = pa[2];
+          y = pb[2];
+          lcp += min(x, y);
+          parted = x != y;
+        }
+        if (parted) lcp |= kLcpExact;
+      }
       gkey[r] = lcp;
     }
   }
@@ -1358,9 +1387,9 @@ extern "C" netkv_status netkv_prefix_match(const void* d_index, uint32_t D,
   const unsigned sgrid = (unsigned)(sblocks < (1u << 24) ? sblocks : (1u << 24));
   group_scan_kernel<<<sgrid, kDirectBlock, 0, s>>>(
       index, (D + kGroup - 1) / kGroup, log2_capacity, n_sets, d_chains, d_chain_off, R, d_set_off,
-      per, tab, lg, set_of, gkey, first_run);
+      per, tab, lg, set_of, gkey, first_run, d_M, D);
   group_resolve_kernel<<<rgrid, 256, 0, s>>>(tab, lg, R, leader_of, set_of, leaders, gkey,
-                                             first_run, counters);
+                                             first_run, d_M, D, counters);
   match_leaders_kernel<<<leader_grid(), kMatchBlock, 0, s>>>(
       index, D, log2_capacity, n_sets, d_chains, d_chain_off, R, d_set_off, set_of, leaders,
       counters, d_M, d_status);

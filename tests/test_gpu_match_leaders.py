@@ -56,3 +56,32 @@ def test_shared_roots(D, copies, first_group):
     M, want, status, _ = _prefix_case(chains, [caches], D, [len(chains)])
     assert status == 0
     np.testing.assert_array_equal(M, want)
+
+
+@pytest.mark.parametrize("D,steps", [(65, 3), (70, 8), (129, 13)])
+def test_paths_over_several_runs(D, steps):
+    """The first group's decodes cache one root ever deeper, with keys of their own between, so
+    its chain is followed over `steps` runs (8 are recorded); chains leave the root before, at
+    and after each run's end, for a tail, another cached chain or a block of hash 0, or end
+    there.  D odd: request rows of M off the 4-byte grid."""
+    rng = np.random.default_rng(D)
+    root, other = _hashes(rng, 40 * steps + 40), _hashes(rng, 400)
+    ends = [40 * (i + 1) for i in range(steps)]
+    chains = []
+    for k in sorted({e + x for e in ends for x in (-20, -1, 0, 1)} | {len(root)}):
+        for tail in (np.zeros(0, np.uint64), _hashes(rng, 3), other[:50], other[50:60],
+                     np.concatenate([other[:20], root[k:k + 30]])):
+            chains.append(np.concatenate([root[:k], tail]))
+    base = len(chains)
+    while len(chains) * -(-D // 64) <= 4864:
+        chains += [np.concatenate([c, _hashes(rng, 2)]) for c in chains[:base]]
+    caches = []
+    for d in range(D):
+        if d < 64:  # deeper and deeper over the first decodes, then any depth
+            depth = ends[d] if d < steps else int(rng.integers(0, ends[-1] + 1))
+        else:
+            depth = int(rng.integers(0, len(root) + 1))
+        caches.append(np.concatenate([root[:depth], _hashes(rng, 5), other[:d % 80]]))
+    M, want, status, _ = _prefix_case(chains, [caches], D, [len(chains)])
+    assert status == 0
+    np.testing.assert_array_equal(M, want)
