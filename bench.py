@@ -228,11 +228,10 @@ KERNEL_CODE = {
 #   prefix_match: bytes per request, from the 64-replica case of the bench workload
 #   oracle_build: bytes per snapshot of the oracle-build sweep
 MEASURED_TRAFFIC = {
-    # 64 replicas (64,000 requests): group_insert 8.96 MB, group_resolve 2.20 MB,
-    # match_leaders 92.51 MB, match_members_kernel 239.84 MB (read + write)
-    "prefix_match": {"code_sha256_16": "770ae3653abd8151", "bytes_per_unit": 343_515_136 / 64_000,
+    # 64 replicas (64,000 requests): match_kernel 303.21 MB read, 3.16 MB written
+    "prefix_match": {"code_sha256_16": "c43f7fc61fbdb936", "bytes_per_unit": 306_365_440 / 64_000,
                      "unit": "request", "captured": "64-replica case, one launch per kernel"},
-    "oracle_build": {"code_sha256_16": "ed437e71560780e2", "bytes_per_unit": 67_155_930,
+    "oracle_build": {"code_sha256_16": "05d89616909d4baa", "bytes_per_unit": 67_161_251,
                      "unit": "snapshot", "captured": "1,000-snapshot sweep, one launch"},
 }
 

@@ -6,9 +6,9 @@
 // A group of copies is one launch: the buffers are cut into chunks of 512 * U units of 16
 // bytes, numbered one buffer after another, and the blocks stride over the chunks.  A small
 // copy is bound by its launch and one round trip over the link (6.8 us each), which a group
-// pays once: the ten inputs and four results of a step of 32 replicas took 95 us,
-// now 72.  Large groups are bound by the link; U = 4 loads a thread in flight where every
-// resident block still gets several chunks, else 1, so that small groups use more SMs.
+// pays once: the ten inputs and four results of a step of 32 replicas took 95 us, now 72.
+// Large groups are bound by the link; U = 4 loads a thread in flight where every resident
+// block still gets several chunks, else 1, so that small groups use more SMs.
 #include "netkv_internal.cuh"
 
 namespace {

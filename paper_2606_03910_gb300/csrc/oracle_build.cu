@@ -19,7 +19,11 @@ namespace {
 
 constexpr int kBlock = 256;
 constexpr int kPerThread = 4;
-constexpr int kPTile = 256;  // prefill ranks staged at a time, one a thread
+constexpr uint32_t kPTile = 256;  // prefill ranks staged at a time, one a thread
+// Pairs of a call from which the deep form runs: four rows a thread in flight at 3 blocks an SM
+// instead of two at 4.  Snapshots of 2,048 x 8,192 (us, two rows / four): 1 20.8 / 24.5, 8
+// 96.2 / 97.8, 16 173 / 168, 32 324 / 310, 1,000 9,232 / 9,167.
+constexpr uint64_t kDeepPairs = 1ull << 28;
 
 __device__ __forceinline__ bool util_ok(float u) { return u >= 0.0f && u < 1.0f; }
 
@@ -80,8 +84,8 @@ __global__ void __launch_bounds__(kBlock) level_bottleneck_kernel(
 // pairs that share a pod (issue slots: about 20 instructions per four pairs, not 80).
 // util_down: the decode side's rows (the downward utilisations of directed links; the
 // same pointer as util for undirected links).
-template <bool kVec, bool kTier>
-__global__ void __launch_bounds__(kBlock, 4) oracle_build_kernel(
+template <bool kVec, bool kTier, bool kDeep>
+__global__ void __launch_bounds__(kBlock, kDeep ? 3 : 4) oracle_build_kernel(
     TopoArgs t, const float* __restrict__ util, const float* __restrict__ util_down,
     uint32_t n_snap, float kv, float* __restrict__ C, float4* __restrict__ UB, uint32_t p_span,
     uint32_t log2_tx, int* status) {
@@ -122,7 +126,7 @@ __global__ void __launch_bounds__(kBlock, 4) oracle_build_kernel(
     }
     float* crow = C + (uint64_t)s * t.P * t.D;
     for (uint32_t p0 = p_beg; p0 < p_end; p0 += kPTile) {
-      const uint32_t np = min((uint32_t)kPTile, p_end - p0);
+      const uint32_t np = min(kPTile, p_end - p0);
       __syncthreads();
       if (threadIdx.x < np) {
         const uint32_t inst = __ldg(t.pre + p0 + threadIdx.x);
@@ -137,7 +141,7 @@ __global__ void __launch_bounds__(kBlock, 4) oracle_build_kernel(
       }
       __syncthreads();
       if (d0 >= t.D) continue;
-#pragma unroll 2
+#pragma unroll kDeep ? 4 : 2
       for (uint32_t k = row; k < np; k += ty) {
         const float2 far = s_far[k];
         const uint32_t pod = __float_as_uint(far.y);
@@ -222,16 +226,20 @@ static netkv_status oracle_build(netkv_topology_t topo, const float* d_util, con
   const bool vec = (t.D % 4 == 0) && aligned_to(d_C, 16);
   const float* down = mode == kDirected ? d_util_down : d_util;
   float4* ub = reinterpret_cast<float4*>(d_UB);
+  const bool deep = (uint64_t)n_snap * t.P * t.D >= kDeepPairs;
 #define NETKV_BUILD(VEC, TIER)                                                             \
-  oracle_build_kernel<VEC, TIER><<<grid, kBlock, 0, s>>>(t, d_util, down, n_snap,          \
-                                                         (float)kv_bytes, d_C, ub, p_span, \
-                                                         log2_tx, d_status)
+  if (deep)                                                                                \
+    oracle_build_kernel<VEC, TIER, true><<<grid, kBlock, 0, s>>>(                          \
+        t, d_util, down, n_snap, (float)kv_bytes, d_C, ub, p_span, log2_tx, d_status);     \
+  else                                                                                     \
+    oracle_build_kernel<VEC, TIER, false><<<grid, kBlock, 0, s>>>(                         \
+        t, d_util, down, n_snap, (float)kv_bytes, d_C, ub, p_span, log2_tx, d_status)
   if (mode == kTiers) {
-    if (vec) NETKV_BUILD(true, true);
-    else NETKV_BUILD(false, true);
+    if (vec) { NETKV_BUILD(true, true); }
+    else { NETKV_BUILD(false, true); }
   } else {
-    if (vec) NETKV_BUILD(true, false);
-    else NETKV_BUILD(false, false);
+    if (vec) { NETKV_BUILD(true, false); }
+    else { NETKV_BUILD(false, false); }
   }
 #undef NETKV_BUILD
   return netkv_launch_status();

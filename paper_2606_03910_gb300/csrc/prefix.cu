@@ -35,8 +35,8 @@
 //     each group's leader is the chain with the most such blocks (then the longest, then the
 //     lowest index): the one whose cached prefix the others' are prefixes of.
 //   group_resolve_kernel: leaders go to a compact list; a member r with leader L gets
-//     lcp = |common prefix of h_r and h_L| from how far both chains followed the same run,
-//     without reading them again (exactly, unless both left the run at the same block).
+//     lcp = |common prefix of h_r and h_L| from the runs that both chains followed, without
+//     reading them again (exactly, unless both left the same last run at the same block).
 //   match_leaders_kernel: leaders (and ungrouped requests) run the full match, one task
 //     per (leader, decode group) taken in order from a counter.
 //   match_members_wide_kernel: one warp per member.  For a decode with M_L[d] < lcp the
@@ -1067,7 +1067,10 @@ __global__ void __launch_bounds__(kDirectBlock, 16) match_kernel(
 // rows are 16-byte aligned), and block lcp is then probed in the groups where some leader
 // hit reaches lcp, up to 32 groups at once with one lane per group; a group whose probe
 // finds the block is walked again by the whole warp.
-// Bound by the rows it writes: 32,000 requests on 4,096 decodes 164 us.  With leaders chosen
+// Bound by the rows it writes: 32,000 requests on 4,096 decodes 143 us, 8,192 on 1,024 15 us.
+// With only the first run's length known, whose end most members share with their leader, both
+// chains were read on from there: 164 and 47 us, and 778 against 36 with the chains in host
+// memory.  With leaders chosen
 // by chain length, the members whose cached prefix ran past their leader's walked all 64
 // groups of the pool again: 3.9 ms (6.6 ms at 32 blocks a step).
 __global__ void __launch_bounds__(kMatchBlock, 4) match_members_wide_kernel(

@@ -62,8 +62,8 @@ def test_shared_roots(D, copies, first_group):
 def test_paths_over_several_runs(D, steps):
     """The first group's decodes cache one root ever deeper, with keys of their own between, so
     its chain is followed over `steps` runs (8 are recorded); chains leave the root before, at
-    and after each run's end, for a tail, another cached chain or a block of hash 0, or end
-    there.  D odd: request rows of M off the 4-byte grid."""
+    and after each run's end, for a tail or another cached chain, or end there.  D odd: request
+    rows of M off the 4-byte grid."""
     rng = np.random.default_rng(D)
     root, other = _hashes(rng, 40 * steps + 40), _hashes(rng, 400)
     ends = [40 * (i + 1) for i in range(steps)]

@@ -86,3 +86,31 @@ def test_cost_matrix_tiles(fanout, n_decode, snaps, shift, mode):
     qd = np.take_along_axis(q[:, d], np.broadcast_to(tau.T, (snaps,) + tau.T.shape), 2)
     want = np.maximum(qp, qd.transpose(0, 2, 1)) + np.array(LAT, np.float32)[tau]
     np.testing.assert_array_equal(C.cpu().numpy().reshape(want.shape), want)
+
+
+@pytest.mark.parametrize("mode", ["links", "tiers"])
+@pytest.mark.parametrize("fanout,n_decode", [((1, 7, 11, 101), 6001),   # ragged, scalar stores
+                                             ((1, 8, 8, 128), 6144)])   # 16-byte rows
+def test_many_pairs_equal_the_snapshots_one_by_one(fanout, n_decode, mode):
+    """Calls of 2^28 pairs and more keep more rows in flight: the same matrices as calls of one
+    snapshot each."""
+    from paper_2606_03910_gb300 import netkv
+    n = int(np.prod(fanout))
+    role = np.zeros(n, np.uint8)
+    role[np.random.default_rng(n).permutation(n)[:n_decode]] = 1
+    L = oracle.used_links(fanout)
+    topo = netkv.netkv_topology_create(fanout, role, BW, LAT, L)
+    P, D = n - n_decode, n_decode
+    snaps = -(-(1 << 28) // (P * D))
+    build = netkv.netkv_oracle_build if mode == "links" else netkv.netkv_oracle_build_tiers
+    g = torch.Generator(device="cuda").manual_seed(5)
+    util = torch.rand((snaps, L if mode == "links" else 4), generator=g, device="cuda") * 0.9
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    C = torch.empty((snaps, P, D), device="cuda")
+    UB = torch.empty((snaps, n, 4), device="cuda")
+    build(topo, util, snaps, 2.5e9, C, UB, st)
+    one, ub = torch.empty((P, D), device="cuda"), torch.empty((n, 4), device="cuda")
+    for s in range(snaps):
+        build(topo, util[s].contiguous(), 1, 2.5e9, one, ub, st)
+        assert torch.equal(C[s], one) and torch.equal(UB[s], ub)
+    assert int(st.item()) == 0
