@@ -271,7 +271,7 @@ typedef struct {
  *   d_UB         [n_snap][N][4] level bottlenecks from netkv_oracle_build
  *   d_events     uint32 codes: bit 31 set = departure, bits 0..30 = request index r;
  *                stream j's events are d_events[d_event_off[j] .. d_event_off[j+1])
- *   d_event_off  [n_streams+1] uint64
+ *   d_event_off  [n_streams+1] uint64; a stream whose offsets decrease has no events
  *   d_load_init  [n_streams][D] int64 initial loads, or NULL for zero (resume support)
  *   d_dec        [R] int32 output: decision of each arrival handled (others untouched)
  *   d_best       [R] fp32 output: minimum score (+inf when rejected)

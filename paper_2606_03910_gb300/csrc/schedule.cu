@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(256, 4) base_kernel(
     // arrivals share their snapshot
     const uint64_t e0 = event_off[stream], e1 = event_off[stream + 1];
     const uint64_t n_seg = (uint64_t)gridDim.y * kSegs;
-    const uint64_t span = (e1 - e0 + n_seg - 1) / n_seg;
+    const uint64_t span = e1 > e0 ? (e1 - e0 + n_seg - 1) / n_seg : 0;
     const uint64_t eb = e0 + ((uint64_t)blockIdx.y * kSegs + seg) * span;
     const uint64_t ee = min(e1, eb + span);
     uint32_t cur_k = 0xffffffffu;

@@ -50,15 +50,18 @@ def _arrays(c, twice):
     return a
 
 
-def _call(c, a, form, pad, load_init=None, model=None, cap=4, bpt=synth.BYTES_PER_TOKEN_SHARD):
+def _call(c, a, form, pad, load_init=None, model=None, cap=4, bpt=synth.BYTES_PER_TOKEN_SHARD,
+          back=False):
     """The greedy `form` with `pad` streams without events after the real ones; the results
-    of the real streams."""
+    of the real streams.  back: the last stream's offsets run back to 0."""
     netkv = nk()
     from paper_2606_03910_gb300.pipeline import weights_tensor
     sc, x, out = c["sc"], c["x"], c["out"]
     R, D, S = x.R, sc.D, x.n_streams + pad
     t32 = lambda v: torch.from_numpy(np.asarray(v).astype(np.uint32).view(np.int32)).cuda()
     off = np.concatenate([c["event_off"], np.full(pad, c["event_off"][-1], np.int64)])
+    if back:
+        off[-1] = 0
     wt = weights_tensor(np.concatenate([c["w"].weights, np.repeat(c["w"].weights[:1], pad, 0)]),
                         THETA, c["cap"], bpt)
     init = None
@@ -88,6 +91,8 @@ def _call(c, a, form, pad, load_init=None, model=None, cap=4, bpt=synth.BYTES_PE
                                           out.UB, *ev, init, n_init, o["dec"], o["best"],
                                           o["second"], o["load"], o["n"], o["status"])
     torch.cuda.synchronize()
+    if back:  # the stream has no events: its loads are the initial ones
+        assert (o["load"][-1] == (model[3] if form == "load" and init is None else 0)).all()
     for k in ("load", "n"):
         if k in o:
             o[k] = o[k][:x.n_streams]
@@ -169,3 +174,16 @@ def test_load_model_with_and_without_more_streams(fanout, D, pad, kind, model, b
 def test_small_pools_against_the_oracle(fanout, D):
     inflight_vs_oracle(fanout, "alternate", D, 2, False)
     load_vs_oracle(fanout, "alternate", D, 4, 10 ** 8, 6 * 10 ** 8)
+
+
+@pytest.mark.parametrize("fanout,D,pad", [((2, 2, 2, 2), 8, 1100), ((2, 2, 2, 4), 16, 1100),
+                                          ((2, 2, 4, 4), 32, 1100), ((2, 4, 8, 9), 288, 1100)])
+@pytest.mark.parametrize("form", ["plain", "inflight", "load"])
+def test_offsets_that_decrease(fanout, D, pad, form):
+    """A stream whose event offsets decrease has no events, in the base-score pass as in the
+    walk; the other streams' results are those of a call without it."""
+    c = _case(fanout, 3, rps=150, seed=D)
+    assert c["sc"].D == D
+    a = _arrays(c, False)
+    kw = dict(model=(4, 0, 10 ** 8, 3 * 10 ** 9)) if form == "load" else {}
+    _same(_call(c, a, form, 0, **kw), _call(c, a, form, pad, back=True, **kw))
