@@ -1455,7 +1455,7 @@ __global__ void __launch_bounds__(32) schedule_listed_kernel(
   __syncwarp();
 
   const uint64_t e0 = event_off[stream], e1 = event_off[stream + 1];
-  const uint64_t n_win = (e1 - e0 + 31) / 32;
+  const uint64_t n_win = e1 > e0 ? (e1 - e0 + 31) / 32 : 0;
   auto codes_of = [&](uint64_t k) -> uint32_t {  // lane i: code of event i of window k
     const uint64_t e = e0 + 32 * k + lane;
     return e < e1 ? __ldg(events + e) : kBad;
@@ -1784,7 +1784,7 @@ __global__ void __launch_bounds__(32 * kWinWarps) schedule_window_kernel(
   for (uint32_t q = sl; q < 33u * LPS; q += LPS) rel[q] = 0u;
 
   const uint64_t e0 = live ? event_off[stream] : 0, e1 = live ? event_off[stream + 1] : 0;
-  const uint32_t my_win = (uint32_t)((e1 - e0 + 31) / 32);
+  const uint32_t my_win = e1 > e0 ? (uint32_t)((e1 - e0 + 31) / 32) : 0u;
   const uint32_t n_win = __reduce_max_sync(0xffffffffu, my_win);
   auto codes_of = [&](uint32_t k, uint32_t* c) {
 #pragma unroll

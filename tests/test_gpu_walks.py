@@ -177,7 +177,9 @@ def test_small_pools_against_the_oracle(fanout, D):
 
 
 @pytest.mark.parametrize("fanout,D,pad", [((2, 2, 2, 2), 8, 1100), ((2, 2, 2, 4), 16, 1100),
-                                          ((2, 2, 4, 4), 32, 1100), ((2, 4, 8, 9), 288, 1100)])
+                                          ((2, 2, 2, 2), 8, 1540), ((2, 2, 2, 4), 16, 1540),
+                                          ((2, 2, 4, 4), 32, 1100), ((2, 4, 8, 9), 288, 1100),
+                                          ((2, 8, 16, 8), 1024, 520), ((1, 1, 1025, 2), 1025, 2)])
 @pytest.mark.parametrize("form", ["plain", "inflight", "load"])
 def test_offsets_that_decrease(fanout, D, pad, form):
     """A stream whose event offsets decrease has no events, in the base-score pass as in the
