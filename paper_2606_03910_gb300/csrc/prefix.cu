@@ -563,7 +563,8 @@ __device__ __forceinline__ void settle(const Mask (&nm)[N], uint32_t p, GroupHit
 }
 
 // Where the lists are not in chain order: blocks from p on looked up 32 at a time, side by
-// side, until the scan is done (p = n) or a run can be followed again from `run`.  Out of
+// side, until the scan is done (p = n) or a run can be followed again from `run`.  A position
+// counts only where the run array holds the block's hash, as when a run is followed.  Out of
 // line, with its state by value, so that the common path keeps its registers.
 template <int kMB>
 struct SideScan {
@@ -573,6 +574,7 @@ struct SideScan {
 };
 template <int kMB>
 __device__ __noinline__ SideScan<kMB> scan_side_by_side(const IndexSlot* __restrict__ hash,
+                                                        const unsigned long long* __restrict__ keys,
                                                         const unsigned char* __restrict__ masks,
                                                         const uint64_t* __restrict__ chain,
                                                         uint32_t n, uint32_t log2_cap,
@@ -584,14 +586,17 @@ __device__ __noinline__ SideScan<kMB> scan_side_by_side(const IndexSlot* __restr
   while (s.p < n && s.alive) {
     const uint32_t i = s.p + lane;
     const uint64_t key = i < n ? __ldcs(chain + i) : 0ull;
-    const unsigned long long pos = key != 0ull ? lookup(hash, key, log2_cap, status) : kNotFound;
+    unsigned long long pos = key != 0ull ? lookup(hash, key, log2_cap, status) : kNotFound;
+    const bool corrupt = pos != kNotFound && (pos >> log2_cap || __ldg(keys + pos) != key);
+    if (corrupt) pos = kNotFound;
     const uint32_t ok = __ballot_sync(0xffffffffu, pos != kNotFound);
     const uint32_t lead = ~ok ? (uint32_t)(__ffs(~ok) - 1) : 32u;
     const Mask nm[1] = {lane < lead ? (Mask)(s.alive & ~(Mask)run_mask<kMB>(ix, pos)) : (Mask)0};
     settle(nm, s.p, s.h, s.alive, lane);
     if (lead < 32u) {
       if (s.p + lead < n) {  // block p + lead is absent from every cache of the group
-        if (lane == lead && key == 0ull && s.alive) flag_status(status, NETKV_DEV_EDOMAIN);
+        if (lane == lead && s.alive && (corrupt || key == 0ull))
+          flag_status(status, corrupt ? NETKV_DEV_EFULL : NETKV_DEV_EDOMAIN);
         miss_all(s.h, lane, s.alive, s.p + lead);
       }
       s.p = n;
@@ -698,8 +703,9 @@ __device__ __forceinline__ void scan_chain(const IndexView& ix, uint32_t log2_ca
     run += lead;
     in_run = lead == 32u * U;  // else the run parts here: look the next block up
     if (out_of_order) {
-      const SideScan<kMB> s = scan_side_by_side<kMB>(ix.hash, ix.masks, chain, n, log2_cap,
-                                                     SideScan<kMB>{h, alive, p, run}, status);
+      const SideScan<kMB> s = scan_side_by_side<kMB>(ix.hash, ix.keys, ix.masks, chain, n,
+                                                     log2_cap, SideScan<kMB>{h, alive, p, run},
+                                                     status);
       h = s.h;
       alive = s.alive;
       p = s.p;

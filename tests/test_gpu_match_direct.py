@@ -92,3 +92,33 @@ def test_zero_hash(at, shuffled):
     M, _, status, _ = _prefix_case([bad], [[keys[:0], chain[:max(at - 1, 0)]]], 2, [1])
     assert status == (nk().NETKV_DEV_EDOMAIN if at == 0 else 0)
     assert M.tolist() == [[0, max(at - 1, 0)]]
+
+
+@pytest.mark.parametrize("at", [1, 2, 5, 40, 99])
+@pytest.mark.parametrize("entry", ["other", "past the end"])
+@pytest.mark.parametrize("shuffled", [False, True])
+@pytest.mark.parametrize("D", [8, 64])
+def test_corrupted_index(D, shuffled, entry, at):
+    """A slot whose position does not hold its hash, or lies past the run array: where the scan
+    looks the block up, it counts as a miss and sets EFULL, in lists in chain order and not."""
+    from tests.gpu_common import host
+    netkv = nk()
+    rng = np.random.default_rng(at)
+    chain = _hashes(rng, 100)
+    keys = rng.permutation(chain) if shuffled else np.concatenate([chain[at:], chain[:at]])
+    _, _, status, index = _prefix_case([chain], [[keys] * D], D, [1])
+    assert status == 0
+    log2_cap = netkv.index_log2_capacity(100)
+    slots = index[:2 << log2_cap].view(-1, 2)
+    hit = (slots[:, 0] == int(chain.view(np.int64)[at])).nonzero()
+    assert hit.numel() == 1
+    slot = int(hit[0, 0])
+    slots[slot, 1] = (int(slots[slot, 1]) + 7) % 100 if entry == "other" else (1 << log2_cap) + 3
+    M = torch.full((1, D), -1, dtype=torch.int16, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    off = torch.tensor([0, 100], device="cuda")
+    netkv.netkv_prefix_match(index, D, log2_cap, 1, torch.from_numpy(chain.view(np.int64)).cuda(),
+                             off, 1, None, M, st)
+    # in chain order the lists wrap at `at`, so that the scan looks that block up there too
+    assert host(M).tolist() == [[at] * D]
+    assert int(st.item()) == netkv.NETKV_DEV_EFULL
