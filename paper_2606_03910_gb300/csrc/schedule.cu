@@ -1565,7 +1565,7 @@ __global__ void __launch_bounds__(32) schedule_listed_kernel(
         if (ce.x == r && (ce.y & ~31u) == tag && (ce.y & 31u) < lane)
           dd = (int32_t)(kInWindow | (ce.y & 31u));
       }
-      if (c == kBad) {
+      if (e0 + 32 * k + lane >= e1) {  // no event
       } else if (r >= R) {
         flag_status(status, NETKV_DEV_ERANGE);
       } else if (c >> 31) {
@@ -1877,7 +1877,7 @@ __global__ void __launch_bounds__(32 * kWinWarps) schedule_window_kernel(
       const uint4 f = b.rec[j];
       l_ev[q] = f.y;
       dd_ev[q] = kBad;
-      if (code == kBad) continue;
+      if (e0 + 32ull * k + j >= e1) continue;  // no event
       if (r >= R) {
         flag_status(status, NETKV_DEV_ERANGE);
         continue;

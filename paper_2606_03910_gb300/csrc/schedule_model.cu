@@ -181,7 +181,8 @@ __device__ __forceinline__ void produce(const ModelArgs& a, const netkv_weights&
   const uint32_t D = t.D, win = a.lay.win;
   const uint32_t ptid = (wid - 1 - wid / 4) * 32 + (threadIdx.x & 31);
   const uint32_t step_q = NP / D, step_d = NP % D;
-  uint32_t code = ptid < win && e0 + ptid < e1 ? __ldg(a.events + e0 + ptid) : kBadCode;
+  bool have = ptid < win && e0 + ptid < e1;  // whether the lane has an event in the window
+  uint32_t code = have ? __ldg(a.events + e0 + ptid) : kBadCode;
   uint32_t prev_r = kBadCode;  // lane j: event j of the window before: its request, if an arrival
   for (uint64_t k = 0; k <= n_win; ++k) {
     if (k < n_win) {
@@ -199,8 +200,9 @@ __device__ __forceinline__ void produce(const ModelArgs& a, const netkv_weights&
         x.dd = -1;
         const uint32_t r = code & 0x7fffffffu;
         const uint64_t e = e0 + (k + 1) * win + ptid;
-        const uint32_t next = ptid < win && e < e1 ? __ldg(a.events + e) : kBadCode;
-        if (code == kBadCode) {
+        const bool have_next = ptid < win && e < e1;
+        const uint32_t next = have_next ? __ldg(a.events + e) : kBadCode;
+        if (!have) {
         } else if (r >= a.R) {
           flag_status(a.status, NETKV_DEV_ERANGE);
         } else if (code >> 31) {
@@ -227,6 +229,7 @@ __device__ __forceinline__ void produce(const ModelArgs& a, const netkv_weights&
           }
         }
         code = next;
+        have = have_next;
         // the window's arrivals, in order, and each departure's arrival when that lies in
         // this window or the one before (their decisions are not recorded yet)
         const bool is_arr = x.type == kArrival || x.type == kBadArrival;

@@ -189,3 +189,24 @@ def test_offsets_that_decrease(fanout, D, pad, form):
     a = _arrays(c, False)
     kw = dict(model=(4, 0, 10 ** 8, 3 * 10 ** 9)) if form == "load" else {}
     _same(_call(c, a, form, 0, **kw), _call(c, a, form, pad, back=True, **kw))
+
+
+@pytest.mark.parametrize("fanout,D,form,pad", [
+    ((2, 2, 2, 2), 8, "plain", 0), ((2, 2, 2, 2), 8, "plain", 1540), ((2, 2, 2, 4), 16, "plain", 1540),
+    ((2, 4, 8, 9), 288, "plain", 0), ((2, 8, 16, 8), 1024, "plain", 520),
+    ((1, 1, 1025, 2), 1025, "plain", 0), ((2, 2, 2, 2), 8, "inflight", 0),
+    ((2, 4, 8, 9), 288, "inflight", 0), ((2, 2, 2, 2), 8, "load", 0), ((2, 4, 8, 9), 288, "load", 0),
+    ((2, 4, 8, 9), 288, "load", 920)])
+def test_event_code_of_all_ones(fanout, D, form, pad):
+    """0xffffffff is the departure of an out-of-range request: skipped, and flagged as such."""
+    c = _case(fanout, 3, rps=150, seed=D)
+    a = _arrays(c, False)
+    kw = dict(model=(4, 0, 10 ** 8, 3 * 10 ** 9)) if form == "load" else {}
+    at = np.flatnonzero(a["events"] >> 31)[40]
+    got = []
+    for code in (0xffffffff, (c["x"].R + 7) | 0x80000000):
+        ev = a["events"].copy()
+        ev[at] = code
+        got.append(_call(c, dict(a, events=ev), form, pad, **kw))
+    _same(*got)
+    assert int(got[0]["status"].item()) == nk().NETKV_DEV_ERANGE
