@@ -1128,8 +1128,7 @@ __global__ void __launch_bounds__(BLOCK) schedule_staged_kernel(
     load[j] = (load_init && d < D) ? load_init[(uint64_t)stream * D + d] : 0;
   }
   auto refresh = [&](int j) {
-    const int64_t h = w.cap_tokens - load[j];
-    hr[j] = tid * NPT + j >= D ? 0u : h <= 0 ? 0u : h >= 0xffffffffll ? 0xffffffffu : (uint32_t)h;
+    hr[j] = tid * NPT + j >= D ? 0u : headroom(w.cap_tokens, load[j]);
     lt[j] = w.theta_s_per_token * (float)load[j];
   };
 #pragma unroll
@@ -1434,9 +1433,8 @@ __global__ void __launch_bounds__(32) schedule_listed_kernel(
     return wide_to_float(x);
   };
   auto hl_of = [&](int64_t ld) -> uint2 {
-    const int64_t h = w.cap_tokens - ld;
-    const uint32_t hr = h <= 0 ? 0u : h >= 0xffffffffll ? 0xffffffffu : (uint32_t)h;
-    return make_uint2(hr, __float_as_uint(w.theta_s_per_token * to_f(ld)));
+    return make_uint2(headroom(w.cap_tokens, ld),
+                      __float_as_uint(w.theta_s_per_token * to_f(ld)));
   };
   int64_t lmin = INT64_MAX;
   for (uint32_t d = lane; d < D; d += 32) {

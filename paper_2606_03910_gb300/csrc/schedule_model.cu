@@ -717,7 +717,7 @@ __global__ void __launch_bounds__(BT, BT >= 256 ? 512 / BT : 1024 / BT)
     return h <= 0 ? 0u : h >= 0xffffffffll ? 0xffffffffu : (uint32_t)h;
   };
   auto hl_of_load = [&](int64_t ld) -> uint2 {
-    return make_uint2(clamp32(w.cap_tokens - ld),
+    return make_uint2(headroom(w.cap_tokens, ld),
                       __float_as_uint(w.theta_s_per_token * load_to_float(ld)));
   };
   // decode d after `delta` tokens more (load model: `delta` missed tokens of `n` requests less)

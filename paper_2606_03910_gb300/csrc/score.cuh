@@ -66,6 +66,13 @@ __device__ __forceinline__ void warp_argmin_keys(uint32_t& key, uint32_t& rank, 
   key2 = sk;
 }
 
+// Tokens that still fit a decode, at most 2^32 - 1: load + l <= cap iff l <= headroom (l >= 1).
+// The unsigned difference is exact where cap > load, also where the signed one overflows.
+__device__ __forceinline__ uint32_t headroom(int64_t cap, int64_t load) {
+  const uint64_t h = (uint64_t)cap - (uint64_t)load;
+  return cap <= load ? 0u : h >= 0xffffffffull ? 0xffffffffu : (uint32_t)h;
+}
+
 // The paper's compute-load model (Sec. III-C, IV-B) as kernel parameters.
 struct LoadModel {
   float t_a, t_b;      // t_iter(beta) = t_a + t_b * beta

@@ -210,3 +210,19 @@ def test_event_code_of_all_ones(fanout, D, form, pad):
         got.append(_call(c, dict(a, events=ev), form, pad, **kw))
     _same(*got)
     assert int(got[0]["status"].item()) == nk().NETKV_DEV_ERANGE
+
+
+@pytest.mark.parametrize("fanout,D,form,pad", [
+    ((2, 2, 2, 2), 8, "plain", 0), ((2, 4, 8, 9), 288, "plain", 0), ((2, 8, 16, 8), 1024, "plain", 520),
+    ((1, 1, 1025, 2), 1025, "plain", 0), ((2, 2, 2, 2), 8, "inflight", 0),
+    ((2, 4, 8, 9), 288, "inflight", 0), ((2, 4, 8, 9), 288, "inflight", 920)])
+def test_no_token_limit_and_negative_loads(fanout, D, form, pad):
+    """A capacity of 2^63 - 1 tokens limits nothing, also where loads are negative (departures
+    of requests that an earlier call dispatched)."""
+    c = _case(fanout, 2, rps=150, seed=D)
+    a = _arrays(c, False)
+    init = _init(c) - 40_000
+    got = []
+    for cap in (2 ** 63 - 1, 2 ** 62):
+        got.append(_call(dict(c, cap=cap), a, form, pad, init))
+    _same(*got)
