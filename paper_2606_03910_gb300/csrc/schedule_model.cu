@@ -713,8 +713,9 @@ __global__ void __launch_bounds__(BT, BT >= 256 ? 512 / BT : 1024 / BT)
   int32_t* s_held = reinterpret_cast<int32_t*>(smem + a.lay.held);
   const int64_t bpt = (int64_t)w.bytes_per_token;
   const bool in_tokens = kWalk != kModel || (bpt > 0 && bpt < (1ll << 31));
-  auto clamp32 = [](int64_t h) -> uint32_t {
-    return h <= 0 ? 0u : h >= 0xffffffffll ? 0xffffffffu : (uint32_t)h;
+  // `tok` whole tokens free: the bound that a candidate's missed tokens stay below
+  auto below = [](int64_t tok) -> uint32_t {
+    return tok < 0 ? 0u : tok >= 0xfffffffell ? 0xffffffffu : (uint32_t)tok + 1u;
   };
   auto hl_of_load = [&](int64_t ld) -> uint2 {
     return make_uint2(headroom(w.cap_tokens, ld),
@@ -728,7 +729,7 @@ __global__ void __launch_bounds__(BT, BT >= 256 ? 512 / BT : 1024 / BT)
       s_state[d] += delta * bpt;
       s_tok[d] = tok;
       s_held[d] = h;
-      s_hl[d] = make_uint2(clamp32(tok + 1), __float_as_uint(load_term(a.lm, h)));
+      s_hl[d] = make_uint2(below(tok), __float_as_uint(load_term(a.lm, h)));
     } else {
       const int64_t ld = s_state[d] + delta;
       s_state[d] = ld;
@@ -740,8 +741,10 @@ __global__ void __launch_bounds__(BT, BT >= 256 ? 512 / BT : 1024 / BT)
     if (a.state_init) x = a.state_init[(uint64_t)stream * D + d];
     s_state[d] = x;
     if (kWalk == kModel) {
-      const int64_t f = x < INT64_MIN / 4 ? INT64_MIN / 2 : x - min(a.lm.m_min, INT64_MAX / 4);
-      s_tok[d] = !in_tokens ? 0 : f >= 0 ? f / bpt : -((-f + bpt - 1) / bpt);
+      // x - m_min in whole tokens, rounded down, kept where a call's changes cannot overflow
+      const int64_t f = x < INT64_MIN + a.lm.m_min ? INT64_MIN : x - a.lm.m_min;
+      const int64_t tok = !in_tokens ? 0 : f / bpt - (f % bpt < 0 ? 1 : 0);
+      s_tok[d] = max(INT64_MIN / 2, min(INT64_MAX / 2, tok));
       s_held[d] = a.held_init ? a.held_init[(uint64_t)stream * D + d] : 0;
       change(d, 0, 0);
     } else {
@@ -852,7 +855,7 @@ __global__ void __launch_bounds__(BT, BT >= 256 ? 512 / BT : 1024 / BT)
           cb = take ? sc : cb;
           cc = take ? d : cc;
         };
-        if (kWalk == kModel && (!in_tokens || l == kNone)) {  // see clamp32: 2^32 - 1 is a bound
+        if (kWalk == kModel && (!in_tokens || l == kNone)) {  // see below(): 2^32 - 1 is a bound
           for (uint32_t d = lane; d < D; d += 32) {  // ranks rise within a lane, as below
             const uint2 c = S.cand[row + d];
             visit(b, s2, ci, d, s_state[d] >= (int64_t)c.y * bpt + a.lm.m_min,

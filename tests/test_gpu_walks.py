@@ -226,3 +226,18 @@ def test_no_token_limit_and_negative_loads(fanout, D, form, pad):
     for cap in (2 ** 63 - 1, 2 ** 62):
         got.append(_call(dict(c, cap=cap), a, form, pad, init))
     _same(*got)
+
+
+@pytest.mark.parametrize("fanout,D,pad", [((2, 2, 2, 2), 8, 0), ((2, 4, 8, 9), 288, 0),
+                                          ((2, 4, 8, 9), 288, 920)])
+def test_load_model_with_memory_near_its_range(fanout, D, pad):
+    """Free memory up to 2^63 - 1 bytes, a token of one byte, and a reserve of 2^62 bytes."""
+    c = _case(fanout, 2, rps=150, seed=D)
+    a = _arrays(c, False)
+    call = lambda m_min, m0, bpt: _call(c, a, "load", pad, model=(64, 0, m_min, m0), bpt=bpt)
+    for other, shift, bpt in (((0, 2 ** 63 - 1), 2 ** 62 - 1, 1),
+                              ((2 ** 62, 2 ** 62 + 2 * 10 ** 8), 0, synth.BYTES_PER_TOKEN_SHARD)):
+        base = (0, 2 ** 62) if bpt == 1 else (0, 2 * 10 ** 8)
+        x, y = call(*other, bpt), call(*base, bpt)
+        x["load"] -= other[1] - base[1]
+        _same(x, y)
