@@ -24,14 +24,16 @@
 // and the table is rebuilt from them.
 //
 // One CTA per stream walks the stream's events in order:
-//   departure  the lead thread returns the request's tokens to its decode's load;
+//   departure  the first thread of the last warp returns the request's tokens to its
+//              decode's load.  It alone writes loads, so departures need no barrier of
+//              their own: those of an arrival separate its writes from the others' reads;
 //   arrival    warps take decodes and find the first miss of the chain by following the
-//              runs the chain's blocks form in the log (32 blocks a step); threads
+//              runs the chain's blocks form in the log (64 or 128 blocks a step); threads
 //              take decodes and score them exactly as netkv_schedule_streams does without
 //              a workspace (base score + w_load * theta * load), then a block-wide
 //              (score, index) argmin; every thread then uses its share of the chain's
-//              blocks on the chosen cache, and the CTA evicts in chunks of 256 log
-//              entries with a block scan over their liveness.
+//              blocks on the chosen cache, and the CTA evicts in chunks of two log entries
+//              a thread with a block scan over their liveness.
 #include <math.h>
 
 #include "score.cuh"
@@ -88,18 +90,19 @@ __device__ __forceinline__ ulonglong2 vload_slot(const LruSlot* p) {
   return __ldcg(reinterpret_cast<const ulonglong2*>(p));
 }
 
-// Latest log position of `key` (non-zero) in a cache's table, by the whole warp (four slots
+// Latest log position of `key` (non-zero) in a cache's table, by the whole warp (kFind slots
 // per step); 0 when the key is absent.
+template <int kFind>
 __device__ __forceinline__ unsigned long long lru_find(const LruSlot* T, uint32_t ls,
                                                        unsigned long long key, uint32_t lane,
                                                        int* status) {
   const unsigned long long n = 1ull << ls;
   const unsigned long long home = home_slot(key, ls);
-  for (unsigned long long seen = 0; seen < n; seen += 4) {
+  for (unsigned long long seen = 0; seen < n; seen += kFind) {
     ulonglong2 s = make_ulonglong2(~key, 0ull);
-    if (lane < 4) s = vload_slot(T + ((home + seen + lane) & (n - 1)));
-    const uint32_t end = __ballot_sync(0xffffffffu, lane < 4 && (s.x == key || s.x == 0ull));
-    if (end) {  // the first of the four that holds the key or nothing decides
+    if (lane < kFind) s = vload_slot(T + ((home + seen + lane) & (n - 1)));
+    const uint32_t end = __ballot_sync(0xffffffffu, lane < kFind && (s.x == key || s.x == 0ull));
+    if (end) {  // the first of them that holds the key or nothing decides
       const uint32_t at = __ffs(end) - 1;
       const bool found = __shfl_sync(0xffffffffu, s.x == key, at);
       const unsigned long long pos = __shfl_sync(0xffffffffu, s.y, at);
@@ -112,8 +115,8 @@ __device__ __forceinline__ unsigned long long lru_find(const LruSlot* T, uint32_
 
 // The slot of `key` (non-zero), claimed when the key is absent (fresh: claimed here).  kWide
 // slots are read at a time: a walk that waits for one chain's blocks reads two (1, 2 and 4:
-// 5.12, 4.93 and 5.19 ms of 300 arrivals on each of 32 streams), an initial fill, bound by
-// the sectors it touches, one.
+// 5.12, 4.93 and 5.19 ms of 300 arrivals on each of 32 streams), an initial fill and the walk
+// of many streams, bound by the sectors they touch, one.
 template <int kWide>
 __device__ __forceinline__ LruSlot* lru_claim(LruSlot* T, uint32_t ls, unsigned long long key,
                                               bool& fresh, int* status) {
@@ -210,15 +213,15 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 // Leading chain blocks cached in one cache: the first miss among blocks [0, n), found by
 // one warp.  The blocks of a chain that entered the cache together sit in the log as one
 // run in reverse order (block j at the run's start position minus j), so the warp looks a
-// block up in the table once and then compares 128 chain blocks with the 128 log entries
+// block up in the table once and then compares 32 U chain blocks with the 32 U log entries
 // below its position per step (coalesced), looking up again only where chain and log part.
 // A log entry in the window that holds the block's hash is its latest use (the others
 // are zero), so a match there is a cached block.
+template <int U, int kFind>
 __device__ __forceinline__ uint32_t lru_match(const LruSlot* T, const unsigned long long* ring,
                                               const LruGeom& g, unsigned long long head,
                                               const uint64_t* __restrict__ chain, uint32_t n,
                                               uint32_t lane, int* status) {
-  constexpr int U = 4;
   const unsigned long long qmask = (1ull << g.log2_ring) - 1;
   uint32_t p = 0;
   unsigned long long rp = 0;  // log position of block p within the current run
@@ -228,12 +231,12 @@ __device__ __forceinline__ uint32_t lru_match(const LruSlot* T, const unsigned l
     if (!in_run) {  // look block p up in the table
       const unsigned long long key = __ldg(chain + p);
       const unsigned long long pos =
-          key != 0ull ? lru_find(T, g.log2_slots, key, lane, status) : 0ull;
+          key != 0ull ? lru_find<kFind>(T, g.log2_slots, key, lane, status) : 0ull;
       if (pos == 0ull || pos < head) return p;  // absent or evicted
       rp = pos;
       in_run = true;
       // the log entries of the next steps into L2, a line a lane
-      const unsigned long long ahead = 128ull + 16ull * lane;
+      const unsigned long long ahead = 32ull * U + 16ull * lane;
       if (p + ahead < n && ahead <= rp - head) prefetch_l2(ring + ((rp - ahead) & qmask));
     }
     unsigned long long ck[U], rk[U];
@@ -465,16 +468,19 @@ __global__ void __launch_bounds__(kLruBlock) lru_export_kernel(const void* state
   }
 }
 
-// One CTA of BLOCK threads per stream.  Bound by the dependent round trips of an arrival
-// (look-up and log comparison, claims and atomics of the chain's blocks, the eviction's
-// scan), so every phase spreads over as many threads as the streams leave room for, the
-// next event's fields are read and its chain is fetched into L2 an event ahead, and
-// departures and the scores of small pools are taken by the last warp, whose loads overlap
-// the others' match.  32 streams x 300 arrivals on 8 decodes of 60,000 blocks: 16 us an
-// arrival, about 4 of them the match, 5 the chain's slots, 4 the eviction and the counts
-// before it, 2 the scores; 35 us with 256 threads and 32 blocks a step (512 threads: 17).
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK) evolving_kernel(
+// One CTA of BLOCK threads per stream, kResident CTAs an SM.  Bound by the dependent round
+// trips of an arrival (look-up and log comparison, claims and atomics of the chain's blocks,
+// the eviction's scan), so every phase spreads over as many threads as the streams leave room
+// for, and departures and the scores of small pools are taken by the last warp, whose loads
+// overlap the others' match.  The wide forms read the next event's fields and fetch its chain
+// into L2 an event ahead and read several slots at once; the narrow ones, whose SMs other
+// streams keep busy, do neither, for fewer registers and sectors (760 streams x 60 arrivals at
+// 5 CTAs an SM: 1,447 us, reading ahead 1,579).  32 streams x 300 arrivals on 8
+// decodes of 60,000 blocks: 16 us an arrival, about 4 of them the match, 5 the chain's slots,
+// 4 the eviction and the counts before it, 2 the scores; 35 us with 256 threads and 32 blocks
+// a step (512 threads: 17).
+template <int BLOCK, int kResident>
+__global__ void __launch_bounds__(BLOCK, kResident) evolving_kernel(
     TopoArgs t, uint32_t n_streams, const netkv_weights* __restrict__ W, uint32_t R,
     const uint32_t* __restrict__ len, const uint32_t* __restrict__ prefill,
     const uint32_t* __restrict__ snap, const float* __restrict__ UB, uint32_t n_snap,
@@ -484,6 +490,10 @@ __global__ void __launch_bounds__(BLOCK) evolving_kernel(
     float* __restrict__ second, uint16_t* __restrict__ M, int64_t* __restrict__ load_final,
     int* status) {
   constexpr int NW = BLOCK / 32;
+  constexpr bool kAhead = BLOCK >= 512;      // the next event is read ahead
+  constexpr int kFind = BLOCK >= 512 ? 4 : 1;   // slots of a look-up read at a time
+  constexpr int kClaim = BLOCK >= 512 ? 2 : 1;  // and of a claim
+  constexpr int kStep = kResident < 6 ? 4 : 2;  // 32 chain blocks each, compared at a time
   constexpr uint32_t kNoEvent = 0xffffffffu;
   extern __shared__ __align__(16) unsigned char evo_smem[];
   __shared__ uint32_t warp_buf[NW];
@@ -538,10 +548,11 @@ __global__ void __launch_bounds__(BLOCK) evolving_kernel(
     f.c1 = __ldg(chain_off + r + 1);
     return f;
   };
-  Fields nf = fields(e0);
+  Fields nf;
+  if (kAhead) nf = fields(e0);
   for (uint64_t e = e0; e < e1; ++e) {
-    const Fields f = nf;
-    nf = fields(e + 1);
+    const Fields f = kAhead ? nf : fields(e);
+    if (kAhead) nf = fields(e + 1);
     const uint32_t code = f.code;
     const uint32_t r = code & 0x7fffffffu;
     if (r >= R) {
@@ -593,15 +604,16 @@ __global__ void __launch_bounds__(BLOCK) evolving_kernel(
       if (one_warp) asm volatile("" : "+f"(ubp0), "+f"(ubd0));  // not read after the barrier
     }
     // the next arrival's chain into L2, a line a thread
-    if (!(nf.code >> 31) && nf.c1 > nf.c0) {
+    if (kAhead && !(nf.code >> 31) && nf.c1 > nf.c0) {
       const uint64_t at = (uint64_t)tid * 16;
       if (at < nf.c1 - nf.c0) prefetch_l2(chains + nf.c0 + at);
     }
 
     // hits against the caches as they are now (Sec. III-B first-miss scan)
     for (uint32_t d = wid; d < D; d += NW) {
-      const uint32_t m = lru_match(lru_slots(state, g, c0_cache + d), lru_ring(state, g, c0_cache + d),
-                                   g, s_head[d], chain, (uint32_t)n, lane, status);
+      const uint32_t m = lru_match<kStep, kFind>(
+          lru_slots(state, g, c0_cache + d), lru_ring(state, g, c0_cache + d), g, s_head[d], chain,
+          (uint32_t)n, lane, status);
       if (lane == 0) {
         s_m[d] = m;
         M[(uint64_t)r * D + d] = (uint16_t)m;
@@ -688,7 +700,7 @@ __global__ void __launch_bounds__(BLOCK) evolving_kernel(
     uint32_t fresh = 0, newly = 0;
     for (uint64_t j = tid; j < n; j += BLOCK) {
       const unsigned long long key = __ldg(chain + j);
-      if (key != 0ull) lru_use<2>(T, ring, g, key, P0 + (n - 1 - j), head, fresh, newly, status);
+      if (key != 0ull) lru_use<kClaim>(T, ring, g, key, P0 + (n - 1 - j), head, fresh, newly, status);
     }
     add_counts(fresh, newly, &s_cnt[0], &s_cnt[1]);
     __syncthreads();
@@ -804,15 +816,22 @@ extern "C" netkv_status netkv_schedule_streams_evolving(
   int dev = 0, sms = 0;
   NETKV_CUDA_TRY(cudaGetDevice(&dev));
   NETKV_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-#define NETKV_EVOLVE(BLOCK)                                                                    \
-  evolving_kernel<BLOCK><<<n_streams, BLOCK, smem, (cudaStream_t)stream>>>(                    \
+#define NETKV_EVOLVE(BLOCK, RESIDENT)                                                          \
+  evolving_kernel<BLOCK, RESIDENT><<<n_streams, BLOCK, smem, (cudaStream_t)stream>>>(          \
       t, n_streams, d_w, R, d_len, d_prefill, d_snap, d_UB, n_snap, d_chains, d_chain_off,     \
       d_events, d_event_off, d_state, g, d_load_init, d_dec, d_best, d_second, d_M,            \
       d_load_final, d_status)
-  // as many threads per stream as keep every stream resident
-  if (n_streams <= 2u * (uint32_t)sms) NETKV_EVOLVE(1024);
-  else if (n_streams <= 4u * (uint32_t)sms) NETKV_EVOLVE(512);
-  else NETKV_EVOLVE(256);
+  // As many threads per stream as keep every stream resident: 1, 2, 4 and 6 CTAs an SM by the
+  // launch bounds.  60 arrivals of 4,096 tokens a stream on 8 decodes (us; 1,024 threads / 512 /
+  // 256 by 4 / 256 by 6): 152 streams 761 / 778 / 948 / 1,023, 153 1,244 / 773 / 922 / -, 304
+  // 1,531 / 938 / 1,130 / 1,229, 456 2,166 / 1,536 / 1,207 / 1,286, 608 2,852 / 1,706 / 1,293 /
+  // 1,361, 760 3,527 / 2,276 / 1,861 / 1,486, 1,024 4,765 / 2,941 / 2,043 / 2,217, 1,824 8,235 /
+  // 4,661 / 3,186 / 2,948.
+  const uint32_t per_sm = (n_streams + (uint32_t)sms - 1) / (uint32_t)sms;
+  if (per_sm <= 1) NETKV_EVOLVE(1024, 1);
+  else if (per_sm <= 2) NETKV_EVOLVE(512, 2);
+  else if (per_sm <= 4) NETKV_EVOLVE(256, 4);
+  else NETKV_EVOLVE(256, 6);
 #undef NETKV_EVOLVE
   return netkv_launch_status();
 }

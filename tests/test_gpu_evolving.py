@@ -10,6 +10,8 @@ order (netkv_lru_export).  Scores are checked within 1e-5.  The cases:
     on pools of 8, 15, 100 and 577 decodes;
   * two calls in a row, the second continuing from the caches and loads the first left,
     equal to one call;
+  * every width of the walk (1,024, 512 and 256 threads a stream, by the number of streams),
+    equal to the widest on the same streams;
   * no dispatch at all (nothing fits): the hits are those of the static match;
   * two whole streams of the 4,096-replica workload with 200,000-block caches;
   * host-side rejections of invalid configurations.
@@ -119,6 +121,40 @@ def test_evolving_streams_vs_oracle(fanout, rule, D, n_keys, cap_blocks):
     assert moved > 0            # dispatches changed later hits
     if n_keys == cap_blocks:
         assert full > 0         # caches stayed at capacity: dispatches evicted
+
+
+@pytest.mark.parametrize("fanout,D", [((1, 1, 3, 2), 3), ((2, 2, 2, 2), 8), ((1, 1, 34, 2), 34)])
+@pytest.mark.parametrize("per_sm", [2, 3, 5])
+def test_evolving_with_more_streams(fanout, D, per_sm):
+    """Streams without events beside the real ones bring the call onto the narrower walks: hits,
+    decisions, scores, loads and caches stay those of the call without them."""
+    netkv = nk()
+    w = synth.make_workload(spec_for(fanout, "alternate", 1500, requests_per_stream=60))
+    assert w.D == D
+    sc, x, out = run_evolving(w, 1500)
+    keys1, lens1 = sc.lru_export()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n, S = x.n_streams, (per_sm - 1) * sms + 1
+    sc2 = make_scorer(w)
+    sc2.lru_setup(S, 1500)
+    sc2.lru_reset(stage.keys(w, 0, w.n_sets), stage.key_offsets(w, w.n_sets * w.D), n_caches=n * D)
+    o2 = sc2.alloc_outputs(x.n_snap, x.R, S)
+    sc2.oracle_build(x, o2)
+    netkv.netkv_schedule_streams_evolving(
+        sc2.topo, S, torch.cat([x.weights, x.weights[:32].repeat(S - n)]), x.R, x.length,
+        x.prefill, x.snap, o2.UB, x.n_snap, x.chains, x.chain_off, x.events,
+        torch.cat([x.event_off, x.event_off[-1:].repeat(S - n)]), sc2.lru_state, sc2.lru_cfg, None,
+        o2.dec, o2.best, o2.second, o2.M, o2.load_final, o2.status)
+    sc2.lru_caches = n * D
+    keys2, lens2 = sc2.lru_export()
+    torch.cuda.synchronize()
+    assert int(o2.status.item()) == 0 and (out.dec >= 0).any()
+    for f in ("M", "dec", "best", "second"):
+        assert torch.equal(getattr(o2, f), getattr(out, f)), f
+    assert torch.equal(o2.load_final[:n], out.load_final)
+    assert torch.equal(lens1, lens2)
+    for c in range(n * D):
+        assert torch.equal(keys1[c, :int(lens1[c])], keys2[c, :int(lens2[c])])
 
 
 def test_evolving_two_calls_equal_one():
