@@ -27,6 +27,7 @@
 //   self-contention with a workspace: schedule_kernel on base scores
 #include <math.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "score.cuh"
@@ -238,137 +239,157 @@ __device__ __forceinline__ uint32_t warp_sort(uint32_t v, uint32_t lane) {
   return v;
 }
 
-// The list and bound of one chunk of up to 1,024 decodes of an arrival's base-score row, one
-// warp per (arrival, chunk).  Lane L holds decodes 128 q + 4 L .. + 3 of the chunk, q = 0 .. 7.
+// The list and bound of decodes c0 .. c0 + n - 1, whose base scores are row[0 .. n), by one warp;
+// cand: kListCand entries of shared memory.
+__device__ __forceinline__ void list_chunk(const float* __restrict__ row, uint32_t c0, uint32_t n,
+                                           bool vec, unsigned long long* cand, uint32_t lane,
+                                           uint2* __restrict__ out, uint2* __restrict__ bound) {
+  const uint32_t below = (1u << lane) - 1u;
+  const float nan = __int_as_float(0x7fffffff);
+  float x[8][4];  // NaN past the chunk: neither below nor at any threshold
+  bool bad = false;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const uint32_t d = 128u * q + 4u * lane;
+    if (vec) {
+      const float4 v = d < n ? __ldg(reinterpret_cast<const float4*>(row + d))
+                             : make_float4(0.f, 0.f, 0.f, 0.f);
+      x[q][0] = v.x;
+      x[q][1] = v.y;
+      x[q][2] = v.z;
+      x[q][3] = v.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[q][j] = d + j < n ? __ldg(row + d + j) : 0.f;
+    }
+  }
+  float mn[2] = {nan, nan};  // minima over the even and the odd q
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      bad |= !(x[q][j] == x[q][j]);
+      if (n < kListChunk && 128u * q + 4u * lane + j >= n) x[q][j] = nan;
+      mn[q & 1] = fminf(mn[q & 1], x[q][j]);
+    }
+  }
+  if (__any_sync(0xffffffffu, bad)) {  // a NaN score: nothing bounds the chunk
+    out[lane] = make_uint2(kNone, 0x7f800000u);
+    if (lane == 0) *bound = make_uint2(0u, kBoundInvalid);
+    return;
+  }
+  const uint32_t a = warp_sort(mn[0] == mn[0] ? score_key(mn[0]) : kNoKey, lane);
+  const uint32_t b = warp_sort(mn[1] == mn[1] ? score_key(mn[1]) : kNoKey, lane);
+  uint32_t tk = __reduce_max_sync(0xffffffffu, min(a, __shfl_sync(0xffffffffu, b, 31 - lane)));
+  tk = min(tk, kInfKey);  // fewer than 32 minima: no score is above infinity
+  float T = key_score(tk);
+  uint32_t m, own, total;  // the lane's pairs below T, their number, the warp's
+  for (uint32_t at = 15;; at >>= 1) {
+    m = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) m |= x[q][j] < T ? 1u << (4 * q + j) : 0u;
+    }
+    own = __popc(m);
+    total = __reduce_add_sync(0xffffffffu, own);
+    if (total <= kListCand) break;
+    tk = min(min(__shfl_sync(0xffffffffu, a, at), __shfl_sync(0xffffffffu, b, at)), kInfKey);
+    T = key_score(tk);
+  }
+  uint32_t pos = own;  // inclusive prefix over the lanes
+#pragma unroll
+  for (uint32_t o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, pos, o);
+    if (lane >= o) pos += y;
+  }
+  pos -= own;
+  __syncwarp();  // the call before is done with `cand`
+  while (m) {
+    const uint32_t i = __ffs(m) - 1;
+    m &= m - 1;
+    const uint32_t d = 128u * (i >> 2) + 4u * lane + (i & 3u);
+    cand[pos++] = ((unsigned long long)score_key(__ldg(row + d)) << 32) | (c0 + d);
+  }
+  __syncwarp();
+  for (uint32_t i = lane; i < total; i += 32) {
+    const unsigned long long v = cand[i];
+    uint32_t p = 0;
+    for (uint32_t o = 0; o < total; ++o) p += cand[o] < v;
+    if (p < (uint32_t)kListLen)
+      out[p] = make_uint2((uint32_t)v, __float_as_uint(key_score((uint32_t)(v >> 32))));
+    else if (p == (uint32_t)kListLen)
+      *bound = make_uint2((uint32_t)v, (uint32_t)(v >> 32));
+  }
+  if (total > (uint32_t)kListLen) return;
+  // pairs at T in rank order, while the list or its bound has room
+  uint32_t cum = total;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const bool any = x[q][0] == T || x[q][1] == T || x[q][2] == T || x[q][3] == T;
+    if (cum <= (uint32_t)kListLen && __any_sync(0xffffffffu, any)) {
+      uint32_t p = cum;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t bl = __ballot_sync(0xffffffffu, x[q][j] == T);
+        p += __popc(bl & below);
+        cum += __popc(bl);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (x[q][j] == T) {
+          const uint32_t d = c0 + 128u * q + 4u * lane + j;
+          if (p < (uint32_t)kListLen)
+            out[p] = make_uint2(d, __float_as_uint(T));
+          else if (p == (uint32_t)kListLen)
+            *bound = make_uint2(d, tk);
+          ++p;
+        }
+      }
+    }
+  }
+  if (cum <= (uint32_t)kListLen) {  // every pair up to T is listed
+    if (lane >= cum) out[lane] = make_uint2(kNone, 0x7f800000u);
+    if (lane == 0) *bound = cum == n ? make_uint2(kNone, kNoKey) : make_uint2(0u, tk + 1u);
+  }
+}
+
+// The list and bound of each chunk of up to 1,024 decodes of an arrival's base-score row.  A
+// warp takes an event of a stream (departures cost it one load) and the chunks of its row one
+// after another, or one of them where the requests are few; so a call lists the requests that
+// arrive in it, not all R.  Lane L holds decodes 128 q + 4 L .. + 3 of a chunk, q = 0 .. 7.
 // The 32nd smallest of the 64 minima over a lane's even and odd q is a threshold T that at
 // least 32 pairs reach and few are below: 31 minima at most are, about 44 pairs of 1,024
 // distinct scores.  The pairs below T are gathered in shared memory and each is placed by
 // counting the pairs before it; then pairs at T follow in rank order until the list and its
 // bound are full.  With more than kListCand pairs below, T falls back to smaller minima (the
 // smallest has none below it), and the list may hold fewer than kListLen pairs.
-// Bound by instruction issue: 32,000 arrivals on 4,096 decodes, 207 us (a read of the rows alone
-// takes 77); walking up at most 8 distinct scores with block barriers inside the base pass
-// added 463 us to it and could leave shorter lists.
+// Bound by instruction issue: 32,000 arrivals on 4,096 decodes 154 us (a read of the rows alone
+// takes 77); a warp per (request, chunk) over all R requests, with two 64-bit divisions each,
+// 210; warps by (8 events, chunk) 242; walking up at most 8 distinct scores with block barriers
+// inside the base pass added 463 us to it and could leave shorter lists.
+template <bool kOneChunk>
 __global__ void __launch_bounds__(256, 4) chunk_lists_kernel(
-    const float* __restrict__ base, uint32_t D, uint32_t n_ch, uint32_t R,
+    const float* __restrict__ base, uint32_t D, uint32_t n_ch, uint32_t R, uint32_t n_streams,
+    const uint32_t* __restrict__ events, const uint64_t* __restrict__ event_off,
     uint2* __restrict__ lists, uint2* __restrict__ bounds) {
   __shared__ unsigned long long s_cand[8][kListCand];
   const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const uint32_t below = (1u << lane) - 1u;
-  unsigned long long* cand = s_cand[wid];
-  const float nan = __int_as_float(0x7fffffff);
   const bool vec = D % 4u == 0 && (reinterpret_cast<uintptr_t>(base) & 15u) == 0;
-  const uint64_t n_tasks = (uint64_t)R * n_ch, n_warps = (uint64_t)gridDim.x * 8;
-  for (uint64_t task = (uint64_t)blockIdx.x * 8 + wid; task < n_tasks; task += n_warps) {
-    const uint32_t c0 = (uint32_t)(task % n_ch) * kListChunk;
-    const uint32_t n = min(D - c0, kListChunk);  // decodes of the chunk
-    const float* row = base + (task / n_ch) * D + c0;
-    uint2* out = lists + task * kListLen;
-    float x[8][4];  // NaN past the chunk: neither below nor at any threshold
-    bool bad = false;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const uint32_t d = 128u * q + 4u * lane;
-      if (vec) {
-        const float4 v = d < n ? __ldg(reinterpret_cast<const float4*>(row + d))
-                               : make_float4(0.f, 0.f, 0.f, 0.f);
-        x[q][0] = v.x;
-        x[q][1] = v.y;
-        x[q][2] = v.z;
-        x[q][3] = v.w;
-      } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) x[q][j] = d + j < n ? __ldg(row + d + j) : 0.f;
+  for (uint32_t stream = blockIdx.x; stream < n_streams; stream += gridDim.x) {
+    const uint64_t e1 = event_off[stream + 1];
+    for (uint64_t e = event_off[stream] + (uint64_t)blockIdx.y * 8 + wid; e < e1;
+         e += (uint64_t)gridDim.y * 8) {
+      const uint32_t r = __ldg(events + e);
+      if (r >> 31 || r >= R) continue;
+#pragma unroll 1
+      for (uint32_t c = kOneChunk ? blockIdx.z : 0u; c < n_ch; ++c) {
+        const uint32_t c0 = c * kListChunk;
+        const uint64_t at = (uint64_t)r * n_ch + c;
+        list_chunk(base + (uint64_t)r * D + c0, c0, min(D - c0, kListChunk), vec, s_cand[wid], lane,
+                   lists + at * kListLen, bounds + at);
+        if (kOneChunk) break;
       }
-    }
-    float mn[2] = {nan, nan};  // minima over the even and the odd q
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        bad |= !(x[q][j] == x[q][j]);
-        if (n < kListChunk && 128u * q + 4u * lane + j >= n) x[q][j] = nan;
-        mn[q & 1] = fminf(mn[q & 1], x[q][j]);
-      }
-    }
-    if (__any_sync(0xffffffffu, bad)) {  // a NaN score: nothing bounds the chunk
-      out[lane] = make_uint2(kNone, 0x7f800000u);
-      if (lane == 0) bounds[task] = make_uint2(0u, kBoundInvalid);
-      continue;
-    }
-    const uint32_t a = warp_sort(mn[0] == mn[0] ? score_key(mn[0]) : kNoKey, lane);
-    const uint32_t b = warp_sort(mn[1] == mn[1] ? score_key(mn[1]) : kNoKey, lane);
-    uint32_t tk = __reduce_max_sync(0xffffffffu, min(a, __shfl_sync(0xffffffffu, b, 31 - lane)));
-    tk = min(tk, kInfKey);  // fewer than 32 minima: no score is above infinity
-    float T = key_score(tk);
-    uint32_t m, own, total;  // the lane's pairs below T, their number, the warp's
-    for (uint32_t at = 15;; at >>= 1) {
-      m = 0;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) m |= x[q][j] < T ? 1u << (4 * q + j) : 0u;
-      }
-      own = __popc(m);
-      total = __reduce_add_sync(0xffffffffu, own);
-      if (total <= kListCand) break;
-      tk = min(min(__shfl_sync(0xffffffffu, a, at), __shfl_sync(0xffffffffu, b, at)), kInfKey);
-      T = key_score(tk);
-    }
-    uint32_t pos = own;  // inclusive prefix over the lanes
-#pragma unroll
-    for (uint32_t o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, pos, o);
-      if (lane >= o) pos += y;
-    }
-    pos -= own;
-    __syncwarp();  // the task before is done with `cand`
-    while (m) {
-      const uint32_t i = __ffs(m) - 1;
-      m &= m - 1;
-      const uint32_t d = 128u * (i >> 2) + 4u * lane + (i & 3u);
-      cand[pos++] = ((unsigned long long)score_key(__ldg(row + d)) << 32) | (c0 + d);
-    }
-    __syncwarp();
-    for (uint32_t i = lane; i < total; i += 32) {
-      const unsigned long long v = cand[i];
-      uint32_t p = 0;
-      for (uint32_t o = 0; o < total; ++o) p += cand[o] < v;
-      if (p < (uint32_t)kListLen)
-        out[p] = make_uint2((uint32_t)v, __float_as_uint(key_score((uint32_t)(v >> 32))));
-      else if (p == (uint32_t)kListLen)
-        bounds[task] = make_uint2((uint32_t)v, (uint32_t)(v >> 32));
-    }
-    if (total > (uint32_t)kListLen) continue;
-    // pairs at T in rank order, while the list or its bound has room
-    uint32_t cum = total;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const bool any = x[q][0] == T || x[q][1] == T || x[q][2] == T || x[q][3] == T;
-      if (cum <= (uint32_t)kListLen && __any_sync(0xffffffffu, any)) {
-        uint32_t p = cum;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t bl = __ballot_sync(0xffffffffu, x[q][j] == T);
-          p += __popc(bl & below);
-          cum += __popc(bl);
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (x[q][j] == T) {
-            const uint32_t d = c0 + 128u * q + 4u * lane + j;
-            if (p < (uint32_t)kListLen)
-              out[p] = make_uint2(d, __float_as_uint(T));
-            else if (p == (uint32_t)kListLen)
-              bounds[task] = make_uint2(d, tk);
-            ++p;
-          }
-        }
-      }
-    }
-    if (cum <= (uint32_t)kListLen) {  // every pair up to T is listed
-      if (lane >= cum) out[lane] = make_uint2(kNone, 0x7f800000u);
-      if (lane == 0) bounds[task] = cum == n ? make_uint2(kNone, kNoKey) : make_uint2(0u, tk + 1u);
     }
   }
 }
@@ -2185,9 +2206,18 @@ netkv_status launch(const TopoArgs& t, uint32_t n_streams, const netkv_weights* 
       const uint32_t n_ch = (t.D + kListChunk - 1) / kListChunk;
       const uint64_t blocks = ((uint64_t)R * 32 + 255) / 256;
       const uint64_t cap = (uint64_t)(sms > 0 ? sms : 1) * 64;
-      const uint64_t cblocks = blocks * n_ch;
-      chunk_lists_kernel<<<(unsigned)(cblocks < cap ? cblocks : cap), 256, 0, s>>>(
-          d_base, t.D, n_ch, R, lw->chunk_lists, lw->chunk_bounds);
+      // a warp for every event that the requests can give (an arrival and a departure each)
+      const uint64_t cblocks = std::min(cap, ((uint64_t)R * 2 + 7) / 8);
+      const unsigned cx = (unsigned)std::min<uint64_t>(n_streams, cblocks);
+      const dim3 cgrid(cx, (unsigned)((cblocks + cx - 1) / cx));
+      if (R <= (uint32_t)sms * 16)
+        chunk_lists_kernel<true><<<dim3(cgrid.x, cgrid.y, n_ch), 256, 0, s>>>(
+            d_base, t.D, n_ch, R, n_streams, d_events, d_event_off, lw->chunk_lists,
+            lw->chunk_bounds);
+      else
+        chunk_lists_kernel<false><<<cgrid, 256, 0, s>>>(d_base, t.D, n_ch, R, n_streams, d_events,
+                                                        d_event_off, lw->chunk_lists,
+                                                        lw->chunk_bounds);
       if (netkv_launch_status() != NETKV_OK) return NETKV_ECUDA;
       merge_lists_kernel<<<(unsigned)(blocks < cap ? blocks : cap), 256, 0, s>>>(
           lw->chunk_lists, lw->chunk_bounds, n_ch, R, lw->lists, lw->bounds);

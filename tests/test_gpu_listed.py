@@ -59,10 +59,10 @@ def _weights(w, scale_load=1.0, cap=60_000, w_load=None):
     return weights_tensor(wt, THETA, cap, synth.BYTES_PER_TOKEN_SHARD)
 
 
-def _run(sc, x, out, weights, load_init, ws_bytes, util=False):
+def _run(sc, x, out, weights, load_init, ws_bytes, util=False, ws=None):
     netkv = nk()
     o = sc.alloc_outputs(x.n_snap, x.R, x.n_streams)
-    ws = torch.empty(ws_bytes, dtype=torch.uint8, device="cuda")
+    ws = torch.empty(ws_bytes, dtype=torch.uint8, device="cuda") if ws is None else ws
     if util:
         netkv.netkv_schedule_streams_util(sc.topo, x.n_streams, weights, x.R, x.length,
                                           x.prefill, x.snap, out.M, x.util, x.n_snap, x.events,
@@ -143,3 +143,31 @@ def test_workspace_size_grows_only_for_listed_pools():
         nc = (D + 1023) // 1024  # chunk lists of the base pass, then the pool's merged list
         lists = r256(1000 * nc * 32 * 8) + r256(1000 * nc * 8) + r256(1000 * 32 * 8) + r256(1000 * 8)
         assert netkv.netkv_schedule_workspace_size(1000, D) == (1000 * D * 4 + 255) // 256 * 256 + lists
+
+
+@pytest.mark.parametrize("fanout,D", [SHAPES[0], SHAPES[3]])
+def test_lists_of_the_events_of_a_call(fanout, D):
+    """A call over a slice of the events lists the requests that arrive in it and no others, and
+    the walk of the slice is the staged walk's."""
+    import dataclasses
+    w, sc, x, out = _workload(fanout)
+    full, rows = _sizes(x.R, D)
+    off = x.event_off.cpu().numpy()
+    lo, hi = int(off[1]) + 3, int(off[1]) + 120  # of the second stream; the others: no events
+    xs = dataclasses.replace(x, event_off=torch.tensor([lo, lo, hi, hi], device="cuda"))
+    wt = _weights(w)
+    ws = torch.full((full,), 0xa5, dtype=torch.uint8, device="cuda")
+    a = _run(sc, xs, out, wt, None, full, ws=ws)
+    ev = x.events.cpu().numpy().view(np.uint32)[lo:hi]
+    arrive = np.zeros(x.R, bool)
+    arrive[ev[ev >> 31 == 0]] = True
+    assert 0 < arrive.sum() < x.R
+    n_ch = (D + 1023) // 1024
+    lists = ws[rows:rows + x.R * n_ch * 256].view(x.R, n_ch * 256)
+    written = (lists != 0xa5).any(1).cpu().numpy()
+    np.testing.assert_array_equal(written, arrive)
+    b = _run(sc, xs, out, wt, None, rows)
+    at = torch.from_numpy(arrive).cuda()
+    for f in ("dec", "best", "second"):
+        assert torch.equal(getattr(a, f)[at], getattr(b, f)[at]), f
+    assert torch.equal(a.load_final, b.load_final)
