@@ -288,8 +288,8 @@ typedef struct {
  *                the rest: the walk then rescores only those and falls
  *                back to the arrival's full row when the bound does not certify the argmin
  *                (the same decisions and scores, bit for bit).  A workspace of only the
- *                rows runs the walk over every candidate.  Overlapping calls need distinct
- *                workspaces.
+ *                rows, or a call of at most 8 requests a stream, runs the walk over every
+ *                candidate.  Overlapping calls need distinct workspaces.
  * Every request index must occur in at most one stream, and its departure after its
  * arrival.  Out-of-range indices set ERANGE and the event is skipped.  The topology
  * may have at most 4096 decode instances.

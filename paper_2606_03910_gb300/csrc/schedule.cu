@@ -315,6 +315,7 @@ __device__ __forceinline__ void list_chunk(const float* __restrict__ row, uint32
   for (uint32_t i = lane; i < total; i += 32) {
     const unsigned long long v = cand[i];
     uint32_t p = 0;
+#pragma unroll 8
     for (uint32_t o = 0; o < total; ++o) p += cand[o] < v;
     if (p < (uint32_t)kListLen)
       out[p] = make_uint2((uint32_t)v, __float_as_uint(key_score((uint32_t)(v >> 32))));
@@ -356,19 +357,17 @@ __device__ __forceinline__ void list_chunk(const float* __restrict__ row, uint32
 
 // The list and bound of each chunk of up to 1,024 decodes of an arrival's base-score row.  A
 // warp takes an event of a stream (departures cost it one load) and the chunks of its row one
-// after another, or one of them where the requests are few; so a call lists the requests that
-// arrive in it, not all R.  Lane L holds decodes 128 q + 4 L .. + 3 of a chunk, q = 0 .. 7.
+// after another, so a call lists the requests that arrive in it, not all R.  Lane L holds decodes 128 q + 4 L .. + 3 of a chunk, q = 0 .. 7.
 // The 32nd smallest of the 64 minima over a lane's even and odd q is a threshold T that at
 // least 32 pairs reach and few are below: 31 minima at most are, about 44 pairs of 1,024
 // distinct scores.  The pairs below T are gathered in shared memory and each is placed by
 // counting the pairs before it; then pairs at T follow in rank order until the list and its
 // bound are full.  With more than kListCand pairs below, T falls back to smaller minima (the
 // smallest has none below it), and the list may hold fewer than kListLen pairs.
-// Bound by instruction issue: 32,000 arrivals on 4,096 decodes 154 us (a read of the rows alone
+// Bound by instruction issue: 32,000 arrivals on 4,096 decodes 147 us (a read of the rows alone
 // takes 77); a warp per (request, chunk) over all R requests, with two 64-bit divisions each,
 // 210; warps by (8 events, chunk) 242; walking up at most 8 distinct scores with block barriers
 // inside the base pass added 463 us to it and could leave shorter lists.
-template <bool kOneChunk>
 __global__ void __launch_bounds__(256, 4) chunk_lists_kernel(
     const float* __restrict__ base, uint32_t D, uint32_t n_ch, uint32_t R, uint32_t n_streams,
     const uint32_t* __restrict__ events, const uint64_t* __restrict__ event_off,
@@ -383,12 +382,11 @@ __global__ void __launch_bounds__(256, 4) chunk_lists_kernel(
       const uint32_t r = __ldg(events + e);
       if (r >> 31 || r >= R) continue;
 #pragma unroll 1
-      for (uint32_t c = kOneChunk ? blockIdx.z : 0u; c < n_ch; ++c) {
+      for (uint32_t c = 0; c < n_ch; ++c) {
         const uint32_t c0 = c * kListChunk;
         const uint64_t at = (uint64_t)r * n_ch + c;
         list_chunk(base + (uint64_t)r * D + c0, c0, min(D - c0, kListChunk), vec, s_cand[wid], lane,
                    lists + at * kListLen, bounds + at);
-        if (kOneChunk) break;
       }
     }
   }
@@ -405,71 +403,100 @@ __device__ __forceinline__ unsigned long long list_pair(uint2 e) {  // (rank, ba
   return e.x == kNone ? ~0ull
                       : ((unsigned long long)score_key(__uint_as_float(e.y)) << 32) | e.x;
 }
+__device__ __forceinline__ void merge_lists(const uint2* chunk_lists, const uint2* chunk_bounds,
+                                            uint32_t n_ch, uint64_t r, uint32_t lane,
+                                            uint2* __restrict__ lists, uint2* __restrict__ bounds) {
+  constexpr uint32_t kMaxCh = kListMaxD / kListChunk;
+  unsigned long long x[kMaxCh], bd[kMaxCh];
+  uint32_t xb[kMaxCh];
+  unsigned long long B = ~0ull;
+#pragma unroll
+  for (uint32_t c = 0; c < kMaxCh; ++c) {
+    x[c] = bd[c] = ~0ull;
+    xb[c] = 0x7f800000u;
+    if (c < n_ch) {
+      const uint2 e = __ldcs(chunk_lists + ((r * n_ch + c) * kListLen + lane));
+      const uint2 b = chunk_bounds[r * n_ch + c];
+      x[c] = list_pair(e);
+      xb[c] = e.y;
+      bd[c] = ((unsigned long long)b.y << 32) | b.x;
+      B = min(B, bd[c]);
+    }
+  }
+  uint2 mine = make_uint2(kNone, 0x7f800000u);
+  bool has_bound = false;  // some pair is the (kListLen + 1)-th below B
+  unsigned long long pb = 0;
+#pragma unroll
+  for (uint32_t c = 0; c < kMaxCh; ++c) {
+    const unsigned long long v = x[c];
+    uint32_t p = lane;  // pairs below v in its own list
+#pragma unroll
+    for (uint32_t o = 0; o < kMaxCh; ++o) {
+      if (o == c || o >= n_ch) continue;
+      uint32_t lo = 0;  // pairs of list o below v, by binary search over its 32 lanes
+#pragma unroll
+      for (uint32_t step = 16; step; step >>= 1) {
+        const unsigned long long u = __shfl_sync(0xffffffffu, x[o], lo + step - 1);
+        if (u < v) lo += step;
+      }
+      const unsigned long long u31 = __shfl_sync(0xffffffffu, x[o], 31);
+      if (lo == 31 && u31 < v) lo = 32;  // every pair of list o is below v
+      p += lo;
+    }
+    const bool real = c < n_ch && v < B && (uint32_t)(v & 0xffffffffu) != kNone;
+    // the real pair at lane `lane` sits at pool position p: list it or make it the bound
+    if (real && p < (uint32_t)kListLen) {
+      lists[r * kListLen + p] = make_uint2((uint32_t)v, xb[c]);
+    }
+    const bool is_b = real && p == (uint32_t)kListLen;
+    if (__any_sync(0xffffffffu, is_b)) {
+      const uint32_t src = __ffs(__ballot_sync(0xffffffffu, is_b)) - 1;
+      pb = __shfl_sync(0xffffffffu, v, src);
+      has_bound = true;
+    }
+  }
+  // how many pairs were listed: positions beyond them are empty
+  uint32_t n_listed = 0;
+#pragma unroll
+  for (uint32_t c = 0; c < kMaxCh; ++c)
+    n_listed += __popc(__ballot_sync(0xffffffffu, c < n_ch && x[c] < B &&
+                                                       (uint32_t)(x[c] & 0xffffffffu) != kNone));
+  if (lane >= n_listed) lists[r * kListLen + lane] = mine;
+  if (lane == 0) {
+    const unsigned long long b = has_bound ? pb : B;
+    bounds[r] = make_uint2((uint32_t)b, (uint32_t)(b >> 32));
+  }
+}
 __global__ void __launch_bounds__(256) merge_lists_kernel(
     const uint2* __restrict__ chunk_lists, const uint2* __restrict__ chunk_bounds, uint32_t n_ch,
     uint32_t R, uint2* __restrict__ lists, uint2* __restrict__ bounds) {
-  constexpr uint32_t kMaxCh = kListMaxD / kListChunk;
-  const uint32_t lane = threadIdx.x & 31;
   const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  for (uint64_t r = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < R; r += n_warps) {
-    unsigned long long x[kMaxCh], bd[kMaxCh];
-    uint32_t xb[kMaxCh];
-    unsigned long long B = ~0ull;
-#pragma unroll
-    for (uint32_t c = 0; c < kMaxCh; ++c) {
-      x[c] = bd[c] = ~0ull;
-      xb[c] = 0x7f800000u;
+  for (uint64_t r = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < R; r += n_warps)
+    merge_lists(chunk_lists, chunk_bounds, n_ch, r, threadIdx.x & 31, lists, bounds);
+}
+
+// Both of one arrival by a block, a chunk per warp: calls of few requests, which another launch
+// and chunks one after another hold up.  On 4,096 decodes (us of the call, this kernel / the
+// two): 16 requests 34.9 / 41.0, 256 42.0 / 47.2, 1,200 85.7 / 87.8, 2,400 148.5 / 144.0.
+__global__ void __launch_bounds__(32 * kListMaxD / kListChunk) arrival_lists_kernel(
+    const float* __restrict__ base, uint32_t D, uint32_t n_ch, uint32_t R, uint32_t n_streams,
+    const uint32_t* __restrict__ events, const uint64_t* __restrict__ event_off, uint2* chunk_lists,
+    uint2* chunk_bounds, uint2* __restrict__ lists, uint2* __restrict__ bounds) {
+  __shared__ unsigned long long s_cand[kListMaxD / kListChunk][kListCand];
+  const uint32_t lane = threadIdx.x & 31, c = threadIdx.x >> 5, c0 = c * kListChunk;
+  const bool vec = D % 4u == 0 && (reinterpret_cast<uintptr_t>(base) & 15u) == 0;
+  for (uint32_t stream = blockIdx.x; stream < n_streams; stream += gridDim.x) {
+    const uint64_t e1 = event_off[stream + 1];
+    for (uint64_t e = event_off[stream] + blockIdx.y; e < e1; e += gridDim.y) {
+      const uint32_t r = __ldg(events + e);
+      if (r >> 31 || r >= R) continue;
       if (c < n_ch) {
-        const uint2 e = __ldcs(chunk_lists + ((r * n_ch + c) * kListLen + lane));
-        const uint2 b = chunk_bounds[r * n_ch + c];
-        x[c] = list_pair(e);
-        xb[c] = e.y;
-        bd[c] = ((unsigned long long)b.y << 32) | b.x;
-        B = min(B, bd[c]);
+        const uint64_t at = (uint64_t)r * n_ch + c;
+        list_chunk(base + (uint64_t)r * D + c0, c0, min(D - c0, kListChunk), vec, s_cand[c], lane,
+                   chunk_lists + at * kListLen, chunk_bounds + at);
       }
-    }
-    uint2 mine = make_uint2(kNone, 0x7f800000u);
-    bool has_bound = false;  // some pair is the (kListLen + 1)-th below B
-    unsigned long long pb = 0;
-#pragma unroll
-    for (uint32_t c = 0; c < kMaxCh; ++c) {
-      const unsigned long long v = x[c];
-      uint32_t p = lane;  // pairs below v in its own list
-#pragma unroll
-      for (uint32_t o = 0; o < kMaxCh; ++o) {
-        if (o == c || o >= n_ch) continue;
-        uint32_t lo = 0;  // pairs of list o below v, by binary search over its 32 lanes
-#pragma unroll
-        for (uint32_t step = 16; step; step >>= 1) {
-          const unsigned long long u = __shfl_sync(0xffffffffu, x[o], lo + step - 1);
-          if (u < v) lo += step;
-        }
-        const unsigned long long u31 = __shfl_sync(0xffffffffu, x[o], 31);
-        if (lo == 31 && u31 < v) lo = 32;  // every pair of list o is below v
-        p += lo;
-      }
-      const bool real = c < n_ch && v < B && (uint32_t)(v & 0xffffffffu) != kNone;
-      // the real pair at lane `lane` sits at pool position p: list it or make it the bound
-      if (real && p < (uint32_t)kListLen) {
-        lists[r * kListLen + p] = make_uint2((uint32_t)v, xb[c]);
-      }
-      const bool is_b = real && p == (uint32_t)kListLen;
-      if (__any_sync(0xffffffffu, is_b)) {
-        const uint32_t src = __ffs(__ballot_sync(0xffffffffu, is_b)) - 1;
-        pb = __shfl_sync(0xffffffffu, v, src);
-        has_bound = true;
-      }
-    }
-    // how many pairs were listed: positions beyond them are empty
-    uint32_t n_listed = 0;
-#pragma unroll
-    for (uint32_t c = 0; c < kMaxCh; ++c)
-      n_listed += __popc(__ballot_sync(0xffffffffu, c < n_ch && x[c] < B &&
-                                                         (uint32_t)(x[c] & 0xffffffffu) != kNone));
-    if (lane >= n_listed) lists[r * kListLen + lane] = mine;
-    if (lane == 0) {
-      const unsigned long long b = has_bound ? pb : B;
-      bounds[r] = make_uint2((uint32_t)b, (uint32_t)(b >> 32));
+      __syncthreads();  // the chunks' lists are visible to the block
+      if (c == 0) merge_lists(chunk_lists, chunk_bounds, n_ch, r, lane, lists, bounds);
     }
   }
 }
@@ -2195,7 +2222,12 @@ netkv_status launch(const TopoArgs& t, uint32_t n_streams, const netkv_weights* 
   const uint32_t per_cta = LPS == 32 ? 1u : 32u / LPS;
   const unsigned grid = (n_streams + per_cta - 1) / per_cta;
   if (d_base) {
-    const bool lists = LPS == 32 && lw != nullptr && lw->lists != nullptr;
+    // Lists pay from about 8 requests a stream: the launch that writes them and the windows of
+    // the walk cost what the staged walk takes for 8 arrivals.  1 stream on 4,096 decodes (us,
+    // lists / staged walk): 1 request 28.7 / 20.5, 8 31.8 / 30.8, 16 34.9 / 41.0; 16 streams of
+    // 4 31.5 / 24.9, 64 of 8 43.2 / 39.0.
+    const bool lists =
+        LPS == 32 && lw != nullptr && lw->lists != nullptr && R > (uint64_t)n_streams * 8;
     if (launch_base<kUtil>(t, n_streams, d_w, R, d_len, d_prefill, d_snap, d_M, d_UB, n_snap,
                            d_events, d_event_off, d_base, nullptr, d_status, s) != NETKV_OK)
       return NETKV_ECUDA;
@@ -2204,23 +2236,25 @@ netkv_status launch(const TopoArgs& t, uint32_t n_streams, const netkv_weights* 
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
       const uint32_t n_ch = (t.D + kListChunk - 1) / kListChunk;
-      const uint64_t blocks = ((uint64_t)R * 32 + 255) / 256;
       const uint64_t cap = (uint64_t)(sms > 0 ? sms : 1) * 64;
-      // a warp for every event that the requests can give (an arrival and a departure each)
-      const uint64_t cblocks = std::min(cap, ((uint64_t)R * 2 + 7) / 8);
-      const unsigned cx = (unsigned)std::min<uint64_t>(n_streams, cblocks);
-      const dim3 cgrid(cx, (unsigned)((cblocks + cx - 1) / cx));
-      if (R <= (uint32_t)sms * 16)
-        chunk_lists_kernel<true><<<dim3(cgrid.x, cgrid.y, n_ch), 256, 0, s>>>(
+      // blocks for every event that the requests can give (an arrival and a departure each)
+      const bool few = R <= (uint32_t)sms * 8;
+      const uint64_t most = few ? (uint64_t)R * 2 : ((uint64_t)R * 2 + 7) / 8;
+      const uint64_t blocks = std::min(cap, most);
+      const unsigned gx = (unsigned)std::min<uint64_t>(n_streams, blocks);
+      const dim3 grid(gx, (unsigned)((blocks + gx - 1) / gx));
+      if (few) {
+        arrival_lists_kernel<<<grid, 32 * kListMaxD / kListChunk, 0, s>>>(
             d_base, t.D, n_ch, R, n_streams, d_events, d_event_off, lw->chunk_lists,
-            lw->chunk_bounds);
-      else
-        chunk_lists_kernel<false><<<cgrid, 256, 0, s>>>(d_base, t.D, n_ch, R, n_streams, d_events,
-                                                        d_event_off, lw->chunk_lists,
-                                                        lw->chunk_bounds);
-      if (netkv_launch_status() != NETKV_OK) return NETKV_ECUDA;
-      merge_lists_kernel<<<(unsigned)(blocks < cap ? blocks : cap), 256, 0, s>>>(
-          lw->chunk_lists, lw->chunk_bounds, n_ch, R, lw->lists, lw->bounds);
+            lw->chunk_bounds, lw->lists, lw->bounds);
+      } else {
+        chunk_lists_kernel<<<grid, 256, 0, s>>>(d_base, t.D, n_ch, R, n_streams, d_events,
+                                                d_event_off, lw->chunk_lists, lw->chunk_bounds);
+        if (netkv_launch_status() != NETKV_OK) return NETKV_ECUDA;
+        const uint64_t mblocks = ((uint64_t)R * 32 + 255) / 256;
+        merge_lists_kernel<<<(unsigned)std::min(mblocks, cap), 256, 0, s>>>(
+            lw->chunk_lists, lw->chunk_bounds, n_ch, R, lw->lists, lw->bounds);
+      }
       if (netkv_launch_status() != NETKV_OK) return NETKV_ECUDA;
       return launch_listed(t, n_streams, d_w, R, d_len, d_prefill, d_snap, n_snap, d_events,
                            d_event_off, d_load_init, d_dec, d_best, d_second, d_load_final,

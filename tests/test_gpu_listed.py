@@ -171,3 +171,16 @@ def test_lists_of_the_events_of_a_call(fanout, D):
     for f in ("dec", "best", "second"):
         assert torch.equal(getattr(a, f)[at], getattr(b, f)[at]), f
     assert torch.equal(a.load_final, b.load_final)
+
+
+@pytest.mark.parametrize("fanout,D", [SHAPES[0], SHAPES[3]])
+@pytest.mark.parametrize("requests", [7, 8, 9, 40, 600])
+def test_few_requests(fanout, D, requests):
+    """Around the request counts from which lists are used at all (more than 8 a stream) and are
+    written by two launches instead of one (more than 8 an SM)."""
+    w, sc, x, out = _workload(fanout, requests=requests)
+    full, rows = _sizes(x.R, D)
+    for wt in (_weights(w), _weights(w, cap=3_000)):
+        a = _run(sc, x, out, wt, None, full)
+        _assert_same(a, _run(sc, x, out, wt, None, rows))
+    assert (a.dec >= 0).any()
