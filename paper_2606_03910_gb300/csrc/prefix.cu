@@ -103,7 +103,8 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t flag, uint32_t* warp_sum
 // 0.060 of it; one block per index walking its lists in chunks of 1,024 took 14.85 ms.
 // An index whose lists are too long for the borrowed memory (T over 8 bits per mask byte,
 // lists that repeat hashes many times) or whose table is nearly full is built by
-// build_serial_kernel instead: one block walks the lists in chunks.
+// build_serial_kernel instead: one block walks the lists in chunks.  So are all indices of a
+// call on small ones (serial_build), where seven launches or the passes over the slots cost more.
 struct GroupLists {
   uint64_t pre[kGroup + 1];  // elements before each decode's list
   uint64_t beg[kGroup];      // where the list starts in the keys
@@ -410,68 +411,116 @@ __global__ void __launch_bounds__(kPassBlock) build_masks_kernel(BuildArgs a) {
   }
 }
 
-// The indices that the passes above left out: one block each, the lists walked in order in
-// chunks; new hashes are claimed by atomicCAS and numbered by a block scan.
-__global__ void __launch_bounds__(kBuildBlock) build_serial_kernel(BuildArgs a) {
-  __shared__ GroupLists L;
-  __shared__ uint32_t warp_sums[32];
-  __shared__ uint32_t chunk_new;
-  const uint64_t cap = 1ull << a.log2_cap, mask = cap - 1;
-  const uint32_t mb = mask_bytes_of(a.D);
-  for (uint64_t idx = blockIdx.x; idx < a.n_index; idx += gridDim.x) {
-    load_lists(L, a, idx, true);
-    const uint64_t T = L.pre[kGroup];
-    const IndexView v = index_view(a.index, idx, a.log2_cap, mb);
-    IndexSlot* hash = v.hash;
-    if (lists_fit(T, cap, mb)) {
-      if (__ldcg(build_counts(v, cap, T) + (T + 255) / 256) == 0u) continue;  // built
-      // the table was nearly full: start over
-      uint4* w = reinterpret_cast<uint4*>(v.hash);
-      __syncthreads();  // every thread has read the count
-      for (uint64_t i = threadIdx.x; i < index_stride(a.log2_cap, mb) / 16; i += kBuildBlock)
-        w[i] = make_uint4(0u, 0u, 0u, 0u);
+// The indices that the passes above left out, or all (kAll: no pass has run): one block each, the
+// lists walked in order in chunks; new hashes are claimed by atomicCAS and numbered by a block
+// scan.  Where a chunk repeats a hash that is new in it, another thread than the first may have
+// claimed it: such an index (lists seldom repeat a hash) is built again, numbering every chunk
+// by first elements, by a call out of line, so that the common path keeps its 32 registers.
+constexpr unsigned long long kTentative = 1ull << 63;  // above every run position
+
+// The lists of one index into it (cleared); kExact: by first elements in a chunk, else whether a
+// chunk repeated a hash that was new in it goes to *repeated (shared).
+template <bool kExact>
+__device__ __forceinline__ void build_lists(const BuildArgs& a, uint64_t idx, uint32_t* warp_sums,
+                                            uint32_t* chunk_new, int* repeated) {
+  const uint32_t cap = 1u << a.log2_cap;  // at most 2^31
+  const uint32_t n_dgroups = (a.D + kGroup - 1) / kGroup;
+  const uint64_t g = idx / n_dgroups;
+  const uint32_t q0 = (uint32_t)(idx - g * n_dgroups) * kGroup;
+  const uint32_t ng = min(kGroup, a.D - q0);
+  const uint64_t* off = a.key_off + g * a.D + q0;
+  const IndexView v = index_view(a.index, idx, a.log2_cap, mask_bytes_of(a.D));
+  IndexSlot* hash = v.hash;
+  uint32_t run_len = 0;  // same value in every thread
+  for (uint32_t d = 0; d < ng; ++d) {
+    const uint64_t beg = __ldg(off + d), end = __ldg(off + d + 1);
+    if (end < beg && threadIdx.x == 0) flag_status(a.status, NETKV_DEV_ERANGE);
+    const unsigned long long bit = 1ull << d;
+    for (uint64_t c = beg; c < end; c += kBuildBlock) {
+      const uint64_t j = c + threadIdx.x;
+      unsigned long long key = j < end ? __ldg(a.keys + j) : 0ull;
+      if (j < end && key == 0ull) flag_status(a.status, NETKV_DEV_EDOMAIN);
+      bool is_new = false, placed = false;
+      uint32_t slot = 0;
+      if (key != 0ull) {
+        slot = (uint32_t)home_slot(key, a.log2_cap);
+        for (uint32_t step = 0; step < cap; ++step) {
+          const unsigned long long prev = atomicCAS(&hash[slot].key, 0ull, key);
+          if (prev == 0ull || prev == key) {
+            is_new = prev == 0ull;
+            placed = true;
+            break;
+          }
+          slot = (slot + 1) & (cap - 1);
+        }
+        if (!placed) flag_status(a.status, NETKV_DEV_EFULL);
+      }
+      if (kExact) {  // of the elements that share a hash new in this chunk, the first counts
+        const unsigned long long own = kTentative | (kBuildBlock - 1 - threadIdx.x);
+        if (is_new) atomicMax(&hash[slot].pos, own);
+        __syncthreads();
+        const bool again =
+            placed && !is_new && *((volatile unsigned long long*)&hash[slot].pos) >= kTentative;
+        if (again) atomicMax(&hash[slot].pos, own);
+        __syncthreads();
+        is_new = (is_new || again) && *((volatile unsigned long long*)&hash[slot].pos) == own;
+      }
+      const uint32_t pos = run_len + block_scan(is_new ? 1u : 0u, warp_sums, chunk_new);
+      if (is_new) {
+        hash[slot].pos = pos;
+        v.keys[pos] = key;
+        run_mask_or(v, pos, bit);  // masks share 32-bit words: set by atomics only
+      }
+      __syncthreads();
+      if (placed && !is_new) {
+        const uint64_t p = *((volatile unsigned long long*)&hash[slot].pos);
+        run_mask_or(v, p, bit);
+        if (!kExact && p >= run_len) *repeated = 1;
+      }
+      run_len += *chunk_new;
       __syncthreads();
     }
-    uint32_t run_len = 0;  // same value in every thread
-    for (uint32_t d = 0; d < kGroup; ++d) {
-      const uint64_t beg = L.beg[d], end = beg + (L.pre[d + 1] - L.pre[d]);
-      if (L.pre[d + 1] == L.pre[d]) continue;
-      const unsigned long long bit = 1ull << d;
-      for (uint64_t c = beg; c < end; c += kBuildBlock) {
-        const uint64_t j = c + threadIdx.x;
-        unsigned long long key = j < end ? __ldg(a.keys + j) : 0ull;
-        if (j < end && key == 0ull) flag_status(a.status, NETKV_DEV_EDOMAIN);
-        bool is_new = false;
-        uint64_t slot = 0;
-        bool placed = false;
-        if (key != 0ull) {
-          slot = home_slot(key, a.log2_cap);
-          for (uint64_t step = 0; step < cap; ++step) {
-            const unsigned long long prev = atomicCAS(&hash[slot].key, 0ull, key);
-            if (prev == 0ull || prev == key) {
-              is_new = prev == 0ull;
-              placed = true;
-              break;
-            }
-            slot = (slot + 1) & mask;
-          }
-          if (!placed) flag_status(a.status, NETKV_DEV_EFULL);
-        }
-        const uint32_t pos = run_len + block_scan(is_new ? 1u : 0u, warp_sums, &chunk_new);
-        if (is_new) {
-          hash[slot].pos = pos;
-          v.keys[pos] = key;
-          run_mask_or(v, pos, bit);  // masks share 32-bit words: set by atomics only
-        }
-        __syncthreads();
-        if (placed && !is_new) {
-          const uint64_t p = *((volatile unsigned long long*)&hash[slot].pos);
-          run_mask_or(v, p, bit);
-        }
-        run_len += chunk_new;
-        __syncthreads();
+  }
+}
+
+__device__ __forceinline__ void clear_index(const BuildArgs& a, uint64_t idx) {
+  const uint32_t mb = mask_bytes_of(a.D);
+  uint4* w = reinterpret_cast<uint4*>(index_view(a.index, idx, a.log2_cap, mb).hash);
+  for (uint64_t i = threadIdx.x; i < index_stride(a.log2_cap, mb) / 16; i += kBuildBlock)
+    w[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+__device__ __noinline__ void rebuild_exact(const BuildArgs& a, uint64_t idx, uint32_t* warp_sums,
+                                           uint32_t* chunk_new) {
+  clear_index(a, idx);
+  __syncthreads();
+  build_lists<true>(a, idx, warp_sums, chunk_new, nullptr);
+}
+
+template <bool kAll>
+__global__ void __launch_bounds__(kBuildBlock, 2) build_serial_kernel(
+    const __grid_constant__ BuildArgs a) {
+  __shared__ uint32_t warp_sums[32];
+  __shared__ uint32_t chunk_new;
+  __shared__ int repeated;
+  for (uint64_t idx = blockIdx.x; idx < a.n_index; idx += gridDim.x) {
+    if (!kAll) {
+      __shared__ GroupLists L;
+      load_lists(L, a, idx, false);
+      const uint64_t cap = 1ull << a.log2_cap, T = L.pre[kGroup];
+      const uint32_t mb = mask_bytes_of(a.D);
+      if (lists_fit(T, cap, mb)) {
+        const IndexView v = index_view(a.index, idx, a.log2_cap, mb);
+        if (__ldcg(build_counts(v, cap, T) + (T + 255) / 256) == 0u) continue;  // built
+        __syncthreads();      // every thread has read the count
+        clear_index(a, idx);  // the table was nearly full: start over
       }
     }
+    if (threadIdx.x == 0) repeated = 0;
+    __syncthreads();
+    build_lists<false>(a, idx, warp_sums, &chunk_new, &repeated);
+    if (repeated) rebuild_exact(a, idx, warp_sums, &chunk_new);
+    __syncthreads();  // every thread has read `repeated`
   }
 }
 
@@ -1296,6 +1345,20 @@ netkv_status launch_match(const void* index, uint32_t D, uint32_t log2_cap, uint
   return netkv_launch_status();
 }
 
+// Whether a call's indices are built by one block each.  Few of them: one list after another
+// takes 3 us a list or more, the passes about 45 us for their launches (us, one block / passes;
+// 1 index of 8 lists: 16 keys each 34 / 46, 1,000 55 / 57, 2,000 92 / 61; 16 lists of 16 41 /
+// 53, of 500 74 / 58).  Many: the blocks fill the card, and the passes go over the slots four
+// times (152 indices of 8 lists with shared prefixes: 2,000 keys each 124 / 179, 8,000 566 /
+// 569, 50,000 3,858 / 1,662; 16 lists of 2,000 245 / 310, of 8,000 1,216 / 817; 608 of 32 lists
+// of 500 448 / 570, of 2,000 1,753 / 2,038).  Lists that share nothing favour one block also
+// beyond (300 indices of 8 lists of 50,000: 7,925 / 9,981), which the host cannot see.
+bool serial_build(uint64_t n_index, uint32_t D, uint32_t log2_cap, uint32_t sms) {
+  const uint32_t lists = D < kGroup ? D : kGroup;
+  if ((lists <= 12 && log2_cap <= 14) || (lists <= 16 && log2_cap <= 11)) return true;
+  return 2 * n_index >= sms && lists <= 32 && log2_cap <= 17;
+}
+
 }  // namespace
 
 extern "C" size_t netkv_cache_index_bytes(uint32_t n_sets, uint32_t D, uint32_t log2_capacity) {
@@ -1324,10 +1387,15 @@ extern "C" netkv_status netkv_cache_build(void* d_index, uint32_t n_sets, uint32
   a.keys = d_keys;
   a.key_off = d_key_off;
   a.status = d_status;
-  // blocks per index: one per 2,048 slots, more where the indices alone leave SMs idle
   int dev = 0, sms = 0;
   NETKV_CUDA_TRY(cudaGetDevice(&dev));
   NETKV_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const unsigned per_index = (unsigned)(a.n_index < (1u << 20) ? a.n_index : (1u << 20));
+  if (serial_build(a.n_index, D, log2_capacity, (uint32_t)sms)) {
+    build_serial_kernel<true><<<per_index, kBuildBlock, 0, s>>>(a);
+    return netkv_launch_status();
+  }
+  // blocks per index: one per 2,048 slots, more where the indices alone leave SMs idle
   uint64_t parts = (1ull << log2_capacity) / 2048;
   const uint64_t fill = ((uint64_t)sms * 8 + a.n_index - 1) / a.n_index;
   if (parts > kPartsMax) parts = kPartsMax;
@@ -1335,14 +1403,13 @@ extern "C" netkv_status netkv_cache_build(void* d_index, uint32_t n_sets, uint32
   a.parts = (uint32_t)parts;
   const uint64_t blocks = a.n_index * a.parts;
   const unsigned grid = (unsigned)(blocks < (1u << 30) ? blocks : (1u << 30));
-  const unsigned per_index = (unsigned)(a.n_index < (1u << 20) ? a.n_index : (1u << 20));
   build_insert_kernel<<<grid, kPassBlock, 0, s>>>(a);
   build_mark_kernel<<<grid, kPassBlock, 0, s>>>(a);
   build_count_kernel<<<per_index, kBuildBlock, 0, s>>>(a);
   build_place_kernel<<<grid, kPassBlock, 0, s>>>(a);
   build_wipe_kernel<<<grid, kPassBlock, 0, s>>>(a);
   build_masks_kernel<<<grid, kPassBlock, 0, s>>>(a);
-  build_serial_kernel<<<per_index, kBuildBlock, 0, s>>>(a);
+  build_serial_kernel<false><<<per_index, kBuildBlock, 0, s>>>(a);
   return netkv_launch_status();
 }
 

@@ -3,7 +3,9 @@ distinct hash once, found by linear probing from its home slot, at the run posit
 first appearance in the lists, with the mask of the decodes that list it, and zeros past
 the last run position.  The cases reach the edges of the build's passes: lists around the
 256 elements of a count, mask widths of 1, 2, 4 and 8 bytes, lists too long for the bitmap
-and tables too full for the counts (both built by one block per index)."""
+and tables too full for the counts (both built by one block per index).  Calls on few lists of
+up to 2^14 slots, and on many indices of up to 2^17, are built by one block per index too: the
+edges of the passes are reached with 17 decodes."""
 import numpy as np
 import pytest
 
@@ -40,6 +42,11 @@ def _repeats(seed, T, distinct):
     return [np.concatenate([h, h[rng.integers(0, distinct, T - distinct)]])]
 
 
+def _among(keys, D):
+    """One list among D - 1 empty ones."""
+    return [[]] * (D // 2) + [keys] + [[]] * (D - 1 - D // 2)
+
+
 CASES = {
     "one key, two slots": ([[5]], 1, 1, "ranked"),
     "no key": ([[], []], 2, 4, "ranked"),
@@ -58,6 +65,25 @@ CASES = {
     "counts fill the keys": ([np.arange(1, 1022)], 1, 10, "ranked"),  # 2 * 1021 + 5 words of 2,048
     "counts past the keys": ([np.arange(1, 1023)], 1, 10, "any"),     # 2 * 1022 + 5
     "full table": ([np.arange(1, 1025)], 1, 10, "any"),
+    # the passes at the same edges: 17 lists of one index are too many for one block
+    "17: 255 elements": (_among(np.arange(1, 256), 17), 17, 10, "ranked"),
+    "17: 256 elements": (_among(np.arange(1, 257), 17), 17, 10, "ranked"),
+    "17: 257 elements": (_among(np.arange(1, 258), 17), 17, 10, "ranked"),
+    "17: bitmap filled": (_among(_repeats(8, 32 * 1024, 100)[0], 17), 17, 10, "ranked"),
+    "17: bitmap too small": (_among(_repeats(9, 32 * 1024 + 1, 100)[0], 17), 17, 10, "ranked"),
+    "17: counts fill the keys": (_among(np.arange(1, 1022), 17), 17, 10, "ranked"),
+    "17: counts past the keys": (_among(np.arange(1, 1023), 17), 17, 10, "any"),
+    "17: full table": (_among(np.arange(1, 1025), 17), 17, 10, "any"),
+    # around the rule
+    "12 decodes of 2^14": (_prefix_lists(10, 12, 900), 12, 14, "ranked"),
+    "12 decodes of 2^15": (_prefix_lists(11, 12, 900), 12, 15, "ranked"),
+    "16 decodes of 2^11": (_prefix_lists(16, 16, 200), 16, 11, "ranked"),
+    "16 decodes of 2^12": (_prefix_lists(17, 16, 200), 16, 12, "ranked"),
+    "300 sets of 3": (_prefix_lists(12, 900, 60), 3, 9, "ranked"),
+    "300 sets of 13": (_prefix_lists(13, 3900, 30), 13, 10, "ranked"),
+    "80 sets of 33": (_prefix_lists(14, 2640, 20), 33, 11, "ranked"),
+    "repeats in a chunk": ([_repeats(15, 3000, 700)[0][::-1], _repeats(15, 3000, 700)[0]], 2, 11,
+                           "ranked"),
 }
 
 
