@@ -21,9 +21,10 @@
 //   base scores      at most 16 decodes and more than kSmallMaxStreams streams: windowed;
 //                    up to 1,024 decodes: the walk with producers (launch_model_plain), or
 //                    staged past its rule on decodes and streams; 1,025 .. 4,096: listed, or
-//                    staged where the workspace has no room for the lists
+//                    staged for a few requests a stream and where the workspace has no room
+//                    for the lists
 //   no workspace     schedule_kernel; self-contention and the load model the walk with
-//                    producers first (launch_model_inflight, launch_model_load)
+//                    producers up to its rules (launch_model_inflight, launch_model_load)
 //   self-contention with a workspace: schedule_kernel on base scores
 #include <math.h>
 
@@ -2335,15 +2336,19 @@ netkv_status launch_inflight(const TopoArgs& t, uint32_t n_streams, const netkv_
         nullptr, d_X);
     return netkv_launch_status();
   }
-  if (smem > 48u * 1024u)  // per device: set before every launch that needs it
-    NETKV_CUDA_TRY(cudaFuncSetAttribute(schedule_kernel<NPT, BLOCK, LPS, false, true>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)kInflightSmemMax));
-  schedule_kernel<NPT, BLOCK, LPS, false, true><<<grid, BLOCK, smem, s>>>(
-      t, n_streams, d_w, R, nullptr, d_len, d_prefill, d_snap, d_M, d_UB, n_snap, d_events,
-      d_event_off, d_load_init, d_dec, d_best, d_second, d_load_final, d_status, d_arrival_us,
-      inflight_cap, d_xfer_us, infl_bytes, heap_cap);
-  return netkv_launch_status();
+  if constexpr (LPS == 32 && BLOCK == 32) {
+    return NETKV_EINVAL;  // the walk above takes every pool of 17 .. 32 decodes
+  } else {
+    if (smem > 48u * 1024u)  // per device: set before every launch that needs it
+      NETKV_CUDA_TRY(cudaFuncSetAttribute(schedule_kernel<NPT, BLOCK, LPS, false, true>,
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)kInflightSmemMax));
+    schedule_kernel<NPT, BLOCK, LPS, false, true><<<grid, BLOCK, smem, s>>>(
+        t, n_streams, d_w, R, nullptr, d_len, d_prefill, d_snap, d_M, d_UB, n_snap, d_events,
+        d_event_off, d_load_init, d_dec, d_best, d_second, d_load_final, d_status, d_arrival_us,
+        inflight_cap, d_xfer_us, infl_bytes, heap_cap);
+    return netkv_launch_status();
+  }
 }
 
 }  // namespace

@@ -956,6 +956,33 @@ netkv_status launch_walk(Kernel kernel, const ModelArgs& a, uint32_t n_streams, 
   return netkv_launch_status();
 }
 
+// Whether a stream's walk by one warp pays.  The rows of a window leave room for few CTAs an SM
+// over large pools, where the other kernels score with several warps a stream, and the packed
+// per-event walk puts 2 or 4 streams of up to 16 decodes into a warp.  60 requests a stream,
+// this walk against the other (us):
+//   base scores      577 decodes, 608 streams 200 / 327, 912 513 / 475; 1,024, 304 141 / 187,
+//                    456 314 / 270
+//   self-contention  16 decodes, 2,432 streams 131 / 140, 4,864 205 / 160; 8, 3,648 144 / 164,
+//                    4,864 178 / 166; 96, 608 145 / 262, 760 350 / 281; 192, 304 119 / 139, 456
+//                    252 / 162, 760 1,024 / 289; 32 and 64 at 4,864 575 / 691 and 1,018 / 1,600
+//   load model       8 decodes, 4,864 streams 102 / 117, 7,296 148 / 124; 16, 2,432 85 / 101,
+//                    3,648 146 / 110; 32, 1,216 72 / 76, 2,432 156 / 90; 192, 608 112 / 203, 760
+//                    256 / 223; 577, 304 121 / 192, 456 445 / 350; 800, 152 98 / 168, 304
+//                    245 / 204
+template <Walk kWalk>
+bool walk_pays(uint32_t D, uint32_t n_streams, uint32_t sms) {
+  const uint32_t per_sm = (n_streams + sms - 1) / sms;
+  const uint64_t pool = (uint64_t)D * n_streams;
+  if (kWalk == kPlain) return D <= 512 || (pool <= 512u * 1024u && per_sm <= (D <= 800 ? 4u : 2u));
+  if (D > 96 && pool > 256u * 1024u) return false;
+  if (kWalk == kContend) {
+    if (D <= 16) return per_sm <= 20;
+    return D <= 64 || per_sm <= (D <= 128 ? 4u : 2u);
+  }
+  if (D <= 32) return per_sm <= (D <= 8 ? 32u : D <= 16 ? 16u : 8u);
+  return D <= 128 || per_sm <= (D <= 400 ? 4u : D <= 600 ? 2u : 1u);
+}
+
 // Launches the walk when the pool fits: false (and nothing launched) otherwise.  Windows of
 // 32 events hide the producers' round trips best; shorter ones where the rows of a larger
 // pool need the memory, or more streams than the card's SMs hold at once.
@@ -970,14 +997,7 @@ bool launch_model(ModelArgs& a, uint32_t n_streams, cudaStream_t s, netkv_status
   }
   const uint32_t D = a.t.D;
   const bool small = D <= 32;
-  // Many streams over large pools keep every SM busy with one CTA of several scoring warps per
-  // stream, and the rows of a window no longer leave room for several CTAs here.  60 requests
-  // a stream, this walk against the per-event one (us): base scores, 1,024 decodes, 400
-  // streams 137 / 151, 1,500 streams 1,374 / 464, 288 decodes 1,500 streams 176 / 463;
-  // self-contention, 288 decodes, 400 streams 245 / 422, 1,500 streams 3,137 / 1,143; load
-  // model, 1,024 decodes, 8 streams 255 / 424, 400 streams 512 / 416.
-  const uint64_t pool = (uint64_t)D * n_streams;
-  if (kWalk == kPlain ? D > 512 && pool > 512u * 1024u : D > 96 && pool > 256u * 1024u) return false;
+  if (!walk_pays<kWalk>(D, n_streams, (uint32_t)sms)) return false;
   // producers enough for a window's candidates (about 16 arrivals) in a few rounds while
   // every stream is resident
   uint32_t bt = 64u;

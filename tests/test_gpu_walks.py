@@ -4,13 +4,16 @@ Which walk a call takes follows from the pool and the number of streams, so stre
 events beside the same real ones bring the same call onto the other walk: more than 1,536
 streams for the windowed walk of pools of at most 16 decodes, more than 512 Ki decodes over all
 streams for the staged walk of 513 .. 1,024 decodes, more than 256 Ki for the per-event walks of
-self-contention and the load model (pools above 96).  Pools of 17 .. 512 decodes with base scores
+self-contention and the load model (pools above 96), and more streams an SM than the rule allows
+(walk_pays) for the packed per-event walks of small pools and the others.  Fewer such streams keep
+the walk and narrow its CTAs (64 and 128 threads, shorter windows), which are compared too.  Pools
+of 17 .. 512 decodes with base scores
 are compared with self-contention at counter cap 0 with its workspace, the same greedy on the
 per-event walk.  The event lists are those of tests/test_gpu_window.py: departures in the same
 window, the next, later or never, twice, requests renumbered at random, 2^27 tokens and more,
-bad events, initial loads.  What has no second walk (self-contention and load model, at most 96
-decodes) is held against the oracle at the edges of the pool sizes and of the counters kept
-in registers (32 prefill ranks)."""
+bad events, initial loads.  What has no second walk (self-contention, 17 .. 32 decodes) is held
+against the oracle at the edges of the pool sizes and of the counters kept in registers (32
+prefill ranks)."""
 import numpy as np
 import pytest
 
@@ -241,3 +244,38 @@ def test_load_model_with_memory_near_its_range(fanout, D, pad):
         x, y = call(*other, bpt), call(*base, bpt)
         x["load"] -= other[1] - base[1]
         _same(x, y)
+
+
+# streams without events beside two real ones, at 152 SMs: (pool, streams, whether the walk stays)
+FLEETS = {
+    "inflight": [((1, 1, 3, 2), 3, 700), ((2, 2, 2, 2), 8, 700), ((2, 2, 2, 4), 16, 700),
+                 ((1, 1, 24, 2), 24, 700), ((2, 2, 4, 4), 32, 1300), ((1, 1, 13, 5), 32, 700),
+                 ((1, 1, 33, 2), 33, 400), ((1, 1, 33, 2), 33, 1300), ((1, 1, 64, 2), 64, 700),
+                 ((1, 1, 96, 2), 96, 400), ((1, 1, 97, 2), 97, 280),
+                 # past the rule: the per-event walks
+                 ((1, 1, 3, 2), 3, 3100), ((2, 2, 2, 2), 8, 3100), ((2, 2, 2, 4), 16, 3100),
+                 ((1, 1, 65, 2), 65, 700), ((1, 1, 129, 2), 129, 400)],
+    "load": [((1, 1, 3, 2), 3, 700), ((2, 2, 2, 2), 8, 1300), ((2, 2, 2, 4), 16, 700),
+             ((2, 2, 4, 4), 32, 700), ((1, 1, 33, 2), 33, 400), ((1, 1, 65, 2), 65, 1300),
+             ((1, 1, 96, 2), 96, 700), ((1, 1, 97, 2), 97, 400), ((2, 4, 8, 9), 288, 400),
+             ((1, 1, 3, 2), 3, 4900), ((2, 2, 2, 4), 16, 2500), ((2, 2, 4, 4), 32, 1300),
+             ((1, 1, 130, 2), 130, 700), ((1, 1, 401, 2), 401, 320)],
+    "plain": [((2, 2, 2, 2), 8, 700), ((2, 2, 4, 4), 32, 1300), ((1, 1, 33, 2), 33, 400),
+              ((1, 1, 65, 2), 65, 1300), ((2, 4, 8, 9), 288, 400), ((2, 4, 8, 9), 288, 1300),
+              ((1, 1, 513, 2), 513, 400), ((1, 1, 513, 2), 513, 650), ((1, 1, 801, 2), 801, 320)],
+}
+
+
+@pytest.mark.parametrize("form,fanout,D,pad", [(f, *v) for f in FLEETS for v in FLEETS[f]])
+@pytest.mark.parametrize("kind", ["plain", "bad", "load_init", "twice"])
+def test_fleets(form, fanout, D, pad, kind):
+    c = _case(fanout, 2, rps=150, seed=D, bad=kind == "bad")
+    assert c["sc"].D == D
+    model = (4, 0, 10 ** 8, 3 * 10 ** 9)
+    init = _init(c) + (model[3] if form == "load" else 0) if kind == "load_init" else None
+    if form == "inflight":
+        c["prefill"][c["prefill"] < c["sc"].P] %= 40
+        c["arrival_us"] = c["arrival_us"] // 50
+    a = _arrays(c, kind == "twice")
+    kw = dict(load_init=init, **(dict(model=model) if form == "load" else {}))
+    _same(_call(c, a, form, 0, **kw), _call(c, a, form, pad, **kw))
