@@ -122,3 +122,19 @@ def test_corrupted_index(D, shuffled, entry, at):
     # in chain order the lists wrap at `at`, so that the scan looks that block up there too
     assert host(M).tolist() == [[at] * D]
     assert int(st.item()) == netkv.NETKV_DEV_EFULL
+
+
+@pytest.mark.parametrize("D", [17, 32, 33, 64])
+@pytest.mark.parametrize("spread", [1, 3, 6, 7, 20, 64, 400])
+def test_misses_of_many_decodes(D, spread):
+    """First misses of a pool over `spread` blocks: of a few decodes, and of more than take a vote
+    each, at one block or many, before, across and after the ends of 32 and 128 blocks."""
+    rng = np.random.default_rng(D * 1000 + spread)
+    root = _hashes(rng, 700)
+    chains = [np.concatenate([root[:k], _hashes(rng, 2)]) for k in (0, 5, 31, 32, 100, 300, 700)]
+    for base in (0, 27, 120):
+        caches = [np.concatenate([root[:base + int(rng.integers(0, spread))], _hashes(rng, 3)])
+                  for _ in range(D)]
+        M, want, status, _ = _prefix_case(chains, [caches], D, [len(chains)])
+        assert status == 0
+        np.testing.assert_array_equal(M, want)
