@@ -1163,18 +1163,39 @@ __global__ void __launch_bounds__(kDirectBlock, 16) match_kernel(
   }
 }
 
+// One group of a member walked on from block lcp, at run position `pos`: the decodes whose
+// leader's hit (ml) reaches lcp go on, the others keep it.  32 blocks a step: few groups come
+// here, and the member pass needs its registers for the rows.
+__device__ __forceinline__ void scan_member(IndexView ix, uint32_t log2_cap,
+                                         const uint64_t* __restrict__ chain, uint32_t lcp,
+                                         uint32_t n, unsigned long long pos,
+                                         const uint16_t* __restrict__ ml,
+                                         uint16_t* __restrict__ mr, uint32_t ng, int* status) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t mlo = lane < ng ? (uint32_t)__ldg(ml + lane) : 0u;
+  const uint32_t mhi = lane + 32 < ng ? (uint32_t)__ldg(ml + lane + 32) : 0u;
+  GroupHits h;
+  h.lo = mlo < lcp ? mlo : n;
+  h.hi = mhi < lcp ? mhi : n;
+  const uint32_t alo = __ballot_sync(0xffffffffu, lane < ng && mlo >= lcp);
+  const uint32_t ahi = __ballot_sync(0xffffffffu, lane + 32 < ng && mhi >= lcp);
+  const unsigned long long alive = (unsigned long long)alo | ((unsigned long long)ahi << 32);
+  scan_chain<1, 8>(ix, log2_cap, chain, lcp, n, alive, h, lane, status, pos);
+  store_hits(mr, 0, 0, ng, lane, h);
+}
+
 // Member pass: one warp per member.  With lcp = |common prefix of h_r and h_L|, every decode
 // has M_r[d] = min(M_L[d], lcp) unless M_L[d] >= lcp and block lcp of h_r is cached on d.  So
 // the member's row is one elementwise pass over the leader's row (16 bytes a lane when the
 // rows are 16-byte aligned), and block lcp is then probed in the groups where some leader
 // hit reaches lcp, up to 32 groups at once with one lane per group; a group whose probe
 // finds the block is walked again by the whole warp.
-// Bound by the rows it writes: 32,000 requests on 4,096 decodes 143 us, 8,192 on 1,024 15 us.
-// With only the first run's length known, whose end most members share with their leader, both
-// chains were read on from there: 164 and 47 us, and 778 against 36 with the chains in host
-// memory.  With leaders chosen
-// by chain length, the members whose cached prefix ran past their leader's walked all 64
-// groups of the pool again: 3.9 ms (6.6 ms at 32 blocks a step).
+// Bound by the rows it writes: 32,000 requests on 4,096 decodes 100 us, 8,192 on 1,024 11 us
+// (147 and 14 with one row chunk a lane in flight and groups noted one by one).  With only the
+// first run's length known, whose end most members share with their leader, both chains were
+// read on from there: 164 and 47 us, and 778 against 36 with the chains in host memory.  With
+// leaders chosen by chain length, the members whose cached prefix ran past their leader's walked
+// all 64 groups of the pool again: 3.9 ms (6.6 ms at 32 blocks a step).
 __global__ void __launch_bounds__(kMatchBlock, 4) match_members_wide_kernel(
     const void* __restrict__ index, uint32_t D, uint32_t log2_cap, uint32_t n_sets,
     const uint64_t* __restrict__ chains, const uint64_t* __restrict__ chain_off, uint32_t R,
@@ -1246,82 +1267,70 @@ __global__ void __launch_bounds__(kMatchBlock, 4) match_members_wide_kernel(
         }
       }
     }
-    const bool probe = lcp < n;  // decodes with M_L >= lcp may hit block lcp
-
-    uint32_t pend_q = 0;  // lane j: the j-th group waiting for its probe of block lcp
-    uint32_t n_pend = 0;
-    auto flush = [&]() {
-      __syncwarp();
+    // M_r = min(M_L, lcp), 32 groups at a time; where a leader hit reaches lcp (bit j of `reached`:
+    // group g0 + j), block lcp is then looked up, a group a lane
+    const uint32_t lcp_u = (uint32_t)lcp, lcp2 = lcp_u | (lcp_u << 16);
+    for (uint32_t g0 = 0; g0 < n_dgroups; g0 += 32) {
+      uint32_t reached = 0;
+      if (vec) {
+#pragma unroll
+        for (uint32_t k0 = 0; k0 < 8; k0 += 4) {  // 256 decodes = 4 groups each
+          if (g0 + 4 * k0 >= n_dgroups) break;
+          uint4 x[4];
+#pragma unroll
+          for (uint32_t k = 0; k < 4; ++k) {
+            const uint32_t c = 8 * g0 + 32 * (k0 + k) + lane;
+            x[k] = make_uint4(0u, 0u, 0u, 0u);
+            if (c < n8) x[k] = __ldg(reinterpret_cast<const uint4*>(ml) + c);
+          }
+#pragma unroll
+          for (uint32_t k = 0; k < 4; ++k) {
+            const uint32_t c = 8 * g0 + 32 * (k0 + k) + lane;
+            const uint32_t m2 = __vmaxu2(__vmaxu2(x[k].x, x[k].y), __vmaxu2(x[k].z, x[k].w));
+            const bool reach = c < n8 && max(m2 & 0xffffu, m2 >> 16) >= lcp_u;
+            if (c < n8)
+              reinterpret_cast<uint4*>(mr)[c] =
+                  make_uint4(__vminu2(x[k].x, lcp2), __vminu2(x[k].y, lcp2),
+                             __vminu2(x[k].z, lcp2), __vminu2(x[k].w, lcp2));
+            // lanes 8 q .. 8 q + 7 hold the q-th of the four groups
+            const uint32_t fb = __ballot_sync(0xffffffffu, reach);
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q)
+              reached |= ((fb >> (8 * q)) & 0xffu) ? 1u << (4 * (k0 + k) + q) : 0u;
+          }
+        }
+      } else {
+        for (uint32_t q = g0; q < min(n_dgroups, g0 + 32); ++q) {
+          const uint32_t q0 = q * kGroup, ng = min(kGroup, D - q0);
+          const uint32_t mlo = lane < ng ? (uint32_t)__ldg(ml + q0 + lane) : 0u;
+          const uint32_t mhi = lane + 32 < ng ? (uint32_t)__ldg(ml + q0 + lane + 32) : 0u;
+          GroupHits h;
+          h.lo = min(mlo, lcp_u);
+          h.hi = min(mhi, lcp_u);
+          store_hits(M, row, q0, ng, lane, h);
+          const bool reach = (lane < ng && mlo >= lcp_u) || (lane + 32 < ng && mhi >= lcp_u);
+          if (__any_sync(0xffffffffu, reach)) reached |= 1u << (q - g0);
+        }
+      }
+      if (lcp >= n || !reached) continue;  // decodes with M_L >= lcp may hit block lcp
       unsigned long long pos = kNotFound;
-      if (lane < n_pend) {
+      if ((reached >> lane) & 1u) {
         const uint64_t key = __ldg(own + lcp);
         if (key == 0ull) flag_status(status, NETKV_DEV_EDOMAIN);
-        else pos = lookup(index_view(index, (uint64_t)set * n_dgroups + pend_q, log2_cap, 8u).hash,
+        else pos = lookup(index_view(index, (uint64_t)set * n_dgroups + g0 + lane, log2_cap, 8u).hash,
                           key, log2_cap, status);
       }
-      uint32_t hit = __ballot_sync(0xffffffffu, lane < n_pend && pos != kNotFound);
+      uint32_t hit = __ballot_sync(0xffffffffu, pos != kNotFound);
       while (hit) {
-        const uint32_t j = __ffs(hit) - 1;
+        const uint32_t j = __ffs(hit) - 1, q = g0 + j;
         hit &= hit - 1;
-        const uint32_t q = __shfl_sync(0xffffffffu, pend_q, j);
         const unsigned long long pj = __shfl_sync(0xffffffffu, pos, j);
-        const uint32_t q0 = q * kGroup, ng = min(kGroup, D - q0);
-        const uint32_t mlo = lane < ng ? (uint32_t)__ldg(ml + q0 + lane) : 0u;
-        const uint32_t mhi = lane + 32 < ng ? (uint32_t)__ldg(ml + q0 + lane + 32) : 0u;
-        GroupHits h;
-        h.lo = (uint64_t)mlo < lcp ? mlo : (uint32_t)n;
-        h.hi = (uint64_t)mhi < lcp ? mhi : (uint32_t)n;
-        const uint32_t alo = __ballot_sync(0xffffffffu, lane < ng && (uint64_t)mlo >= lcp);
-        const uint32_t ahi = __ballot_sync(0xffffffffu, lane + 32 < ng && (uint64_t)mhi >= lcp);
-        const unsigned long long alive = (unsigned long long)alo | ((unsigned long long)ahi << 32);
-        scan_chain<4, 8>(index_view(index, (uint64_t)set * n_dgroups + q, log2_cap, 8u),
-                   log2_cap, own, lcp, n, alive, h, lane, status, pj);
-        store_hits(M, row, q0, ng, lane, h);
-      }
-      n_pend = 0;
-    };
-    auto pend = [&](uint32_t q) {
-      if (lane == n_pend) pend_q = q;
-      if (++n_pend == 32) flush();
-    };
-
-    // M_r = min(M_L, lcp); note the groups where a leader hit reaches lcp
-    const uint32_t lcp_u = (uint32_t)lcp;
-    if (vec) {
-      const uint32_t lcp2 = lcp_u | (lcp_u << 16);
-      for (uint32_t c0v = 0; c0v < n8; c0v += 32) {
-        const uint32_t c = c0v + lane;
-        bool reach = false;
-        if (c < n8) {
-          uint4 v = __ldg(reinterpret_cast<const uint4*>(ml) + c);
-          const uint32_t m2 = __vmaxu2(__vmaxu2(v.x, v.y), __vmaxu2(v.z, v.w));
-          reach = max(m2 & 0xffffu, m2 >> 16) >= lcp_u;
-          v.x = __vminu2(v.x, lcp2);
-          v.y = __vminu2(v.y, lcp2);
-          v.z = __vminu2(v.z, lcp2);
-          v.w = __vminu2(v.w, lcp2);
-          reinterpret_cast<uint4*>(mr)[c] = v;
-        }
-        // 8 chunks per group: lanes 8k .. 8k+7 hold group c0v / 8 + k
-        const uint32_t fb = __ballot_sync(0xffffffffu, probe && reach);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if ((fb >> (8 * k)) & 0xffu) pend(c0v / 8u + (uint32_t)k);
-      }
-    } else {
-      for (uint32_t q = 0; q < n_dgroups; ++q) {
-        const uint32_t q0 = q * kGroup, ng = min(kGroup, D - q0);
-        const uint32_t mlo = lane < ng ? (uint32_t)__ldg(ml + q0 + lane) : 0u;
-        const uint32_t mhi = lane + 32 < ng ? (uint32_t)__ldg(ml + q0 + lane + 32) : 0u;
-        GroupHits h;
-        h.lo = min(mlo, lcp_u);
-        h.hi = min(mhi, lcp_u);
-        store_hits(M, row, q0, ng, lane, h);
-        const bool reach = (lane < ng && mlo >= lcp_u) || (lane + 32 < ng && mhi >= lcp_u);
-        if (__any_sync(0xffffffffu, probe && reach)) pend(q);
+        __syncwarp();  // the row's minima are written
+        scan_member(index_view(index, (uint64_t)set * n_dgroups + q, log2_cap, 8u), log2_cap, own,
+                    lcp_u, (uint32_t)n, pj, ml + q * kGroup, mr + q * kGroup,
+                    min(kGroup, D - q * kGroup), status);
       }
     }
-    if (n_pend) flush();
   }
 }
 

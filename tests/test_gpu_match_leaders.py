@@ -25,7 +25,7 @@ def _hashes(rng, n):
 
 
 @pytest.mark.parametrize("first_group", ["deepest", "shallow", "none", "shuffled"])
-@pytest.mark.parametrize("D,copies", [(65, 1), (72, 60), (130, 40)])
+@pytest.mark.parametrize("D,copies", [(65, 1), (72, 60), (130, 40), (2120, 6), (2123, 6)])
 def test_shared_roots(D, copies, first_group):
     """copies = 1: few enough tasks for the direct match; else sharing (more than 4,864
     (request, group) tasks).  The first group caches the roots deepest, to a shallow depth
