@@ -578,8 +578,9 @@ __device__ __forceinline__ unsigned long long lookup_warp(const IndexSlot* __res
 
 // First-miss scan of blocks [start, n) of one chain for the `alive` decodes of a group.
 // Decodes found missing at position p get p; decodes never missing keep their value.
-// A step compares 32 * U chain blocks with the run; where a looked-up block's run ends at
-// once (lists that are not in chain order) the next 32 blocks are looked up side by side.
+// A step compares 32 * U chain blocks with the run; where a looked-up block's run ends at once,
+// or two short ones follow one another (lists that are not in chain order), the next 32 blocks
+// are looked up side by side.
 // start_pos: the run position of block `start` when the caller has already looked it up.
 // n is at most 65,535.  U: a wide step has more loads in flight per warp, but reads up to 32 * U - 1 blocks past
 // the last one needed.  kMB: the run masks' width.
@@ -701,7 +702,7 @@ __device__ __noinline__ SideScan<kMB> scan_side_by_side(const IndexSlot* __restr
     s.p += 32;
     const unsigned long long before = __shfl_up_sync(0xffffffffu, pos, 1);
     const uint32_t follows = __ballot_sync(0xffffffffu, lane > 0 && pos == before + 1);
-    if (__popc(follows) >= 16) {  // in order here
+    if (__popc(follows) == 31) {  // in order here
       s.run = (uint32_t)__shfl_sync(0xffffffffu, pos, 31) + 1;
       return s;
     }
@@ -722,6 +723,7 @@ __device__ __forceinline__ void scan_chain(const IndexView& ix, uint32_t log2_ca
   uint32_t p = start;
   uint32_t run = (uint32_t)min(start_pos, (unsigned long long)cap);  // block p's run position
   bool in_run = start_pos != kNotFound, looked_up = in_run;
+  bool was_short = false;  // the run before had fewer than 32 blocks
   while (p < n && alive) {
     if (!in_run) {
       const uint64_t key = __ldg(chain + p);
@@ -793,11 +795,13 @@ __device__ __forceinline__ void scan_chain(const IndexView& ix, uint32_t log2_ca
       miss_all(h, lane, alive, p);
       return;
     }
-    const bool out_of_order = looked_up && lead < 3;
+    // a run that ends at once, or two short ones: the lists are not in chain order here
+    const bool out_of_order = looked_up && (lead < 3 || (was_short && lead < 32u));
     looked_up = false;
     p += lead;
     run += lead;
     in_run = lead == 32u * U;  // else the run parts here: look the next block up
+    was_short = lead < 32u;
     if (out_of_order) {
       const SideScan<kMB> s = scan_side_by_side<kMB>(ix.hash, ix.keys, ix.masks, chain, n,
                                                      log2_cap, SideScan<kMB>{h, alive, p, run},
@@ -1102,8 +1106,10 @@ __global__ void __launch_bounds__(kMatchBlock, 2) match_leaders_kernel(
 // a grouping and a leader pass, took 1.38 ms there, 130 us against 14 for 1,000 requests,
 // 37 against 4 for one, and 1.20 ms against 0.60 for 32,000 requests whose chains lie in
 // host memory, where the leader's chain crosses the link for every member.  Steps of 64 and
-// 96 blocks: 1.10 and 1.01 ms; 24 blocks an SM (40 registers): spills, no faster.
-
+// 96 blocks: 1.39 and 1.18 ms (in host memory 0.59 and 0.58); 32 blocks first: 1.26 ms; 24
+// blocks an SM (40 registers): spills, no faster.  Many requests on shallow caches of 33 .. 64
+// decodes still favour the grouping: 64,000 requests whose hits end within 1,024 blocks 197 us
+// against 125, within 16 101 against 93.
 template <int kMB>
 __global__ void __launch_bounds__(kDirectBlock, 16) match_kernel(
     const void* __restrict__ index, uint32_t D, uint32_t log2_cap, uint32_t n_sets,

@@ -27,7 +27,7 @@ def _hashes(rng, n):
 EDGES = [0, 1, 2, 3, 31, 32, 33, 127, 128, 129, 130, 255, 256, 257, 383, 384, 385, 640]
 
 
-@pytest.mark.parametrize("order", ["chain", "shuffled", "both"])
+@pytest.mark.parametrize("order", ["chain", "shuffled", "both", "runs of 4", "runs of 16"])
 @pytest.mark.parametrize("D", [1, 8, 9, 16, 17, 32, 33, 64])
 def test_step_edges(D, order):
     rng = np.random.default_rng(D)
@@ -41,6 +41,9 @@ def test_step_edges(D, order):
             keys = rng.permutation(keys)
         elif order == "both":  # in order, out of order, in order again
             keys[100:200] = rng.permutation(keys[100:200])
+        elif order.startswith("runs"):
+            k = int(order[8:])
+            keys = np.concatenate([keys[k * i:k * i + k] for i in rng.permutation(-(-len(keys) // k))])
         caches.append(keys)
     M, want, status, _ = _prefix_case(chains, [caches], D, [len(chains)])
     assert status == 0
