@@ -696,12 +696,6 @@ __global__ void __launch_bounds__(BT, BT >= 256 ? 512 / BT : 1024 / BT)
   const ModelShared S(smem, a.lay);
   const uint64_t e0 = a.event_off[stream], e1 = a.event_off[stream + 1];
   const uint64_t n_win = e1 > e0 ? (e1 - e0 + win - 1) / win : 0;
-  if (threadIdx.x >= 32) {
-    produce<kWalk, BT>(a, w, S, e0, e1, n_win);
-    return;
-  }
-
-  // ---- the walker: lane i takes decodes 2 i, 2 i + 1, 2 i + 64, ...
   int32_t* s_wd = reinterpret_cast<int32_t*>(smem + a.lay.wd);          // [2][kMaxWindow]
   uint32_t* s_wmiss = reinterpret_cast<uint32_t*>(smem + a.lay.wmiss);  // [2][kMaxWindow]
   uint32_t* s_wb = reinterpret_cast<uint32_t*>(smem + a.lay.wb);
@@ -736,7 +730,7 @@ __global__ void __launch_bounds__(BT, BT >= 256 ? 512 / BT : 1024 / BT)
       s_hl[d] = hl_of_load(ld);
     }
   };
-  for (uint32_t d = lane; d < D; d += 32) {
+  for (uint32_t d = threadIdx.x; d < D; d += BT) {  // the initial state, by the whole block
     int64_t x = kWalk == kModel ? a.lm.m0 : 0;
     if (a.state_init) x = a.state_init[(uint64_t)stream * D + d];
     s_state[d] = x;
@@ -751,11 +745,17 @@ __global__ void __launch_bounds__(BT, BT >= 256 ? 512 / BT : 1024 / BT)
       s_hl[d] = hl_of_load(x);
     }
   }
-  Completions<false> done_at;
-  if (lane == 0 && (D & 1u)) s_hl[D] = make_uint2(0u, 0u);  // the padding fits nothing
+  if (threadIdx.x == 0 && (D & 1u)) s_hl[D] = make_uint2(0u, 0u);  // the padding fits nothing
   if (kWalk == kContend)
-    for (uint32_t p = lane; p < t.P; p += 32) S.cnt[p] = 0u;
-  __syncwarp();
+    for (uint32_t p = threadIdx.x; p < t.P; p += BT) S.cnt[p] = 0u;
+  __syncthreads();
+  if (threadIdx.x >= 32) {
+    produce<kWalk, BT>(a, w, S, e0, e1, n_win);
+    return;
+  }
+
+  // ---- the walker: lane i takes decodes 2 i, 2 i + 1, 2 i + 64, ...
+  Completions<false> done_at;
   for (uint64_t k = 0; k <= n_win; ++k) {
     if (k > 0) {
       const uint32_t buf = (uint32_t)((k - 1) & 1);
