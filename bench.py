@@ -565,6 +565,15 @@ def match_launches(sc, R: int, dev) -> int:
     return 4 if sc.share_prefixes and sc.D > 64 and tasks > resident else 1
 
 
+def list_launches(sc, R: int, n_streams: int, dev) -> int:
+    """Kernels of the candidate lists of a plain greedy with its full workspace: pools of 1,025 ..
+    4,096 decodes with more than 8 requests a stream; one for up to 8 requests an SM, else two."""
+    import torch
+    if not (1025 <= sc.D <= 4096 and R > 8 * n_streams):
+        return 0
+    return 1 if R <= 8 * torch.cuda.get_device_properties(dev).multi_processor_count else 2
+
+
 def run_netkv(args):
     import torch
     import synth
@@ -632,12 +641,13 @@ def run_netkv(args):
 
     R, D = x.R, sc.D
     # level bottlenecks 1; prefix match 4 (group scan, group resolve, leaders, members) or 1;
-    # greedy 2 (base scores + walk) with a workspace, 4 for pools of 1,025 .. 4,096 decodes
-    # (base scores, chunk lists, list merge, listed walk), or 1
+    # greedy 2 (base scores + walk) with a workspace, with candidate lists the launches that
+    # write them besides, or 1
     plain_greedy = not (sc.inflight_cap > 0 or sc.load_model is not None)
-    listed = plain_greedy and sc.precompute_scores and 1025 <= sc.D <= 4096
+    lists = (list_launches(sc, R, x.n_streams, dev) if plain_greedy and sc.precompute_scores else 0)
+    listed = lists > 0
     launches_per_step = (0 if fused else 1) + match_launches(sc, R, dev) + (
-        1 if not plain_greedy else (4 if listed else 2) if sc.precompute_scores else 1)
+        1 if not plain_greedy else 2 + lists if sc.precompute_scores else 1)
     decisions = R * world
     value = decisions / (ms / 1e3)
 

@@ -204,9 +204,9 @@ static netkv_status oracle_build(netkv_topology_t topo, const float* d_util, con
   // Thread columns to cover D four decodes a thread, at most 256; then the prefill ranks are
   // split until the card has kBlocksPerSm blocks an SM.  A block's set-up (16 gathers
   // and divisions a thread) is worth at least kMinRows prefill ranks per thread row.
-  // 2,048 x 8,192 pairs with UB (kernel time): one snapshot, 21.2 us (24.5 us at 3 blocks
-  // resident an SM; 491 us as 8 blocks of all prefill ranks); 32 snapshots, 323 us = 6.65
-  // TB/s (528 us as 256 blocks; 387 us at 4 blocks an SM).
+  // 2,048 x 8,192 pairs with UB (kernel time): one snapshot 20.8 us (491 us as 8 blocks of all
+  // prefill ranks); 32 snapshots, in the two-row form, 324 us (528 us as 256 blocks; 387 us with
+  // 4 blocks an SM wanted), in the deep form that they take 310 us = 6.9 TB/s of writes.
   constexpr uint32_t kBlocksPerSm = 16, kMinRows = 16;
   uint32_t log2_tx = 0;
   while (log2_tx < 8 && (uint32_t)kPerThread << log2_tx < t.D) ++log2_tx;

@@ -1060,7 +1060,7 @@ __device__ __forceinline__ void store_hits(uint16_t* __restrict__ M, uint64_t ro
 // Leader pass: one task per (leader, decode group), taken in order from a global counter
 // by whole warps, so long and short chains balance across the GPU.  Bound by the dependent
 // steps of the longest chains, so steps are 256 blocks: 8 leaders x 16 groups of up to 7,680
-// blocks 57 us (69 at 128 a step), 50 leaders x 64 groups 93 us.  A block of 8 warps per long
+// blocks 57 us (69 at 128 a step), 50 leaders x 64 groups 97 us.  A block of 8 warps per long
 // leader, 1,024 blocks a step: 58 and 209 us.
 __global__ void __launch_bounds__(kMatchBlock, 2) match_leaders_kernel(
     const void* __restrict__ index, uint32_t D, uint32_t log2_cap, uint32_t n_sets,

@@ -157,8 +157,8 @@ struct DoneHeap {
 
 }  // namespace
 
-// The walks with producers (schedule_model.cu); false when the pool or its tables do not fit:
-// nothing is launched.
+// The walks with producers (schedule_model.cu); false when the pool or its tables do not fit, or
+// another walk serves so many streams faster: nothing is launched.
 bool launch_model_plain(const TopoArgs& t, uint32_t n_streams, const netkv_weights* d_w,
                         uint32_t R, const uint32_t* d_len, const uint32_t* d_prefill,
                         const uint32_t* d_snap, uint32_t n_snap, const uint32_t* d_events,
