@@ -976,7 +976,7 @@ bool walk_pays(uint32_t D, uint32_t n_streams, uint32_t sms) {
   if (kWalk == kPlain) return D <= 512 || (pool <= 512u * 1024u && per_sm <= (D <= 800 ? 4u : 2u));
   if (D > 96 && pool > 256u * 1024u) return false;
   if (kWalk == kContend) {
-    if (D <= 16) return per_sm <= 20;
+    if (D <= 16) return per_sm <= (D <= 8 ? 28u : 20u);
     return D <= 64 || per_sm <= (D <= 128 ? 4u : 2u);
   }
   if (D <= 32) return per_sm <= (D <= 8 ? 32u : D <= 16 ? 16u : 8u);

@@ -253,7 +253,7 @@ FLEETS = {
                  ((1, 1, 33, 2), 33, 400), ((1, 1, 33, 2), 33, 1300), ((1, 1, 64, 2), 64, 700),
                  ((1, 1, 96, 2), 96, 400), ((1, 1, 97, 2), 97, 280),
                  # past the rule: the per-event walks
-                 ((1, 1, 3, 2), 3, 3100), ((2, 2, 2, 2), 8, 3100), ((2, 2, 2, 4), 16, 3100),
+                 ((1, 1, 3, 2), 3, 4300), ((2, 2, 2, 2), 8, 4300), ((2, 2, 2, 4), 16, 3100),
                  ((1, 1, 65, 2), 65, 700), ((1, 1, 129, 2), 129, 400)],
     "load": [((1, 1, 3, 2), 3, 700), ((2, 2, 2, 2), 8, 1300), ((2, 2, 2, 4), 16, 700),
              ((2, 2, 4, 4), 32, 700), ((1, 1, 33, 2), 33, 400), ((1, 1, 65, 2), 65, 1300),
