@@ -1409,16 +1409,16 @@ netkv_status launch_match(const void* index, uint32_t D, uint32_t log2_cap, uint
 
 // Whether a call's indices are built by one block each.  Few of them: one list after another
 // takes 3 us a list or more, the passes about 45 us for their launches (us, one block / passes;
-// 1 index of 8 lists: 16 keys each 34 / 46, 1,000 55 / 57, 2,000 92 / 61; 16 lists of 16 41 /
+// 1 index of 8 lists of 16 keys 34 / 46, of 500 35 / 53, of 2,000 92 / 61; 16 lists of 16 41 /
 // 53, of 500 74 / 58).  Many: the blocks fill the card, and the passes go over the slots four
-// times (152 indices of 8 lists with shared prefixes: 2,000 keys each 124 / 179, 8,000 566 /
-// 569, 50,000 3,858 / 1,662; 16 lists of 2,000 245 / 310, of 8,000 1,216 / 817; 608 of 32 lists
-// of 500 448 / 570, of 2,000 1,753 / 2,038).  Lists that share nothing favour one block also
-// beyond (300 indices of 8 lists of 50,000: 7,925 / 9,981), which the host cannot see.
+// times (256 indices of 8 lists: 1,000 keys each 68 / 114, 2,000 137 / 184, 10,000 968 / 672;
+// of 16 lists: 1,000 121 / 155, 2,000 237 / 244, 10,000 1,916 / 911).  Larger lists that share
+// nothing favour one block too (300 indices of 8 lists of 50,000: 7,925 / 9,981), but the host
+// cannot tell them from lists with shared prefixes.
 bool serial_build(uint64_t n_index, uint32_t D, uint32_t log2_cap, uint32_t sms) {
   const uint32_t lists = D < kGroup ? D : kGroup;
-  if ((lists <= 12 && log2_cap <= 14) || (lists <= 16 && log2_cap <= 11)) return true;
-  return 2 * n_index >= sms && lists <= 32 && log2_cap <= 17;
+  if ((lists <= 12 && log2_cap <= 13) || (lists <= 16 && log2_cap <= 11)) return true;
+  return 2 * n_index >= sms && (lists <= 12 ? log2_cap <= 14 : lists <= 32 && log2_cap <= 13);
 }
 
 }  // namespace

@@ -4,7 +4,7 @@ first appearance in the lists, with the mask of the decodes that list it, and ze
 the last run position.  The cases reach the edges of the build's passes: lists around the
 256 elements of a count, mask widths of 1, 2, 4 and 8 bytes, lists too long for the bitmap
 and tables too full for the counts (both built by one block per index).  Calls on few lists of
-up to 2^14 slots, and on many indices of up to 2^17, are built by one block per index too: the
+up to 2^13 slots, and on many indices of up to 2^14, are built by one block per index too: the
 edges of the passes are reached with 17 decodes."""
 import numpy as np
 import pytest
@@ -75,8 +75,10 @@ CASES = {
     "17: counts past the keys": (_among(np.arange(1, 1023), 17), 17, 10, "any"),
     "17: full table": (_among(np.arange(1, 1025), 17), 17, 10, "any"),
     # around the rule
-    "12 decodes of 2^14": (_prefix_lists(10, 12, 900), 12, 14, "ranked"),
-    "12 decodes of 2^15": (_prefix_lists(11, 12, 900), 12, 15, "ranked"),
+    "12 decodes of 2^13": (_prefix_lists(10, 12, 900), 12, 13, "ranked"),
+    "12 decodes of 2^14": (_prefix_lists(11, 12, 900), 12, 14, "ranked"),
+    "80 sets of 12 of 2^14": (_prefix_lists(18, 960, 20), 12, 14, "ranked"),
+    "80 sets of 12 of 2^15": (_prefix_lists(19, 960, 20), 12, 15, "ranked"),
     "16 decodes of 2^11": (_prefix_lists(16, 16, 200), 16, 11, "ranked"),
     "16 decodes of 2^12": (_prefix_lists(17, 16, 200), 16, 12, "ranked"),
     "300 sets of 3": (_prefix_lists(12, 900, 60), 3, 9, "ranked"),
