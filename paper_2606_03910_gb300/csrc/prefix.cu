@@ -576,15 +576,6 @@ __device__ __forceinline__ unsigned long long lookup_warp(const IndexSlot* __res
   return kNotFound;
 }
 
-// First-miss scan of blocks [start, n) of one chain for the `alive` decodes of a group.
-// Decodes found missing at position p get p; decodes never missing keep their value.
-// A step compares 32 * U chain blocks with the run; where a looked-up block's run ends at
-// once (lists that are not in chain order) the next 32 blocks are looked up side by side.  (Two
-// runs of fewer than 32 blocks in a row taken for lists out of order: pieces of 4 blocks 2,095
-// -> 592 us, but lists of a dozen decodes in order, whose depths lie that close, 13.1 -> 16.1.)
-// start_pos: the run position of block `start` when the caller has already looked it up.
-// n is at most 65,535.  U: a wide step has more loads in flight per warp, but reads up to 32 * U - 1 blocks past
-// the last one needed.  kMB: the run masks' width.
 template <int kMB>  // masks of at most 32 decodes are reduced as one word
 using DecodeMask = std::conditional_t<kMB == 8, unsigned long long, uint32_t>;
 
@@ -600,8 +591,10 @@ __device__ __forceinline__ Mask warp_or(Mask m) {
 // The decodes of nm[u] miss block p + 32 u + lane: the first miss of each counts, and the
 // decode leaves `alive`.  A few decodes take a vote each per 32 blocks; more are settled by the
 // blocks where some decode misses first (a prefix OR over the lanes), of which there are at most
-// as many.  32,000 requests on 64 decodes whose hits end within 16 blocks: 53 us, 161 with votes
-// over all blocks, 105 with votes over the 32 of the miss.
+// as many.  32,000 requests on 64 decodes whose hits end within 16 blocks: 59 us, 161 with votes
+// over all blocks, 105 with votes over the 32 of the miss.  Up to 8 that miss in one step vote
+// over all its blocks: 57 us from 3 up instead, but 24 streams of 4 requests on 42 decodes 20.8
+// -> 21.4.
 constexpr int kVotes = 6;
 template <bool kMany, int N, typename Mask>
 __device__ __forceinline__ void settle(const Mask (&nm)[N], uint32_t p, GroupHits& h, Mask& alive,
@@ -611,7 +604,7 @@ __device__ __forceinline__ void settle(const Mask (&nm)[N], uint32_t p, GroupHit
   for (int u = 1; u < N; ++u) m |= nm[u];
   Mask a = warp_or(m);
   if (!a) return;  // usually
-  if (!kMany || (N > 1 && __popcll((unsigned long long)a) <= 3)) {  // over all blocks at once
+  if (!kMany || (N > 1 && __popcll((unsigned long long)a) <= 8)) {  // over all blocks at once
     alive &= ~a;
     while (a) {
       const uint32_t j = __ffsll((long long)a) - 1;
@@ -712,6 +705,15 @@ __device__ __noinline__ SideScan<kMB> scan_side_by_side(const IndexSlot* __restr
   return s;
 }
 
+// First-miss scan of blocks [start, n) of one chain for the `alive` decodes of a group; n is at
+// most 65,535.  Decodes found missing at position p get p; decodes never missing keep their
+// value.  start_pos: the run position of block `start` when the caller has already looked it up.
+// kMB: the run masks' width.  U: a step compares 32 * U chain blocks with the run; a wide step
+// has more loads in flight per warp, but reads up to 32 * U - 1 blocks past the last one needed.
+// Where a looked-up block's run ends at once (lists that are not in chain order) the next 32
+// blocks are looked up side by side.  (Two runs of fewer than 32 blocks in a row taken for lists
+// out of order: pieces of 4 blocks 2,105 -> 592 us, but lists of a dozen decodes in order, whose
+// depths lie that close, 13.1 -> 16.1.)
 template <int U, int kMB>
 __device__ __forceinline__ void scan_chain(const IndexView& ix, uint32_t log2_cap,
                                            const uint64_t* __restrict__ chain, uint32_t start,
@@ -1106,7 +1108,7 @@ __global__ void __launch_bounds__(kMatchBlock, 2) match_leaders_kernel(
 // host memory, where the leader's chain crosses the link for every member.  Steps of 64 and
 // 96 blocks: 1.39 and 1.18 ms (in host memory 0.59 and 0.58); 32 blocks first: 1.26 ms; 24
 // blocks an SM (40 registers): spills, no faster.  Many requests on shallow caches of 33 .. 64
-// decodes still favour the grouping: 64,000 requests whose hits end within 1,024 blocks 197 us
+// decodes still favour the grouping: 64,000 requests whose hits end within 1,024 blocks 202 us
 // against 125, within 16 101 against 93.
 template <int kMB>
 __global__ void __launch_bounds__(kDirectBlock, 16) match_kernel(
@@ -1168,8 +1170,8 @@ __global__ void __launch_bounds__(kDirectBlock, 16) match_kernel(
 }
 
 // One group of a member walked on from block lcp, at run position `pos`: the decodes whose
-// leader's hit (ml) reaches lcp go on, the others keep it.  32 blocks a step: few groups come
-// here, and the member pass needs its registers for the rows.
+// leader's hit (ml) reaches lcp go on, the others keep it.  (32 blocks a step instead of 128:
+// 32,000 requests of 1,024 blocks on deep caches of 4,096 decodes 435 us, now 322.)
 __device__ __forceinline__ void scan_member(IndexView ix, uint32_t log2_cap,
                                          const uint64_t* __restrict__ chain, uint32_t lcp,
                                          uint32_t n, unsigned long long pos,
@@ -1184,7 +1186,7 @@ __device__ __forceinline__ void scan_member(IndexView ix, uint32_t log2_cap,
   const uint32_t alo = __ballot_sync(0xffffffffu, lane < ng && mlo >= lcp);
   const uint32_t ahi = __ballot_sync(0xffffffffu, lane + 32 < ng && mhi >= lcp);
   const unsigned long long alive = (unsigned long long)alo | ((unsigned long long)ahi << 32);
-  scan_chain<1, 8>(ix, log2_cap, chain, lcp, n, alive, h, lane, status, pos);
+  scan_chain<4, 8>(ix, log2_cap, chain, lcp, n, alive, h, lane, status, pos);
   store_hits(mr, 0, 0, ng, lane, h);
 }
 
