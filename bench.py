@@ -228,10 +228,10 @@ KERNEL_CODE = {
 #   prefix_match: bytes per request, from the 64-replica case of the bench workload
 #   oracle_build: bytes per snapshot of the oracle-build sweep
 MEASURED_TRAFFIC = {
-    # 64 replicas (64,000 requests): match_kernel 303.21 MB read, 3.16 MB written
-    "prefix_match": {"code_sha256_16": "c43f7fc61fbdb936", "bytes_per_unit": 306_365_440 / 64_000,
+    # 64 replicas (64,000 requests): match_kernel 303.19 MB read, 3.17 MB written
+    "prefix_match": {"code_sha256_16": "89de750ed1f7b274", "bytes_per_unit": 306_365_184 / 64_000,
                      "unit": "request", "captured": "64-replica case, one launch per kernel"},
-    "oracle_build": {"code_sha256_16": "05d89616909d4baa", "bytes_per_unit": 67_161_251,
+    "oracle_build": {"code_sha256_16": "0fe7069cea46de05", "bytes_per_unit": 67_161_251,
                      "unit": "snapshot", "captured": "1,000-snapshot sweep, one launch"},
 }
 

@@ -358,7 +358,8 @@ __device__ __forceinline__ void list_chunk(const float* __restrict__ row, uint32
 
 // The list and bound of each chunk of up to 1,024 decodes of an arrival's base-score row.  A
 // warp takes an event of a stream (departures cost it one load) and the chunks of its row one
-// after another, so a call lists the requests that arrive in it, not all R.  Lane L holds decodes 128 q + 4 L .. + 3 of a chunk, q = 0 .. 7.
+// after another, so a call lists the requests that arrive in it, not all R.  Lane L holds
+// decodes 128 q + 4 L .. + 3 of a chunk, q = 0 .. 7.
 // The 32nd smallest of the 64 minima over a lane's even and odd q is a threshold T that at
 // least 32 pairs reach and few are below: 31 minima at most are, about 44 pairs of 1,024
 // distinct scores.  The pairs below T are gathered in shared memory and each is placed by
